@@ -345,9 +345,16 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
     g.P = (int)std::min<long long>(ctx->num_sms - 1, (K + 31) / 32);
   }
   const int sbp = g.sbp, P = g.P;
+  // FP64 X: runs of full steps go to one persistent launch (ca_persist64.cu)
+  // of P64 column CTAs, with two sets of partials
+  const long long nch = (K + 31) / 32;
+  const int P64 = (int)std::min<long long>(ctx->num_sms - 1, nch);
+  bool persist64 = ctx->persist && pb.xfmt == CA_DENSE_F64 && !f64solve && P64 >= 1 &&
+                   persist64_fits(b, sbm);
+  const int Pmax = persist64 ? std::max(P, 2 * P64) : P;
   void* part = g.tc ? (void*)cv.take<float>((size_t)P * sbp * sbp)
-                    : (void*)cv.take<double>((size_t)P * sbp * sbp);
-  double* ppart = cv.take<double>((size_t)P * sbp);
+                    : (void*)cv.take<double>((size_t)Pmax * sbp * sbp);
+  double* ppart = cv.take<double>((size_t)Pmax * sbp);
   double* R = cv.take<double>((size_t)sbp * sbp);
   double* pvec = cv.take<double>((size_t)sbp);
   double* delta2[2] = {cv.take<double>((size_t)sbp), cv.take<double>((size_t)sbp)};
@@ -417,15 +424,62 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
     const int sb = sk * b;
     const int* idx = idx_all + (size_t)s * k * b;
     double* delta = delta2[k & 1];
-    if (pending && (!fuse || due(k - 1))) {
+    // (a persistent FP64 launch applies a pending update itself)
+    const bool fuse_k = fuse || (persist64 && sk == s && k + 1 < n_outer &&
+                                 (long long)s * (k + 2) <= H && !boundary_after(k));
+    if (pending && (!fuse_k || due(k - 1))) {
       CA_TRY(update_alone());                                   // a5 of step k-1 (clears after_rc)
       if (due(k - 1)) CA_TRY(launch_recompute(ctx, pb, pb.v, pb.y0, pb.c0, pb.c1));  // a6
     }
     long long k1 = k + 1;  // end of the run that starts at k
-    if (persist_ok && sk == s)
+    if ((persist_ok || persist64) && sk == s)
       while (k1 < n_outer && (long long)s * (k1 + 1) <= H && !boundary_after(k1 - 1)) ++k1;
     bool persisted = false;
-    if (persist_ok && sk == s && k1 - k >= 2) {
+    if (persist64 && sk == s && k1 - k >= 2) {
+      Persist64Args pa{};
+      pa.A = static_cast<const double*>(pb.A);
+      pa.lda = pb.lda;
+      pa.N = pb.N;
+      pa.K = K;
+      pa.idx_all = idx_all;
+      pa.sb = sb;
+      pa.k0 = k;
+      pa.npass = (int)(k1 - k);
+      pa.prev_idx = pending ? prev_idx : nullptr;
+      pa.prev_sb = pending ? prev_sb : 0;
+      pa.delta2[0] = delta2[0];
+      pa.delta2[1] = delta2[1];
+      pa.v = pb.v;
+      pa.cU = pb.cU;
+      pa.part = static_cast<double*>(part);
+      pa.ppart = ppart;
+      pa.Rs[0] = Rs;
+      pa.Rs[1] = reinterpret_cast<float2*>(R);  // (R itself is not formed here)
+      pa.Ginv[0] = Ginv;
+      pa.Ginv[1] = Ginv + (size_t)sbp * (CA_FAST_B / 2);  // b <= 16
+      pa.pvec = pvec;
+      pa.sa = SolveArgs{nullptr, pb.N, b, s, sb, sbp, pb.cG, pb.cI, pb.cP, pb.cY, pb.x, pb.yv, nullptr};
+      pa.cnt = ctx->d_cnt;
+      CA_TRY_CUDA(cudaMemsetAsync(ctx->d_cnt, 0, 4 * sizeof(unsigned), ctx->stream));
+      prof_mark(ctx, PC_GRAM);
+      const int e = launch_persist64(pa, P64, chain_smem(b, sb), ctx->d_err, ctx->stream);
+      prof_mark(ctx, PC_GRAM);
+      if (e == (int)cudaErrorCooperativeLaunchTooLarge || e == (int)cudaErrorInvalidConfiguration) {
+        (void)cudaGetLastError();  // not resident at once here: the launches per step instead
+        persist64 = false;
+        if (pending) CA_TRY(update_alone());
+      } else if (e != 0) {
+        return cuda_fail((cudaError_t)e, __LINE__);
+      } else {
+        ctx->prof.kernel_launches += 1;
+        persisted = true;
+        k = k1 - 1;  // the last step of the run; its update is pending
+        pending = true;
+        prev_idx = idx_all + (size_t)s * k * b;
+        prev_sb = sb;
+        prev_delta = delta2[k & 1];
+      }
+    } else if (persist_ok && sk == s && k1 - k >= 2) {
       PersistArgs pa{};
       pa.A = static_cast<const float*>(pb.A);
       pa.N = pb.N;

@@ -94,6 +94,42 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   }
 }
 
+// Bounded wait on a count another CTA raises: true once *p >= target; gives
+// up (CA_DEV_ERR_TIMEOUT) after the limit or as soon as another wait of the
+// grid has given up.
+__device__ __forceinline__ bool wait_count(const unsigned* p, unsigned target, unsigned* err) {
+  const uint64_t t0 = ca_globaltimer();
+  for (uint32_t it = 0;; ++it) {
+    if (*(volatile const unsigned*)p >= target) {
+      __threadfence();
+      return true;
+    }
+    if ((it & 63u) == 63u) {
+      if (*(volatile unsigned*)err & CA_DEV_ERR_TIMEOUT) return false;
+      if (ca_globaltimer() - t0 > CA_WAIT_LIMIT_NS) {
+        ca_flag(err, CA_DEV_ERR_TIMEOUT);
+        return false;
+      }
+    }
+  }
+}
+
+// mbarrier wait that also gives up once another wait of the grid has.
+__device__ __forceinline__ bool mbar_wait_grid(uint64_t* bar, uint32_t parity, unsigned* err) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = ca_globaltimer();
+  for (uint32_t it = 1;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 255u) == 0u) {
+      if (*(volatile unsigned*)err & CA_DEV_ERR_TIMEOUT) return false;
+      if (ca_globaltimer() - t0 > CA_WAIT_LIMIT_NS) {
+        ca_flag(err, CA_DEV_ERR_TIMEOUT);
+        return false;
+      }
+    }
+  }
+}
+
 __device__ __forceinline__ void cp_async_16_zfill(uint32_t dst, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes)
                : "memory");

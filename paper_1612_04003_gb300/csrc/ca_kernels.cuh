@@ -136,6 +136,34 @@ int launch_persist(const PersistArgs& a, int grid, int sbp, int mode, unsigned* 
 // Depth of the persistent kernel's load ring (stages in flight per CTA).
 int persist_load_ring(int sbp, int mode);
 
+// Consecutive outer steps k0 .. k0+npass-1 of one dense FP64 solve in one
+// persistent cooperative launch of P column CTAs + 1 chain CTA
+// (ca_persist64.cu).
+struct Persist64Args {
+  const double* A;       // N x K row-major, leading dimension lda
+  long long lda, N, K;
+  const int* idx_all;    // sampled indices: step k at idx_all + k * sb
+  int sb;                // s * b of every step of the launch
+  long long k0;
+  int npass;
+  const int* prev_idx;   // rows of step k0 - 1, update pending (prev_sb = 0: none)
+  int prev_sb;
+  double* delta2[2];     // Delta of step k in delta2[k & 1]
+  double* v;             // K, updated in place
+  double cU;
+  double* part;          // 2 x P x sbp^2 Gram partials (transposed), by step parity
+  double* ppart;         // P x sbp projection partials
+  float2* Rs[2];         // by step parity
+  float2* Ginv[2];
+  double* pvec;
+  SolveArgs sa;          // solve constants (idx and delta are set per step); ldr = sbp
+  unsigned* cnt;         // 4 counts, zero on entry
+};
+bool persist64_fits(int b, int sb);
+// P <= number of SMs - 1 and <= ceil(K / 32).  Returns a cudaError_t.
+int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,
+                     cudaStream_t st);
+
 // Shared launch of P CTAs; sbp = 32, 64 or 128 (>= every problem's s*b).
 int launch_gram_tc_batch(const GramBatchArgs& bt, int P, int sbp, int three_pass, unsigned* err,
                          cudaStream_t stream);

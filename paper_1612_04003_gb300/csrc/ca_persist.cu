@@ -89,42 +89,6 @@ struct PCfg {
   static_assert(kSmem <= 232448, "shared memory");
 };
 
-// Bounded wait on a count another CTA raises: true once *p >= target; gives
-// up (CA_DEV_ERR_TIMEOUT) after the limit or as soon as another wait of the
-// grid has given up.
-__device__ __forceinline__ bool wait_count(const unsigned* p, unsigned target, unsigned* err) {
-  const uint64_t t0 = ca_globaltimer();
-  for (uint32_t it = 0;; ++it) {
-    if (*(volatile const unsigned*)p >= target) {
-      __threadfence();
-      return true;
-    }
-    if ((it & 63u) == 63u) {
-      if (*(volatile unsigned*)err & CA_DEV_ERR_TIMEOUT) return false;
-      if (ca_globaltimer() - t0 > CA_WAIT_LIMIT_NS) {
-        ca_flag(err, CA_DEV_ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-}
-
-// mbarrier wait that also gives up once another wait of the grid has.
-__device__ __forceinline__ bool mbar_wait_grid(uint64_t* bar, uint32_t parity, unsigned* err) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = ca_globaltimer();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 255u) == 0u) {
-      if (*(volatile unsigned*)err & CA_DEV_ERR_TIMEOUT) return false;
-      if (ca_globaltimer() - t0 > CA_WAIT_LIMIT_NS) {
-        ca_flag(err, CA_DEV_ERR_TIMEOUT);
-        return false;
-      }
-    }
-  }
-}
-
 __device__ __forceinline__ uint64_t l2_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));

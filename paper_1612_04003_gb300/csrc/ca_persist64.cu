@@ -1,0 +1,365 @@
+// ca_persist64.cu -- consecutive outer steps of a dense FP64 CA-BCD (Alg. 2) /
+// CA-BDCD (Alg. 4) solve in one persistent, cooperative launch.
+//
+// The Gram of step k+1 needs only the sampled indices, so it is formed and
+// reduced while the chain of step k runs; what depends on Delta_k is the
+// deferred update of v and the projection p_{k+1} = Y_{k+1} v, one sweep over
+// the CTA's own columns.  Grid = P column CTAs + 1 chain CTA, all resident
+// (cooperative launch); every wait is bounded and gives up once any wait of
+// the grid has.
+//   column CTA, step k:  wait Delta_{k-1} -> v -= cU Y_{k-1}^T Delta_{k-1} on
+//     its columns, p partial -> count P  |  Gram partial of step k+1 -> count
+//     G -> all G: its share of the reduction (Rs, inverted diagonal blocks)
+//     -> count R
+//   chain CTA, step k:   counts R and P of step k -> p summed -> the s
+//     dependent solves -> Delta_k -> count D
+// Buffers written ahead (partials, Rs, Ginv) alternate by step parity: the
+// buffers of step k+1 were last read for step k-1, whose Delta this CTA has
+// seen before it writes them.
+//
+// Bound by latency.  X 64 x 1024, b = 4: 10.9 us a step at s = 1 and 14 us at
+// s = 4, against 58 and 62 us with four launches a step and a Gram tile of
+// 64 x 64 FP64 products whatever s b; X^T 1500 x 8190, b = 8, s = 4: 34 us
+// against 107 us.
+#include <algorithm>
+#include <atomic>
+
+#include "ca_kernels.cuh"
+#include "ca_solve.cuh"
+
+namespace {
+
+constexpr int kT = 256;      // threads of a CTA
+constexpr int kSmemMax = 200 * 1024;  // dynamic shared memory a launch may ask for
+constexpr int kSmallSB = 32;  // rows of a step the CUDA-core Gram covers
+
+struct Cnt {  // counts in cnt[]
+  enum { G = 0, R = 1, P = 2, D = 3 };
+};
+
+// thread 0 waits, the CTA follows; false once a wait of the grid gave up
+__device__ __forceinline__ bool cta_wait(const unsigned* p, unsigned target, unsigned* err, bool ok) {
+  int good = ok;
+  if (threadIdx.x == 0 && ok) good = wait_count(p, target, err);
+  return __syncthreads_and(threadIdx.x == 0 ? good : 1) != 0 && ok;
+}
+__device__ __forceinline__ void cta_count(unsigned* p) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(p, 1u);
+  }
+}
+
+// Row offsets of the sampled rows (element offset, -1: out of range, flagged).
+__device__ __forceinline__ void row_offsets(const int* idx, int sb, long long N, long long lda,
+                                            long long* out, unsigned* err) {
+  for (int r = threadIdx.x; r < sb; r += kT) {
+    const long long gi = idx[r];
+    const bool in = gi >= 0 && gi < N;
+    if (!in) ca_flag(err, CA_DEV_ERR_ARG);
+    out[r] = in ? gi * lda : -1;
+  }
+}
+
+// Gram partial of sb <= 32 rows over columns [k0, k1) on CUDA cores: the
+// FP64 pipe does two FMAs a clock and SM, so only the lower triangle is
+// formed.  Warp w takes columns 4 w .. 4 w + 3 of each 32-column tile, lane l
+// the entries l, l + 32, ...; the warps' sums meet in shared memory.
+// smem: tile [sb][33], then sums [8][entries].
+__device__ void gram_small(const double* __restrict__ A, const long long* off, int sb, long long k0,
+                           long long k1, double* sm, double* __restrict__ part, int sbp) {
+  constexpr int kSlots = kSmallSB * (kSmallSB + 1) / 2 / 32 + 1;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int E = sb * (sb + 1) / 2;
+  double* tile = sm;
+  double* red = sm + kSmallSB * 33;
+  int ij[kSlots];
+  double acc[kSlots];
+#pragma unroll
+  for (int q = 0; q < kSlots; ++q) {
+    int i = 0, j = 0;
+    if (lane + 32 * q < E) tri_decode(lane + 32 * q, i, j);
+    ij[q] = i * 33 | (j * 33) << 16;
+    acc[q] = 0.0;
+  }
+  for (long long kt = k0; kt < k1; kt += 32) {
+    __syncthreads();
+    const long long k = kt + lane;
+#pragma unroll
+    for (int q = 0; q < kSmallSB / 8; ++q) {
+      const int r = warp + 8 * q;
+      if (r < sb) tile[r * 33 + lane] = (off[r] >= 0 && k < k1) ? __ldg(A + off[r] + k) : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kSlots; ++q) {
+      if (32 * q < E) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          acc[q] = fma(tile[(ij[q] & 0xffff) + 4 * warp + c], tile[(ij[q] >> 16) + 4 * warp + c], acc[q]);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kSlots; ++q)
+    if (lane + 32 * q < E) red[warp * E + lane + 32 * q] = acc[q];
+  __syncthreads();
+  for (int e = threadIdx.x; e < E; e += kT) {
+    double s = red[e];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += red[w * E + e];
+    int i, j;
+    tri_decode(e, i, j);
+    part[(long long)j * sbp + i] = s;
+  }
+}
+
+// Sum over the warp's 32 lanes of RQ values per lane by halving exchanges (RQ
+// + 5 - log2 RQ additions a lane instead of 5 RQ): returns, on lanes whose low
+// bits are zero, the sum of value q = (lane >> 1's bits, most significant
+// first); lane of value q: see the caller.
+template <int RQ>
+__device__ __forceinline__ double halving_sum(double (&y)[RQ], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int w = RQ / 2; w >= 1; w /= 2, o /= 2) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < w; ++j) {
+      const double keep = up ? y[j + w] : y[j], send = up ? y[j] : y[j + w];
+      y[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+#pragma unroll
+  for (; o >= 1; o /= 2) y[0] += __shfl_xor_sync(0xffffffffu, y[0], o);
+  return y[0];
+}
+
+// v -= cU Yprev^T Delta (psb > 0) and the projection partial p = Y v of the
+// CTA's columns [k0, k1), FP64.  Lane = column of a 32-column tile, warp w the
+// rows w, w + 8, ...; one exchange of the warps' column sums a tile.
+template <int RQ>
+__device__ void update_project(const Persist64Args& a, const long long* off, const long long* poff,
+                               const double* sdl, int sb, int psb, long long k0, long long k1,
+                               double* ured, double* __restrict__ pp) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double pacc[RQ];
+#pragma unroll
+  for (int q = 0; q < RQ; ++q) pacc[q] = 0.0;
+  int par = 0;
+  for (long long kt = k0; kt < k1; kt += 32, par ^= 1) {
+    const long long k = kt + lane;
+    const bool in = k < k1;
+    double y[RQ], u = 0.0;
+#pragma unroll
+    for (int q = 0; q < RQ; ++q) {
+      const int r = warp + 8 * q;
+      y[q] = (r < sb && in && off[r] >= 0) ? __ldg(a.A + off[r] + k) : 0.0;
+    }
+    double vk = in ? a.v[k] : 0.0;
+    if (psb > 0) {
+      double x[RQ];
+#pragma unroll
+      for (int q = 0; q < RQ; ++q) {
+        const int r = warp + 8 * q;
+        x[q] = (r < psb && in && poff[r] >= 0) ? __ldg(a.A + poff[r] + k) : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < RQ; ++q)
+        if (warp + 8 * q < psb) u = fma(x[q], sdl[warp + 8 * q], u);
+      ured[par * 256 + threadIdx.x] = u;
+      __syncthreads();
+      double s = ured[par * 256 + lane];
+#pragma unroll
+      for (int w = 1; w < 8; ++w) s += ured[par * 256 + 32 * w + lane];
+      vk -= a.cU * s;
+      if (warp == 0 && in) a.v[k] = vk;
+    }
+#pragma unroll
+    for (int q = 0; q < RQ; ++q)
+      if (warp + 8 * q < sb) pacc[q] = fma(y[q], vk, pacc[q]);
+  }
+  const double s = halving_sum<RQ>(pacc, lane);
+  constexpr int low = 32 / RQ;  // lanes holding the same sum
+  const int q = lane / low;      // (the exchanges sort the values by the lane's high bits)
+  const int r = warp + 8 * q;
+  if (lane % low == 0 && r < sb) pp[r] = s;
+}
+
+template <int BMAX, int DEPTH, int RQ>
+__global__ void __launch_bounds__(kT, 1) k_persist64(Persist64Args a, unsigned* __restrict__ err) {
+  extern __shared__ double smem_d[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int P = (int)gridDim.x - 1, c = blockIdx.x;
+  const int sb = a.sb, sbp = a.sa.ldr, npass = a.npass;
+  const int b = a.sa.b, s = a.sa.s_cur;
+  const long long sq = (long long)sbp * sbp;
+  bool ok = true;
+
+  if (c == P) {  // ------------------------------------------------ chain CTA
+    for (int p = 0; p < npass; ++p) {
+      const long long k = a.k0 + p;
+      SolveArgs sa = a.sa;
+      sa.idx = a.idx_all + k * sb;
+      sa.delta = a.delta2[k & 1];
+      ok = cta_wait(a.cnt + Cnt::R, (unsigned)(P * (p + 1)), err, ok);
+      ok = cta_wait(a.cnt + Cnt::P, (unsigned)(P * (p + 1)), err, ok);
+      if (!ok) return;
+      // p = sum of the P partials, a warp per row
+      for (int r = warp; r < sb; r += kT / 32) {
+        double t = 0.0;
+        for (int q = lane; q < P; q += 32) t += __ldcg(a.ppart + (long long)q * sbp + r);
+        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) a.pvec[r] = t;
+      }
+      __syncthreads();
+      chain_la_body<BMAX, DEPTH>(a.Rs[k & 1], a.pvec, a.Ginv[k & 1], sa, err, smem_d);
+      cta_count(a.cnt + Cnt::D);
+    }
+    return;
+  }
+
+  // --------------------------------------------------------------- column CTA
+  __shared__ long long soff[2][8 * RQ];
+  __shared__ double sdl[8 * RQ];
+  __shared__ double ured[2 * kT];
+  __shared__ float2 Mb[256];
+  __shared__ float2 colbuf[66];
+  const long long nch = (a.K + 31) / 32;
+  const long long c0 = nch * c / P * 32, c1 = min(a.K, nch * (c + 1) / P * 32);
+  const float2 cG2 = split_f64(a.sa.cG), cI2 = split_f64(a.sa.cI);
+  const int E = sb * (sb + 1) / 2;
+  // Gram partial of step k0 + p into its parity's buffer, then this CTA's
+  // share of the reduction: roles 0 .. s-1 invert a diagonal block, the others
+  // take 64 entries each, four threads an entry
+  auto gram = [&](int p, const long long* off) {
+    const long long k = a.k0 + p;
+    double* part = a.part + (k & 1) * (long long)P * sq;
+    gram_small(a.A, off, sb, c0, c1, smem_d, part + c * sq, sbp);
+    cta_count(a.cnt + Cnt::G);
+    ok = cta_wait(a.cnt + Cnt::G, (unsigned)(P * (p + 1)), err, ok);
+    if (!ok) return;
+    float2* Rs = a.Rs[k & 1];
+    const int nrole = s + (E + 63) / 64;
+    double* red = smem_d;
+    for (int role = c; role < nrole; role += P) {
+      const int ent = tid & 63, sub = tid >> 6;
+      int i = -1, j = 0;
+      if (role < s) {  // entry (i, j) of block `role`, b <= 8; larger b: loop below
+        for (int e0 = 0; e0 < b * b; e0 += 64) {
+          const int e = e0 + ent;
+          i = e / b;
+          j = e - i * b;
+          double t = 0.0;
+          if (e < b * b && i >= j)
+#pragma unroll 8
+            for (int q = sub; q < P; q += 4)
+              t += __ldcg(part + q * sq + (long long)(role * b + j) * sbp + role * b + i);
+          red[tid] = t;
+          __syncthreads();
+          if (tid < 64 && e < b * b && i >= j) {
+            const double g = (red[tid] + red[64 + tid]) + (red[128 + tid] + red[192 + tid]);
+            float2 m = df_mul(cG2, split_f64(g));
+            if (i == j) m = df_add(m, cI2);
+            Mb[i * b + j] = m;
+            Mb[j * b + i] = m;
+          }
+          __syncthreads();
+        }
+        float2* out = a.Ginv[k & 1] + (long long)role * b * b;
+        float2 m[1] = {tid < b * b ? Mb[tid] : make_float2(0.f, 0.f)};
+        if (b <= 8) {
+          if (tid < 64) cta_sweep_inverse<1, 64>(m, b, colbuf, out, err);
+        } else {
+          cta_sweep_inverse<1>(m, b, colbuf, out, err);
+        }
+        __syncthreads();
+        continue;
+      }
+      const int e = (role - s) * 64 + ent;
+      double t = 0.0;
+      if (e < E) {  // column-major over the lower triangle: lanes along i
+        int ir, jr;
+        tri_decode(e, ir, jr);
+        i = sb - 1 - jr;
+        j = sb - 1 - ir;
+#pragma unroll 8
+        for (int q = sub; q < P; q += 4) t += __ldcg(part + q * sq + (long long)j * sbp + i);
+      }
+      red[tid] = t;
+      __syncthreads();
+      if (tid < 64 && e < E)
+        Rs[(long long)j * sbp + i] =
+            df_mul(cG2, split_f64((red[tid] + red[64 + tid]) + (red[128 + tid] + red[192 + tid])));
+      __syncthreads();
+    }
+    cta_count(a.cnt + Cnt::R);
+  };
+
+  row_offsets(a.idx_all + a.k0 * sb, sb, a.N, a.lda, soff[0], err);
+  if (a.prev_sb > 0) row_offsets(a.prev_idx, a.prev_sb, a.N, a.lda, soff[1], err);
+  __syncthreads();
+  gram(0, soff[0]);
+  for (int p = 0; p < npass && ok; ++p) {
+    const long long k = a.k0 + p;
+    const int psb = p == 0 ? a.prev_sb : sb;
+    if (p > 0) ok = cta_wait(a.cnt + Cnt::D, (unsigned)p, err, ok);
+    if (!ok) break;
+    if (psb > 0) {
+      for (int r = tid; r < psb; r += kT) sdl[r] = __ldcg(a.delta2[(k - 1) & 1] + r);
+      __syncthreads();
+    }
+    update_project<RQ>(a, soff[p & 1], soff[(p + 1) & 1], sdl, sb, psb, c0, c1, ured,
+                       a.ppart + (long long)c * sbp);
+    cta_count(a.cnt + Cnt::P);
+    if (p + 1 < npass) {
+      row_offsets(a.idx_all + (k + 1) * sb, sb, a.N, a.lda, soff[(p + 1) & 1], err);
+      __syncthreads();
+      gram(p + 1, soff[(p + 1) & 1]);
+    }
+  }
+}
+
+template <int BMAX, int DEPTH, int RQ>
+int launch_one(const Persist64Args& a, int P, size_t chain_smem, unsigned* err, cudaStream_t st) {
+  const size_t gsm = (kSmallSB * 33 + 8 * (size_t)(kSmallSB * (kSmallSB + 1) / 2)) * 8;
+  const size_t smem = std::max(chain_smem, gsm);
+  if (smem > (size_t)kSmemMax) return (int)cudaErrorInvalidConfiguration;
+  auto kern = k_persist64<BMAX, DEPTH, RQ>;
+  static std::atomic<unsigned long long> configured{0ull};  // devices (a bit each)
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return (int)e;
+  const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;
+  if (!bit || !(configured.load(std::memory_order_acquire) & bit)) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    if (e != cudaSuccess) return (int)e;
+    configured.fetch_or(bit, std::memory_order_release);
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(P + 1);
+  cfg.blockDim = dim3(kT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, kern, a, err);
+  return (int)(e != cudaSuccess ? e : cudaGetLastError());
+}
+
+}  // namespace
+
+// Rows of a step and block sizes the launch covers.
+bool persist64_fits(int b, int sb) { return b <= 16 && sb <= kSmallSB; }
+
+int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,
+                     cudaStream_t st) {
+  const bool small = a.sa.b <= 8;
+  return small ? launch_one<8, 4, 4>(a, P, chain_smem, err, st)
+               : launch_one<16, 3, 4>(a, P, chain_smem, err, st);
+}
