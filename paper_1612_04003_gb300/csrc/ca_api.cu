@@ -222,6 +222,10 @@ GramPlan gram_plan(ca_ctx* ctx, int xfmt, int prec, int sbm, long long K) {
     const int t = g.sbp / 64;
     g.ntiles = t * (t + 1) / 2;
     const long long nchunks = (K + 31) / 32;
+    if (xfmt == CA_DENSE_F64 && sbm <= gram64_max_sb()) {  // k_gram64: a CTA per SM
+      g.P = (int)std::min<long long>(ctx->num_sms, nchunks);
+      return g;
+    }
     long long Pm = std::max(1LL, (long long)(2 * ctx->num_sms) / g.ntiles);
     Pm = std::min(Pm, nchunks);
     const long long cap = std::max(1LL, (long long)((256ull << 20) / ((size_t)g.sbp * g.sbp * 8)));
@@ -247,6 +251,11 @@ int launch_gram(ca_ctx* ctx, const GramPlan& g, int xfmt, const void* A, long lo
                                  static_cast<float*>(part), ppart, ctx->d_err, g.three, ctx->stream,
                                  &none, panel);
     return e == 0 ? CA_OK : CA_ERR_CUDA;
+  }
+  if (xfmt == CA_DENSE_F64 && g.chunks_per_split == 0) {
+    const int e = launch_gram64(static_cast<const double*>(A), lda, N, K, idx, sb, v, g.P, g.sbp,
+                                static_cast<double*>(part), ppart, ctx->d_err, ctx->stream);
+    return e == 0 ? CA_OK : cuda_fail((cudaError_t)e, __LINE__);
   }
   launch_gram_simt(xfmt == CA_DENSE_F64, dim3(g.P, g.ntiles), ctx->stream, A, lda, N, K, idx, sb, v,
                    g.chunks_per_split, g.sbp, static_cast<double*>(part), ppart, ctx->d_err);

@@ -1,0 +1,264 @@
+// ca_digits.cuh -- the FP64 Gram Y Y^T of sampled rows on the BF16 tensor
+// cores, by exact digit products (the error-free splitting of Ozaki, Ogita,
+// Oishi and Rump, Numer. Algorithms 59, 2012, with integer digits and FP32
+// accumulation as Mukunoki, Ozaki, Ogita and Imamura, ISC 2020, use it).
+//
+// A segment of at most kSeg columns: every row gets one power of two above its
+// largest magnitude there, each element becomes a 55-bit fixed-point integer
+// (to nearest) and the integer seven signed base-256 digits.  A digit is exact
+// in BF16; so is every product, and the sums of the products of digits i and
+// j with one i + j = l stay below 2^24 (l - 1 pairs of at most 2^14 over kSeg
+// columns, l <= 6), so the FP32 accumulators of the levels l = 2 .. 6 are
+// exact integers.  Levels 7 .. 9 share one accumulator (their FP32 rounding is
+// below 2^-54 of the product of the two rows' largest magnitudes); higher
+// levels are below that and left out.  The levels are put together in 64-bit
+// integers and converted once.  Rows with an infinity, a NaN or a magnitude
+// outside 2^-480 .. 2^490 take the plain FP64 sums instead.
+//
+// Why: the FP64 pipe does two FMAs a clock and SM (1.25 TFLOP/s).  The 34
+// digit products of a 128-row tile and 32 columns take ~4,400 cycles of the
+// tensor pipe where 128 x 129 / 2 x 32 FMAs take 132,000 of the FP64 pipe.
+#pragma once
+#include "ca_common.cuh"
+#include "ca_tc.cuh"
+
+namespace {
+
+constexpr int kSeg = 192;  // columns whose level sums stay exact in FP32
+constexpr int kDigits = 7;
+
+// SBP rows (32, 64 or 128), a CTA of 256 threads.  Tensor memory: one
+// accumulator of SBP columns a level.  SBP = 128 holds four of the six at
+// once: levels 2 .. 5, then (the columns converted again) levels 6 .. 9.
+template <int SBP>
+struct DigitGram {
+  static constexpr int kSlice = SBP * 64;              // 32 BF16 digits a row
+  static constexpr int kStage = kDigits * kSlice;
+  // the M = 128 MMA reads 128 rows of a slice: slack behind the last one
+  static constexpr int kSmem = 2 * kStage + (128 - (SBP < 128 ? SBP : 128)) * 64 + 1024;
+  static constexpr int kTmemCols = SBP == 32 ? 256 : 512;
+
+  unsigned char* dig;   // 1024-byte aligned digits of two stages
+  uint64_t* bars;       // [0], [1]: stage buffer read by the MMAs; [2]: all MMAs
+  uint32_t tmem;
+  int* emax;            // [SBP] largest biased exponent of each row
+  uint32_t gt = 0;      // stages so far (buffers and phases run on)
+  uint32_t ph = 0;      // passes so far
+
+  // one stage of 32 columns: digits 1 .. ND of every row
+  template <int ND>
+  __device__ __forceinline__ void convert(const double* __restrict__ A, const long long* off, int sb,
+                                          long long k, long long k1, unsigned char* buf) const {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int l = lane & 15;
+    const long long kk = k + 2 * l;
+#pragma unroll 4
+    for (int i = 0; i < SBP / 16; ++i) {
+      const int r = 2 * (warp + 8 * i) + (lane >> 4);
+      if (r >= sb) continue;
+      const long long o = off[r];
+      const double x0 = (o >= 0 && kk < k1) ? __ldg(A + o + kk) : 0.0;
+      const double x1 = (o >= 0 && kk + 1 < k1) ? __ldg(A + o + kk + 1) : 0.0;
+      const int em = emax[r];
+      uint32_t hi[2], lo[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const uint64_t u = (uint64_t)__double_as_longlong(e ? x1 : x0);
+        const int ex = (int)(u >> 52) & 0x7ff;
+        const uint64_t m = ((u & 0xfffffffffffffull) | ((uint64_t)(ex != 0) << 52)) << 2;
+        const int sh = min(em - (ex ? ex : 1), 63);  // >= 0
+        const uint64_t q = (m + ((1ull << sh) >> 1)) >> sh;
+        const uint64_t t = ((int64_t)u < 0 ? (uint64_t)0 - q : q) + 0x0080808080808080ull;
+        hi[e] = (uint32_t)(t >> 32);
+        lo[e] = (uint32_t)t;
+      }
+      const uint32_t at = (uint32_t)((r >> 3) * 512 + (r & 7) * 64 +
+                                     (((l >> 2) ^ ((r >> 1) & 3)) << 4) + (l & 3) * 4);
+#pragma unroll
+      for (int d = 0; d < ND; ++d) {  // digit d + 1, scaled by 256^-d
+        const uint32_t sel = d == 0 ? 0x7632u : d == 1 ? 0x7651u : d == 2 ? 0x7650u
+                             : d == 3 ? 0x7653u : d == 4 ? 0x7652u : d == 5 ? 0x7651u : 0x7650u;
+        const float w = __uint_as_float((uint32_t)(127 - 8 * d) << 23);
+        float f[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e)  // 2^23 + byte, less 2^23 + 128
+          f[e] = fmaf(__uint_as_float(__byte_perm(d < 3 ? hi[e] : lo[e], 0x4B000000u, sel)), w,
+                      -8388736.0f * w);
+        *reinterpret_cast<uint32_t*>(buf + d * kSlice + at) = bf16x2_rn(f[0], f[1]);
+      }
+    }
+  }
+
+  // MMAs of one stage: pairs (i, j) of digits with level i + j in [L0, L1],
+  // level l into accumulator min(l, 7) - L0
+  template <int L0, int L1>
+  __device__ __forceinline__ void issue(uint32_t buf, int nb, bool first) const {
+    const uint32_t id = idesc_bf16(128, nb);
+#pragma unroll
+    for (int l = L0; l <= L1; ++l) {
+      const uint32_t d = tmem + (uint32_t)(SBP * ((l < 7 ? l : 7) - L0));
+#pragma unroll
+      for (int i = 1; i <= kDigits; ++i) {
+        const int j = l - i;
+        if (j < 1 || j > kDigits) continue;
+        const bool start = l <= 7 && i == (l > 7 ? l - 7 : 1);
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk)
+          mma_bf16(d, sw64_kmajor_desc(buf + (i - 1) * kSlice + kk * 32),
+                   sw64_kmajor_desc(buf + (j - 1) * kSlice + kk * 32), id,
+                   first && start && kk == 0 ? 0u : 1u);
+      }
+    }
+  }
+
+  // one pass over the segment: levels L0 .. L1 into tensor memory
+  template <int L0, int L1>
+  __device__ bool pass(const double* __restrict__ A, const long long* off, int sb, long long k0,
+                       long long k1, unsigned* err, bool ok) {
+    const int nb = (sb + 15) & ~15;
+    for (long long k = k0; k < k1; k += 32, ++gt) {
+      const uint32_t bi = gt & 1;
+      unsigned char* buf = dig + bi * kStage;
+      if (gt >= 2 && ok) ok = mbar_wait_grid(&bars[bi], ((gt >> 1) - 1) & 1, err);
+      convert<(L1 - 1 < kDigits ? L1 - 1 : kDigits)>(A, off, sb, k, k1, buf);
+      fence_proxy_async_smem();
+      tc_fence_before();
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        tc_fence_after();
+        issue<L0, L1>(smem_u32(buf), nb, k == k0);
+        mma_commit(&bars[bi]);
+        if (k + 32 >= k1) mma_commit(&bars[2]);
+      }
+    }
+    if (ok) ok = mbar_wait_grid(&bars[2], ph & 1, err);
+    ++ph;
+    tc_fence_after();
+    return ok;
+  }
+
+  // Gram of rows off[0 .. sb) over columns [k0, k1), added to (add) or stored
+  // in part[j * sbp + i], i >= j.  All 256 threads; false once a wait gave up.
+  __device__ bool gram(const double* __restrict__ A, const long long* off, int sb, long long k0,
+                       long long k1, double* __restrict__ part, int sbp, bool add, unsigned* err,
+                       bool ok) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // largest exponent of each row in the segment
+    bool plain = false;
+    for (int r = warp; r < sb; r += 8) {
+      uint32_t h = 0;
+      if (off[r] >= 0)
+#pragma unroll
+        for (int q = 0; q < kSeg / 32; ++q) {
+          const long long k = k0 + 32 * q + lane;
+          if (k < k1)
+            h = max(h, __ldg(reinterpret_cast<const uint32_t*>(A + off[r] + k) + 1) & 0x7fffffffu);
+        }
+      h = __reduce_max_sync(0xffffffffu, h);
+      int e = (int)(h >> 20);
+      if (e == 0) {  // zeros (or subnormal numbers only: the plain sums)
+        bool nz = false;
+        if (off[r] >= 0)
+          for (long long k = k0 + lane; k < k1; k += 32) nz |= __ldg(A + off[r] + k) != 0.0;
+        if (!__any_sync(0xffffffffu, nz)) e = 1023;
+      }
+      plain |= e < 543 || e > 1513;
+      if (lane == 0) emax[r] = e;
+    }
+    if (__syncthreads_or(plain)) {
+      for (int e = tid; e < sb * (sb + 1) / 2; e += 256) {
+        int i, j;
+        tri_decode(e, i, j);
+        double s = add ? part[(long long)j * sbp + i] : 0.0;
+        if (off[i] >= 0 && off[j] >= 0)
+          for (long long k = k0; k < k1; ++k) s = fma(__ldg(A + off[i] + k), __ldg(A + off[j] + k), s);
+        part[(long long)j * sbp + i] = s;
+      }
+      __syncthreads();
+      return ok;
+    }
+    // warp w: tensor-memory lanes (rows) 32 (w % 4) .. + 31, column chunks of
+    // parity w / 4
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t tbase = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    const bool act = (warp & 3) * 32 < sb;  // (rows past sb hold garbage)
+    auto put = [&](int cc, const int64_t (&v)[32], const float (&low)[32]) {
+      if (row >= sb) return;
+      const int er = emax[row];
+#pragma unroll
+      for (int q = 0; q < 32; ++q) {
+        const int j = cc + q;
+        if (j > row) break;
+        // units of level 7 (2^-40 of level 2), then 2^(er + ej - 2098)
+        double g = (double)(v[q] * 256 + __float2int_rn(low[q] * 1099511627776.0f));
+        if (g != 0.0)
+          g = __hiloint2double(__double2hiint(g) + ((er + emax[j] - 2098) << 20), __double2loint(g));
+        double* at = part + (long long)j * sbp + row;
+        *at = add ? *at + g : g;
+      }
+    };
+    auto level = [&](int a, int cc, float scale, int64_t (&v)[32]) {
+      uint32_t x[32];
+      tmem_ld32(tbase + (uint32_t)(SBP * a + cc), x);
+#pragma unroll
+      for (int q = 0; q < 32; ++q) v[q] = v[q] * 256 + __float2int_rn(__uint_as_float(x[q]) * scale);
+    };
+    if constexpr (SBP <= 64) {
+      ok = pass<2, 9>(A, off, sb, k0, k1, err, ok);
+      for (int cc = 32 * (warp >> 2); act && cc < sb && cc <= (warp & 3) * 32; cc += 64) {
+        int64_t v[32];
+#pragma unroll
+        for (int q = 0; q < 32; ++q) v[q] = 0;
+        level(0, cc, 1.0f, v);
+        level(1, cc, 256.0f, v);
+        level(2, cc, 65536.0f, v);
+        level(3, cc, 16777216.0f, v);
+        level(4, cc, 4294967296.0f, v);
+        uint32_t x[32];
+        float low[32];
+        tmem_ld32(tbase + (uint32_t)(SBP * 5 + cc), x);
+#pragma unroll
+        for (int q = 0; q < 32; ++q) low[q] = __uint_as_float(x[q]);
+        put(cc, v, low);
+      }
+    } else {
+      // levels 2 .. 5: their integers wait in the thread's own memory
+      int64_t keep[2][32];
+      const int cc0 = 32 * (warp >> 2), ccn = (warp & 3) * 32;
+      ok = pass<2, 5>(A, off, sb, k0, k1, err, ok);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int cc = cc0 + 64 * h;
+        if (act && cc < sb && cc <= ccn) {
+#pragma unroll
+          for (int q = 0; q < 32; ++q) keep[h][q] = 0;
+          level(0, cc, 1.0f, keep[h]);
+          level(1, cc, 256.0f, keep[h]);
+          level(2, cc, 65536.0f, keep[h]);
+          level(3, cc, 16777216.0f, keep[h]);
+        }
+      }
+      tc_fence_before();
+      __syncthreads();
+      ok = pass<6, 9>(A, off, sb, k0, k1, err, ok);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int cc = cc0 + 64 * h;
+        if (act && cc < sb && cc <= ccn) {
+          level(0, cc, 4294967296.0f, keep[h]);
+          uint32_t x[32];
+          float low[32];
+          tmem_ld32(tbase + (uint32_t)(SBP + cc), x);
+#pragma unroll
+          for (int q = 0; q < 32; ++q) low[q] = __uint_as_float(x[q]);
+          put(cc, keep[h], low);
+        }
+      }
+    }
+    tc_fence_before();
+    __syncthreads();  // the accumulators are read
+    return ok;
+  }
+};
+
+}  // namespace

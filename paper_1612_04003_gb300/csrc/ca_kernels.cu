@@ -243,8 +243,8 @@ __device__ void block_solve(const double* __restrict__ R, const double* __restri
 // into Ginv[j] (cta_sweep_inverse; two warps for b <= 8); the other CTAs take
 // 64 entries per pass (warps 0-3: the first 32, one per lane; warps 4-7: the
 // next 32), the 4 warps of a group splitting the P partials, so that every
-// load of a pass is in flight at once.  Sums are double-float; R is written
-// in FP64.
+// load of a pass is in flight at once.  Sums are double-float for FP32 partials
+// (R holds them in FP64) and FP64 for FP64 partials.
 template <typename PT>
 __device__ void reduce_body(const PT* __restrict__ part, const double* __restrict__ ppart, int P,
                             int sbp, double* __restrict__ R, float2* __restrict__ Rs,
@@ -332,24 +332,33 @@ __device__ void reduce_body(const PT* __restrict__ part, const double* __restric
       kind = 2;
       i = (int)(e - nlow);
     }
-    if (kind == 1) {
-      s2 = sum_partials<PT, 40>(part + (long long)j * sbp + i, sub, P, 4, sq);
-    } else if (kind == 2) {
-      const float2 q = sum_partials<double, 40>(ppart + i, sub, P, 4, (long long)sbp);
-      sp = (double)q.x + (double)q.y;
+    if constexpr (sizeof(PT) == 8) {  // FP64 partials: FP64 sums
+      if (kind == 1) sp = sum_partials64<40>(part + (long long)j * sbp + i, sub, P, 4, sq);
+      else if (kind == 2) sp = sum_partials64<40>(ppart + i, sub, P, 4, (long long)sbp);
+    } else {
+      if (kind == 1) {
+        s2 = sum_partials<PT, 40>(part + (long long)j * sbp + i, sub, P, 4, sq);
+      } else if (kind == 2) {
+        const float2 q = sum_partials<double, 40>(ppart + i, sub, P, 4, (long long)sbp);
+        sp = (double)q.x + (double)q.y;
+      }
+      red[warp][lane] = s2;
     }
-    red[warp][lane] = s2;
     redp[warp][lane] = sp;
     __syncthreads();
     if (sub == 0 && kind) {  // warps 0 and 4: the group's four sums
       const int w = warp;
-      if (kind == 1) {
+      const double t64 = (redp[w][lane] + redp[w + 1][lane]) + (redp[w + 2][lane] + redp[w + 3][lane]);
+      if (kind == 2) {
+        pvec[i] = t64;
+      } else if constexpr (sizeof(PT) == 8) {
+        R[(long long)i * ldr + j] = t64;
+        if (Rs) Rs[(long long)j * ldr + i] = df_mul(cG2, split_f64(t64));
+      } else {
         const float2 t = df_add(df_add(red[w][lane], red[w + 1][lane]),
                                 df_add(red[w + 2][lane], red[w + 3][lane]));
         R[(long long)i * ldr + j] = (double)t.x + (double)t.y;
         if (Rs) Rs[(long long)j * ldr + i] = df_mul(cG2, t);
-      } else {
-        pvec[i] = (redp[w][lane] + redp[w + 1][lane]) + (redp[w + 2][lane] + redp[w + 3][lane]);
       }
     }
     __syncthreads();

@@ -159,6 +159,12 @@ struct Persist64Args {
   SolveArgs sa;          // solve constants (idx and delta are set per step); ldr = sbp
   unsigned* cnt;         // 4 counts, zero on entry
 };
+// The Gram pass of dense FP64 X alone, sb <= gram64_max_sb(): P <= ceil(K / 32)
+// split-K partials (P x sbp^2, transposed) and projections (P x sbp).
+int gram64_max_sb();
+int launch_gram64(const double* A, long long lda, long long N, long long K, const int* idx, int sb,
+                  const double* v, int P, int sbp, double* part, double* ppart, unsigned* err,
+                  cudaStream_t st);
 bool persist64_fits(int b, int sb);
 // P <= number of SMs - 1 and <= ceil(K / 32).  Returns a cudaError_t.
 int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,

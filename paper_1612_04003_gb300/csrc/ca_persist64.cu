@@ -24,6 +24,7 @@
 #include <algorithm>
 #include <atomic>
 
+#include "ca_digits.cuh"
 #include "ca_kernels.cuh"
 #include "ca_solve.cuh"
 
@@ -31,7 +32,7 @@ namespace {
 
 constexpr int kT = 256;      // threads of a CTA
 constexpr int kSmemMax = 200 * 1024;  // dynamic shared memory a launch may ask for
-constexpr int kSmallSB = 32;  // rows of a step the CUDA-core Gram covers
+constexpr int kSmallSB = 16;  // rows of a step the CUDA-core Gram takes
 
 struct Cnt {  // counts in cnt[]
   enum { G = 0, R = 1, P = 2, D = 3 };
@@ -62,7 +63,7 @@ __device__ __forceinline__ void row_offsets(const int* idx, int sb, long long N,
   }
 }
 
-// Gram partial of sb <= 32 rows over columns [k0, k1) on CUDA cores: the
+// Gram partial of sb <= 16 rows over columns [k0, k1) on CUDA cores: the
 // FP64 pipe does two FMAs a clock and SM, so only the lower triangle is
 // formed.  Warp w takes columns 4 w .. 4 w + 3 of each 32-column tile, lane l
 // the entries l, l + 32, ...; the warps' sums meet in shared memory.
@@ -188,6 +189,88 @@ __device__ void update_project(const Persist64Args& a, const long long* off, con
   if (lane % low == 0 && r < sb) pp[r] = s;
 }
 
+// Shared state of a column CTA's digit Gram; digits_begin / digits_end by all
+// threads (tensor memory is held in between).
+template <int RQ>
+struct DigitShared {
+  int emax[8 * RQ];
+  uint64_t bars[3];
+  uint32_t tmem_holder;
+};
+template <int RQ>
+__device__ __forceinline__ void digits_begin(DigitGram<8 * RQ>& dg, DigitShared<RQ>& sh, void* smem) {
+  dg.dig = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem) + 1023) &
+                                            ~uintptr_t(1023));
+  dg.bars = sh.bars;
+  dg.emax = sh.emax;
+  if (threadIdx.x == 0) {
+    for (int q = 0; q < 3; ++q) mbar_init(&sh.bars[q], 1);
+    fence_mbar_init();
+  }
+  if (threadIdx.x < 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&sh.tmem_holder)),
+                 "r"((uint32_t)DigitGram<8 * RQ>::kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_proxy_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  dg.tmem = sh.tmem_holder;
+}
+template <int RQ>
+__device__ __forceinline__ void digits_end(const DigitGram<8 * RQ>& dg) {
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(dg.tmem),
+                 "r"((uint32_t)DigitGram<8 * RQ>::kTmemCols)
+                 : "memory");
+  }
+}
+
+// Gram partial of the CTA's columns [c0, c1).
+template <int RQ>
+__device__ __forceinline__ bool gram_columns(DigitGram<8 * RQ>& dg, const double* __restrict__ A,
+                                             const long long* off, int sb, long long c0,
+                                             long long c1, double* smem_d, double* __restrict__ part,
+                                             int sbp, unsigned* err, bool ok) {
+  if (sb <= kSmallSB) {
+    gram_small(A, off, sb, c0, c1, smem_d, part, sbp);
+    return ok;
+  }
+  // segments of equal length, whole 32-column stages
+  const long long nst = (c1 - c0 + 31) / 32, nseg = (nst + kSeg / 32 - 1) / (kSeg / 32);
+  for (long long g = 0; g < nseg && ok; ++g)
+    ok = dg.gram(A, off, sb, c0 + nst * g / nseg * 32, min(c1, c0 + nst * (g + 1) / nseg * 32), part,
+                 sbp, g > 0, err, ok);
+  return ok;
+}
+
+// The Gram pass alone (steps a2+a3): split-K partials over gridDim.x CTAs and
+// the projection partials on v.
+template <int RQ>
+__global__ void __launch_bounds__(kT, 1)
+k_gram64(Persist64Args a, unsigned* __restrict__ err) {
+  extern __shared__ double smem_d[];
+  __shared__ long long soff[8 * RQ];
+  __shared__ double ured[2 * kT];
+  __shared__ DigitShared<RQ> sh;
+  const int P = (int)gridDim.x, c = blockIdx.x, sb = a.sb, sbp = a.sa.ldr;
+  const long long nch = (a.K + 31) / 32;
+  const long long c0 = nch * c / P * 32, c1 = min(a.K, nch * (c + 1) / P * 32);
+  DigitGram<8 * RQ> dg;
+  if (sb > kSmallSB) digits_begin<RQ>(dg, sh, smem_d);
+  row_offsets(a.idx_all, sb, a.N, a.lda, soff, err);
+  __syncthreads();
+  gram_columns<RQ>(dg, a.A, soff, sb, c0, c1, smem_d, a.part + (long long)c * sbp * sbp, sbp, err, true);
+  update_project<RQ>(a, soff, soff, nullptr, sb, 0, c0, c1, ured, a.ppart + (long long)c * sbp);
+  if (sb > kSmallSB) digits_end<RQ>(dg);
+}
+
 template <int BMAX, int DEPTH, int RQ>
 __global__ void __launch_bounds__(kT, 1) k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
@@ -227,6 +310,10 @@ __global__ void __launch_bounds__(kT, 1) k_persist64(Persist64Args a, unsigned* 
   __shared__ double ured[2 * kT];
   __shared__ float2 Mb[256];
   __shared__ float2 colbuf[66];
+  __shared__ DigitShared<RQ> sh;
+  DigitGram<8 * RQ> dg;
+  const bool digits = sb > kSmallSB;
+  if (digits) digits_begin<RQ>(dg, sh, smem_d);
   const long long nch = (a.K + 31) / 32;
   const long long c0 = nch * c / P * 32, c1 = min(a.K, nch * (c + 1) / P * 32);
   const float2 cG2 = split_f64(a.sa.cG), cI2 = split_f64(a.sa.cI);
@@ -237,7 +324,7 @@ __global__ void __launch_bounds__(kT, 1) k_persist64(Persist64Args a, unsigned* 
   auto gram = [&](int p, const long long* off) {
     const long long k = a.k0 + p;
     double* part = a.part + (k & 1) * (long long)P * sq;
-    gram_small(a.A, off, sb, c0, c1, smem_d, part + c * sq, sbp);
+    ok = gram_columns<RQ>(dg, a.A, off, sb, c0, c1, smem_d, part + c * sq, sbp, err, ok);
     cta_count(a.cnt + Cnt::G);
     ok = cta_wait(a.cnt + Cnt::G, (unsigned)(P * (p + 1)), err, ok);
     if (!ok) return;
@@ -320,46 +407,93 @@ __global__ void __launch_bounds__(kT, 1) k_persist64(Persist64Args a, unsigned* 
       gram(p + 1, soff[(p + 1) & 1]);
     }
   }
+  if (digits) digits_end<RQ>(dg);
 }
 
-template <int BMAX, int DEPTH, int RQ>
-int launch_one(const Persist64Args& a, int P, size_t chain_smem, unsigned* err, cudaStream_t st) {
-  const size_t gsm = (kSmallSB * 33 + 8 * (size_t)(kSmallSB * (kSmallSB + 1) / 2)) * 8;
-  const size_t smem = std::max(chain_smem, gsm);
+// Dynamic shared memory of a column CTA.  With digits more than half of an
+// SM's: two launches never share an SM, so neither can hold the tensor memory
+// that a CTA of the other, which its grid waits for, needs.
+template <int RQ>
+size_t column_smem(int sb) {
+  if (sb <= kSmallSB) return (kSmallSB * 33 + 8 * (size_t)(kSmallSB * (kSmallSB + 1) / 2)) * 8;
+  return std::max<size_t>(DigitGram<8 * RQ>::kSmem, 118 * 1024);
+}
+
+template <typename Kern>
+int launch64(Kern kern, std::atomic<unsigned long long>& configured, const Persist64Args& a,
+             int grid, size_t smem, bool coop, unsigned* err, cudaStream_t st) {
   if (smem > (size_t)kSmemMax) return (int)cudaErrorInvalidConfiguration;
-  auto kern = k_persist64<BMAX, DEPTH, RQ>;
-  static std::atomic<unsigned long long> configured{0ull};  // devices (a bit each)
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return (int)e;
-  const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;
+  const unsigned long long bit = dev < 64 ? (1ull << dev) : 0ull;  // a bit per device
   if (!bit || !(configured.load(std::memory_order_acquire) & bit)) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e != cudaSuccess) return (int)e;
     configured.fetch_or(bit, std::memory_order_release);
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(P + 1);
+  cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].id = cudaLaunchAttributeCooperative;  // every CTA resident at once
   at[0].val.cooperative = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = coop ? 1 : 0;
   e = cudaLaunchKernelEx(&cfg, kern, a, err);
   return (int)(e != cudaSuccess ? e : cudaGetLastError());
 }
 
+template <int BMAX, int DEPTH, int RQ>
+int launch_steps(const Persist64Args& a, int P, size_t chain_smem, unsigned* err, cudaStream_t st) {
+  static std::atomic<unsigned long long> configured{0ull};
+  return launch64(k_persist64<BMAX, DEPTH, RQ>, configured, a, P + 1,
+                  std::max(chain_smem, column_smem<RQ>(a.sb)), true, err, st);
+}
+
+template <int RQ>
+int launch_gram(const Persist64Args& a, int P, unsigned* err, cudaStream_t st) {
+  static std::atomic<unsigned long long> configured{0ull};
+  return launch64(k_gram64<RQ>, configured, a, P, column_smem<RQ>(a.sb), false, err, st);
+}
+
 }  // namespace
 
-// Rows of a step and block sizes the launch covers.
-bool persist64_fits(int b, int sb) { return b <= 16 && sb <= kSmallSB; }
+int gram64_max_sb() { return 128; }
+
+int launch_gram64(const double* A, long long lda, long long N, long long K, const int* idx, int sb,
+                  const double* v, int P, int sbp, double* part, double* ppart, unsigned* err,
+                  cudaStream_t st) {
+  Persist64Args a{};
+  a.A = A;
+  a.lda = lda;
+  a.N = N;
+  a.K = K;
+  a.idx_all = idx;
+  a.sb = sb;
+  a.v = const_cast<double*>(v);  // read only: no update is pending
+  a.part = part;
+  a.ppart = ppart;
+  a.sa.ldr = sbp;
+  if (sb <= 32) return launch_gram<4>(a, P, err, st);
+  if (sb <= 64) return launch_gram<8>(a, P, err, st);
+  if (sb <= 128) return launch_gram<16>(a, P, err, st);
+  return (int)cudaErrorInvalidValue;
+}
+
+// Block sizes and rows of a step the persistent launch covers.
+bool persist64_fits(int b, int sb) { return b <= 16 && sb <= 128; }
 
 int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,
                      cudaStream_t st) {
-  const bool small = a.sa.b <= 8;
-  return small ? launch_one<8, 4, 4>(a, P, chain_smem, err, st)
-               : launch_one<16, 3, 4>(a, P, chain_smem, err, st);
+#define CA_P64(RQ)                                                       \
+  return a.sa.b <= 8 ? launch_steps<8, 4, RQ>(a, P, chain_smem, err, st) \
+                     : launch_steps<16, 3, RQ>(a, P, chain_smem, err, st);
+  if (a.sb <= 32) CA_P64(4)
+  if (a.sb <= 64) CA_P64(8)
+  if (a.sb <= 128) CA_P64(16)
+#undef CA_P64
+  return (int)cudaErrorInvalidValue;
 }

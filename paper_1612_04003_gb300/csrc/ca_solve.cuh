@@ -68,6 +68,34 @@ __device__ void cta_sweep_inverse(float2 (&a)[EPT], int b, float2* __restrict__ 
     if (ri[q] >= 0) out[t + NT * q] = df_neg(a[q]);
 }
 
+// FP64 sum of the partials c = c0, c0 + step, ... < P of one entry (stride sq
+// between partials): U (U >= 32, else 16) loads in flight, a pairwise tree.
+template <int U>
+__device__ __forceinline__ double sum_partials64(const double* __restrict__ src, int c0, int P,
+                                                 int step, long long sq) {
+  constexpr int UD = U >= 32 ? U : 16;
+  double acc = 0.0;
+  for (int base = c0; base < P; base += UD * step) {
+    double v[UD];
+#pragma unroll
+    for (int i = 0; i < UD; ++i) {
+      const int c = base + i * step;
+      const double x = __ldcg(src + (long long)min(c, P - 1) * sq);
+      v[i] = c < P ? x : 0.0;
+    }
+    // pairwise tree over UD <= 128 values: at width w, v[i + w] folds onto
+    // v[i] where it exists
+    static_assert(UD <= 128, "tree depth");
+#pragma unroll
+    for (int w = 64; w >= 1; w /= 2)
+#pragma unroll
+      for (int i = 0; i < w; ++i)
+        if (i + w < UD) v[i] += v[i + w];
+    acc += v[0];
+  }
+  return acc;
+}
+
 // Sum of the partials c = c0, c0 + step, ... < P of one entry (stride sq
 // between partials), as a double-float value.  Up to U (FP32; FP64: U when
 // U >= 32, else 16) loads are in flight at once (independent of the sums); FP32 partials are
@@ -92,27 +120,7 @@ __device__ __forceinline__ float2 sum_partials(const PT* __restrict__ src, int c
     return df_add(df_add(df_norm(h[0], l[0]), df_norm(h[1], l[1])),
                   df_add(df_norm(h[2], l[2]), df_norm(h[3], l[3])));
   } else {
-    constexpr int UD = U >= 32 ? U : 16;
-    double acc = 0.0;
-    for (int base = c0; base < P; base += UD * step) {
-      double v[UD];
-#pragma unroll
-      for (int i = 0; i < UD; ++i) {
-        const int c = base + i * step;
-        const double x = __ldcg(src + (long long)min(c, P - 1) * sq);
-        v[i] = c < P ? x : 0.0;
-      }
-      // pairwise tree over UD <= 128 values: at width w, v[i + w] folds onto
-      // v[i] where it exists
-      static_assert(UD <= 128, "tree depth");
-#pragma unroll
-      for (int w = 64; w >= 1; w /= 2)
-#pragma unroll
-        for (int i = 0; i < w; ++i)
-          if (i + w < UD) v[i] += v[i + w];
-      acc += v[0];
-    }
-    return split_f64(acc);
+    return split_f64(sum_partials64<U>(src, c0, P, step, sq));
   }
 }
 

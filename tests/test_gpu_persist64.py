@@ -39,12 +39,19 @@ def _rel(a, b):
 
 
 CASES = [  # method, d, n, b, s, H, recompute_every, check_every
+    # s*b = 16 | 17 .. 128: the Gram on CUDA cores | by digit products
     ("primal", 40, 17, 1, 1, 23, 0, 0),
     ("primal", 64, 1024, 4, 4, 202, 0, 0),
     ("primal", 33, 1057, 8, 4, 61, 4, 0),
     ("primal", 60, 5003, 16, 2, 31, 0, 3),
     ("dual", 4832, 48, 8, 3, 40, 0, 0),
     ("dual", 31, 200, 16, 1, 37, 5, 0),
+    ("primal", 90, 4999, 8, 4, 41, 0, 0),
+    ("dual", 1500, 90, 1, 17, 70, 0, 2),
+    ("primal", 70, 33, 16, 4, 18, 0, 0),
+    ("dual", 5001, 160, 16, 8, 28, 2, 0),
+    ("primal", 130, 777, 8, 16, 50, 0, 0),
+    ("primal", 40, 36001, 8, 5, 33, 0, 0),  # two segments of columns a CTA
 ]
 
 
@@ -73,3 +80,46 @@ def test_persistent_fp64_steps(ctx, method, d, n, b, s, H, every, check):
     for i in range(2):
         assert _rel(got[0][i], np.asarray(ref[i])) < 1e-10
         assert _rel(got[0][i], got[1][i]) < 1e-10
+
+
+@pytest.mark.parametrize("rows,K,scale", [(1, 1, 0), (16, 40, 0), (17, 31, 0), (32, 4000, 0),
+                                          (33, 999, 1), (64, 32, 0), (100, 5000, 1),
+                                          (128, 30011, 0), (128, 70, 2)])
+def test_gram_fp64(ctx, rows, K, scale):
+    """G = Y Y^T and p = Y v of FP64 rows against extended precision.  Digit products: each
+    element is rounded to 2^-55 of its row's largest magnitude m in the segment, the levels left
+    out and the one rounded accumulator are smaller, so an entry is within 2^-52 K m_i m_j (an
+    FP64 sum: 2^-53 K times the sum of |products|, about the same).  scale 1: rows of magnitudes
+    1e-6 .. 1e6 and single large elements; 2: rows outside the digits' exponent range."""
+    rng = np.random.default_rng(rows + K)
+    A = rng.standard_normal((rows + 3, K))
+    if scale == 1:
+        A *= 10.0 ** rng.uniform(-6, 6, size=(rows + 3, 1))
+        A[np.arange(rows), rng.integers(0, K, rows)] *= 1e9
+        A[5] = 0.0
+    if scale == 2:
+        A *= (1e-150 ** rng.integers(0, 2, size=(rows + 3, 1)))
+    idx = rng.permutation(rows + 3)[:rows].astype(np.int32)
+    v = rng.standard_normal(K)
+    G = torch.empty(rows, rows, dtype=torch.float64, device="cuda")
+    p = torch.empty(rows, dtype=torch.float64, device="cuda")
+    ctx.ca_gram_project(_dev(A), _dev(idx), _dev(v), G, p, prec="f64")
+    Y = A[idx].astype(np.longdouble)
+    m = np.abs(A[idx]).max(1)
+    assert (np.abs(G.cpu().numpy() - Y @ Y.T) <= 2.0 ** -52 * K * np.outer(m, m)).all()
+    assert (np.abs(p.cpu().numpy() - Y @ v) <= 2.0 ** -52 * K * m * np.abs(v).max()).all()
+
+
+def test_gram_fp64_non_finite(ctx):
+    """An infinity or a NaN in one row reaches exactly the entries FP64 arithmetic gives."""
+    rng = np.random.default_rng(1)
+    A = rng.standard_normal((40, 500))
+    A[3, 100], A[7, 20] = np.inf, np.nan
+    G = torch.empty(40, 40, dtype=torch.float64, device="cuda")
+    p = torch.empty(40, dtype=torch.float64, device="cuda")
+    ctx.ca_gram_project(_dev(A), torch.arange(40, dtype=torch.int32, device="cuda"),
+                        _dev(rng.standard_normal(500)), G, p, prec="f64")
+    g, ref = G.cpu().numpy(), A @ A.T
+    assert (np.isnan(g) == np.isnan(ref)).all() and (np.isinf(g) == np.isinf(ref)).all()
+    fin = np.isfinite(ref)
+    assert np.abs(g[fin] - ref[fin]).max() <= 2.0 ** -52 * 500 * 25
