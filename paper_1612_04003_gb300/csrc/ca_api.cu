@@ -469,7 +469,7 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
       pa.pvec = pvec;
       pa.sa = SolveArgs{nullptr, pb.N, b, s, sb, sbp, pb.cG, pb.cI, pb.cP, pb.cY, pb.x, pb.yv, nullptr};
       pa.cnt = ctx->d_cnt;
-      CA_TRY_CUDA(cudaMemsetAsync(ctx->d_cnt, 0, 4 * sizeof(unsigned), ctx->stream));
+      CA_TRY_CUDA(cudaMemsetAsync(ctx->d_cnt, 0, 6 * sizeof(unsigned), ctx->stream));
       prof_mark(ctx, PC_GRAM);
       const int e = launch_persist64(pa, P64, chain_smem(b, sb), ctx->d_err, ctx->stream);
       prof_mark(ctx, PC_GRAM);

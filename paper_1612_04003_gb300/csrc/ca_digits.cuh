@@ -27,7 +27,37 @@ namespace {
 constexpr int kSeg = 192;  // columns whose level sums stay exact in FP32
 constexpr int kDigits = 7;
 
-// SBP rows (32, 64 or 128), a CTA of 256 threads.  Tensor memory: one
+// Named barrier 1 over the eight warps that form a Gram partial (a CTA may have
+// others), and the same with a vote.
+__device__ __forceinline__ void main_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ bool main_any(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 256, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)v)
+      : "memory");
+  return r != 0;
+}
+
+// v 2^e, rounded to nearest, on the integer pipe (a conversion of the FP64
+// pipe holds a scheduler for 64 cycles); the result is a normal number.
+__device__ __forceinline__ double fixed_to_double(int64_t v, int e) {
+  uint64_t m = v < 0 ? (uint64_t)0 - (uint64_t)v : (uint64_t)v;
+  int lz = __clzll((long long)m);
+  m <<= lz & 63;
+  uint64_t t = m + 0x400u;
+  if (t < m) {  // rounded up to the next power of two
+    t = 1ull << 63;
+    --lz;
+  }
+  const uint64_t b = ((uint64_t)(uint32_t)(1086 - lz + e) << 52) | ((t >> 11) & 0xfffffffffffffull) |
+                     ((uint64_t)v & (1ull << 63));
+  return v == 0 ? 0.0 : __longlong_as_double((long long)b);
+}
+
+// SBP rows (32, 64 or 128), the eight main warps of a CTA.  Tensor memory: one
 // accumulator of SBP columns a level.  SBP = 128 holds four of the six at
 // once: levels 2 .. 5, then (the columns converted again) levels 6 .. 9.
 template <int SBP>
@@ -42,31 +72,51 @@ struct DigitGram {
   uint64_t* bars;       // [0], [1]: stage buffer read by the MMAs; [2]: all MMAs
   uint32_t tmem;
   int* emax;            // [SBP] largest biased exponent of each row
+  int64_t* diag;        // [SBP] (SBP = 128)
   uint32_t gt = 0;      // stages so far (buffers and phases run on)
   uint32_t ph = 0;      // passes so far
 
-  // one stage of 32 columns: digits 1 .. ND of every row
+  // This thread's rows 2 (warp + 8 i) + lane / 16, columns 2 (lane % 16) and
+  // the next of a stage.
+  static constexpr int kRows = SBP / 16;
+  struct Rows {
+    long long off[kRows];  // (rows past sb: the last row again, never stored)
+    int em[kRows];
+  };
+  // (unconditional loads at clamped columns, then a select: a condition on
+  // each load makes branches that wait for one load after another)
+  __device__ __forceinline__ void load(const double* __restrict__ A, const Rows& rw, long long k,
+                                       long long k1, double (&x)[kRows][2]) const {
+    const long long kk = k + 2 * (threadIdx.x & 15);
+    const long long ka = min(kk, k1 - 1), kb = min(kk + 1, k1 - 1);
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      x[i][0] = __ldg(A + rw.off[i] + ka);
+      x[i][1] = __ldg(A + rw.off[i] + kb);
+    }
+    if (kk + 1 >= k1) {
+#pragma unroll
+      for (int i = 0; i < kRows; ++i) {
+        x[i][1] = 0.0;
+        if (kk >= k1) x[i][0] = 0.0;
+      }
+    }
+  }
+  // one stage of 32 columns: digits 1 .. ND of every row (rows past sb: zero)
   template <int ND>
-  __device__ __forceinline__ void convert(const double* __restrict__ A, const long long* off, int sb,
-                                          long long k, long long k1, unsigned char* buf) const {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int l = lane & 15;
-    const long long kk = k + 2 * l;
-#pragma unroll 4
-    for (int i = 0; i < SBP / 16; ++i) {
+  __device__ __forceinline__ void convert(const Rows& rw, const double (&x)[kRows][2],
+                                          unsigned char* buf) const {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane & 15;
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
       const int r = 2 * (warp + 8 * i) + (lane >> 4);
-      if (r >= sb) continue;
-      const long long o = off[r];
-      const double x0 = (o >= 0 && kk < k1) ? __ldg(A + o + kk) : 0.0;
-      const double x1 = (o >= 0 && kk + 1 < k1) ? __ldg(A + o + kk + 1) : 0.0;
-      const int em = emax[r];
       uint32_t hi[2], lo[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
-        const uint64_t u = (uint64_t)__double_as_longlong(e ? x1 : x0);
+        const uint64_t u = (uint64_t)__double_as_longlong(x[i][e]);
         const int ex = (int)(u >> 52) & 0x7ff;
         const uint64_t m = ((u & 0xfffffffffffffull) | ((uint64_t)(ex != 0) << 52)) << 2;
-        const int sh = min(em - (ex ? ex : 1), 63);  // >= 0
+        const int sh = min(rw.em[i] - (ex ? ex : 1), 63);  // >= 0
         const uint64_t q = (m + ((1ull << sh) >> 1)) >> sh;
         const uint64_t t = ((int64_t)u < 0 ? (uint64_t)0 - q : q) + 0x0080808080808080ull;
         hi[e] = (uint32_t)(t >> 32);
@@ -94,6 +144,7 @@ struct DigitGram {
   template <int L0, int L1>
   __device__ __forceinline__ void issue(uint32_t buf, int nb, bool first) const {
     const uint32_t id = idesc_bf16(128, nb);
+    const uint64_t base = sw64_kmajor_desc(buf);  // (the address field is in 16-byte units)
 #pragma unroll
     for (int l = L0; l <= L1; ++l) {
       const uint32_t d = tmem + (uint32_t)(SBP * ((l < 7 ? l : 7) - L0));
@@ -104,31 +155,39 @@ struct DigitGram {
         const bool start = l <= 7 && i == (l > 7 ? l - 7 : 1);
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk)
-          mma_bf16(d, sw64_kmajor_desc(buf + (i - 1) * kSlice + kk * 32),
-                   sw64_kmajor_desc(buf + (j - 1) * kSlice + kk * 32), id,
-                   first && start && kk == 0 ? 0u : 1u);
+          mma_bf16(d, base + (uint32_t)(((i - 1) * kSlice + kk * 32) >> 4),
+                   base + (uint32_t)(((j - 1) * kSlice + kk * 32) >> 4), id,
+                   start && kk == 0 ? (first ? 0u : 1u) : 1u);
       }
     }
   }
 
   // one pass over the segment: levels L0 .. L1 into tensor memory
   template <int L0, int L1>
-  __device__ bool pass(const double* __restrict__ A, const long long* off, int sb, long long k0,
+  __device__ bool pass(const double* __restrict__ A, const Rows& rw, int sb, long long k0,
                        long long k1, unsigned* err, bool ok) {
     const int nb = (sb + 15) & ~15;
+    double x[kRows][2];
+    load(A, rw, k0, k1, x);
     for (long long k = k0; k < k1; k += 32, ++gt) {
       const uint32_t bi = gt & 1;
       unsigned char* buf = dig + bi * kStage;
       if (gt >= 2 && ok) ok = mbar_wait_grid(&bars[bi], ((gt >> 1) - 1) & 1, err);
-      convert<(L1 - 1 < kDigits ? L1 - 1 : kDigits)>(A, off, sb, k, k1, buf);
+      convert<(L1 - 1 < kDigits ? L1 - 1 : kDigits)>(rw, x, buf);
+      load(A, rw, k + 32, k1, x);  // (lands while the MMAs of this stage run)
       fence_proxy_async_smem();
       tc_fence_before();
-      __syncthreads();
-      if (threadIdx.x == 0) {
+      main_sync();
+      // (a warp-uniform branch and one elected lane: the descriptors stay in
+      // uniform registers)
+      if (__shfl_sync(0xffffffffu, threadIdx.x >> 5, 0) == 0) {
         tc_fence_after();
-        issue<L0, L1>(smem_u32(buf), nb, k == k0);
-        mma_commit(&bars[bi]);
-        if (k + 32 >= k1) mma_commit(&bars[2]);
+        if (elect_one()) {
+          issue<L0, L1>(smem_u32(buf), nb, k == k0);
+          mma_commit(&bars[bi]);
+          if (k + 32 >= k1) mma_commit(&bars[2]);
+        }
+        __syncwarp();
       }
     }
     if (ok) ok = mbar_wait_grid(&bars[2], ph & 1, err);
@@ -145,118 +204,135 @@ struct DigitGram {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // largest exponent of each row in the segment
     bool plain = false;
-    for (int r = warp; r < sb; r += 8) {
-      uint32_t h = 0;
-      if (off[r] >= 0)
+    constexpr int RB = 4;  // rows in flight a warp
+    for (int r0 = warp; r0 < sb; r0 += 8 * RB) {
+      uint32_t h[RB];
 #pragma unroll
-        for (int q = 0; q < kSeg / 32; ++q) {
-          const long long k = k0 + 32 * q + lane;
-          if (k < k1)
-            h = max(h, __ldg(reinterpret_cast<const uint32_t*>(A + off[r] + k) + 1) & 0x7fffffffu);
-        }
-      h = __reduce_max_sync(0xffffffffu, h);
-      int e = (int)(h >> 20);
-      if (e == 0) {  // zeros (or subnormal numbers only: the plain sums)
-        bool nz = false;
-        if (off[r] >= 0)
-          for (long long k = k0 + lane; k < k1; k += 32) nz |= __ldg(A + off[r] + k) != 0.0;
-        if (!__any_sync(0xffffffffu, nz)) e = 1023;
+      for (int u = 0; u < RB; ++u) {
+        const double* row = A + off[min(r0 + 8 * u, sb - 1)];
+        h[u] = 0;
+#pragma unroll
+        for (int q = 0; q < kSeg / 32; ++q)
+          h[u] = max(h[u], __ldg(reinterpret_cast<const uint32_t*>(
+                               row + min(k0 + 32 * q + lane, k1 - 1)) + 1) & 0x7fffffffu);
       }
-      plain |= e < 543 || e > 1513;
-      if (lane == 0) emax[r] = e;
+#pragma unroll
+      for (int u = 0; u < RB; ++u) {
+        const int r = r0 + 8 * u;
+        if (r >= sb) break;
+        int e = (int)(__reduce_max_sync(0xffffffffu, h[u]) >> 20);
+        if (e == 0) {  // zeros (or subnormal numbers only: the plain sums)
+          bool nz = false;
+          for (long long k = k0 + lane; k < k1; k += 32) nz |= __ldg(A + off[r] + k) != 0.0;
+          if (!__any_sync(0xffffffffu, nz)) e = 1023;
+        }
+        plain |= e < 543 || e > 1513;
+        if (lane == 0) emax[r] = e;
+      }
     }
-    if (__syncthreads_or(plain)) {
+    if (main_any(plain)) {
       for (int e = tid; e < sb * (sb + 1) / 2; e += 256) {
         int i, j;
         tri_decode(e, i, j);
         double s = add ? part[(long long)j * sbp + i] : 0.0;
-        if (off[i] >= 0 && off[j] >= 0)
-          for (long long k = k0; k < k1; ++k) s = fma(__ldg(A + off[i] + k), __ldg(A + off[j] + k), s);
+        for (long long k = k0; k < k1; ++k) s = fma(__ldg(A + off[i] + k), __ldg(A + off[j] + k), s);
         part[(long long)j * sbp + i] = s;
       }
-      __syncthreads();
+      main_sync();
       return ok;
+    }
+    Rows rw;
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      const int r = 2 * (warp + 8 * i) + (lane >> 4);
+      rw.off[i] = off[min(r, sb - 1)];
+      rw.em[i] = emax[min(r, sb - 1)];
     }
     // warp w: tensor-memory lanes (rows) 32 (w % 4) .. + 31, column chunks of
     // parity w / 4
     const int row = (warp & 3) * 32 + lane;
     const uint32_t tbase = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const bool act = (warp & 3) * 32 < sb;  // (rows past sb hold garbage)
-    auto put = [&](int cc, const int64_t (&v)[32], const float (&low)[32]) {
+    // chunks of 16 columns, shared by the two warps of a lane quadrant
+    auto put = [&](int cc, const int64_t (&v)[16], const uint32_t (&low)[16]) {
       if (row >= sb) return;
-      const int er = emax[row];
+      const int er = emax[row] - 2098;
 #pragma unroll
-      for (int q = 0; q < 32; ++q) {
+      for (int q = 0; q < 16; ++q) {
         const int j = cc + q;
         if (j > row) break;
         // units of level 7 (2^-40 of level 2), then 2^(er + ej - 2098)
-        double g = (double)(v[q] * 256 + __float2int_rn(low[q] * 1099511627776.0f));
-        if (g != 0.0)
-          g = __hiloint2double(__double2hiint(g) + ((er + emax[j] - 2098) << 20), __double2loint(g));
+        const double g = fixed_to_double(
+            v[q] * 256 + __float2int_rn(__uint_as_float(low[q]) * 1099511627776.0f), er + emax[j]);
         double* at = part + (long long)j * sbp + row;
         *at = add ? *at + g : g;
       }
     };
-    auto level = [&](int a, int cc, float scale, int64_t (&v)[32]) {
-      uint32_t x[32];
-      tmem_ld32(tbase + (uint32_t)(SBP * a + cc), x);
+    auto level = [&](int a, int cc, float scale, int64_t (&v)[16]) {
+      uint32_t x[16];
+      tmem_ld16(tbase + (uint32_t)(SBP * a + cc), x);
 #pragma unroll
-      for (int q = 0; q < 32; ++q) v[q] = v[q] * 256 + __float2int_rn(__uint_as_float(x[q]) * scale);
+      for (int q = 0; q < 16; ++q) v[q] = v[q] * 256 + __float2int_rn(__uint_as_float(x[q]) * scale);
+    };
+    const int ccn = (warp & 3) * 32 + 31;  // last column of the quadrant's triangle
+    auto chunks = [&](auto&& f) {
+      if (act)
+        for (int cc = 16 * (warp >> 2); cc < sb && cc <= ccn; cc += 32) f(cc);
     };
     if constexpr (SBP <= 64) {
-      ok = pass<2, 9>(A, off, sb, k0, k1, err, ok);
-      for (int cc = 32 * (warp >> 2); act && cc < sb && cc <= (warp & 3) * 32; cc += 64) {
-        int64_t v[32];
+      ok = pass<2, 9>(A, rw, sb, k0, k1, err, ok);
+      chunks([&](int cc) {
+        int64_t v[16];
 #pragma unroll
-        for (int q = 0; q < 32; ++q) v[q] = 0;
+        for (int q = 0; q < 16; ++q) v[q] = 0;
         level(0, cc, 1.0f, v);
         level(1, cc, 256.0f, v);
         level(2, cc, 65536.0f, v);
         level(3, cc, 16777216.0f, v);
         level(4, cc, 4294967296.0f, v);
-        uint32_t x[32];
-        float low[32];
-        tmem_ld32(tbase + (uint32_t)(SBP * 5 + cc), x);
-#pragma unroll
-        for (int q = 0; q < 32; ++q) low[q] = __uint_as_float(x[q]);
+        uint32_t low[16];
+        tmem_ld16(tbase + (uint32_t)(SBP * 5 + cc), low);
         put(cc, v, low);
-      }
+      });
     } else {
-      // levels 2 .. 5: their integers wait in the thread's own memory
-      int64_t keep[2][32];
-      const int cc0 = 32 * (warp >> 2), ccn = (warp & 3) * 32;
-      ok = pass<2, 5>(A, off, sb, k0, k1, err, ok);
+      // the integers of levels 2 .. 5 wait in the half of the partial that holds
+      // no entry: (row, j) at [row * sbp + j], j < row, and the diagonal in diag
+      int64_t* hold = reinterpret_cast<int64_t*>(part) + (long long)min(row, sb - 1) * sbp;
+      ok = pass<2, 5>(A, rw, sb, k0, k1, err, ok);
+      chunks([&](int cc) {
+        int64_t v[16];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int cc = cc0 + 64 * h;
-        if (act && cc < sb && cc <= ccn) {
+        for (int q = 0; q < 16; ++q) v[q] = 0;
+        level(0, cc, 1.0f, v);
+        level(1, cc, 256.0f, v);
+        level(2, cc, 65536.0f, v);
+        level(3, cc, 16777216.0f, v);
+        if (row < sb) {
 #pragma unroll
-          for (int q = 0; q < 32; ++q) keep[h][q] = 0;
-          level(0, cc, 1.0f, keep[h]);
-          level(1, cc, 256.0f, keep[h]);
-          level(2, cc, 65536.0f, keep[h]);
-          level(3, cc, 16777216.0f, keep[h]);
+          for (int q = 0; q < 16; ++q) {
+            if (cc + q < row) hold[cc + q] = v[q];
+            if (cc + q == row) diag[row] = v[q];
+          }
         }
-      }
+      });
       tc_fence_before();
-      __syncthreads();
-      ok = pass<6, 9>(A, off, sb, k0, k1, err, ok);
+      main_sync();
+      ok = pass<6, 9>(A, rw, sb, k0, k1, err, ok);
+      chunks([&](int cc) {
+        int64_t v[16];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int cc = cc0 + 64 * h;
-        if (act && cc < sb && cc <= ccn) {
-          level(0, cc, 4294967296.0f, keep[h]);
-          uint32_t x[32];
-          float low[32];
-          tmem_ld32(tbase + (uint32_t)(SBP + cc), x);
+        for (int q = 0; q < 16; ++q) v[q] = hold[min(cc + q, SBP - 1)];
 #pragma unroll
-          for (int q = 0; q < 32; ++q) low[q] = __uint_as_float(x[q]);
-          put(cc, keep[h], low);
-        }
-      }
+        for (int q = 0; q < 16; ++q)
+          if (cc + q == row) v[q] = diag[row];
+        level(0, cc, 4294967296.0f, v);
+        uint32_t low[16];
+        tmem_ld16(tbase + (uint32_t)(SBP + cc), low);
+        put(cc, v, low);
+      });
     }
     tc_fence_before();
-    __syncthreads();  // the accumulators are read
+    main_sync();  // the accumulators are read
     return ok;
   }
 };

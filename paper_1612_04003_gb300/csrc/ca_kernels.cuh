@@ -157,7 +157,7 @@ struct Persist64Args {
   float2* Ginv[2];
   double* pvec;
   SolveArgs sa;          // solve constants (idx and delta are set per step); ldr = sbp
-  unsigned* cnt;         // 4 counts, zero on entry
+  unsigned* cnt;         // 6 counts, zero on entry
 };
 // The Gram pass of dense FP64 X alone, sb <= gram64_max_sb(): P <= ceil(K / 32)
 // split-K partials (P x sbp^2, transposed) and projections (P x sbp).

@@ -30,36 +30,43 @@
 
 namespace {
 
-constexpr int kT = 256;      // threads of a CTA
+constexpr int kT = 256;      // main threads of a CTA (the Gram pass, the chain)
+constexpr int kSide = 128;   // side threads of a column CTA (reduction, inverses)
+constexpr int kBarSide = 7, kBarInv = 8;  // named barriers of the side warps
 constexpr int kSmemMax = 200 * 1024;  // dynamic shared memory a launch may ask for
 constexpr int kSmallSB = 16;  // rows of a step the CUDA-core Gram takes
 
-struct Cnt {  // counts in cnt[]
-  enum { G = 0, R = 1, P = 2, D = 3 };
+// Counts in cnt[].  A fast CTA may form the Gram partial of step p + 1 (and its
+// side warps reduce it) before a slow one has done step p, but not that of
+// step p + 2, which follows Delta_p: G and R count even and odd steps apart,
+// each to (p / 2 + 1) times its CTAs.
+struct Cnt {
+  enum { G = 0, R = 2, P = 4, D = 5 };
 };
 
-// thread 0 waits, the CTA follows; false once a wait of the grid gave up
-__device__ __forceinline__ bool cta_wait(const unsigned* p, unsigned target, unsigned* err, bool ok) {
-  int good = ok;
-  if (threadIdx.x == 0 && ok) good = wait_count(p, target, err);
-  return __syncthreads_and(threadIdx.x == 0 ? good : 1) != 0 && ok;
+// thread 0 waits, the main warps follow; false once a wait of the grid gave up
+__device__ __forceinline__ bool main_wait(const unsigned* p, unsigned target, unsigned* err, bool ok) {
+  bool gone = !ok;
+  if (threadIdx.x == 0 && ok) gone = !wait_count(p, target, err);
+  return !main_any(gone);
 }
-__device__ __forceinline__ void cta_count(unsigned* p) {
-  __syncthreads();
+__device__ __forceinline__ void main_count(unsigned* p) {
+  main_sync();
   if (threadIdx.x == 0) {
     __threadfence();
     atomicAdd(p, 1u);
   }
 }
 
-// Row offsets of the sampled rows (element offset, -1: out of range, flagged).
+// Element offsets of the sampled rows (an index out of range is flagged, and
+// row 0 stands in for it).
 __device__ __forceinline__ void row_offsets(const int* idx, int sb, long long N, long long lda,
                                             long long* out, unsigned* err) {
   for (int r = threadIdx.x; r < sb; r += kT) {
     const long long gi = idx[r];
     const bool in = gi >= 0 && gi < N;
     if (!in) ca_flag(err, CA_DEV_ERR_ARG);
-    out[r] = in ? gi * lda : -1;
+    out[r] = in ? gi * lda : 0;
   }
 }
 
@@ -85,14 +92,15 @@ __device__ void gram_small(const double* __restrict__ A, const long long* off, i
     acc[q] = 0.0;
   }
   for (long long kt = k0; kt < k1; kt += 32) {
-    __syncthreads();
+    main_sync();
     const long long k = kt + lane;
 #pragma unroll
     for (int q = 0; q < kSmallSB / 8; ++q) {
       const int r = warp + 8 * q;
-      if (r < sb) tile[r * 33 + lane] = (off[r] >= 0 && k < k1) ? __ldg(A + off[r] + k) : 0.0;
+      const double x = __ldg(A + off[min(r, sb - 1)] + min(k, k1 - 1));
+      if (r < sb) tile[r * 33 + lane] = k < k1 ? x : 0.0;
     }
-    __syncthreads();
+    main_sync();
 #pragma unroll
     for (int q = 0; q < kSlots; ++q) {
       if (32 * q < E) {
@@ -102,11 +110,11 @@ __device__ void gram_small(const double* __restrict__ A, const long long* off, i
       }
     }
   }
-  __syncthreads();
+  main_sync();
 #pragma unroll
   for (int q = 0; q < kSlots; ++q)
     if (lane + 32 * q < E) red[warp * E + lane + 32 * q] = acc[q];
-  __syncthreads();
+  main_sync();
   for (int e = threadIdx.x; e < E; e += kT) {
     double s = red[e];
 #pragma unroll
@@ -117,76 +125,72 @@ __device__ void gram_small(const double* __restrict__ A, const long long* off, i
   }
 }
 
-// Sum over the warp's 32 lanes of RQ values per lane by halving exchanges (RQ
-// + 5 - log2 RQ additions a lane instead of 5 RQ): returns, on lanes whose low
-// bits are zero, the sum of value q = (lane >> 1's bits, most significant
-// first); lane of value q: see the caller.
-template <int RQ>
-__device__ __forceinline__ double halving_sum(double (&y)[RQ], int lane) {
-  int o = 16;
-#pragma unroll
-  for (int w = RQ / 2; w >= 1; w /= 2, o /= 2) {
-    const bool up = lane & o;
-#pragma unroll
-    for (int j = 0; j < w; ++j) {
-      const double keep = up ? y[j + w] : y[j], send = up ? y[j] : y[j + w];
-      y[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-#pragma unroll
-  for (; o >= 1; o /= 2) y[0] += __shfl_xor_sync(0xffffffffu, y[0], o);
-  return y[0];
-}
-
 // v -= cU Yprev^T Delta (psb > 0) and the projection partial p = Y v of the
-// CTA's columns [k0, k1), FP64.  Lane = column of a 32-column tile, warp w the
-// rows w, w + 8, ...; one exchange of the warps' column sums a tile.
+// CTA's columns [k0, k1), FP64.  A warp takes four columns at a time (lane =
+// 4 row group + column, rows g, g + 8, ...): the eight row groups' sums of a
+// column meet by three shuffles, no exchange between warps until the end, and
+// the next four columns load while these are summed.  Bound by the FP64 pipe
+// (2 FMAs a clock and SM): 2 s b K / (2 P) clocks.
+// red: 8 x 8 RQ.
 template <int RQ>
 __device__ void update_project(const Persist64Args& a, const long long* off, const long long* poff,
                                const double* sdl, int sb, int psb, long long k0, long long k1,
-                               double* ured, double* __restrict__ pp) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double pacc[RQ];
+                               double* red, double* __restrict__ pp) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2;
+  double pacc[RQ], y[RQ], x[RQ], vk;
 #pragma unroll
   for (int q = 0; q < RQ; ++q) pacc[q] = 0.0;
-  int par = 0;
-  for (long long kt = k0; kt < k1; kt += 32, par ^= 1) {
-    const long long k = kt + lane;
-    const bool in = k < k1;
-    double y[RQ], u = 0.0;
+  auto rows = [&](const long long* o, int n, long long k, double (&z)[RQ]) {
+    const long long kc = min(k, k1 - 1);  // (unconditional loads, then selects)
 #pragma unroll
-    for (int q = 0; q < RQ; ++q) {
-      const int r = warp + 8 * q;
-      y[q] = (r < sb && in && off[r] >= 0) ? __ldg(a.A + off[r] + k) : 0.0;
-    }
-    double vk = in ? a.v[k] : 0.0;
+    for (int q = 0; q < RQ; ++q) z[q] = __ldg(a.A + o[min(g + 8 * q, n - 1)] + kc);
+#pragma unroll
+    for (int q = 0; q < RQ; ++q)
+      if (g + 8 * q >= n || k >= k1) z[q] = 0.0;
+  };
+  const long long kw = k0 + 4 * warp + (lane & 3);
+  if (psb > 0) rows(poff, psb, kw, x);
+  vk = kw < k1 ? a.v[kw] : 0.0;
+  rows(off, sb, kw, y);
+  for (long long k = kw; k - (lane & 3) < k1; k += 32) {
+    double vn = vk;
+    vk = k + 32 < k1 ? a.v[k + 32] : 0.0;
     if (psb > 0) {
-      double x[RQ];
-#pragma unroll
-      for (int q = 0; q < RQ; ++q) {
-        const int r = warp + 8 * q;
-        x[q] = (r < psb && in && poff[r] >= 0) ? __ldg(a.A + poff[r] + k) : 0.0;
-      }
+      double u = 0.0;
 #pragma unroll
       for (int q = 0; q < RQ; ++q)
-        if (warp + 8 * q < psb) u = fma(x[q], sdl[warp + 8 * q], u);
-      ured[par * 256 + threadIdx.x] = u;
-      __syncthreads();
-      double s = ured[par * 256 + lane];
+        if (8 * q < psb) u = fma(x[q], sdl[g + 8 * q], u);  // (x = 0 past psb)
+      rows(poff, psb, k + 32, x);
 #pragma unroll
-      for (int w = 1; w < 8; ++w) s += ured[par * 256 + 32 * w + lane];
-      vk -= a.cU * s;
-      if (warp == 0 && in) a.v[k] = vk;
+      for (int o = 4; o <= 16; o <<= 1) u += __shfl_xor_sync(0xffffffffu, u, o);
+      vn -= a.cU * u;
+      if (g == 0 && k < k1) a.v[k] = vn;
     }
 #pragma unroll
     for (int q = 0; q < RQ; ++q)
-      if (warp + 8 * q < sb) pacc[q] = fma(y[q], vk, pacc[q]);
+      if (8 * q < sb) pacc[q] = fma(y[q], vn, pacc[q]);
+    rows(off, sb, k + 32, y);
   }
-  const double s = halving_sum<RQ>(pacc, lane);
-  constexpr int low = 32 / RQ;  // lanes holding the same sum
-  const int q = lane / low;      // (the exchanges sort the values by the lane's high bits)
-  const int r = warp + 8 * q;
-  if (lane % low == 0 && r < sb) pp[r] = s;
+  // the four columns' sums of a row, by halving exchanges: lane bit 0 keeps
+  // the upper or lower half of the values, bit 1 a quarter
+#pragma unroll
+  for (int j = 0; j < RQ / 2; ++j) {
+    const double keep = (lane & 1) ? pacc[j + RQ / 2] : pacc[j];
+    pacc[j] = keep + __shfl_xor_sync(0xffffffffu, (lane & 1) ? pacc[j] : pacc[j + RQ / 2], 1);
+  }
+#pragma unroll
+  for (int j = 0; j < RQ / 4; ++j) {
+    const double keep = (lane & 2) ? pacc[j + RQ / 4] : pacc[j];
+    pacc[j] = keep + __shfl_xor_sync(0xffffffffu, (lane & 2) ? pacc[j] : pacc[j + RQ / 4], 2);
+    red[warp * 8 * RQ + g + 8 * (j + (lane & 1) * (RQ / 2) + ((lane >> 1) & 1) * (RQ / 4))] = pacc[j];
+  }
+  main_sync();
+  for (int r = threadIdx.x; r < sb; r += kT) {
+    double t = red[r];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) t += red[w * 8 * RQ + r];
+    pp[r] = t;
+  }
 }
 
 // Shared state of a column CTA's digit Gram; digits_begin / digits_end by all
@@ -194,6 +198,7 @@ __device__ void update_project(const Persist64Args& a, const long long* off, con
 template <int RQ>
 struct DigitShared {
   int emax[8 * RQ];
+  int64_t diag[RQ == 16 ? 128 : 1];
   uint64_t bars[3];
   uint32_t tmem_holder;
 };
@@ -203,6 +208,7 @@ __device__ __forceinline__ void digits_begin(DigitGram<8 * RQ>& dg, DigitShared<
                                             ~uintptr_t(1023));
   dg.bars = sh.bars;
   dg.emax = sh.emax;
+  dg.diag = sh.diag;
   if (threadIdx.x == 0) {
     for (int q = 0; q < 3; ++q) mbar_init(&sh.bars[q], 1);
     fence_mbar_init();
@@ -216,14 +222,14 @@ __device__ __forceinline__ void digits_begin(DigitGram<8 * RQ>& dg, DigitShared<
   }
   fence_proxy_async_smem();
   tc_fence_before();
-  __syncthreads();
+  main_sync();
   tc_fence_after();
   dg.tmem = sh.tmem_holder;
 }
 template <int RQ>
 __device__ __forceinline__ void digits_end(const DigitGram<8 * RQ>& dg) {
   tc_fence_before();
-  __syncthreads();
+  main_sync();
   if (threadIdx.x < 32) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(dg.tmem),
@@ -257,7 +263,7 @@ __global__ void __launch_bounds__(kT, 1)
 k_gram64(Persist64Args a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
   __shared__ long long soff[8 * RQ];
-  __shared__ double ured[2 * kT];
+  __shared__ double ured[64 * RQ];
   __shared__ DigitShared<RQ> sh;
   const int P = (int)gridDim.x, c = blockIdx.x, sb = a.sb, sbp = a.sa.ldr;
   const long long nch = (a.K + 31) / 32;
@@ -265,145 +271,181 @@ k_gram64(Persist64Args a, unsigned* __restrict__ err) {
   DigitGram<8 * RQ> dg;
   if (sb > kSmallSB) digits_begin<RQ>(dg, sh, smem_d);
   row_offsets(a.idx_all, sb, a.N, a.lda, soff, err);
-  __syncthreads();
+  main_sync();
   gram_columns<RQ>(dg, a.A, soff, sb, c0, c1, smem_d, a.part + (long long)c * sbp * sbp, sbp, err, true);
   update_project<RQ>(a, soff, soff, nullptr, sb, 0, c0, c1, ured, a.ppart + (long long)c * sbp);
   if (sb > kSmallSB) digits_end<RQ>(dg);
 }
 
+// p[r] = the sum of the P partials, all threads.  An FP64 addition holds a
+// scheduler for 64 cycles whatever the lanes in use: for few rows a warp sums
+// a row (lanes over the partials), for more the lanes take 32 rows and the
+// warps share the partials (sm: 256 sums).
+__device__ __forceinline__ void sum_rows(const Persist64Args& a, int P, int sbp, int sb, double* sm) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (sb <= 8) {
+    if (warp < sb) {
+      double t = 0.0;
+#pragma unroll 5
+      for (int q = lane; q < P; q += 32) t += __ldcg(a.ppart + (long long)q * sbp + warp);
+      for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) a.pvec[warp] = t;
+    }
+  } else {
+    const int ng = (sb + 31) / 32;             // groups of 32 rows (1 .. 4; three as four)
+    const int gw = ng == 1 ? 8 : ng == 2 ? 4 : 2;  // warps a group
+    const int grp = warp / gw, sub = warp % gw, r = 32 * grp + lane;
+    double t = 0.0;
+    if (r < sb) {
+#pragma unroll 16
+      for (int q = sub; q < P; q += gw) t += __ldcg(a.ppart + (long long)q * sbp + r);
+    }
+    sm[threadIdx.x] = t;
+    main_sync();
+    if (sub == 0 && r < sb) {
+      for (int w = 1; w < gw; ++w) t += sm[threadIdx.x + 32 * w];
+      a.pvec[r] = t;
+    }
+  }
+  main_sync();
+}
+
 template <int BMAX, int DEPTH, int RQ>
-__global__ void __launch_bounds__(kT, 1) k_persist64(Persist64Args a, unsigned* __restrict__ err) {
+__global__ void __launch_bounds__(kT + kSide, 1)
+k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x;
   const int P = (int)gridDim.x - 1, c = blockIdx.x;
   const int sb = a.sb, sbp = a.sa.ldr, npass = a.npass;
   const int b = a.sa.b, s = a.sa.s_cur;
   const long long sq = (long long)sbp * sbp;
   bool ok = true;
-
   if (c == P) {  // ------------------------------------------------ chain CTA
+    if (tid >= kT) return;
+    const int nred = min(P, s + (sb * (sb + 1) / 2 + 63) / 64);  // CTAs that reduce
     for (int p = 0; p < npass; ++p) {
       const long long k = a.k0 + p;
       SolveArgs sa = a.sa;
       sa.idx = a.idx_all + k * sb;
       sa.delta = a.delta2[k & 1];
-      ok = cta_wait(a.cnt + Cnt::R, (unsigned)(P * (p + 1)), err, ok);
-      ok = cta_wait(a.cnt + Cnt::P, (unsigned)(P * (p + 1)), err, ok);
+      ok = main_wait(a.cnt + Cnt::R + (p & 1), (unsigned)(nred * (p / 2 + 1)), err, ok);
+      ok = main_wait(a.cnt + Cnt::P, (unsigned)(P * (p + 1)), err, ok);
       if (!ok) return;
-      // p = sum of the P partials, a warp per row
-      for (int r = warp; r < sb; r += kT / 32) {
-        double t = 0.0;
-        for (int q = lane; q < P; q += 32) t += __ldcg(a.ppart + (long long)q * sbp + r);
-        for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (lane == 0) a.pvec[r] = t;
-      }
-      __syncthreads();
+      sum_rows(a, P, sbp, sb, smem_d);
       chain_la_body<BMAX, DEPTH>(a.Rs[k & 1], a.pvec, a.Ginv[k & 1], sa, err, smem_d);
-      cta_count(a.cnt + Cnt::D);
+      main_count(a.cnt + Cnt::D);
     }
     return;
   }
 
   // --------------------------------------------------------------- column CTA
   __shared__ long long soff[2][8 * RQ];
-  __shared__ double sdl[8 * RQ];
-  __shared__ double ured[2 * kT];
-  __shared__ float2 Mb[256];
-  __shared__ float2 colbuf[66];
+  __shared__ double sdl[8 * RQ];  // zero past the rows
+  __shared__ double ured[64 * RQ];
+  if (tid >= kT) {
+    // side warps: this CTA's share of each step's reduction.  Roles 0 .. s-1
+    // invert a diagonal block, the others take 64 entries each, two threads an
+    // entry
+    __shared__ double red[kSide];
+    __shared__ float2 Mb[256];
+    __shared__ float2 colbuf[66];
+    const int st = tid - kT, ent = st & 63, sub = st >> 6;
+    const float2 cG2 = split_f64(a.sa.cG), cI2 = split_f64(a.sa.cI);
+    const int E = sb * (sb + 1) / 2, nrole = s + (E + 63) / 64;
+    auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"n"(kBarSide), "n"(kSide) : "memory"); };
+    for (int p = 0; p < npass; ++p) {
+      const long long k = a.k0 + p;
+      if (c >= nrole) break;
+      if (st == 0) wait_count(a.cnt + Cnt::G + (p & 1), (unsigned)(P * (p / 2 + 1)), err);
+      sync();
+      const double* part = a.part + (k & 1) * (long long)P * sq;
+      auto sum = [&](int i, int j) {  // this thread's half of entry (i, j)
+        double t = 0.0;
+        const double* src = part + (long long)j * sbp + i;
+#pragma unroll 16
+        for (int q = sub; q < P; q += 2) t += __ldcg(src + q * sq);
+        return t;
+      };
+      for (int role = c; role < nrole; role += P) {
+        if (role < s) {
+          for (int e0 = 0; e0 < b * b; e0 += 64) {
+            const int e = e0 + ent, i = e / b, j = e - i * b;
+            const bool low = e < b * b && i >= j;
+            red[st] = low ? sum(role * b + i, role * b + j) : 0.0;
+            sync();
+            if (st < 64 && low) {
+              float2 m = df_mul(cG2, split_f64(red[st] + red[64 + st]));
+              if (i == j) m = df_add(m, cI2);
+              Mb[i * b + j] = m;
+              Mb[j * b + i] = m;
+            }
+            sync();
+          }
+          float2* out = a.Ginv[k & 1] + (long long)role * b * b;
+          if (b <= 8) {
+            float2 m[1] = {st < b * b ? Mb[st] : make_float2(0.f, 0.f)};
+            if (st < 64) cta_sweep_inverse<1, 64, kBarInv>(m, b, colbuf, out, err, st);
+          } else {
+            float2 m[2];
+            for (int q = 0; q < 2; ++q)
+              m[q] = st + kSide * q < b * b ? Mb[st + kSide * q] : make_float2(0.f, 0.f);
+            cta_sweep_inverse<2, kSide, kBarInv>(m, b, colbuf, out, err, st);
+          }
+        } else {
+          const int e = (role - s) * 64 + ent;
+          int i = 0, j = 0;
+          if (e < E) {  // column-major over the lower triangle: lanes along i
+            int ir, jr;
+            tri_decode(e, ir, jr);
+            i = sb - 1 - jr;
+            j = sb - 1 - ir;
+          }
+          red[st] = e < E ? sum(i, j) : 0.0;
+          sync();
+          if (st < 64 && e < E)
+            a.Rs[k & 1][(long long)j * sbp + i] = df_mul(cG2, split_f64(red[st] + red[64 + st]));
+        }
+        sync();
+      }
+      if (st == 0) {
+        __threadfence();
+        atomicAdd(a.cnt + Cnt::R + (p & 1), 1u);
+      }
+    }
+    return;
+  }
   __shared__ DigitShared<RQ> sh;
   DigitGram<8 * RQ> dg;
   const bool digits = sb > kSmallSB;
   if (digits) digits_begin<RQ>(dg, sh, smem_d);
   const long long nch = (a.K + 31) / 32;
   const long long c0 = nch * c / P * 32, c1 = min(a.K, nch * (c + 1) / P * 32);
-  const float2 cG2 = split_f64(a.sa.cG), cI2 = split_f64(a.sa.cI);
-  const int E = sb * (sb + 1) / 2;
-  // Gram partial of step k0 + p into its parity's buffer, then this CTA's
-  // share of the reduction: roles 0 .. s-1 invert a diagonal block, the others
-  // take 64 entries each, four threads an entry
-  auto gram = [&](int p, const long long* off) {
-    const long long k = a.k0 + p;
-    double* part = a.part + (k & 1) * (long long)P * sq;
+  auto gram = [&](int p, const long long* off) {  // the partial of step k0 + p
+    double* part = a.part + ((a.k0 + p) & 1) * (long long)P * sq;
     ok = gram_columns<RQ>(dg, a.A, off, sb, c0, c1, smem_d, part + c * sq, sbp, err, ok);
-    cta_count(a.cnt + Cnt::G);
-    ok = cta_wait(a.cnt + Cnt::G, (unsigned)(P * (p + 1)), err, ok);
-    if (!ok) return;
-    float2* Rs = a.Rs[k & 1];
-    const int nrole = s + (E + 63) / 64;
-    double* red = smem_d;
-    for (int role = c; role < nrole; role += P) {
-      const int ent = tid & 63, sub = tid >> 6;
-      int i = -1, j = 0;
-      if (role < s) {  // entry (i, j) of block `role`, b <= 8; larger b: loop below
-        for (int e0 = 0; e0 < b * b; e0 += 64) {
-          const int e = e0 + ent;
-          i = e / b;
-          j = e - i * b;
-          double t = 0.0;
-          if (e < b * b && i >= j)
-#pragma unroll 8
-            for (int q = sub; q < P; q += 4)
-              t += __ldcg(part + q * sq + (long long)(role * b + j) * sbp + role * b + i);
-          red[tid] = t;
-          __syncthreads();
-          if (tid < 64 && e < b * b && i >= j) {
-            const double g = (red[tid] + red[64 + tid]) + (red[128 + tid] + red[192 + tid]);
-            float2 m = df_mul(cG2, split_f64(g));
-            if (i == j) m = df_add(m, cI2);
-            Mb[i * b + j] = m;
-            Mb[j * b + i] = m;
-          }
-          __syncthreads();
-        }
-        float2* out = a.Ginv[k & 1] + (long long)role * b * b;
-        float2 m[1] = {tid < b * b ? Mb[tid] : make_float2(0.f, 0.f)};
-        if (b <= 8) {
-          if (tid < 64) cta_sweep_inverse<1, 64>(m, b, colbuf, out, err);
-        } else {
-          cta_sweep_inverse<1>(m, b, colbuf, out, err);
-        }
-        __syncthreads();
-        continue;
-      }
-      const int e = (role - s) * 64 + ent;
-      double t = 0.0;
-      if (e < E) {  // column-major over the lower triangle: lanes along i
-        int ir, jr;
-        tri_decode(e, ir, jr);
-        i = sb - 1 - jr;
-        j = sb - 1 - ir;
-#pragma unroll 8
-        for (int q = sub; q < P; q += 4) t += __ldcg(part + q * sq + (long long)j * sbp + i);
-      }
-      red[tid] = t;
-      __syncthreads();
-      if (tid < 64 && e < E)
-        Rs[(long long)j * sbp + i] =
-            df_mul(cG2, split_f64((red[tid] + red[64 + tid]) + (red[128 + tid] + red[192 + tid])));
-      __syncthreads();
-    }
-    cta_count(a.cnt + Cnt::R);
+    main_count(a.cnt + Cnt::G + (p & 1));
   };
 
   row_offsets(a.idx_all + a.k0 * sb, sb, a.N, a.lda, soff[0], err);
   if (a.prev_sb > 0) row_offsets(a.prev_idx, a.prev_sb, a.N, a.lda, soff[1], err);
-  __syncthreads();
+  main_sync();
   gram(0, soff[0]);
   for (int p = 0; p < npass && ok; ++p) {
     const long long k = a.k0 + p;
     const int psb = p == 0 ? a.prev_sb : sb;
-    if (p > 0) ok = cta_wait(a.cnt + Cnt::D, (unsigned)p, err, ok);
+    if (p > 0) ok = main_wait(a.cnt + Cnt::D, (unsigned)p, err, ok);
     if (!ok) break;
     if (psb > 0) {
-      for (int r = tid; r < psb; r += kT) sdl[r] = __ldcg(a.delta2[(k - 1) & 1] + r);
-      __syncthreads();
+      for (int r = tid; r < 8 * RQ; r += kT)
+        sdl[r] = r < psb ? __ldcg(a.delta2[(k - 1) & 1] + r) : 0.0;
+      main_sync();
     }
     update_project<RQ>(a, soff[p & 1], soff[(p + 1) & 1], sdl, sb, psb, c0, c1, ured,
                        a.ppart + (long long)c * sbp);
-    cta_count(a.cnt + Cnt::P);
+    main_count(a.cnt + Cnt::P);
     if (p + 1 < npass) {
       row_offsets(a.idx_all + (k + 1) * sb, sb, a.N, a.lda, soff[(p + 1) & 1], err);
-      __syncthreads();
+      main_sync();
       gram(p + 1, soff[(p + 1) & 1]);
     }
   }
@@ -434,7 +476,7 @@ int launch64(Kern kern, std::atomic<unsigned long long>& configured, const Persi
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kT);
+  cfg.blockDim = dim3(coop ? kT + kSide : kT);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
