@@ -356,10 +356,9 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
   const int sbp = g.sbp, P = g.P;
   // FP64 X: runs of full steps go to one persistent launch (ca_persist64.cu)
   // of P64 column CTAs, with two sets of partials
-  const long long nch = (K + 31) / 32;
-  const int P64 = (int)std::min<long long>(ctx->num_sms - 1, nch);
-  bool persist64 = ctx->persist && pb.xfmt == CA_DENSE_F64 && !f64solve && P64 >= 1 &&
-                   persist64_fits(b, sbm);
+  const int P64 = pb.xfmt == CA_DENSE_F64 && !f64solve
+                      ? persist64_columns(b, sbm / b, K, ctx->num_sms) : 0;
+  bool persist64 = ctx->persist && P64 > 0;
   const int Pmax = persist64 ? std::max(P, 2 * P64) : P;
   void* part = g.tc ? (void*)cv.take<float>((size_t)P * sbp * sbp)
                     : (void*)cv.take<double>((size_t)Pmax * sbp * sbp);
@@ -469,7 +468,7 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
       pa.pvec = pvec;
       pa.sa = SolveArgs{nullptr, pb.N, b, s, sb, sbp, pb.cG, pb.cI, pb.cP, pb.cY, pb.x, pb.yv, nullptr};
       pa.cnt = ctx->d_cnt;
-      CA_TRY_CUDA(cudaMemsetAsync(ctx->d_cnt, 0, 6 * sizeof(unsigned), ctx->stream));
+      CA_TRY_CUDA(cudaMemsetAsync(ctx->d_cnt, 0, 9 * sizeof(unsigned), ctx->stream));
       prof_mark(ctx, PC_GRAM);
       const int e = launch_persist64(pa, P64, chain_smem(b, sb), ctx->d_err, ctx->stream);
       prof_mark(ctx, PC_GRAM);
@@ -712,7 +711,7 @@ int ca_bcd_init(ca_ctx** out, int device, void* cuda_stream, size_t scratch_byte
     return CA_ERR_CUDA;
   }
   ctx->d_ticket = ctx->d_err + 32;
-  ctx->d_cnt = ctx->d_err + 48;
+  ctx->d_cnt = ctx->d_err + 40;
   cudaMemset(ctx->d_err, 0, 256);
   if (set_solve_smem_limit(kSolveSmemMax) != 0) {
     cudaGetLastError();

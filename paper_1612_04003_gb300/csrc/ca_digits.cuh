@@ -1,4 +1,4 @@
-// ca_digits.cuh -- the FP64 Gram Y Y^T of sampled rows on the BF16 tensor
+// ca_digits.cuh -- the FP64 Gram Y Y^T of sampled rows on the FP16 tensor
 // cores, by exact digit products (the error-free splitting of Ozaki, Ogita,
 // Oishi and Rump, Numer. Algorithms 59, 2012, with integer digits and FP32
 // accumulation as Mukunoki, Ozaki, Ogita and Imamura, ISC 2020, use it).
@@ -41,6 +41,12 @@ __device__ __forceinline__ bool main_any(bool v) {
   return r != 0;
 }
 
+__device__ __forceinline__ uint32_t h2_sub(uint32_t a, uint32_t b) {
+  uint32_t d;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+
 // v 2^e, rounded to nearest, on the integer pipe (a conversion of the FP64
 // pipe holds a scheduler for 64 cycles); the result is a normal number.
 __device__ __forceinline__ double fixed_to_double(int64_t v, int e) {
@@ -58,18 +64,20 @@ __device__ __forceinline__ double fixed_to_double(int64_t v, int e) {
 }
 
 // SBP rows (32, 64 or 128), the eight main warps of a CTA.  Tensor memory: one
-// accumulator of SBP columns a level.  SBP = 128 holds four of the six at
+// accumulator of SBP columns a level.  SBP = 128 holds four of the eight at
 // once: levels 2 .. 5, then (the columns converted again) levels 6 .. 9.
 template <int SBP>
 struct DigitGram {
-  static constexpr int kSlice = SBP * 64;              // 32 BF16 digits a row
+  static constexpr int kSlice = SBP * 64;              // 32 FP16 digits a row
   static constexpr int kStage = kDigits * kSlice;
   // the M = 128 MMA reads 128 rows of a slice: slack behind the last one
   static constexpr int kSmem = 2 * kStage + (128 - (SBP < 128 ? SBP : 128)) * 64 + 1024;
   static constexpr int kTmemCols = SBP == 32 ? 256 : 512;
 
   unsigned char* dig;   // 1024-byte aligned digits of two stages
-  uint64_t* bars;       // [0], [1]: stage buffer read by the MMAs; [2]: all MMAs
+  uint64_t* bars;       // [0], [1]: stage buffer read by the MMAs; [2]: all MMAs of a
+                        // pass; [3], [4]: stage buffer converted (a warp each)
+  uint32_t* cmd;        // [2]: what the MMA warp does with each buffer
   uint32_t tmem;
   int* emax;            // [SBP] largest biased exponent of each row
   int64_t* diag;        // [SBP] (SBP = 128)
@@ -125,40 +133,75 @@ struct DigitGram {
       const uint32_t at = (uint32_t)((r >> 3) * 512 + (r & 7) * 64 +
                                      (((l >> 2) ^ ((r >> 1) & 3)) << 4) + (l & 3) * 4);
 #pragma unroll
-      for (int d = 0; d < ND; ++d) {  // digit d + 1, scaled by 256^-d
-        const uint32_t sel = d == 0 ? 0x7632u : d == 1 ? 0x7651u : d == 2 ? 0x7650u
-                             : d == 3 ? 0x7653u : d == 4 ? 0x7652u : d == 5 ? 0x7651u : 0x7650u;
-        const float w = __uint_as_float((uint32_t)(127 - 8 * d) << 23);
-        float f[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e)  // 2^23 + byte, less 2^23 + 128
-          f[e] = fmaf(__uint_as_float(__byte_perm(d < 3 ? hi[e] : lo[e], 0x4B000000u, sel)), w,
-                      -8388736.0f * w);
-        *reinterpret_cast<uint32_t*>(buf + d * kSlice + at) = bf16x2_rn(f[0], f[1]);
+      for (int d = 0; d < ND; ++d) {  // digit d + 1 of both columns
+        // byte 6 - d of the two (the first digit has nine bits) under the FP16
+        // exponent of 1024, less 1024 + 128
+        const uint32_t w0 = d < 3 ? hi[0] : lo[0], w1 = d < 3 ? hi[1] : lo[1];
+        const uint32_t sel = d == 0 ? 0x7632u : d == 1 ? 0x0501u : d == 2 ? 0x0400u
+                             : d == 3 ? 0x0703u : d == 4 ? 0x0602u : d == 5 ? 0x0501u : 0x0400u;
+        const uint32_t f = (__byte_perm(w0, w1, sel) & (d == 0 ? 0x01ff01ffu : 0x00ff00ffu)) | 0x64006400u;
+        *reinterpret_cast<uint32_t*>(buf + d * kSlice + at) = h2_sub(f, 0x64806480u);
       }
     }
   }
 
   // MMAs of one stage: pairs (i, j) of digits with level i + j in [L0, L1],
-  // level l into accumulator min(l, 7) - L0
+  // level l into accumulator l - L0
   template <int L0, int L1>
-  __device__ __forceinline__ void issue(uint32_t buf, int nb, bool first) const {
-    const uint32_t id = idesc_bf16(128, nb);
+  __device__ __forceinline__ void issue(uint32_t buf, int nb, bool first, bool half) const {
+    const uint32_t id = idesc_f16(128, nb);
     const uint64_t base = sw64_kmajor_desc(buf);  // (the address field is in 16-byte units)
 #pragma unroll
     for (int l = L0; l <= L1; ++l) {
-      const uint32_t d = tmem + (uint32_t)(SBP * ((l < 7 ? l : 7) - L0));
+      const uint32_t d = tmem + (uint32_t)(SBP * (l - L0));
 #pragma unroll
       for (int i = 1; i <= kDigits; ++i) {
         const int j = l - i;
         if (j < 1 || j > kDigits) continue;
-        const bool start = l <= 7 && i == (l > 7 ? l - 7 : 1);
+        const bool start = i == (l > 8 ? l - kDigits : 1);
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk)
-          mma_bf16(d, base + (uint32_t)(((i - 1) * kSlice + kk * 32) >> 4),
-                   base + (uint32_t)(((j - 1) * kSlice + kk * 32) >> 4), id,
-                   start && kk == 0 ? (first ? 0u : 1u) : 1u);
+          if (kk == 0 || !half)
+            mma_bf16(d, base + (uint32_t)(((i - 1) * kSlice + kk * 32) >> 4),
+                     base + (uint32_t)(((j - 1) * kSlice + kk * 32) >> 4), id,
+                     start && kk == 0 ? (first ? 0u : 1u) : 1u);
       }
+    }
+  }
+
+  // The MMA warp (a warp of its own: an issue waits until the tensor pipe takes
+  // it, which in a converting warp held the conversion of the next stage):
+  // stages in order until stop().
+  static constexpr uint32_t kFirst = 16u, kLast = 32u, kStop = 64u, kHalf = 128u;
+  __device__ void mma_loop(unsigned* err) const {
+    for (uint32_t g = 0;; ++g) {
+      const uint32_t bi = g & 1;
+      if (!mbar_wait_grid(&bars[3 + bi], (g >> 1) & 1, err)) return;
+      const uint32_t c = *(volatile uint32_t*)&cmd[bi];
+      if (c & kStop) return;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint32_t buf = smem_u32(dig + bi * kStage);
+        const int nb = (int)(c >> 8);
+        const bool first = c & kFirst, half = c & kHalf;  // (half: at most 16 columns)
+        if constexpr (SBP <= 64) {
+          issue<2, 9>(buf, nb, first, half);
+        } else {
+          if ((c & 3u) == 1u) issue<2, 5>(buf, nb, first, half);
+          else issue<6, 9>(buf, nb, first, half);
+        }
+        mma_commit(&bars[bi]);
+        if (c & kLast) mma_commit(&bars[2]);
+      }
+      __syncwarp();
+    }
+  }
+  // ends mma_loop (every pass so far is complete)
+  __device__ void stop() {
+    main_sync();
+    if (threadIdx.x == 0) {
+      cmd[gt & 1] = kStop;
+      for (int q = 0; q < 8; ++q) mbar_arrive(&bars[3 + (gt & 1)]);
     }
   }
 
@@ -175,20 +218,13 @@ struct DigitGram {
       if (gt >= 2 && ok) ok = mbar_wait_grid(&bars[bi], ((gt >> 1) - 1) & 1, err);
       convert<(L1 - 1 < kDigits ? L1 - 1 : kDigits)>(rw, x, buf);
       load(A, rw, k + 32, k1, x);  // (lands while the MMAs of this stage run)
+      if (threadIdx.x == 0)
+        cmd[bi] = (uint32_t)(L0 == 6 ? 2 : (L1 == 5 ? 1 : 0)) | (k == k0 ? kFirst : 0u) |
+                  (k + 32 >= k1 ? kLast : 0u) | (k + 16 >= k1 ? kHalf : 0u) | (uint32_t)nb << 8;
       fence_proxy_async_smem();
       tc_fence_before();
-      main_sync();
-      // (a warp-uniform branch and one elected lane: the descriptors stay in
-      // uniform registers)
-      if (__shfl_sync(0xffffffffu, threadIdx.x >> 5, 0) == 0) {
-        tc_fence_after();
-        if (elect_one()) {
-          issue<L0, L1>(smem_u32(buf), nb, k == k0);
-          mma_commit(&bars[bi]);
-          if (k + 32 >= k1) mma_commit(&bars[2]);
-        }
-        __syncwarp();
-      }
+      __syncwarp();
+      if ((threadIdx.x & 31) == 0) mbar_arrive(&bars[3 + bi]);
     }
     if (ok) ok = mbar_wait_grid(&bars[2], ph & 1, err);
     ++ph;
@@ -254,7 +290,20 @@ struct DigitGram {
     const uint32_t tbase = tmem + ((uint32_t)((warp & 3) * 32) << 16);
     const bool act = (warp & 3) * 32 < sb;  // (rows past sb hold garbage)
     // chunks of 16 columns, shared by the two warps of a lane quadrant
-    auto put = [&](int cc, const int64_t (&v)[16], const uint32_t (&low)[16]) {
+    // levels 7 .. 9 of a chunk, in units of level 7
+    auto lows = [&](int a, int cc, float (&low)[16]) {
+      uint32_t x[16];
+      tmem_ld16(tbase + (uint32_t)(SBP * a + cc), x);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) low[q] = __uint_as_float(x[q]);
+      tmem_ld16(tbase + (uint32_t)(SBP * (a + 1) + cc), x);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) low[q] = fmaf(__uint_as_float(x[q]), 0x1p-8f, low[q]);
+      tmem_ld16(tbase + (uint32_t)(SBP * (a + 2) + cc), x);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) low[q] = fmaf(__uint_as_float(x[q]), 0x1p-16f, low[q]);
+    };
+    auto put = [&](int cc, const int64_t (&v)[16], const float (&low)[16]) {
       if (row >= sb) return;
       const int er = emax[row] - 2098;
 #pragma unroll
@@ -262,17 +311,16 @@ struct DigitGram {
         const int j = cc + q;
         if (j > row) break;
         // units of level 7 (2^-40 of level 2), then 2^(er + ej - 2098)
-        const double g = fixed_to_double(
-            v[q] * 256 + __float2int_rn(__uint_as_float(low[q]) * 1099511627776.0f), er + emax[j]);
+        const double g = fixed_to_double(v[q] * 256 + __float2int_rn(low[q]), er + emax[j]);
         double* at = part + (long long)j * sbp + row;
         *at = add ? *at + g : g;
       }
     };
-    auto level = [&](int a, int cc, float scale, int64_t (&v)[16]) {
+    auto level = [&](int a, int cc, int64_t (&v)[16]) {
       uint32_t x[16];
       tmem_ld16(tbase + (uint32_t)(SBP * a + cc), x);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) v[q] = v[q] * 256 + __float2int_rn(__uint_as_float(x[q]) * scale);
+      for (int q = 0; q < 16; ++q) v[q] = v[q] * 256 + __float2int_rn(__uint_as_float(x[q]));
     };
     const int ccn = (warp & 3) * 32 + 31;  // last column of the quadrant's triangle
     auto chunks = [&](auto&& f) {
@@ -285,13 +333,13 @@ struct DigitGram {
         int64_t v[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) v[q] = 0;
-        level(0, cc, 1.0f, v);
-        level(1, cc, 256.0f, v);
-        level(2, cc, 65536.0f, v);
-        level(3, cc, 16777216.0f, v);
-        level(4, cc, 4294967296.0f, v);
-        uint32_t low[16];
-        tmem_ld16(tbase + (uint32_t)(SBP * 5 + cc), low);
+        level(0, cc, v);
+        level(1, cc, v);
+        level(2, cc, v);
+        level(3, cc, v);
+        level(4, cc, v);
+        float low[16];
+        lows(5, cc, low);
         put(cc, v, low);
       });
     } else {
@@ -303,10 +351,10 @@ struct DigitGram {
         int64_t v[16];
 #pragma unroll
         for (int q = 0; q < 16; ++q) v[q] = 0;
-        level(0, cc, 1.0f, v);
-        level(1, cc, 256.0f, v);
-        level(2, cc, 65536.0f, v);
-        level(3, cc, 16777216.0f, v);
+        level(0, cc, v);
+        level(1, cc, v);
+        level(2, cc, v);
+        level(3, cc, v);
         if (row < sb) {
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
@@ -325,9 +373,9 @@ struct DigitGram {
 #pragma unroll
         for (int q = 0; q < 16; ++q)
           if (cc + q == row) v[q] = diag[row];
-        level(0, cc, 4294967296.0f, v);
-        uint32_t low[16];
-        tmem_ld16(tbase + (uint32_t)(SBP + cc), low);
+        level(0, cc, v);
+        float low[16];
+        lows(1, cc, low);
         put(cc, v, low);
       });
     }

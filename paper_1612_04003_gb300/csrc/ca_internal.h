@@ -46,7 +46,7 @@ struct ca_ctx {
   unsigned* d_err = nullptr;     // device error word
   unsigned* d_ticket = nullptr;  // count of the reducing CTAs of the reduce/solve kernel
                                  // (d_err + 32; both cleared where a call starts)
-  unsigned* d_cnt = nullptr;     // 6 counts of the persistent solves (d_err + 48; cleared
+  unsigned* d_cnt = nullptr;     // counts of the persistent solves (d_err + 40 .. 48; cleared
                                  // before each persistent launch); d_err + 56: whether
                                  // the x of a recomputation has a nonzero entry
   unsigned* h_err = nullptr;     // pinned copy (128 bytes: error word; check sums at +32)

@@ -137,8 +137,7 @@ int launch_persist(const PersistArgs& a, int grid, int sbp, int mode, unsigned* 
 int persist_load_ring(int sbp, int mode);
 
 // Consecutive outer steps k0 .. k0+npass-1 of one dense FP64 solve in one
-// persistent cooperative launch of P column CTAs + 1 chain CTA
-// (ca_persist64.cu).
+// persistent cooperative launch (ca_persist64.cu).
 struct Persist64Args {
   const double* A;       // N x K row-major, leading dimension lda
   long long lda, N, K;
@@ -157,7 +156,7 @@ struct Persist64Args {
   float2* Ginv[2];
   double* pvec;
   SolveArgs sa;          // solve constants (idx and delta are set per step); ldr = sbp
-  unsigned* cnt;         // 6 counts, zero on entry
+  unsigned* cnt;         // 9 counts, zero on entry
 };
 // The Gram pass of dense FP64 X alone, sb <= gram64_max_sb(): P <= ceil(K / 32)
 // split-K partials (P x sbp^2, transposed) and projections (P x sbp).
@@ -165,8 +164,9 @@ int gram64_max_sb();
 int launch_gram64(const double* A, long long lda, long long N, long long K, const int* idx, int sb,
                   const double* v, int P, int sbp, double* part, double* ppart, unsigned* err,
                   cudaStream_t st);
-bool persist64_fits(int b, int sb);
-// P <= number of SMs - 1 and <= ceil(K / 32).  Returns a cudaError_t.
+// Column CTAs of the persistent launch: 0 where it does not cover the call.
+int persist64_columns(int b, int s, long long K, int num_sms);
+// P = persist64_columns().  Returns a cudaError_t.
 int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,
                      cudaStream_t st);
 

@@ -4,15 +4,19 @@
 // The Gram of step k+1 needs only the sampled indices, so it is formed and
 // reduced while the chain of step k runs; what depends on Delta_k is the
 // deferred update of v and the projection p_{k+1} = Y_{k+1} v, one sweep over
-// the CTA's own columns.  Grid = P column CTAs + 1 chain CTA, all resident
-// (cooperative launch); every wait is bounded and gives up once any wait of
-// the grid has.
-//   column CTA, step k:  wait Delta_{k-1} -> v -= cU Y_{k-1}^T Delta_{k-1} on
-//     its columns, p partial -> count P  |  Gram partial of step k+1 -> count
-//     G -> all G: its share of the reduction (Rs, inverted diagonal blocks)
-//     -> count R
-//   chain CTA, step k:   counts R and P of step k -> p summed -> the s
-//     dependent solves -> Delta_k -> count D
+// the CTA's own columns.  Grid = P column CTAs + up to 16 inverse CTAs + 1
+// chain CTA, all resident (cooperative launch); every wait is bounded and gives
+// up once any wait of the grid has.
+//   column CTA, step k, main warps: wait Delta_{k-1} -> v -= cU Y_{k-1}^T
+//     Delta_{k-1} on its columns, p partial -> count P -> Gram partial of step
+//     k+1 -> count G; side warps: all G -> its share of the entries summed (Rs,
+//     the diagonal blocks) -> count E (s b >= 64: then all P -> its rows of p
+//     -> count Q)
+//   inverse CTA, step k:  all E -> its diagonal blocks inverted -> count R
+//   chain CTA, step k:    all R and P (or Q) -> p -> the s dependent solves ->
+//     Delta_k -> count D
+// (an inverse CTA that sums its blocks from the partials itself took 11.5 us
+// after the last partial of X^T 1500 x 8190, s b = 32; through E 8.3 us)
 // Buffers written ahead (partials, Rs, Ginv) alternate by step parity: the
 // buffers of step k+1 were last read for step k-1, whose Delta this CTA has
 // seen before it writes them.
@@ -31,18 +35,22 @@
 namespace {
 
 constexpr int kT = 256;      // main threads of a CTA (the Gram pass, the chain)
-constexpr int kSide = 128;   // side threads of a column CTA (reduction, inverses)
-constexpr int kBarSide = 7, kBarInv = 8;  // named barriers of the side warps
+constexpr int kSide = 96;    // side threads of a column CTA (reduction); twelve warps in all
+                             // leave 168 registers a thread
+constexpr int kMma = 32;     // and the warp that issues the MMAs of the digit Gram
+constexpr int kBarSide = 7;  // named barrier of the side warps
 constexpr int kSmemMax = 200 * 1024;  // dynamic shared memory a launch may ask for
 constexpr int kSmallSB = 16;  // rows of a step the CUDA-core Gram takes
 
 // Counts in cnt[].  A fast CTA may form the Gram partial of step p + 1 (and its
 // side warps reduce it) before a slow one has done step p, but not that of
-// step p + 2, which follows Delta_p: G and R count even and odd steps apart,
+// step p + 2, which follows Delta_p: G, E and R count even and odd steps apart,
 // each to (p / 2 + 1) times its CTAs.
 struct Cnt {
-  enum { G = 0, R = 2, P = 4, D = 5 };
+  enum { G = 0, E = 2, R = 4, P = 6, Q = 7, D = 8 };
 };
+constexpr int kMaxInv = 16;  // inverse CTAs
+constexpr int kRowsSB = 64;  // s b from which the column CTAs sum p
 
 // thread 0 waits, the main warps follow; false once a wait of the grid gave up
 __device__ __forceinline__ bool main_wait(const unsigned* p, unsigned target, unsigned* err, bool ok) {
@@ -199,9 +207,15 @@ template <int RQ>
 struct DigitShared {
   int emax[8 * RQ];
   int64_t diag[RQ == 16 ? 128 : 1];
-  uint64_t bars[3];
+  uint64_t bars[5];
+  uint32_t cmd[2];
   uint32_t tmem_holder;
 };
+// digits_begin, digits_end: the main warps and the MMA warp together (named
+// barrier 9).
+__device__ __forceinline__ void digit_sync() {
+  asm volatile("bar.sync 9, %0;" ::"n"(kT + kMma) : "memory");
+}
 template <int RQ>
 __device__ __forceinline__ void digits_begin(DigitGram<8 * RQ>& dg, DigitShared<RQ>& sh, void* smem) {
   dg.dig = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem) + 1023) &
@@ -209,8 +223,9 @@ __device__ __forceinline__ void digits_begin(DigitGram<8 * RQ>& dg, DigitShared<
   dg.bars = sh.bars;
   dg.emax = sh.emax;
   dg.diag = sh.diag;
+  dg.cmd = sh.cmd;
   if (threadIdx.x == 0) {
-    for (int q = 0; q < 3; ++q) mbar_init(&sh.bars[q], 1);
+    for (int q = 0; q < 5; ++q) mbar_init(&sh.bars[q], q < 3 ? 1 : 8);
     fence_mbar_init();
   }
   if (threadIdx.x < 32) {
@@ -222,14 +237,14 @@ __device__ __forceinline__ void digits_begin(DigitGram<8 * RQ>& dg, DigitShared<
   }
   fence_proxy_async_smem();
   tc_fence_before();
-  main_sync();
+  digit_sync();
   tc_fence_after();
   dg.tmem = sh.tmem_holder;
 }
 template <int RQ>
 __device__ __forceinline__ void digits_end(const DigitGram<8 * RQ>& dg) {
   tc_fence_before();
-  main_sync();
+  digit_sync();
   if (threadIdx.x < 32) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(dg.tmem),
@@ -259,22 +274,33 @@ __device__ __forceinline__ bool gram_columns(DigitGram<8 * RQ>& dg, const double
 // The Gram pass alone (steps a2+a3): split-K partials over gridDim.x CTAs and
 // the projection partials on v.
 template <int RQ>
-__global__ void __launch_bounds__(kT, 1)
+__global__ void __launch_bounds__(kT + kMma, 1)
 k_gram64(Persist64Args a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
   __shared__ long long soff[8 * RQ];
   __shared__ double ured[64 * RQ];
   __shared__ DigitShared<RQ> sh;
   const int P = (int)gridDim.x, c = blockIdx.x, sb = a.sb, sbp = a.sa.ldr;
-  const long long nch = (a.K + 31) / 32;
-  const long long c0 = nch * c / P * 32, c1 = min(a.K, nch * (c + 1) / P * 32);
+  const long long nch = (a.K + 15) / 16;
+  const long long c0 = nch * c / P * 16, c1 = min(a.K, nch * (c + 1) / P * 16);
   DigitGram<8 * RQ> dg;
-  if (sb > kSmallSB) digits_begin<RQ>(dg, sh, smem_d);
+  const bool digits = sb > kSmallSB;
+  if (digits) digits_begin<RQ>(dg, sh, smem_d);
+  if (threadIdx.x >= kT) {
+    if (digits) {
+      dg.mma_loop(err);
+      digits_end<RQ>(dg);
+    }
+    return;
+  }
   row_offsets(a.idx_all, sb, a.N, a.lda, soff, err);
   main_sync();
   gram_columns<RQ>(dg, a.A, soff, sb, c0, c1, smem_d, a.part + (long long)c * sbp * sbp, sbp, err, true);
   update_project<RQ>(a, soff, soff, nullptr, sb, 0, c0, c1, ured, a.ppart + (long long)c * sbp);
-  if (sb > kSmallSB) digits_end<RQ>(dg);
+  if (digits) {
+    dg.stop();
+    digits_end<RQ>(dg);
+  }
 }
 
 // p[r] = the sum of the P partials, all threads.  An FP64 addition holds a
@@ -292,8 +318,7 @@ __device__ __forceinline__ void sum_rows(const Persist64Args& a, int P, int sbp,
       if (lane == 0) a.pvec[warp] = t;
     }
   } else {
-    const int ng = (sb + 31) / 32;             // groups of 32 rows (1 .. 4; three as four)
-    const int gw = ng == 1 ? 8 : ng == 2 ? 4 : 2;  // warps a group
+    const int gw = sb <= 32 ? 8 : 4;  // warps a group of 32 rows
     const int grp = warp / gw, sub = warp % gw, r = 32 * grp + lane;
     double t = 0.0;
     if (r < sb) {
@@ -310,30 +335,57 @@ __device__ __forceinline__ void sum_rows(const Persist64Args& a, int P, int sbp,
   main_sync();
 }
 
+// Entries of the lower triangle a reducing CTA takes: as few as spread the E
+// entries over the P CTAs (a power of two, 4 .. 32).
+__device__ __forceinline__ int entries_a_role(int E, int P) {
+  int epr = 4;
+  while (epr < 32 && epr * P < E) epr *= 2;
+  return epr;
+}
+
 template <int BMAX, int DEPTH, int RQ>
-__global__ void __launch_bounds__(kT + kSide, 1)
+__global__ void __launch_bounds__(kT + kMma + kSide, 1)
 k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
   const int tid = threadIdx.x;
-  const int P = (int)gridDim.x - 1, c = blockIdx.x;
   const int sb = a.sb, sbp = a.sa.ldr, npass = a.npass;
   const int b = a.sa.b, s = a.sa.s_cur;
+  const int ninv = min(s, kMaxInv), P = (int)gridDim.x - 1 - ninv, c = blockIdx.x;
   const long long sq = (long long)sbp * sbp;
+  const int E = sb * (sb + 1) / 2, epr = entries_a_role(E, P);
+  const int nrole = (E + epr - 1) / epr, nred = min(P, nrole);  // roles and CTAs that reduce
   bool ok = true;
-  if (c == P) {  // ------------------------------------------------ chain CTA
+
+  if (c == P + ninv) {  // ----------------------------------------- chain CTA
     if (tid >= kT) return;
-    const int nred = min(P, s + (sb * (sb + 1) / 2 + 63) / 64);  // CTAs that reduce
     for (int p = 0; p < npass; ++p) {
       const long long k = a.k0 + p;
       SolveArgs sa = a.sa;
       sa.idx = a.idx_all + k * sb;
       sa.delta = a.delta2[k & 1];
-      ok = main_wait(a.cnt + Cnt::R + (p & 1), (unsigned)(nred * (p / 2 + 1)), err, ok);
-      ok = main_wait(a.cnt + Cnt::P, (unsigned)(P * (p + 1)), err, ok);
+      ok = main_wait(a.cnt + Cnt::R + (p & 1), (unsigned)(ninv * (p / 2 + 1)), err, ok);
+      ok = sb >= kRowsSB ? main_wait(a.cnt + Cnt::Q, (unsigned)(min(P, sb) * (p + 1)), err, ok)
+                         : main_wait(a.cnt + Cnt::P, (unsigned)(P * (p + 1)), err, ok);
       if (!ok) return;
-      sum_rows(a, P, sbp, sb, smem_d);
+      if (sb < kRowsSB) sum_rows(a, P, sbp, sb, smem_d);
       chain_la_body<BMAX, DEPTH>(a.Rs[k & 1], a.pvec, a.Ginv[k & 1], sa, err, smem_d);
       main_count(a.cnt + Cnt::D);
+    }
+    return;
+  }
+
+  if (c >= P) {  // ------------------------------------------------ inverse CTA
+    if (tid >= kT) return;
+    __shared__ float2 colbuf[66];
+    for (int p = 0; p < npass && ok; ++p) {
+      ok = main_wait(a.cnt + Cnt::E + (p & 1), (unsigned)(nred * (p / 2 + 1)), err, ok);
+      for (int j = c - P; j < s; j += ninv) {  // (each block replaced by its inverse)
+        float2* out = a.Ginv[(a.k0 + p) & 1] + (long long)j * b * b;
+        float2 m[1] = {tid < b * b ? __ldcg(out + tid) : make_float2(0.f, 0.f)};
+        if (BMAX > 8) cta_sweep_inverse<1, kT, 8>(m, b, colbuf, out, err, tid);
+        else if (tid < 64) cta_sweep_inverse<1, 64, 8>(m, b, colbuf, out, err, tid);
+      }
+      main_count(a.cnt + Cnt::R + (p & 1));
     }
     return;
   }
@@ -342,74 +394,70 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   __shared__ long long soff[2][8 * RQ];
   __shared__ double sdl[8 * RQ];  // zero past the rows
   __shared__ double ured[64 * RQ];
-  if (tid >= kT) {
-    // side warps: this CTA's share of each step's reduction.  Roles 0 .. s-1
-    // invert a diagonal block, the others take 64 entries each, two threads an
-    // entry
+  if (tid >= kT + kMma) {
+    // side warps: this CTA's share of each step's reduction, epr entries a role,
+    // 96 / epr threads an entry
     __shared__ double red[kSide];
-    __shared__ float2 Mb[256];
-    __shared__ float2 colbuf[66];
-    const int st = tid - kT, ent = st & 63, sub = st >> 6;
+    const int st = tid - kT - kMma, sw = st >> 5, lane = st & 31;
     const float2 cG2 = split_f64(a.sa.cG), cI2 = split_f64(a.sa.cI);
-    const int E = sb * (sb + 1) / 2, nrole = s + (E + 63) / 64;
     auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"n"(kBarSide), "n"(kSide) : "memory"); };
+    auto count = [&](unsigned* p) {
+      sync();
+      if (st == 0) {
+        __threadfence();
+        atomicAdd(p, 1u);
+      }
+    };
     for (int p = 0; p < npass; ++p) {
       const long long k = a.k0 + p;
-      if (c >= nrole) break;
-      if (st == 0) wait_count(a.cnt + Cnt::G + (p & 1), (unsigned)(P * (p / 2 + 1)), err);
-      sync();
-      const double* part = a.part + (k & 1) * (long long)P * sq;
-      auto sum = [&](int i, int j) {  // this thread's half of entry (i, j)
-        double t = 0.0;
-        const double* src = part + (long long)j * sbp + i;
-#pragma unroll 16
-        for (int q = sub; q < P; q += 2) t += __ldcg(src + q * sq);
-        return t;
-      };
-      for (int role = c; role < nrole; role += P) {
-        if (role < s) {
-          for (int e0 = 0; e0 < b * b; e0 += 64) {
-            const int e = e0 + ent, i = e / b, j = e - i * b;
-            const bool low = e < b * b && i >= j;
-            red[st] = low ? sum(role * b + i, role * b + j) : 0.0;
-            sync();
-            if (st < 64 && low) {
-              float2 m = df_mul(cG2, split_f64(red[st] + red[64 + st]));
-              if (i == j) m = df_add(m, cI2);
-              Mb[i * b + j] = m;
-              Mb[j * b + i] = m;
-            }
-            sync();
-          }
-          float2* out = a.Ginv[k & 1] + (long long)role * b * b;
-          if (b <= 8) {
-            float2 m[1] = {st < b * b ? Mb[st] : make_float2(0.f, 0.f)};
-            if (st < 64) cta_sweep_inverse<1, 64, kBarInv>(m, b, colbuf, out, err, st);
-          } else {
-            float2 m[2];
-            for (int q = 0; q < 2; ++q)
-              m[q] = st + kSide * q < b * b ? Mb[st + kSide * q] : make_float2(0.f, 0.f);
-            cta_sweep_inverse<2, kSide, kBarInv>(m, b, colbuf, out, err, st);
-          }
-        } else {
-          const int e = (role - s) * 64 + ent;
+      if (c < nrole) {
+        if (st == 0) wait_count(a.cnt + Cnt::G + (p & 1), (unsigned)(P * (p / 2 + 1)), err);
+        sync();
+        const double* part = a.part + (k & 1) * (long long)P * sq;
+        float2* Gi = a.Ginv[k & 1];
+        const int en = lane & (epr - 1), wsub = 32 / epr;  // threads of an entry in a warp
+        for (int role = c; role < nrole; role += P) {
+          const int e = role * epr + en;
           int i = 0, j = 0;
+          double t = 0.0;
           if (e < E) {  // column-major over the lower triangle: lanes along i
             int ir, jr;
             tri_decode(e, ir, jr);
             i = sb - 1 - jr;
             j = sb - 1 - ir;
+            const double* src = part + (long long)j * sbp + i;
+#pragma unroll 16
+            for (int q = sw * wsub + lane / epr; q < P; q += 3 * wsub) t += __ldcg(src + q * sq);
           }
-          red[st] = e < E ? sum(i, j) : 0.0;
+          for (int o = 16; o >= epr; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+          red[st] = t;
           sync();
-          if (st < 64 && e < E)
-            a.Rs[k & 1][(long long)j * sbp + i] = df_mul(cG2, split_f64(red[st] + red[64 + st]));
+          if (st < epr && e < E) {
+            float2 g = df_mul(cG2, split_f64((t + red[32 + st]) + red[64 + st]));
+            const int bj = j / b, ii = i - bj * b, jj = j - bj * b;
+            if (ii < b) {  // diagonal block bj: Gamma, for its inverse
+              if (i == j) g = df_add(g, cI2);
+              Gi[((long long)bj * b + ii) * b + jj] = g;
+              Gi[((long long)bj * b + jj) * b + ii] = g;
+            } else {
+              a.Rs[k & 1][(long long)j * sbp + i] = g;
+            }
+          }
+          sync();
         }
-        sync();
+        count(a.cnt + Cnt::E + (p & 1));
       }
-      if (st == 0) {
-        __threadfence();
-        atomicAdd(a.cnt + Cnt::R + (p & 1), 1u);
+      if (sb >= kRowsSB && c < sb) {  // rows c, c + P, ... of p: lanes over the partials
+        if (st == 0) wait_count(a.cnt + Cnt::P, (unsigned)(P * (p + 1)), err);
+        sync();
+        for (int r = c + P * sw; r < sb; r += 3 * P) {
+          double t = 0.0;
+#pragma unroll 5
+          for (int q = lane; q < P; q += 32) t += __ldcg(a.ppart + (long long)q * sbp + r);
+          for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+          if (lane == 0) a.pvec[r] = t;
+        }
+        count(a.cnt + Cnt::Q);
       }
     }
     return;
@@ -418,8 +466,15 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   DigitGram<8 * RQ> dg;
   const bool digits = sb > kSmallSB;
   if (digits) digits_begin<RQ>(dg, sh, smem_d);
-  const long long nch = (a.K + 31) / 32;
-  const long long c0 = nch * c / P * 32, c1 = min(a.K, nch * (c + 1) / P * 32);
+  if (tid >= kT) {
+    if (digits) {
+      dg.mma_loop(err);
+      digits_end<RQ>(dg);
+    }
+    return;
+  }
+  const long long nch = (a.K + 15) / 16;  // (half stages: even shares)
+  const long long c0 = nch * c / P * 16, c1 = min(a.K, nch * (c + 1) / P * 16);
   auto gram = [&](int p, const long long* off) {  // the partial of step k0 + p
     double* part = a.part + ((a.k0 + p) & 1) * (long long)P * sq;
     ok = gram_columns<RQ>(dg, a.A, off, sb, c0, c1, smem_d, part + c * sq, sbp, err, ok);
@@ -449,7 +504,10 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
       gram(p + 1, soff[(p + 1) & 1]);
     }
   }
-  if (digits) digits_end<RQ>(dg);
+  if (digits) {
+    dg.stop();
+    digits_end<RQ>(dg);
+  }
 }
 
 // Dynamic shared memory of a column CTA.  With digits more than half of an
@@ -476,7 +534,7 @@ int launch64(Kern kern, std::atomic<unsigned long long>& configured, const Persi
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(coop ? kT + kSide : kT);
+  cfg.blockDim = dim3(coop ? kT + kMma + kSide : kT + kMma);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -491,7 +549,7 @@ int launch64(Kern kern, std::atomic<unsigned long long>& configured, const Persi
 template <int BMAX, int DEPTH, int RQ>
 int launch_steps(const Persist64Args& a, int P, size_t chain_smem, unsigned* err, cudaStream_t st) {
   static std::atomic<unsigned long long> configured{0ull};
-  return launch64(k_persist64<BMAX, DEPTH, RQ>, configured, a, P + 1,
+  return launch64(k_persist64<BMAX, DEPTH, RQ>, configured, a, P + 1 + std::min(a.sa.s_cur, kMaxInv),
                   std::max(chain_smem, column_smem<RQ>(a.sb)), true, err, st);
 }
 
@@ -525,8 +583,12 @@ int launch_gram64(const double* A, long long lda, long long N, long long K, cons
   return (int)cudaErrorInvalidValue;
 }
 
-// Block sizes and rows of a step the persistent launch covers.
-bool persist64_fits(int b, int sb) { return b <= 16 && sb <= 128; }
+// Column CTAs of the persistent launch (0: not for this block size, rows of a
+// step or GPU).
+int persist64_columns(int b, int s, long long K, int num_sms) {
+  if (b > 16 || s * b > 128) return 0;
+  return (int)std::max(0LL, std::min<long long>(num_sms - 1 - std::min(s, kMaxInv), (K + 31) / 32));
+}
 
 int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,
                      cudaStream_t st) {

@@ -19,14 +19,15 @@
 // of this part.  NT = 256: every thread of the CTA calls this; NT = 64 (b <= 8,
 // EPT = 1): two warps alone call it (warps 0-1, or the two warps whose
 // threads pass their index 0..63 as tix) and the barrier per pivot is named
-// barrier BAR over their 64 threads; NT = 128: four warps likewise.
+// barrier BAR over their 64 threads (NT = 256 with BAR other than 1: named
+// barrier BAR over 256 threads of a larger CTA).
 // Writes Gamma^{-1} (FP32 pairs, row-major) to out; a non-positive pivot
 // raises CA_DEV_ERR_NOT_SPD.
 template <int EPT, int NT = 256, int BAR = 1>
 __device__ void cta_sweep_inverse(float2 (&a)[EPT], int b, float2* __restrict__ colbuf,
                                   float2* __restrict__ out, unsigned* __restrict__ err,
                                   int tix = -1) {
-  static_assert(NT == 256 || NT == 128 || NT == 64, "a CTA of 256 threads or some of its warps");
+  static_assert(NT == 256 || NT == 64, "a CTA of 256 threads or two of its warps");
   const int t = tix >= 0 ? tix : (int)(threadIdx.x % NT);  // index among the NT threads
   int ri[EPT], ci[EPT];
 #pragma unroll
@@ -45,7 +46,7 @@ __device__ void cta_sweep_inverse(float2 (&a)[EPT], int b, float2* __restrict__ 
         if (ri[q] == k && !(a[q].x > 0.f)) ca_flag(err, CA_DEV_ERR_NOT_SPD);
       }
     }
-    if constexpr (NT < 256) asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
+    if constexpr (NT < 256 || BAR != 1) asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
     else __syncthreads();
     if (active) {
       // every thread forms 1 / a_kk itself (shorter than a broadcast)
