@@ -731,95 +731,105 @@ template __global__ void k_update_dense<float, true>(const float*, long long, lo
 // ---------------------------------------------------------------------------
 // a6: full recompute  v[k] = c0 * y0[k] + c1 * sum_{r < N} A[r][k] x[r]
 // (primal: rho = y - X^T w, or z = X^T w; dual: w = -X alpha/(lambda n)).
-// Grid (K-blocks, row splits); row splits add into v with FP64 atomics after
-// split 0 wrote the c0 * y0 term.  FP32 A: x split in two FP32 halves,
-// exact products summed in double-float over the split's rows, then FP64.
-// PANEL (FP32 only): A stored as 32-column panels [K/32][N][32]
-// (zero-padded).
+// k_recompute_prep writes the c0 * y0 term; a warp of k_recompute_dense takes 32
+// columns (a lane each) of one row split and streams the split's rows, 128
+// contiguous bytes a row (in panels the whole split is contiguous), sixteen
+// rows in flight; the warps of a CTA that hold the same columns add their sums
+// before one FP64 atomic addition a column.  FP32 A: x split in two FP32
+// halves, exact products summed in double-float over the split's rows, then
+// FP64.  PANEL (FP32 only): A stored as 32-column panels [K/32][N][32]
+// (zero-padded).  Bound by HBM (FP32) or the FP64 pipe.
 // ---------------------------------------------------------------------------
 template <typename T, bool PANEL>
 __global__ void __launch_bounds__(256)
 k_recompute_dense(const T* __restrict__ A, long long lda, long long N, long long K,
                   const double* __restrict__ x, const float2* __restrict__ x2, double c1,
-                  long long rows_per_split, double* __restrict__ v,
-                  const unsigned* __restrict__ nz) {
+                  long long rows_per_split, int ysplit, double* __restrict__ v,
+                  const unsigned* __restrict__ nz, unsigned epoch) {
+  __shared__ double red[8][32];
+  pdl_wait();  // x2, the c0 y0 term and the flag (k_recompute_prep)
+  pdl_trigger();
   // x = 0 (a solve started from zero): sum_r A[r] x[r] = 0, A is not read
-  if (nz && *nz == 0u) return;
-  const long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * 4;
-  if (k >= K) return;
-  const int nk = (int)min(4ll, K - k);
-  const long long r0 = (long long)blockIdx.y * rows_per_split;
-  const long long r1 = min(N, r0 + rows_per_split);
-  double acc[4] = {0, 0, 0, 0};
-  if constexpr (sizeof(T) == 8) {
-    for (long long r = r0; r < r1; ++r) {
-      const double xr = x[r];
-      const T* row = A + r * lda + k;
+  if (*(volatile const unsigned*)nz != epoch) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long natoms = (K + 31) / 32;
+  const long long item0 = (long long)blockIdx.x * 8, items = natoms * ysplit;
+  const long long item = item0 + warp;
+  const long long a = item / ysplit, k = a * 32 + lane;
+  double acc = 0.0;
+  if (item < items) {
+    const long long r0 = (item - a * ysplit) * rows_per_split;
+    const int n = (int)max(0LL, min(N, r0 + rows_per_split) - r0);
+    const long long st = PANEL ? 32 : lda;
+    const T* p = A + (PANEL ? a * N * 32 + lane : min(k, K - 1)) + r0 * st;
+    constexpr int U = 8;
+    T cur[U], nxt[U];
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (e < nk) acc[e] = fma((double)row[e], xr, acc[e]);
-    }
-  } else {
-    // x split in FP32 halves (x2); exact products, double-float sums
-    const bool vec = PANEL || ((nk == 4) && ((lda & 3) == 0) &&
-                               ((reinterpret_cast<uintptr_t>(A) & 15) == 0));
-    const long long pbase = (k >> 5) * N * 32 + (k & 31);
-    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-    for (long long r = r0; r < r1; ++r) {
-      const float2 xs = __ldg(x2 + r);
-      const float* row = reinterpret_cast<const float*>(A) + (PANEL ? pbase + r * 32 : r * lda + k);
-      float q[4];
-      if (vec) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(row));
-        q[0] = t.x; q[1] = t.y; q[2] = t.z; q[3] = t.w;
+    for (int u = 0; u < U; ++u) cur[u] = u < n ? __ldg(p + u * st) : T(0);
+    float hi = 0.f, lo = 0.f;
+    for (int r = 0; r < n; r += U) {
+      if (r + 2 * U <= n) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) nxt[u] = __ldg(p + (r + U + u) * st);
       } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e) q[e] = (e < nk) ? row[e] : 0.f;
+        for (int u = 0; u < U; ++u) nxt[u] = r + U + u < n ? __ldg(p + (r + U + u) * st) : T(0);
       }
 #pragma unroll
-      for (int e = 0; e < 4; ++e) df_dot_acc(q[e], xs.x, xs.y, hi[e], lo[e]);
+      for (int u = 0; u < U; ++u) {
+        if (r + u < n) {
+          if constexpr (sizeof(T) == 8) {
+            acc = fma((double)cur[u], __ldca(x + r0 + r + u), acc);
+          } else {
+            const float2 xs = __ldca(x2 + r0 + r + u);
+            df_dot_acc(cur[u], xs.x, xs.y, hi, lo);
+          }
+        }
+        cur[u] = nxt[u];
+      }
     }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[e] = (double)hi[e] + (double)lo[e];
+    if constexpr (sizeof(T) == 4) acc = (double)hi + (double)lo;
+    acc *= c1;
   }
-  for (int e = 0; e < nk; ++e) atomicAdd(v + k + e, c1 * acc[e]);
+  red[warp][lane] = acc;
+  __syncthreads();
+  if (item < items && (warp == 0 || (item - 1) / ysplit != a)) {  // first of its columns here
+    for (int w = warp + 1; w < 8 && (item0 + w) / ysplit == a; ++w) acc += red[w][lane];
+    if (k < K) {
+      if (ysplit == 1) v[k] += acc;
+      else atomicAdd(v + k, acc);
+    }
+  }
 }
-
-template __global__ void k_recompute_dense<double, false>(const double*, long long, long long,
-                                                          long long, const double*, const float2*,
-                                                          double, long long, double*,
-                                                          const unsigned*);
-template __global__ void k_recompute_dense<float, true>(const float*, long long, long long, long long,
-                                                        const double*, const float2*, double,
-                                                        long long, double*, const unsigned*);
-template __global__ void k_recompute_dense<float, false>(const float*, long long, long long, long long,
-                                                  const double*, const float2*, double, long long,
-                                                  double*, const unsigned*);
 
 // v2[k] = (hi, lo) FP32 split of v[k]; zero for K <= k < Kpad
 __global__ void k_split(const double* __restrict__ v, long long K, long long Kpad,
                         float2* __restrict__ v2) {
+  pdl_wait();
+  pdl_trigger();
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < Kpad) v2[k] = k < K ? split_f64(v[k]) : make_float2(0.f, 0.f);
 }
 
-// v = c0 * y0 (or 0 when y0 is null); clears *nz (when not null) for k_nonzero
+// v = c0 * y0 (or 0 when y0 is null)
 __global__ void k_axpby_init(const double* __restrict__ y0, double c0, long long K,
-                             double* __restrict__ v, unsigned* __restrict__ nz) {
+                             double* __restrict__ v) {
   const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k < K) v[k] = y0 ? c0 * y0[k] : 0.0;
-  if (nz && k == 0) *nz = 0u;
 }
 
-// *nz = 1 if any x[r] != 0 (r < N); x2 (when not null) receives the (hi, lo)
-// FP32 split of x
-__global__ void k_nonzero(const double* __restrict__ x, long long N, float2* __restrict__ x2,
-                          unsigned* __restrict__ nz) {
-  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const double xv = r < N ? x[r] : 0.0;
-  if (x2 && r < N) x2[r] = split_f64(xv);
-  if (__any_sync(0xffffffffu, xv != 0.0) && (threadIdx.x & 31) == 0) atomicOr(nz, 1u);
+// Before a recomputation: v = c0 * y0 (or 0 when y0 is null); *nz = epoch if any
+// x[r] != 0 (r < N); x2 (when not null) receives the (hi, lo) FP32 split of x.
+__global__ void k_recompute_prep(const double* __restrict__ y0, double c0, long long K,
+                                 double* __restrict__ v, const double* __restrict__ x, long long N,
+                                 float2* __restrict__ x2, unsigned* __restrict__ nz, unsigned epoch) {
+  pdl_wait();
+  pdl_trigger();
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < K) v[t] = y0 ? c0 * y0[t] : 0.0;
+  const double xv = t < N ? x[t] : 0.0;
+  if (x2 && t < N) x2[t] = split_f64(xv);
+  if (xv != 0.0) *nz = epoch;  // (the same value from every thread)
 }
 
 // ---------------------------------------------------------------------------
@@ -1633,47 +1643,51 @@ k_rowdot_dense(const T* __restrict__ A, long long lda, long long N, long long K,
   const long long natoms = (K + 31) / 32;
   const long long a0 = (long long)blockIdx.y * chunks_per_split;
   const long long a1 = min(natoms, a0 + chunks_per_split);
-  if constexpr (sizeof(T) == 8) {
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long a = a0; a < a1; ++a) {
-      const long long k = a * 32 + lane;
+  constexpr bool F64 = sizeof(T) == 8;
+  // row j of the warp's eight, column 32 a + lane (rows past N: row N - 1 again)
+  auto load = [&](long long a, T (&x)[8]) {
+    const long long k = a * 32 + lane;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const long long r = min(r0 + j, N - 1);
+      x[j] = __ldg(A + (PANEL ? (a * N + r) * 32 + lane : r * lda + min(k, K - 1)));
+    }
+  };
+  T cur[8], nxt[8];
+  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  float hi[8], lo[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) hi[j] = lo[j] = 0.f;
+  if (a0 < a1) load(a0, cur);
+  for (long long a = a0; a < a1; ++a) {
+    load(min(a + 1, a1 - 1), nxt);
+    const long long k = a * 32 + lane;
+    if constexpr (F64) {
       const double vk = k < K ? __ldcg(v + k) : 0.0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (r0 + j < N && k < K) acc[j] = fma((double)__ldg(A + (r0 + j) * lda + k), vk, acc[j]);
+      for (int j = 0; j < 8; ++j) acc[j] = fma((double)cur[j], vk, acc[j]);
+    } else {
+      const float2 vk = __ldcg(v2 + k);  // (zero past K, as A's panels)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) df_dot_acc(PANEL || k < K ? cur[j] : 0.f, vk.x, vk.y, hi[j], lo[j]);
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      double t = acc[j];
+    for (int j = 0; j < 8; ++j) cur[j] = nxt[j];
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    double t;
+    if constexpr (F64) {
+      t = acc[j];
       for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      if (lane == 0 && r0 + j < N) atomicAdd(q + r0 + j, t);
-    }
-  } else {
-    float hi[8], lo[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) hi[j] = lo[j] = 0.f;
-    for (long long a = a0; a < a1; ++a) {
-      const float2 vk = __ldcg(v2 + a * 32 + lane);
-      const long long k = a * 32 + lane;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const long long r = r0 + j;
-        float x = 0.f;
-        if (r < N) {
-          if constexpr (PANEL) x = __ldg(reinterpret_cast<const float*>(A) + (a * N + r) * 32 + lane);
-          else if (k < K) x = __ldg(reinterpret_cast<const float*>(A) + r * lda + k);
-        }
-        df_dot_acc(x, vk.x, vk.y, hi[j], lo[j]);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      float2 t = df_norm(hi[j], lo[j]);
+    } else {
+      float2 f = df_norm(hi[j], lo[j]);
       for (int o = 16; o; o >>= 1)
-        t = df_add(t, make_float2(__shfl_xor_sync(0xffffffffu, t.x, o),
-                                  __shfl_xor_sync(0xffffffffu, t.y, o)));
-      if (lane == 0 && r0 + j < N) atomicAdd(q + r0 + j, (double)t.x + (double)t.y);
+        f = df_add(f, make_float2(__shfl_xor_sync(0xffffffffu, f.x, o),
+                                  __shfl_xor_sync(0xffffffffu, f.y, o)));
+      t = (double)f.x + (double)f.y;
     }
+    if (lane == 0 && r0 + j < N) atomicAdd(q + r0 + j, t);
   }
 }
 
@@ -1812,18 +1826,43 @@ void launch_update_dense(bool f64, unsigned grid, size_t smem, cudaStream_t st, 
                                                            idx, sb, delta, cU, v, v2, err);
 }
 
-void launch_recompute_dense(bool f64, dim3 grid, cudaStream_t st, const void* A, long long lda,
-                            long long N, long long K, const double* x, const float2* x2, double c1,
-                            long long rows_per_split, double* v, bool panel, const unsigned* nz) {
+int launch_recompute_dense(bool f64, int num_sms, cudaStream_t st, const void* A, long long lda,
+                           long long N, long long K, const double* x, float2* x2, const double* y0,
+                           double c0, double c1, double* v, bool panel, unsigned* nz,
+                           unsigned epoch) {
+  const long long natoms = (K + 31) / 32;
+  // row splits: FP32 a few thousand warps' worth in splits of at least 64 rows;
+  // FP64 (short on arithmetic, not on warps) at least eight rows
+  long long ysplit;
+  if (f64) {
+    ysplit = std::max(1LL, std::min((32LL * num_sms + natoms - 1) / natoms, (N + 7) / 8));
+  } else {
+    const long long gx = (K + 1023) / 1024;
+    ysplit = std::max(1LL, std::min((4LL * num_sms + gx - 1) / gx, (N + 63) / 64));
+  }
+  const long long rps = (N + ysplit - 1) / ysplit;
+  ysplit = (N + rps - 1) / rps;
+  const unsigned grid = (unsigned)((natoms * ysplit + 7) / 8);
+  launch_programmatic(k_recompute_prep, (unsigned)((std::max(N, K) + 255) / 256), 0, st, y0, c0, K, v,
+                      x, N, x2, nz, epoch);
+  const unsigned* nzc = nz;
+  const float2* x2c = x2;
   if (f64)
-    k_recompute_dense<double, false><<<grid, 256, 0, st>>>(static_cast<const double*>(A), lda, N, K,
-                                                            x, x2, c1, rows_per_split, v, nz);
-  else if (panel)
-    k_recompute_dense<float, true><<<grid, 256, 0, st>>>(static_cast<const float*>(A), lda, N, K, x,
-                                                          x2, c1, rows_per_split, v, nz);
-  else
-    k_recompute_dense<float, false><<<grid, 256, 0, st>>>(static_cast<const float*>(A), lda, N, K,
-                                                           x, x2, c1, rows_per_split, v, nz);
+    return (int)launch_programmatic(k_recompute_dense<double, false>, grid, 0, st,
+                                    static_cast<const double*>(A), lda, N, K, x, x2c, c1, rps,
+                                    (int)ysplit, v, nzc, epoch);
+  if (panel)
+    return (int)launch_programmatic(k_recompute_dense<float, true>, grid, 0, st,
+                                    static_cast<const float*>(A), lda, N, K, x, x2c, c1, rps,
+                                    (int)ysplit, v, nzc, epoch);
+  return (int)launch_programmatic(k_recompute_dense<float, false>, grid, 0, st,
+                                  static_cast<const float*>(A), lda, N, K, x, x2c, c1, rps,
+                                  (int)ysplit, v, nzc, epoch);
+}
+
+void launch_split(cudaStream_t st, const double* v, long long K, float2* v2) {
+  const long long Kp = (K + 31) / 32 * 32;
+  launch_programmatic(k_split, (unsigned)((Kp + 255) / 256), 0, st, v, K, Kp, v2);
 }
 
 // Repack a row-major N x K FP32 matrix (leading dimension lda, 16-byte aligned
