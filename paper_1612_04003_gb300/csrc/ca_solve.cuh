@@ -4,6 +4,8 @@
 // inversion of the diagonal blocks, the sums of split-K partials and the
 // lookahead chain.
 #pragma once
+#include <type_traits>
+
 #include "ca_common.cuh"
 
 // Gamma_j^{-1} for one b x b block by the Gauss-Jordan sweep operator on a
@@ -153,6 +155,17 @@ __device__ __forceinline__ void chain_cta_sync() {
   asm volatile("bar.sync 6, 256;" ::: "memory");
 }
 
+__device__ __forceinline__ bool chain_cta_any(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 6, 256, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)v)
+      : "memory");
+  return r != 0;
+}
+
 // The dependent chain with lookahead (one CTA of 256 threads; b <= BMAX <= 16,
 // sb <= 256), from Rs (cG-scaled, transposed), p and the diagonal-block
 // inverses Ginv.  Warp 0 runs only the dependent path: for step j it forms
@@ -219,6 +232,16 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
     }
     sidx[tid] = gi;
   }
+  // does an index recur across the blocks (none does inside one)?  Found while
+  // the reduction still runs.
+  chain_cta_sync();
+  bool rep = false;
+  for (int t = tid; t < sb * 2; t += 256) {  // two threads a row, half of the earlier rows each
+    const int r = t >> 1, gi = sidx[r], h = (r + 1) >> 1;
+    const int q1 = (t & 1) ? r : h;
+    for (int q = (t & 1) ? h : 0; q < q1; ++q) rep |= sidx[q] == gi;
+  }
+  const bool dup = chain_cta_any(rep);
   if (ticket) {  // the reducing CTAs of this grid: R, Rs, p and Ginv complete
     if (tid == 0) {
       const uint64_t t0 = ca_globaltimer();
@@ -246,107 +269,120 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
   chain_cta_sync();
   const float2 cI2 = split_f64(a.cI);
   const float2 z2 = make_float2(0.f, 0.f);
-  if (warp == 0) {
-    const int i = lane / LPR, c0 = (lane % LPR) * CPL;
-    float2 rbv = i < b ? rhs0s[i] : z2;  // rb of the current block, row i
-    for (int j = 0; j < s; ++j) {
-      const int jb = j * b;
-      float2 pr[CPL];
+  // the index-overlap terms only where a sampled index recurs (dup)
+  auto steps = [&](auto overlap) {
+    constexpr bool OV = decltype(overlap)::value;
+    if (warp == 0) {
+      const int i = lane / LPR, c0 = (lane % LPR) * CPL;
+      float2 g[CPL];  // this lane's entries of Gamma_j^{-1}, loaded a step ahead
+      auto load_g = [&](int j) {
 #pragma unroll
-      for (int cc = 0; cc < CPL; ++cc) {
-        const int c = c0 + cc;
-        const float2 rbc = shfl_df(rbv, c * LPR);
-        pr[cc] = (i < b && c < b) ? df_mul(Gs[(size_t)j * b * b + i * b + c], rbc) : z2;
-      }
-      float2 dl = df_tree_sum(pr);
+        for (int cc = 0; cc < CPL; ++cc)
+          g[cc] = (i < b && c0 + cc < b) ? Gs[(size_t)j * b * b + i * b + c0 + cc] : z2;
+      };
+      load_g(0);
+      float2 rbv = i < b ? rhs0s[i] : z2;  // rb of the current block, row i
+      for (int j = 0; j < s; ++j) {
+        const int jb = j * b;
+        float2 pr[CPL];
 #pragma unroll
-      for (int o = LPR / 2; o >= 1; o /= 2) dl = df_add(dl, shfl_xor_df(dl, o));
-      if (i < b && (lane % LPR) == 0) dall[jb + i] = dl;
-      __syncwarp();
-      named_bar_arrive(2 + (j & 1));  // D(j): Delta_j published
-      if (j + 1 < s) {
-        if (j >= 1) named_bar_sync(4 + ((j - 1) & 1));  // F(j-1): sums of block j+1, columns of step j
-        const int rowp = (j + 1) * b + i;
-        const bool rv = i < b && rowp < sb;
-        const int gp = rv ? sidx[rowp] : -2;
-        const float2* slot = ring + (size_t)(j % DEPTH) * BMAX * 256;
-        float2 u[CPL];
-        float2 ov = z2;
-        bool hit = false;
+        for (int cc = 0; cc < CPL; ++cc) pr[cc] = df_mul(g[cc], shfl_df(rbv, (c0 + cc) * LPR));
+        float2 dl = df_tree_sum(pr);
 #pragma unroll
-        for (int cc = 0; cc < CPL; ++cc) {
-          const int c = c0 + cc;
-          const float2 dc = shfl_df(dl, c * LPR);
-          u[cc] = z2;
-          if (rv && c < b) {
-            u[cc] = df_mul(slot[c * 256 + rowp], dc);
-            if (sidx[jb + c] == gp) {
-              ov = df_add(ov, dc);
-              hit = true;
+        for (int o = LPR / 2; o >= 1; o /= 2) dl = df_add(dl, shfl_xor_df(dl, o));
+        if (i < b && (lane % LPR) == 0) dall[jb + i] = dl;
+        __syncwarp();
+        named_bar_arrive(2 + (j & 1));  // D(j): Delta_j published
+        if (j + 1 < s) {
+          load_g(j + 1);
+          const int rowp = (j + 1) * b + i;
+          const bool rv = i < b && rowp < sb;
+          const float2 rh = rv ? rhs0s[rowp] : z2;
+          float2 dc[CPL];
+#pragma unroll
+          for (int cc = 0; cc < CPL; ++cc) dc[cc] = shfl_df(dl, (c0 + cc) * LPR);
+          float2 ov = z2;
+          if constexpr (OV) {
+            const int gp = rv ? sidx[rowp] : -2;
+            bool hit = false;
+#pragma unroll
+            for (int cc = 0; cc < CPL; ++cc) {
+              if (rv && c0 + cc < b && sidx[jb + c0 + cc] == gp) {
+                ov = df_add(ov, dc[cc]);
+                hit = true;
+              }
+            }
+            if (__any_sync(FULL, hit)) {
+#pragma unroll
+              for (int o = LPR / 2; o >= 1; o /= 2) ov = df_add(ov, shfl_xor_df(ov, o));
             }
           }
-        }
-        float2 us = df_tree_sum(u);
+          if (j >= 1) named_bar_sync(4 + ((j - 1) & 1));  // F(j-1): sums of block j+1, columns of step j
+          const float2* slot = ring + (size_t)(j % DEPTH) * BMAX * 256;
+          float2 u[CPL];
 #pragma unroll
-        for (int o = LPR / 2; o >= 1; o /= 2) us = df_add(us, shfl_xor_df(us, o));
-        if (__any_sync(FULL, hit)) {
+          for (int cc = 0; cc < CPL; ++cc)
+            u[cc] = (rv && c0 + cc < b) ? slot[(c0 + cc) * 256 + rowp] : z2;
+          const int hb = ((j + 1) & 1) * 16 + i;
+          const float2 accv = (j >= 1 && rv) ? accb[hb] : z2;
 #pragma unroll
-          for (int o = LPR / 2; o >= 1; o /= 2) ov = df_add(ov, shfl_xor_df(ov, o));
+          for (int cc = 0; cc < CPL; ++cc) u[cc] = df_mul(u[cc], dc[cc]);
+          float2 us = df_tree_sum(u);
+#pragma unroll
+          for (int o = LPR / 2; o >= 1; o /= 2) us = df_add(us, shfl_xor_df(us, o));
+          us = df_add(accv, us);
+          if constexpr (OV) {
+            const float2 ovv = (j >= 1 && rv) ? ovlb[hb] : z2;
+            us = df_add(us, df_mul(cI2, df_add(ovv, ov)));
+          }
+          rbv = rv ? df_add(rh, df_neg(us)) : z2;
         }
-        const int hb = ((j + 1) & 1) * 16 + i;
-        const float2 accv = (j >= 1 && rv) ? accb[hb] : z2;
-        const float2 ovv = (j >= 1 && rv) ? ovlb[hb] : z2;
-        rbv = rv ? df_add(rhs0s[rowp], df_neg(df_add(df_add(accv, us), df_mul(cI2, df_add(ovv, ov)))))
-                 : z2;
       }
+    } else {
+      const int r1 = cu, r2 = cu + 224;
+      const int g1 = r1 < sb ? sidx[r1] : -2, g2 = r2 < sb ? sidx[r2] : -2;
+      float2 acc1 = z2, acc2 = z2, ov1 = z2, ov2 = z2;
+      for (int j = 0; j < s; ++j) {
+        const int jb = j * b, lo = (j + 2) * b;
+        named_bar_sync(2 + (j & 1));  // D(j)
+        const float2* slot = ring + (size_t)(j % DEPTH) * BMAX * 256;
+        auto fold = [&](int r, int g, float2& acc, float2& ov) {
+          float2 pr[BMAX];
+          unsigned m = 0;
+#pragma unroll
+          for (int q = 0; q < BMAX; ++q) {
+            pr[q] = q < b ? df_mul(slot[q * 256 + r], dall[jb + q]) : z2;
+            if constexpr (OV) m |= (q < b && sidx[jb + q] == g) ? (1u << q) : 0u;
+          }
+          acc = df_add(acc, df_tree_sum(pr));
+          if constexpr (OV) {
+            while (m) {  // sampled index shared with an earlier row (rare)
+              const int q = __ffs(m) - 1;
+              ov = df_add(ov, dall[jb + q]);
+              m &= m - 1;
+            }
+          }
+        };
+        if (r1 >= lo && r1 < sb) fold(r1, g1, acc1, ov1);
+        if (r2 >= lo && r2 < sb) fold(r2, g2, acc2, ov2);
+        const int hb = ((j + 2) & 1) * 16;
+        if (r1 >= lo && r1 < lo + b && r1 < sb) {
+          accb[hb + r1 - lo] = acc1;
+          if constexpr (OV) ovlb[hb + r1 - lo] = ov1;
+        }
+        if (r2 >= lo && r2 < lo + b && r2 < sb) {
+          accb[hb + r2 - lo] = acc2;
+          if constexpr (OV) ovlb[hb + r2 - lo] = ov2;
+        }
+        fetch(j + DEPTH - 1);        // into the slot of step j-1 (warp 0 is done with it)
+        cp_async_wait<DEPTH - 2>();  // this thread's columns of step j+1 have landed
+        if (j + 2 < s) named_bar_arrive(4 + (j & 1));  // F(j)
+      }
+      cp_async_wait<0>();
     }
-  } else {
-    const int r1 = cu, r2 = cu + 224;
-    const int g1 = r1 < sb ? sidx[r1] : -2, g2 = r2 < sb ? sidx[r2] : -2;
-    float2 acc1 = z2, acc2 = z2, ov1 = z2, ov2 = z2;
-    for (int j = 0; j < s; ++j) {
-      const int jb = j * b, lo = (j + 2) * b;
-      named_bar_sync(2 + (j & 1));  // D(j)
-      const float2* slot = ring + (size_t)(j % DEPTH) * BMAX * 256;
-      float2 dq[BMAX];
-      int iq[BMAX];
-#pragma unroll
-      for (int q = 0; q < BMAX; ++q) {
-        dq[q] = q < b ? dall[jb + q] : z2;
-        iq[q] = q < b ? sidx[jb + q] : -3;
-      }
-      auto fold = [&](int r, int g, float2& acc, float2& ov) {
-        float2 pr[BMAX];
-        unsigned m = 0;
-#pragma unroll
-        for (int q = 0; q < BMAX; ++q) {
-          pr[q] = q < b ? df_mul(slot[q * 256 + r], dq[q]) : z2;
-          m |= (iq[q] == g) ? (1u << q) : 0u;
-        }
-        acc = df_add(acc, df_tree_sum(pr));
-        while (m) {  // sampled index shared with an earlier row (rare)
-          const int q = __ffs(m) - 1;
-          ov = df_add(ov, dall[jb + q]);
-          m &= m - 1;
-        }
-      };
-      if (r1 >= lo && r1 < sb) fold(r1, g1, acc1, ov1);
-      if (r2 >= lo && r2 < sb) fold(r2, g2, acc2, ov2);
-      const int hb = ((j + 2) & 1) * 16;
-      if (r1 >= lo && r1 < lo + b && r1 < sb) {
-        accb[hb + r1 - lo] = acc1;
-        ovlb[hb + r1 - lo] = ov1;
-      }
-      if (r2 >= lo && r2 < lo + b && r2 < sb) {
-        accb[hb + r2 - lo] = acc2;
-        ovlb[hb + r2 - lo] = ov2;
-      }
-      fetch(j + DEPTH - 1);        // into the slot of step j-1 (warp 0 is done with it)
-      cp_async_wait<DEPTH - 2>();  // this thread's columns of step j+1 have landed
-      if (j + 2 < s) named_bar_arrive(4 + (j & 1));  // F(j)
-    }
-    cp_async_wait<0>();
-  }
+  };
+  if (dup) steps(std::true_type{});
+  else steps(std::false_type{});
   chain_cta_sync();
   if (tid < sb) {  // Delta out, x += Delta (atomic: an index may recur across blocks)
     const float2 d2 = dall[tid];
