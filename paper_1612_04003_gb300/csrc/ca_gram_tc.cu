@@ -261,12 +261,13 @@ k_gram_tc(const float* __restrict__ A, long long lda, long long N, long long K,
         const uint32_t dst = raw0 + (uint32_t)(slot * C::kRawBytes);
 #pragma unroll
         for (int i = 0; i < RPT; ++i)
-          if (rowoff[i] >= 0) cp_async_16_zfill(dst + dsto[i], U.A + rowoff[i] + col, bytes);
+          // (a row that is not there is zeros: no branch here or where it is read)
+          cp_async_16_zfill(dst + dsto[i], U.A + max(rowoff[i], 0LL) + col, rowoff[i] >= 0 ? bytes : 0u);
         if constexpr (UPD) {
 #pragma unroll
           for (int i = 0; i < RPT; ++i)
-            if (prevoff[i] >= 0)
-              cp_async_16_zfill(dst + C::kPrevOff + dsto[i], U.A + prevoff[i] + col, bytes);
+            cp_async_16_zfill(dst + C::kPrevOff + dsto[i], U.A + max(prevoff[i], 0LL) + col,
+                              prevoff[i] >= 0 ? bytes : 0u);
         }
         if (tid < 16)  // the stage's 32 (hi, lo) pairs of v (zero-padded to a multiple of 32)
           cp_async_16_zfill(vring0 + (uint32_t)(((g0 + t) % (2 * NS)) * 256 + tid * 16),
@@ -324,13 +325,11 @@ k_gram_tc(const float* __restrict__ A, long long lda, long long N, long long K,
           float up[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int i = 0; i < RPT; ++i) {
-            if (prevoff[i] >= 0) {
-              const float4 x = *reinterpret_cast<const float4*>(big + C::kPrevOff + dsto[i]);
-              up[0] = fmaf(x.x, dph[i], fmaf(x.x, dpl[i], up[0]));
-              up[1] = fmaf(x.y, dph[i], fmaf(x.y, dpl[i], up[1]));
-              up[2] = fmaf(x.z, dph[i], fmaf(x.z, dpl[i], up[2]));
-              up[3] = fmaf(x.w, dph[i], fmaf(x.w, dpl[i], up[3]));
-            }
+            const float4 x = *reinterpret_cast<const float4*>(big + C::kPrevOff + dsto[i]);
+            up[0] = fmaf(x.x, dph[i], fmaf(x.x, dpl[i], up[0]));
+            up[1] = fmaf(x.y, dph[i], fmaf(x.y, dpl[i], up[1]));
+            up[2] = fmaf(x.z, dph[i], fmaf(x.z, dpl[i], up[2]));
+            up[3] = fmaf(x.w, dph[i], fmaf(x.w, dpl[i], up[3]));
           }
 #pragma unroll
           for (int e = 0; e < 4; ++e) {

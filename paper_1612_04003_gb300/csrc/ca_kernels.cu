@@ -381,7 +381,7 @@ template __global__ void k_reduce<float>(const float*, const double*, int, int, 
 
 // Gamma_j^{-1} for every diagonal block j = blockIdx.x from R (FP64 lower
 // triangle), one CTA each (b <= 32).
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 1)
 k_factor(const double* __restrict__ R, SolveArgs sa, float2* __restrict__ Ginv,
          unsigned* __restrict__ err) {
   __shared__ float2 colbuf[66];
@@ -519,13 +519,13 @@ __device__ void chain_body(const float2* __restrict__ Rs, const double* __restri
 }
 
 template <int BMAX, int DEPTH>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 1)
 k_chain(const float2* __restrict__ Rs, const double* __restrict__ pvec,
         const float2* __restrict__ Ginv, SolveArgs a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
   pdl_wait();  // (as a programmatic dependent: p from the launch before it)
   if constexpr (BMAX <= 16)
-    chain_la_body<BMAX, DEPTH>(Rs, pvec, Ginv, a, err, smem_d);
+    chain_la_body<BMAX, DEPTH>(Rs, pvec, Ginv, a, err, smem_d, [] { return true; });
   else
     chain_body<BMAX, DEPTH>(Rs, pvec, Ginv, a, err, smem_d);
 }
@@ -540,8 +540,10 @@ k_chain(const float2* __restrict__ Rs, const double* __restrict__ pvec,
 // waits for that grid, then lets the next Gram pass launch its CTAs, which
 // prepare and start their loads on the SMs this grid frees while the chain
 // runs.  *ticket is zero on entry and left zero.
+// (One CTA per SM: without the bound the compiler stayed at 80 registers, short
+// of the 40 loads a reducing thread keeps in flight.)
 template <typename PT, int BMAX, int DEPTH>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 1)
 k_reduce_chain(const PT* __restrict__ part, const double* __restrict__ ppart, int P, int sbp,
                double* __restrict__ R, float2* __restrict__ Rs, double* __restrict__ pvec,
                float2* __restrict__ Ginv, int ndiag, SolveArgs sa, unsigned* __restrict__ err,
@@ -559,7 +561,8 @@ k_reduce_chain(const PT* __restrict__ part, const double* __restrict__ ppart, in
     }
     return;
   }
-  chain_la_body<BMAX, DEPTH>(Rs, pvec, Ginv, sa, err, smem_d, ticket, (unsigned)nred);
+  chain_la_body<BMAX, DEPTH>(Rs, pvec, Ginv, sa, err, smem_d,
+                             [&] { return chain_wait(ticket, (unsigned)nred, true, err); });
 }
 
 template __global__ void k_reduce_chain<float, 8, 4>(const float*, const double*, int, int, double*,
@@ -579,7 +582,7 @@ template __global__ void k_reduce_chain<double, 16, 3>(const double*, const doub
 // reduces every problem's split-K partials (role table: problem and CTA index
 // within it), one grid runs one chain CTA per problem.  No CTA waits on
 // another, so neither grid needs its CTAs resident at once.
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
 k_reduce_batch(const RedInst* __restrict__ insts, const RedRole* __restrict__ roles,
                unsigned* __restrict__ err) {
   pdl_wait();
@@ -591,13 +594,13 @@ k_reduce_batch(const RedInst* __restrict__ insts, const RedRole* __restrict__ ro
 }
 
 template <int BMAX, int DEPTH>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 1)
 k_chain_batch(const RedInst* __restrict__ insts, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
   pdl_wait();
   pdl_trigger();
   const RedInst ri = insts[blockIdx.x];
-  chain_la_body<BMAX, DEPTH>(ri.Rs, ri.pvec, ri.Ginv, ri.sa, err, smem_d);
+  chain_la_body<BMAX, DEPTH>(ri.Rs, ri.pvec, ri.Ginv, ri.sa, err, smem_d, [] { return true; });
 }
 
 template __global__ void k_chain<8, 4>(const float2*, const double*, const float2*, SolveArgs,

@@ -94,9 +94,11 @@ __device__ __forceinline__ uint64_t l2_evict_first() {
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-__device__ __forceinline__ void cp_async_16_pol(uint32_t dst, const void* src, uint64_t pol) {
-  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(dst), "l"(src),
-               "l"(pol)
+// 16 bytes, or (bytes = 0) zeros
+__device__ __forceinline__ void cp_async_16_pol(uint32_t dst, const void* src, uint32_t bytes,
+                                                uint64_t pol) {
+  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;" ::"r"(dst),
+               "l"(src), "r"(bytes), "l"(pol)
                : "memory");
 }
 
@@ -134,8 +136,9 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_persist(PersistArgs a, unsigne
       SolveArgs sa = a.sa;
       sa.idx = a.idx_all + k * sb;
       sa.delta = a.delta2[k & 1];
-      chain_la_body<8, 4>(a.Rs, a.pvec, a.Ginv, sa, err, smem_d, a.cnt + 1,
-                          (unsigned)(Pg * (p + 1)), false);
+      chain_la_body<8, 4>(a.Rs, a.pvec, a.Ginv, sa, err, smem_d, [&] {
+        return chain_wait(a.cnt + 1, (unsigned)(Pg * (p + 1)), false, err);
+      });
       chain_cta_sync();  // Delta_k and x written by every thread of the chain
       if (tid == 0) {
         __threadfence();
@@ -255,20 +258,22 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_persist(PersistArgs a, unsigne
       const long long atom = a0 + t;
       const uint32_t dst = raw0 + (uint32_t)(slot * C::kRaw);
       const float* base = a.A + atom * N * 32 + 4 * l;
+      // (a row that is not there is zeros: no branch here or where it is read)
+      auto row_copy = [&](uint32_t to, int r) {
+        cp_async_16_pol(to, base + (long long)max(r, 0) * 32, r >= 0 ? 16u : 0u, pol_stream);
+      };
       if (!fin) {
 #pragma unroll
         for (int i = 0; i < RPT; ++i)
-          if (icur[i] >= 0) cp_async_16_pol(dst + dsto[i], base + (long long)icur[i] * 32, pol_stream);
+          row_copy(dst + dsto[i], icur[i]);
       }
 #pragma unroll
       for (int i = 0; i < RPT; ++i)
-        if (iprv[i] >= 0)
-          cp_async_16_pol(dst + C::kTile + dsto[i], base + (long long)iprv[i] * 32, pol_stream);
+        row_copy(dst + C::kTile + dsto[i], iprv[i]);
       if (regA2) {
 #pragma unroll
         for (int i = 0; i < RPT; ++i)
-          if (iprv2[i] >= 0)
-            cp_async_16_pol(dst + 2 * C::kTile + dsto[i], base + (long long)iprv2[i] * 32, pol_stream);
+          row_copy(dst + 2 * C::kTile + dsto[i], iprv2[i]);
       }
       if (tid < 16)  // the stage's 32 (hi, lo) pairs of v
         cp_async_16_zfill(vring0 + (uint32_t)((gs % (2 * NS)) * 256 + tid * 16),
@@ -327,15 +332,12 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_persist(PersistArgs a, unsigne
         float up[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-          const int vr = KIND == 1 ? vprev2[i] : vprev[i];
           const float dh = KIND == 1 ? dph2[i] : dph[i], dlo = KIND == 1 ? dpl2[i] : dpl[i];
-          if (vr >= 0) {
-            const float4 x = *reinterpret_cast<const float4*>(big + UOFF + dsto[i]);
-            up[0] = fmaf(x.x, dh, fmaf(x.x, dlo, up[0]));
-            up[1] = fmaf(x.y, dh, fmaf(x.y, dlo, up[1]));
-            up[2] = fmaf(x.z, dh, fmaf(x.z, dlo, up[2]));
-            up[3] = fmaf(x.w, dh, fmaf(x.w, dlo, up[3]));
-          }
+          const float4 x = *reinterpret_cast<const float4*>(big + UOFF + dsto[i]);
+          up[0] = fmaf(x.x, dh, fmaf(x.x, dlo, up[0]));
+          up[1] = fmaf(x.y, dh, fmaf(x.y, dlo, up[1]));
+          up[2] = fmaf(x.z, dh, fmaf(x.z, dlo, up[2]));
+          up[3] = fmaf(x.w, dh, fmaf(x.w, dlo, up[3]));
         }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
@@ -354,8 +356,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_persist(PersistArgs a, unsigne
       if constexpr (REGA) {
 #pragma unroll
         for (int i = 0; i < RPT; ++i)
-          xp[i] = vprev[i] >= 0 ? *reinterpret_cast<const float4*>(big + C::kTile + dsto[i])
-                                : make_float4(0.f, 0.f, 0.f, 0.f);
+          xp[i] = *reinterpret_cast<const float4*>(big + C::kTile + dsto[i]);
       }
       // every loader has read its FP32 chunks of this stage (the tiles below
       // overwrite them) and written its column sums; every copy (v slice

@@ -363,12 +363,15 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
       SolveArgs sa = a.sa;
       sa.idx = a.idx_all + k * sb;
       sa.delta = a.delta2[k & 1];
-      ok = main_wait(a.cnt + Cnt::R + (p & 1), (unsigned)(ninv * (p / 2 + 1)), err, ok);
-      ok = sb >= kRowsSB ? main_wait(a.cnt + Cnt::Q, (unsigned)(min(P, sb) * (p + 1)), err, ok)
-                         : main_wait(a.cnt + Cnt::P, (unsigned)(P * (p + 1)), err, ok);
-      if (!ok) return;
-      if (sb < kRowsSB) sum_rows(a, P, sbp, sb, smem_d);
-      chain_la_body<BMAX, DEPTH>(a.Rs[k & 1], a.pvec, a.Ginv[k & 1], sa, err, smem_d);
+      const bool done = chain_la_body<BMAX, DEPTH>(
+          a.Rs[k & 1], a.pvec, a.Ginv[k & 1], sa, err, smem_d, [&] {
+            ok = main_wait(a.cnt + Cnt::R + (p & 1), (unsigned)(ninv * (p / 2 + 1)), err, ok);
+            ok = sb >= kRowsSB ? main_wait(a.cnt + Cnt::Q, (unsigned)(min(P, sb) * (p + 1)), err, ok)
+                               : main_wait(a.cnt + Cnt::P, (unsigned)(P * (p + 1)), err, ok);
+            if (ok && sb < kRowsSB) sum_rows(a, P, sbp, sb, smem_d);
+            return ok;
+          });
+      if (!done) return;
       main_count(a.cnt + Cnt::D);
     }
     return;

@@ -182,16 +182,13 @@ __device__ __forceinline__ bool chain_cta_any(bool v) {
 // analogue) is added where the sampled indices coincide.  All arithmetic on
 // the dependent path is double-float; FP64 converts in and out.  Only warps
 // 0-7 of the CTA take part (CTA-wide steps use named barrier 6 over 256
-// threads), so a larger CTA may give its other warps other work.  With a
-// ticket the chain first waits (bounded) until *ticket >= nready; the count
-// is cleared afterwards unless reset_ticket is false (a count that keeps
-// growing across outer steps).
-template <int BMAX, int DEPTH>
-__device__ void chain_la_body(const float2* __restrict__ Rs, const double* __restrict__ pvec,
+// threads), so a larger CTA may give its other warps other work.  What does
+// not depend on R, Rs, p and Ginv comes first; then ready() (by all 256
+// threads) returns once they are complete, or false: the chain ends there.
+template <int BMAX, int DEPTH, typename Ready>
+__device__ bool chain_la_body(const float2* __restrict__ Rs, const double* __restrict__ pvec,
                               const float2* __restrict__ Ginv, const SolveArgs& a,
-                              unsigned* __restrict__ err, double* smem_d,
-                              unsigned* __restrict__ ticket = nullptr, unsigned nready = 0,
-                              bool reset_ticket = true) {
+                              unsigned* __restrict__ err, double* smem_d, Ready&& ready) {
   static_assert(BMAX == 8 || BMAX == 16, "lookahead chain: BMAX 8 or 16");
   constexpr int LPR = 32 / BMAX, CPL = BMAX / LPR;  // warp 0: lanes per row, columns per lane
   constexpr unsigned FULL = 0xffffffffu;
@@ -210,13 +207,13 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
   const int cu = tid - 32;  // index among warps 1-7
   auto fetch = [&](int j) {  // warps 1-7: columns jb .. jb+b of rows >= jb + b, slot j % DEPTH
     const int jb = j * b;
-    if (j < s && ld_ok) {
-      const int p0 = (jb + b) >> 1, np = ((sb + 1) >> 1) - p0;
-      for (int u = cu; u < b * np; u += 224) {
-        const int q = u / np, pr = 2 * (p0 + u - q * np);
-        cp_async_16_zfill(ring0 + 8u * (uint32_t)(((j % DEPTH) * BMAX + q) * 256 + pr),
-                          Rs + (long long)(jb + q) * ldr + pr, 16u);
-      }
+    const int pr = ((jb + b) & ~1) + 2 * cu;  // this thread's row pair (at most 128 of them)
+    if (j < s && ld_ok && pr < sb) {
+      const uint32_t dst = ring0 + 8u * (uint32_t)((j % DEPTH) * BMAX * 256 + pr);
+      const float2* src = Rs + (long long)jb * ldr + pr;
+#pragma unroll
+      for (int q = 0; q < BMAX; ++q)
+        if (q < b) cp_async_16_zfill(dst + 8u * 256u * q, src + (long long)q * ldr, 16u);
     }
     cp_async_commit();
   };
@@ -242,25 +239,7 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
     for (int q = (t & 1) ? h : 0; q < q1; ++q) rep |= sidx[q] == gi;
   }
   const bool dup = chain_cta_any(rep);
-  if (ticket) {  // the reducing CTAs of this grid: R, Rs, p and Ginv complete
-    if (tid == 0) {
-      const uint64_t t0 = ca_globaltimer();
-      // gives up after the limit, or at once when another wait of the
-      // grid has already given up
-      for (uint32_t it = 1; *(volatile unsigned*)ticket < nready; ++it) {
-        if ((it & 255u) == 0u) {
-          if (*(volatile unsigned*)err & CA_DEV_ERR_TIMEOUT) break;
-          if (ca_globaltimer() - t0 > CA_WAIT_LIMIT_NS) {
-            ca_flag(err, CA_DEV_ERR_TIMEOUT);
-            break;
-          }
-        }
-      }
-      if (reset_ticket) *ticket = 0u;  // for the next launch (which starts after this grid ends)
-      __threadfence();
-    }
-    chain_cta_sync();
-  }
+  if (!ready()) return false;  // R, Rs, p and Ginv complete, seen by every thread
   if (warp > 0)
     for (int d = 0; d < DEPTH - 1; ++d) fetch(d);
   for (int e = tid; e < sb * b; e += 256) Gs[e] = __ldcg(Ginv + e);
@@ -278,7 +257,12 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
       auto load_g = [&](int j) {
 #pragma unroll
         for (int cc = 0; cc < CPL; ++cc)
-          g[cc] = (i < b && c0 + cc < b) ? Gs[(size_t)j * b * b + i * b + c0 + cc] : z2;
+          g[cc] = Gs[j * b * b + min(i, b - 1) * b + min(c0 + cc, b - 1)];
+        // (unconditional loads, then selects: a condition on each load makes
+        // branches that wait for one load after another)
+#pragma unroll
+        for (int cc = 0; cc < CPL; ++cc)
+          if (i >= b || c0 + cc >= b) g[cc] = z2;
       };
       load_g(0);
       float2 rbv = i < b ? rhs0s[i] : z2;  // rb of the current block, row i
@@ -297,7 +281,8 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
           load_g(j + 1);
           const int rowp = (j + 1) * b + i;
           const bool rv = i < b && rowp < sb;
-          const float2 rh = rv ? rhs0s[rowp] : z2;
+          const int rowc = min(rowp, sb - 1);
+          const float2 rh = rhs0s[rowc];
           float2 dc[CPL];
 #pragma unroll
           for (int cc = 0; cc < CPL; ++cc) dc[cc] = shfl_df(dl, (c0 + cc) * LPR);
@@ -322,9 +307,13 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
           float2 u[CPL];
 #pragma unroll
           for (int cc = 0; cc < CPL; ++cc)
-            u[cc] = (rv && c0 + cc < b) ? slot[(c0 + cc) * 256 + rowp] : z2;
+            u[cc] = slot[(c0 + cc) * 256 + rowc];
           const int hb = ((j + 1) & 1) * 16 + i;
-          const float2 accv = (j >= 1 && rv) ? accb[hb] : z2;
+          float2 accv = accb[hb];
+#pragma unroll
+          for (int cc = 0; cc < CPL; ++cc)
+            if (!rv || c0 + cc >= b) u[cc] = z2;
+          if (j < 1 || !rv) accv = z2;
 #pragma unroll
           for (int cc = 0; cc < CPL; ++cc) u[cc] = df_mul(u[cc], dc[cc]);
           float2 us = df_tree_sum(u);
@@ -347,11 +336,16 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
         named_bar_sync(2 + (j & 1));  // D(j)
         const float2* slot = ring + (size_t)(j % DEPTH) * BMAX * 256;
         auto fold = [&](int r, int g, float2& acc, float2& ov) {
-          float2 pr[BMAX];
+          float2 pr[BMAX], dq[BMAX];
           unsigned m = 0;
 #pragma unroll
+          for (int q = 0; q < BMAX; ++q) {  // (columns past b: whatever is there, not used)
+            pr[q] = slot[q * 256 + r];
+            dq[q] = dall[jb + q];
+          }
+#pragma unroll
           for (int q = 0; q < BMAX; ++q) {
-            pr[q] = q < b ? df_mul(slot[q * 256 + r], dall[jb + q]) : z2;
+            pr[q] = q < b ? df_mul(pr[q], dq[q]) : z2;
             if constexpr (OV) m |= (q < b && sidx[jb + q] == g) ? (1u << q) : 0u;
           }
           acc = df_add(acc, df_tree_sum(pr));
@@ -392,5 +386,20 @@ __device__ void chain_la_body(const float2* __restrict__ Rs, const double* __res
     const int g = sidx[tid];
     if (g >= 0 && g < a.N) atomicAdd(a.x + g, dv);
   }
+  return true;
+}
+
+// ready() of the chain: thread 0 waits (bounded; at once when another wait of
+// the grid has given up) until *p >= target, the 256 threads follow.  A wait
+// that gave up is flagged, and the chain goes on with what is there.
+__device__ __forceinline__ bool chain_wait(unsigned* p, unsigned target, bool reset,
+                                           unsigned* err) {
+  if (threadIdx.x == 0) {
+    wait_count(p, target, err);
+    if (reset) *p = 0u;  // for the next launch (which starts after this grid ends)
+    __threadfence();
+  }
+  chain_cta_sync();
+  return true;
 }
 
