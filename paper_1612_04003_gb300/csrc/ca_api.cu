@@ -88,7 +88,17 @@ int finish(ca_ctx* ctx) {
     }
     pr.cls.clear();
   }
+  ctx->err_clean = *ctx->h_err == 0;
   return status_from_err(*ctx->h_err);
+}
+
+// The error word and the ticket behind it at zero where a call starts: they are
+// when the last call ended (finish()) without an error.
+int clear_err(ca_ctx* ctx) {
+  if (!ctx->err_clean)
+    CA_TRY_CUDA(cudaMemsetAsync(ctx->d_err, 0, 33 * sizeof(unsigned), ctx->stream));
+  ctx->err_clean = false;
+  return CA_OK;
 }
 
 // Record an event of class cls on the context's stream (profiling only).
@@ -620,13 +630,17 @@ size_t dense_base_need(ca_ctx* ctx, const ca_opts* o, int method, int xf, bool p
   return need;
 }
 
-void launch_pack(ca_ctx* ctx, const float* A, long long N, long long K, long long lda, float* out) {
-  const long long units = N * ((K + 31) / 32);
-  const long long blocks = std::min<long long>((units * 8 + 255) / 256, 16LL * ctx->num_sms);
+// The panels of A; with rscale (scaled FP16) its rows' multipliers from the
+// same pass.
+int launch_pack(ca_ctx* ctx, const float* A, long long N, long long K, long long lda, float* out,
+                float* rscale) {
+  if (rscale) CA_TRY_CUDA(cudaMemsetAsync(rscale, 0, (size_t)N * 4, ctx->stream));
   prof_mark(ctx, PC_OTHER);
-  k_pack_panels<<<(unsigned)std::max(1LL, blocks), 256, 0, ctx->stream>>>(A, N, K, lda, out);
+  launch_pack_panels(ctx->stream, A, N, K, lda, out, reinterpret_cast<unsigned*>(rscale));
+  if (rscale) launch_row_scale_of(ctx->stream, rscale, N);
   prof_mark(ctx, PC_OTHER);
-  ctx->prof.kernel_launches += 1;
+  ctx->prof.kernel_launches += rscale ? 2 : 1;
+  return cuda_status(cudaGetLastError());
 }
 
 // Stage a caller array on the device (copy in when `in`), return the device pointer.
@@ -644,11 +658,12 @@ T* stage(ca_ctx* ctx, Carve& cv, const T* p, size_t count, bool in, bool* staged
 
 int launch_update_alone(ca_ctx* ctx, const DenseProblem& pb, const int* prev_idx, int prev_sb,
                         const double* prev_delta) {
-  const size_t usm = align256((size_t)prev_sb * 4) + (size_t)prev_sb * 8;  // sidx | delta
-  const unsigned ug = (unsigned)((pb.K + 255) / 256);
+  if (prev_sb <= 0) return CA_OK;
   prof_mark(ctx, PC_UPDATE);
-  launch_update_dense(pb.xfmt == CA_DENSE_F64, ug, usm, ctx->stream, pb.A, pb.lda, pb.N, pb.K,
-                      prev_idx, prev_sb, prev_delta, pb.cU, pb.v, pb.v2, ctx->d_err, pb.panel);
+  const int e = launch_update_dense(pb.xfmt == CA_DENSE_F64, ctx->stream, pb.A, pb.lda, pb.N, pb.K,
+                                    prev_idx, prev_sb, prev_delta, pb.cU, pb.v, pb.v2, ctx->d_err,
+                                    pb.panel);
+  if (e != 0) return cuda_fail((cudaError_t)e, __LINE__);
   prof_mark(ctx, PC_UPDATE);
   ctx->prof.kernel_launches += 1;
   return cuda_status(cudaGetLastError());
@@ -796,14 +811,15 @@ int ca_bcd_solve(ca_ctx* ctx, int xfmt, const void* X, long long d, long long n,
     Xd = p;
   }
   bool panel = pre;
+  float* rsc = nullptr;  // scaled FP16 Gram: row multipliers, from the packing where there is one
   if (tc && !pre) {  // the gather reads 32-column panels (ca_pack_panels layout)
     float* pk = cv.take<float>(panel_bytes(d, n) / 4);
-    launch_pack(ctx, static_cast<const float*>(Xd), d, n, ld, pk);
+    if (f16) rsc = cv.take<float>((size_t)d);
+    CA_TRY(launch_pack(ctx, static_cast<const float*>(Xd), d, n, ld, pk, rsc));
     Xd = pk;
     panel = true;
   }
-  float* rsc = nullptr;  // scaled FP16 Gram: per-feature multipliers (one pass over X)
-  if (f16) {
+  if (f16 && !rsc) {  // scaled FP16 Gram: per-feature multipliers (one pass over X)
     rsc = cv.take<float>((size_t)d);
     launch_row_scale(ctx->stream, static_cast<const float*>(Xd), ld, d, n, panel, rsc);
     ctx->prof.kernel_launches += 1;
@@ -824,7 +840,7 @@ int ca_bcd_solve(ca_ctx* ctx, int xfmt, const void* X, long long d, long long n,
     CA_TRY_CUDA(cudaMemsetAsync(rq, 0, (size_t)rows * 8, ctx->stream));
   }
   char* work = static_cast<char*>(ctx->arena) + align256(cv.off);  // after every carve above
-  CA_TRY_CUDA(cudaMemsetAsync(ctx->d_err, 0, 33 * sizeof(unsigned), ctx->stream));
+  CA_TRY(clear_err(ctx));
 
   DenseProblem pb;
   pb.xfmt = xf;
@@ -940,7 +956,7 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
     float2* GinvB[2] = {Ginv, cv.take<float2>(sbp * CA_FAST_B)};
     double* rn = cv.take<double>((size_t)n);  // row norms (the Grams' diagonals)
     double* pp1 = cv.take<double>(sbp);       // its projections
-    CA_TRY_CUDA(cudaMemsetAsync(ctx->d_err, 0, 33 * sizeof(unsigned), ctx->stream));
+    CA_TRY(clear_err(ctx));
     double* rq = nullptr;
     double* racc = nullptr;
     if (o->check_every > 0) {  // stopping test scratch (zero between uses)
@@ -1184,14 +1200,15 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
     Xd = p;
   }
   bool panel = pre;
+  float* rsc = nullptr;  // scaled FP16 Gram: row multipliers, from the packing where there is one
   if (tc && !pre) {  // the gather reads 32-column panels (ca_pack_panels layout)
     float* pk = cv.take<float>(panel_bytes(n, d) / 4);
-    launch_pack(ctx, static_cast<const float*>(Xd), n, d, ld, pk);
+    if (f16) rsc = cv.take<float>((size_t)n);
+    CA_TRY(launch_pack(ctx, static_cast<const float*>(Xd), n, d, ld, pk, rsc));
     Xd = pk;
     panel = true;
   }
-  float* rsc = nullptr;  // scaled FP16 Gram: per-sample multipliers (one pass over X)
-  if (f16) {
+  if (f16 && !rsc) {  // scaled FP16 Gram: per-sample multipliers (one pass over X)
     rsc = cv.take<float>((size_t)n);
     launch_row_scale(ctx->stream, static_cast<const float*>(Xd), ld, n, d, panel, rsc);
     ctx->prof.kernel_launches += 1;
@@ -1211,7 +1228,7 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
     CA_TRY_CUDA(cudaMemsetAsync(rq, 0, (size_t)rows * 8, ctx->stream));
   }
   char* work = static_cast<char*>(ctx->arena) + align256(cv.off);  // after every carve above
-  CA_TRY_CUDA(cudaMemsetAsync(ctx->d_err, 0, 33 * sizeof(unsigned), ctx->stream));
+  CA_TRY(clear_err(ctx));
   DenseProblem pb;
   pb.xfmt = xf;
   pb.A = Xd;
@@ -1255,8 +1272,7 @@ int ca_pack_panels(ca_ctx* ctx, const float* A, long long N, long long K, long l
     return CA_ERR_ARG;
   if (!is_device_ptr(A) || !is_device_ptr(out)) return CA_ERR_ARG;
   CA_TRY_CUDA(cudaSetDevice(ctx->device));
-  launch_pack(ctx, A, N, K, ld, out);
-  return cuda_status(cudaGetLastError());
+  return launch_pack(ctx, A, N, K, ld, out, nullptr);
 }
 
 const char* ca_last_error(ca_ctx* ctx) { return ctx ? ctx->last_error : "no context"; }
@@ -1326,15 +1342,16 @@ int ca_gram_project(ca_ctx* ctx, int xfmt, int prec, const void* A, long long N,
   void* part = g.tc ? (void*)cv.take<float>((size_t)g.P * g.sbp * g.sbp)
                     : (void*)cv.take<double>((size_t)g.P * g.sbp * g.sbp);
   double* ppart = cv.take<double>((size_t)g.P * g.sbp);
-  double* R = cv.take<double>((size_t)g.sbp * g.sbp);
   float2* v2 = cv.take<float2>((size_t)Kp);
-  CA_TRY_CUDA(cudaMemsetAsync(ctx->d_err, 0, 33 * sizeof(unsigned), ctx->stream));
-  k_split<<<(unsigned)((Kp + 255) / 256), 256, 0, ctx->stream>>>(v, K, Kp, v2);
+  CA_TRY(clear_err(ctx));
+  if (g.tc) launch_split(ctx->stream, v, K, v2);
   if (f16) launch_row_scale(ctx->stream, static_cast<const float*>(A), ld, N, K, false, rsc);
   CA_TRY(launch_gram(ctx, g, xfmt, A, ld, N, K, idx, sb, v, v2, part, ppart, false, rsc));
   SolveArgs sa{idx, N, 1, 0, sb, g.sbp, 0.0, 0.0, 0.0, 0.0, nullptr, nullptr, nullptr};
-  CA_TRY(launch_reduce_solve(ctx, g, part, ppart, R, nullptr, p, nullptr, sa));
-  k_symmetrize<<<(unsigned)(((long long)sb * sb + 255) / 256), 256, 0, ctx->stream>>>(R, g.sbp, sb, G);
+  const long long entries = (long long)sb * (sb + 1) / 2 + sb;
+  launch_reduce(g.tc, (int)std::min<long long>((entries + 63) / 64, 8LL * ctx->num_sms), 0,
+                ctx->stream, part, ppart, g.P, g.sbp, nullptr, nullptr, p, nullptr, 0, sa,
+                ctx->d_err, G);
   CA_TRY_CUDA(cudaGetLastError());
   return finish(ctx);
 }
@@ -1382,7 +1399,7 @@ int ca_selftest_wait_timeout(ca_ctx* ctx, long long limit_ns) {
   t_cur_ctx = ctx;
   if (!ctx || limit_ns < 1 || limit_ns > 1000000000LL) return CA_ERR_ARG;
   CA_TRY_CUDA(cudaSetDevice(ctx->device));
-  CA_TRY_CUDA(cudaMemsetAsync(ctx->d_err, 0, 33 * sizeof(unsigned), ctx->stream));
+  CA_TRY(clear_err(ctx));
   k_selftest_wait<<<1, 32, 0, ctx->stream>>>((unsigned long long)limit_ns, ctx->d_err);
   CA_TRY_CUDA(cudaGetLastError());
   return finish(ctx);

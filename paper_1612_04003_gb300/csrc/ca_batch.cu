@@ -170,7 +170,7 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
   const size_t max_roles = max_roles_of(count);
   CA_TRY(ensure_arena(ctx, need));
   Carve cv{static_cast<char*>(ctx->arena)};
-  CA_TRY_CUDA(cudaMemsetAsync(ctx->d_err, 0, 33 * sizeof(unsigned), ctx->stream));
+  CA_TRY(clear_err(ctx));
 
   // per-problem set-up: panels, v0 = its definition, the sampled indices
   for (int i = 0; i < count; ++i) {
@@ -198,7 +198,7 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
     const float* Ap = static_cast<const float*>(r.X);
     if (r.xfmt != CA_DENSE_F32_PANELS) {
       float* pk = cv.take<float>(panel_bytes(N, K) / 4);
-      launch_pack(ctx, Ap, N, K, r.ld, pk);
+      CA_TRY(launch_pack(ctx, Ap, N, K, r.ld, pk, nullptr));
       Ap = pk;
     }
     pb.A = Ap;

@@ -49,6 +49,7 @@ struct ca_ctx {
   unsigned* d_cnt = nullptr;     // counts of the persistent solves (d_err + 40 .. 48; cleared
                                  // before each persistent launch); d_err + 56: the
                                  // last recomputation whose x has a nonzero entry
+  bool err_clean = false;        // the error word and the ticket are zero
   unsigned nz_epoch = 0;         // recomputations so far
   unsigned* h_err = nullptr;     // pinned copy (128 bytes: error word; check sums at +32)
   // tuning (ca_set_tuning): persistent launches for runs of outer steps, and
@@ -83,12 +84,14 @@ int cuda_status_at(cudaError_t e, int line);
 bool is_device_ptr(const void* p);
 int ensure_arena(ca_ctx* ctx, size_t bytes);
 int finish(ca_ctx* ctx);
+int clear_err(ca_ctx* ctx);
 void prof_mark(ca_ctx* ctx, int cls);
 int check_opts(const ca_opts* o, long long N);
 bool tc_prec(int prec);
 size_t chain_smem(int b, int sb);
 size_t panel_bytes(long long N, long long K);
-void launch_pack(ca_ctx* ctx, const float* A, long long N, long long K, long long lda, float* out);
+int launch_pack(ca_ctx* ctx, const float* A, long long N, long long K, long long lda, float* out,
+                float* rscale);
 void launch_row_scale_ctx(ca_ctx* ctx, const float* A, long long N, long long K, float* rscale);
 
 // The dense outer-step loop shared by both methods.

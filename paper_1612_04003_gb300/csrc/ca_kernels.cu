@@ -249,7 +249,8 @@ template <typename PT>
 __device__ void reduce_body(const PT* __restrict__ part, const double* __restrict__ ppart, int P,
                             int sbp, double* __restrict__ R, float2* __restrict__ Rs,
                             double* __restrict__ pvec, float2* __restrict__ Ginv, int ndiag,
-                            const SolveArgs& sa, unsigned* __restrict__ err, int cta, int ncta) {
+                            const SolveArgs& sa, unsigned* __restrict__ err, int cta, int ncta,
+                            double* __restrict__ Gout = nullptr) {
   __shared__ float2 red[8][32];
   __shared__ float2 Mb[256];
   __shared__ float2 colbuf[66];
@@ -351,6 +352,15 @@ __device__ void reduce_body(const PT* __restrict__ part, const double* __restric
       const double t64 = (redp[w][lane] + redp[w + 1][lane]) + (redp[w + 2][lane] + redp[w + 3][lane]);
       if (kind == 2) {
         pvec[i] = t64;
+      } else if (Gout) {  // the full symmetric matrix
+        double g = t64;
+        if constexpr (sizeof(PT) == 4) {
+          const float2 t = df_add(df_add(red[w][lane], red[w + 1][lane]),
+                                  df_add(red[w + 2][lane], red[w + 3][lane]));
+          g = (double)t.x + (double)t.y;
+        }
+        Gout[(long long)i * sb + j] = g;
+        Gout[(long long)j * sb + i] = g;
       } else if constexpr (sizeof(PT) == 8) {
         R[(long long)i * ldr + j] = t64;
         if (Rs) Rs[(long long)j * ldr + i] = df_mul(cG2, split_f64(t64));
@@ -369,35 +379,38 @@ template <typename PT>
 __global__ void __launch_bounds__(256)
 k_reduce(const PT* __restrict__ part, const double* __restrict__ ppart, int P, int sbp,
          double* __restrict__ R, float2* __restrict__ Rs, double* __restrict__ pvec,
-         float2* __restrict__ Ginv, int ndiag, SolveArgs sa, unsigned* __restrict__ err) {
+         float2* __restrict__ Ginv, int ndiag, SolveArgs sa, double* __restrict__ Gout,
+         unsigned* __restrict__ err) {
+  pdl_wait();
+  pdl_trigger();
   reduce_body<PT>(part, ppart, P, sbp, R, Rs, pvec, Ginv, ndiag, sa, err, (int)blockIdx.x,
-                  (int)gridDim.x);
+                  (int)gridDim.x, Gout);
 }
 
 template __global__ void k_reduce<double>(const double*, const double*, int, int, double*, float2*,
-                                          double*, float2*, int, SolveArgs, unsigned*);
+                                          double*, float2*, int, SolveArgs, double*, unsigned*);
 template __global__ void k_reduce<float>(const float*, const double*, int, int, double*, float2*,
-                                         double*, float2*, int, SolveArgs, unsigned*);
+                                         double*, float2*, int, SolveArgs, double*, unsigned*);
 
 // Gamma_j^{-1} for every diagonal block j = blockIdx.x from R (FP64 lower
-// triangle), one CTA each (b <= 32).
-__global__ void __launch_bounds__(256, 1)
+// triangle), one CTA each (b <= 32), a thread an entry: a pivot is a barrier and
+// one entry's products (with 256 threads and four entries each 0.9 us a pivot,
+// 29 us at b = 32).
+__global__ void __launch_bounds__(1024)
 k_factor(const double* __restrict__ R, SolveArgs sa, float2* __restrict__ Ginv,
          unsigned* __restrict__ err) {
   __shared__ float2 colbuf[66];
-  const int b = sa.b, base = (int)blockIdx.x * b;
-  float2 a[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int e = (int)threadIdx.x + 256 * q;
-    a[q] = make_float2(0.f, 0.f);
-    if (e < b * b) {
-      const int i = e / b, c = e - (e / b) * b;
-      const int hi = i > c ? i : c, lo = i > c ? c : i;
-      a[q] = split_f64(sa.cG * R[(long long)(base + hi) * sa.ldr + (base + lo)] + (i == c ? sa.cI : 0.0));
-    }
+  pdl_wait();
+  pdl_trigger();
+  const int b = sa.b, base = (int)blockIdx.x * b, e = (int)threadIdx.x;
+  float2 a[1] = {make_float2(0.f, 0.f)};
+  if (e < b * b) {
+    const int i = e / b, c = e - (e / b) * b;
+    const int hi = i > c ? i : c, lo = i > c ? c : i;
+    a[0] = split_f64(sa.cG * __ldcg(R + (long long)(base + hi) * sa.ldr + (base + lo)) +
+                     (i == c ? sa.cI : 0.0));
   }
-  cta_sweep_inverse<4>(a, b, colbuf, Ginv + (long long)blockIdx.x * b * b, err);
+  cta_sweep_inverse<1, 1024>(a, b, colbuf, Ginv + (long long)blockIdx.x * b * b, err);
 }
 
 // The dependent chain (one CTA of 256 threads), for sb <= 256, b <= BMAX <= 32,
@@ -627,96 +640,88 @@ k_solve(const double* __restrict__ R, const double* __restrict__ pvec, SolveArgs
 // rebuilds v with exact products before each check, so these FP32 roundings
 // never reach its gap or f(w).)
 // ---------------------------------------------------------------------------
-// CTA = 4 row groups x 64 threads; thread t of group g handles the 4
-// consecutive k at (64 blockIdx + t) * 4 and the rows r = g (mod 4); group 0
-// adds the groups' partial sums and writes v (and its FP32 split v2).
-// PANEL (FP32 only): A stored as 32-column panels [K/32][N][32] (zero-padded).
+// CTA = 4 row groups x 2 sets of 32 columns; a warp (lane = column) takes the
+// rows r = g (mod 4) of its columns, sixteen in flight; the group 0 warps add
+// the groups' sums and write v (and its FP32 split v2).  The first rows of X
+// load before the wait for Delta.  PANEL (FP32 only): A stored as 32-column
+// panels [K/32][N][32] (zero-padded).  Bound by HBM; at few columns by the
+// latency of a warp's loads (four columns a thread and 64 threads a group left
+// four CTAs to K = 1000: 22 us).
 template <typename T, bool PANEL>
 __global__ void __launch_bounds__(256)
 k_update_dense(const T* __restrict__ A, long long lda, long long N, long long K,
                const int* __restrict__ idx, int sb, const double* __restrict__ delta, double cU,
                double* __restrict__ v, float2* __restrict__ v2, unsigned* __restrict__ err) {
   using Acc = typename std::conditional<sizeof(T) == 8, double, float>::type;
+  constexpr int U = 16;
   extern __shared__ unsigned char smem_u[];
-  __shared__ Acc red[3][64][4];
+  __shared__ Acc red[2][3][32];
   int* sidx = reinterpret_cast<int*>(smem_u);
   double* sdl = reinterpret_cast<double*>(smem_u + ((sb * 4 + 255) & ~255));
   float2* sdl2 = reinterpret_cast<float2*>(sdl);  // FP32 path: Delta as (hi, lo)
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, grp = warp & 3, set = warp >> 2;
   for (int r = threadIdx.x; r < sb; r += blockDim.x) {
-    int gi = idx[r];
-    double dl = delta[r];
-    if (gi < 0 || (long long)gi >= N) {  // flagged; the row is skipped
-      if (blockIdx.x == 0) ca_flag(err, CA_DEV_ERR_ARG);
-      gi = 0;
-      dl = 0.0;
-    }
-    sidx[r] = gi;
+    const int gi = idx[r];
+    sidx[r] = gi >= 0 && (long long)gi < N ? gi : -1;  // out of range: flagged, no update from it
+    if (sidx[r] < 0 && blockIdx.x == 0) ca_flag(err, CA_DEV_ERR_ARG);
+  }
+  __syncthreads();
+  const long long a = (long long)blockIdx.x * 2 + set, k = a * 32 + lane;
+  const bool any = a * 32 < K;
+  const T* base = A + (PANEL ? (any ? a : 0) * N * 32 + lane : min(k, K - 1));
+  const long long st = PANEL ? 32 : lda;
+  const int n = sb > grp ? (sb - grp + 3) / 4 : 0;  // rows grp, grp + 4, ...
+  T x[U];
+  auto load = [&](int q0) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      x[u] = __ldg(base + (long long)max(sidx[min(grp + 4 * (q0 + u), sb - 1)], 0) * st);
+  };
+  load(0);
+  pdl_wait();  // Delta and v
+  pdl_trigger();
+  for (int r = threadIdx.x; r < sb; r += blockDim.x) {
+    const double dl = sidx[r] >= 0 ? __ldcg(delta + r) : 0.0;
     if constexpr (sizeof(T) == 8) sdl[r] = dl;
     else sdl2[r] = split_f64(dl);
   }
   __syncthreads();
-  const int grp = threadIdx.x >> 6, t = threadIdx.x & 63;
-  const long long k = ((long long)blockIdx.x * 64 + t) * 4;
-  const int nk = k < K ? (int)min(4ll, K - k) : 0;
-  Acc acc[4] = {0, 0, 0, 0};
-  if (nk > 0) {
-    if constexpr (sizeof(T) == 8) {
-      for (int r = grp; r < sb; r += 4) {
-        const T* row = A + (long long)sidx[r] * lda + k;
-        const double dl = sdl[r];
+  Acc acc = 0;
+  for (int q0 = 0; q0 < n; q0 += U) {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (e < nk) acc[e] = fma((double)row[e], dl, acc[e]);
-      }
-    } else {
-      const bool vec = PANEL || ((nk == 4) && ((lda & 3) == 0) &&
-                                 ((reinterpret_cast<uintptr_t>(A) & 15) == 0));
-      const long long pbase = (k >> 5) * N * 32 + (k & 31);
-#pragma unroll 8
-      for (int r = grp; r < sb; r += 4) {
-        const float* row = reinterpret_cast<const float*>(A) +
-                           (PANEL ? pbase + (long long)sidx[r] * 32 : (long long)sidx[r] * lda + k);
-        const float2 d2 = sdl2[r];
-        float x[4];
-        if (vec) {
-          const float4 q = __ldg(reinterpret_cast<const float4*>(row));
-          x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+    for (int u = 0; u < U; ++u) {
+      if (q0 + u < n) {
+        const int r = grp + 4 * (q0 + u);
+        if constexpr (sizeof(T) == 8) {
+          acc = fma((double)x[u], sdl[r], acc);
         } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) x[e] = (e < nk) ? row[e] : 0.f;
+          const float2 d2 = sdl2[r];
+          acc = fmaf(x[u], d2.x, fmaf(x[u], d2.y, acc));
         }
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[e] = fmaf(x[e], d2.x, fmaf(x[e], d2.y, acc[e]));
       }
     }
+    if (q0 + U < n) load(q0 + U);
   }
-  if (grp > 0) {
-#pragma unroll
-    for (int e = 0; e < 4; ++e) red[grp - 1][t][e] = acc[e];
-  }
+  if (grp > 0) red[set][grp - 1][lane] = acc;
   __syncthreads();
-  if (grp == 0 && nk > 0) {
+  if (grp == 0 && k < K) {
     if constexpr (sizeof(T) == 8) {
-      for (int e = 0; e < nk; ++e) {
-        const double nv = v[k + e] - cU * (acc[e] + red[0][t][e] + red[1][t][e] + red[2][t][e]);
-        v[k + e] = nv;
-        if (v2) v2[k + e] = split_f64(nv);
-      }
+      const double nv = __ldcg(v + k) - cU * (acc + red[set][0][lane] + red[set][1][lane] + red[set][2][lane]);
+      v[k] = nv;
+      if (v2) v2[k] = split_f64(nv);
     } else {
       // FP32 X: the FP32-pair copy v2 is the state the tensor-core passes
       // keep current; update it in double-float and refresh v from it
       const float2 cU2 = split_f64(cU);
-      for (int e = 0; e < nk; ++e) {
-        float hi = acc[e], lo = 0.f;
-        comp_add(hi, lo, red[0][t][e]);
-        comp_add(hi, lo, red[1][t][e]);
-        comp_add(hi, lo, red[2][t][e]);
-        float th, tl;
-        two_sum(hi, lo, th, tl);
-        const float2 nv = df_add(v2[k + e], df_neg(df_mul(cU2, make_float2(th, tl))));
-        v2[k + e] = nv;
-        v[k + e] = (double)nv.x + (double)nv.y;
-      }
+      float hi = acc, lo = 0.f;
+      comp_add(hi, lo, red[set][0][lane]);
+      comp_add(hi, lo, red[set][1][lane]);
+      comp_add(hi, lo, red[set][2][lane]);
+      float th, tl;
+      two_sum(hi, lo, th, tl);
+      const float2 nv = df_add(__ldcg(v2 + k), df_neg(df_mul(cU2, make_float2(th, tl))));
+      v2[k] = nv;
+      v[k] = (double)nv.x + (double)nv.y;
     }
   }
 }
@@ -1541,14 +1546,6 @@ __global__ void k_selftest_wait(unsigned long long limit_ns, unsigned* __restric
   if (threadIdx.x == 0) mbar_wait_bounded(&bar, 0u, err, limit_ns);
 }
 
-// G[i][j] = R[max(i,j)][min(i,j)] (full symmetric copy of the lower triangle)
-__global__ void k_symmetrize(const double* __restrict__ R, int ldr, int sb, double* __restrict__ G) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (long long)sb * sb) return;
-  const int i = (int)(e / sb), j = (int)(e % sb);
-  G[e] = i >= j ? R[(long long)i * ldr + j] : R[(long long)j * ldr + i];
-}
-
 // ---------------------------------------------------------------------------
 // Host launchers of the templated kernels.
 // ---------------------------------------------------------------------------
@@ -1564,19 +1561,24 @@ void launch_gram_simt(bool f64, dim3 grid, cudaStream_t st, const void* A, long 
                                              chunks_per_split, sbp, part, ppart, err);
 }
 
-void launch_reduce(bool f32_partials, int grid, size_t smem, cudaStream_t st, const void* part,
-                   const double* ppart, int P, int sbp, double* R, float2* Rs, double* pvec,
-                   float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err) {
-  if (f32_partials)
-    k_reduce<float><<<grid, 256, smem, st>>>(static_cast<const float*>(part), ppart, P, sbp, R, Rs,
-                                              pvec, Ginv, ndiag, sa, err);
-  else
-    k_reduce<double><<<grid, 256, smem, st>>>(static_cast<const double*>(part), ppart, P, sbp, R,
-                                               Rs, pvec, Ginv, ndiag, sa, err);
-}
-
 template <typename K, typename... Args>
 cudaError_t launch_programmatic(K kernel, unsigned grid, size_t smem, cudaStream_t st, Args... args);
+template <typename K, typename... Args>
+cudaError_t launch_programmatic_t(K kernel, unsigned grid, unsigned threads, size_t smem,
+                                  cudaStream_t st, Args... args);
+
+void launch_reduce(bool f32_partials, int grid, size_t smem, cudaStream_t st, const void* part,
+                   const double* ppart, int P, int sbp, double* R, float2* Rs, double* pvec,
+                   float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err, double* Gout) {
+  if (f32_partials)
+    launch_programmatic(k_reduce<float>, (unsigned)grid, smem, st, static_cast<const float*>(part),
+                        ppart, P, sbp, R, Rs, pvec, Ginv, ndiag, sa, Gout, err);
+  else
+    launch_programmatic(k_reduce<double>, (unsigned)grid, smem, st,
+                        static_cast<const double*>(part), ppart, P, sbp, R, Rs, pvec, Ginv, ndiag,
+                        sa, Gout, err);
+}
+
 
 void launch_chain(int b, size_t smem, cudaStream_t st, const float2* Rs, const double* pvec,
                   const float2* Ginv, const SolveArgs& sa, unsigned* err) {
@@ -1590,9 +1592,15 @@ void launch_chain(int b, size_t smem, cudaStream_t st, const float2* Rs, const d
 
 template <typename K, typename... Args>
 cudaError_t launch_programmatic(K kernel, unsigned grid, size_t smem, cudaStream_t st, Args... args) {
+  return launch_programmatic_t(kernel, grid, 256u, smem, st, args...);
+}
+
+template <typename K, typename... Args>
+cudaError_t launch_programmatic_t(K kernel, unsigned grid, unsigned threads, size_t smem,
+                                  cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -1657,25 +1665,35 @@ k_rowdot_dense(const T* __restrict__ A, long long lda, long long N, long long K,
     }
   };
   T cur[8], nxt[8];
+  using V = typename std::conditional<F64, double, float2>::type;
+  auto load_v = [&](long long a) -> V {
+    const long long k = a * 32 + lane;
+    if constexpr (F64) return k < K ? __ldcg(v + k) : 0.0;
+    else return __ldcg(v2 + k);  // (zero past K, as A's panels)
+  };
+  V vk{}, vn{};
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   float hi[8], lo[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) hi[j] = lo[j] = 0.f;
-  if (a0 < a1) load(a0, cur);
+  if (a0 < a1) {
+    load(a0, cur);
+    vk = load_v(a0);
+  }
   for (long long a = a0; a < a1; ++a) {
     load(min(a + 1, a1 - 1), nxt);
+    vn = load_v(min(a + 1, a1 - 1));
     const long long k = a * 32 + lane;
     if constexpr (F64) {
-      const double vk = k < K ? __ldcg(v + k) : 0.0;
 #pragma unroll
       for (int j = 0; j < 8; ++j) acc[j] = fma((double)cur[j], vk, acc[j]);
     } else {
-      const float2 vk = __ldcg(v2 + k);  // (zero past K, as A's panels)
 #pragma unroll
       for (int j = 0; j < 8; ++j) df_dot_acc(PANEL || k < K ? cur[j] : 0.f, vk.x, vk.y, hi[j], lo[j]);
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) cur[j] = nxt[j];
+    vk = vn;
   }
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
@@ -1771,6 +1789,13 @@ void launch_sumsq(cudaStream_t st, int num_sms, double* q, const double* x, cons
 // the FP16 range (largest finite 65504), and G_ij of the scaled rows is the
 // true one times rscale[i] rscale[j] exactly.  A zero or non-finite row gets
 // 1.  One warp per row.
+__device__ __forceinline__ float row_scale(float mx) {
+  if (!(mx > 0.f && mx <= 3.4028234e38f)) return 1.f;
+  int e = 0;
+  frexpf(mx, &e);
+  return ldexpf(1.f, min(max(15 - e, -120), 120));
+}
+
 __global__ void __launch_bounds__(256)
 k_row_scale(const float* __restrict__ A, long long lda, long long N, long long K, int panel,
             float* __restrict__ rscale) {
@@ -1790,15 +1815,7 @@ k_row_scale(const float* __restrict__ A, long long lda, long long N, long long K
   }
   float mx = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
   for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) {
-    float sc = 1.f;
-    if (mx > 0.f && mx <= 3.4028234e38f) {
-      int e = 0;
-      frexpf(mx, &e);
-      sc = ldexpf(1.f, min(max(15 - e, -120), 120));
-    }
-    rscale[r] = sc;
-  }
+  if (lane == 0) rscale[r] = row_scale(mx);
 }
 
 void launch_row_scale(cudaStream_t st, const float* A, long long lda, long long N, long long K,
@@ -1808,25 +1825,28 @@ void launch_row_scale(cudaStream_t st, const float* A, long long lda, long long 
 
 void launch_factor(cudaStream_t st, const double* R, const SolveArgs& sa, float2* Ginv,
                    unsigned* err) {
-  k_factor<<<sa.s_cur, 256, 0, st>>>(R, sa, Ginv, err);
+  launch_programmatic_t(k_factor, (unsigned)sa.s_cur, 1024u, 0, st, R, sa, Ginv, err);
 }
 
 // Rs[j][i] = FP32 split of cG R[i][j] (transposed, as k_reduce writes it) for
 // the lower-triangle entries outside the diagonal blocks (the sparse path
 
-void launch_update_dense(bool f64, unsigned grid, size_t smem, cudaStream_t st, const void* A,
-                         long long lda, long long N, long long K, const int* idx, int sb,
-                         const double* delta, double cU, double* v, float2* v2, unsigned* err,
-                         bool panel) {
+int launch_update_dense(bool f64, cudaStream_t st, const void* A, long long lda, long long N,
+                        long long K, const int* idx, int sb, const double* delta, double cU,
+                        double* v, float2* v2, unsigned* err, bool panel) {
+  const unsigned grid = (unsigned)((K + 63) / 64);
+  const size_t smem = (((size_t)sb * 4 + 255) & ~(size_t)255) + (size_t)sb * 8;  // sidx | delta
   if (f64)
-    k_update_dense<double, false><<<grid, 256, smem, st>>>(static_cast<const double*>(A), lda, N, K,
-                                                            idx, sb, delta, cU, v, v2, err);
-  else if (panel)
-    k_update_dense<float, true><<<grid, 256, smem, st>>>(static_cast<const float*>(A), lda, N, K,
-                                                          idx, sb, delta, cU, v, v2, err);
-  else
-    k_update_dense<float, false><<<grid, 256, smem, st>>>(static_cast<const float*>(A), lda, N, K,
-                                                           idx, sb, delta, cU, v, v2, err);
+    return (int)launch_programmatic(k_update_dense<double, false>, grid, smem, st,
+                                    static_cast<const double*>(A), lda, N, K, idx, sb, delta, cU, v,
+                                    v2, err);
+  if (panel)
+    return (int)launch_programmatic(k_update_dense<float, true>, grid, smem, st,
+                                    static_cast<const float*>(A), lda, N, K, idx, sb, delta, cU, v,
+                                    v2, err);
+  return (int)launch_programmatic(k_update_dense<float, false>, grid, smem, st,
+                                  static_cast<const float*>(A), lda, N, K, idx, sb, delta, cU, v, v2,
+                                  err);
 }
 
 int launch_recompute_dense(bool f64, int num_sms, cudaStream_t st, const void* A, long long lda,
@@ -1870,31 +1890,59 @@ void launch_split(cudaStream_t st, const double* v, long long K, float2* v2) {
 
 // Repack a row-major N x K FP32 matrix (leading dimension lda, 16-byte aligned
 // rows) into 32-column panels: P[(a N + r) 32 + c] = A[r][32 a + c], zero past
-// K.  Units of 128 bytes (one row of one panel), 8 lanes each; consecutive
-// units run along a row, so a warp reads 512 contiguous bytes and writes four
-// full 128-byte lines.
+// K.  A CTA takes 8 rows x 64 panels: a warp reads 512 contiguous bytes of its
+// row (four panels), the eight warps write 1 KB of each panel.  rmax (when not
+// null, zero on entry): the bits of each row's largest magnitude, NaN left out.
 __global__ void __launch_bounds__(256)
 k_pack_panels(const float* __restrict__ A, long long N, long long K, long long lda,
-              float* __restrict__ Pn) {
+              float* __restrict__ Pn, unsigned* __restrict__ rmax) {
   const long long na = (K + 31) / 32;
-  const long long units = N * na;
-  const int q = threadIdx.x & 7;
-  for (long long u = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3; u < units;
-       u += ((long long)gridDim.x * blockDim.x) >> 3) {
-    const long long r = u / na, a = u - r * na;
-    const long long k = a * 32 + 4 * q;
-    const float* src = A + r * lda + k;
-    float4 x;
-    if (k + 4 <= K) {
-      x = __ldg(reinterpret_cast<const float4*>(src));
-    } else {
-      x.x = k < K ? src[0] : 0.f;
-      x.y = k + 1 < K ? src[1] : 0.f;
-      x.z = k + 2 < K ? src[2] : 0.f;
-      x.w = 0.f;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = lane & 7;
+  const long long nrb = (N + 7) / 8;
+  const long long rb = blockIdx.x % nrb, ab = blockIdx.x / nrb;
+  const long long r = rb * 8 + warp;
+  if (r >= N) return;
+  const float* row = A + r * lda;
+  float m = 0.f;
+#pragma unroll 4
+  for (int it = 0; it < 16; ++it) {
+    const long long a = ab * 64 + it * 4 + (lane >> 3), k = a * 32 + 4 * q;
+    if (a < na) {
+      float4 x;
+      if (k + 4 <= K) {
+        x = __ldg(reinterpret_cast<const float4*>(row + k));
+      } else {
+        x.x = k < K ? row[k] : 0.f;
+        x.y = k + 1 < K ? row[k + 1] : 0.f;
+        x.z = k + 2 < K ? row[k + 2] : 0.f;
+        x.w = 0.f;
+      }
+      *reinterpret_cast<float4*>(Pn + (a * N + r) * 32 + 4 * q) = x;
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
     }
-    *reinterpret_cast<float4*>(Pn + (a * N + r) * 32 + 4 * q) = x;
   }
+  if (rmax) {
+    const unsigned mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    if (lane == 0) atomicMax(rmax + r, mb);
+  }
+}
+
+void launch_pack_panels(cudaStream_t st, const float* A, long long N, long long K, long long lda,
+                        float* Pn, unsigned* rmax) {
+  const long long na = (K + 31) / 32;
+  k_pack_panels<<<(unsigned)(((N + 7) / 8) * ((na + 63) / 64)), 256, 0, st>>>(A, N, K, lda, Pn, rmax);
+}
+
+// The scaled-FP16 multipliers of k_row_scale from the rows' largest magnitudes
+// (in place).
+__global__ void __launch_bounds__(256)
+k_row_scale_of(float* __restrict__ rscale, long long N) {
+  const long long r = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (r < N) rscale[r] = row_scale(rscale[r]);
+}
+
+void launch_row_scale_of(cudaStream_t st, float* rscale, long long N) {
+  k_row_scale_of<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(rscale, N);
 }
 
 // Raise the dynamic shared-memory limit of the solve kernels to `bytes`, less

@@ -16,7 +16,8 @@ void launch_gram_simt(bool f64, dim3 grid, cudaStream_t st, const void* A, long 
 // chain (fast form) or the general solve.
 void launch_reduce(bool f32_partials, int grid, size_t smem, cudaStream_t st, const void* part,
                    const double* ppart, int P, int sbp, double* R, float2* Rs, double* pvec,
-                   float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err);
+                   float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err,
+                   double* Gout = nullptr);
 void launch_chain(int b, size_t smem, cudaStream_t st, const float2* Rs, const double* pvec,
                   const float2* Ginv, const SolveArgs& sa, unsigned* err);
 void launch_factor(cudaStream_t st, const double* R, const SolveArgs& sa, float2* Ginv,
@@ -28,14 +29,12 @@ int launch_reduce_chain(int grid, size_t smem, cudaStream_t st, const float* par
                         const double* ppart, int P, int sbp, double* R, float2* Rs, double* pvec,
                         float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err,
                         unsigned* ticket);
-__global__ void k_factor(const double* R, SolveArgs sa, float2* Ginv, unsigned* err);
 #define CA_FAST_B 32
 #define CA_FAST_SB 256
 // panel: FP32 A stored as 32-column panels [K/32][N][32] (k_pack_panels).
-void launch_update_dense(bool f64, unsigned grid, size_t smem, cudaStream_t st, const void* A,
-                         long long lda, long long N, long long K, const int* idx, int sb,
-                         const double* delta, double cU, double* v, float2* v2, unsigned* err,
-                         bool panel);
+int launch_update_dense(bool f64, cudaStream_t st, const void* A, long long lda, long long N,
+                        long long K, const int* idx, int sb, const double* delta, double cU,
+                        double* v, float2* v2, unsigned* err, bool panel);
 // v = c0 y0 + c1 A^T x (two launches); x2: N pairs of scratch (FP32 A); *nz is set
 // to epoch (new for each call) when x has a nonzero entry.  Returns a cudaError_t.
 int launch_recompute_dense(bool f64, int num_sms, cudaStream_t st, const void* A, long long lda,
@@ -43,7 +42,11 @@ int launch_recompute_dense(bool f64, int num_sms, cudaStream_t st, const void* A
                            double c0, double c1, double* v, bool panel, unsigned* nz,
                            unsigned epoch);
 void launch_split(cudaStream_t st, const double* v, long long K, float2* v2);
-__global__ void k_pack_panels(const float* A, long long N, long long K, long long lda, float* Pn);
+// rmax (N words, zero): the rows' largest magnitudes as bits, which
+// launch_row_scale_of turns into the scaled-FP16 multipliers.
+void launch_pack_panels(cudaStream_t st, const float* A, long long N, long long K, long long lda,
+                        float* Pn, unsigned* rmax);
+void launch_row_scale_of(cudaStream_t st, float* rscale, long long N);
 int set_solve_smem_limit(int bytes);
 
 __global__ void k_solve(const double* R, const double* pvec, SolveArgs sa, unsigned* err);
@@ -57,7 +60,6 @@ __global__ void k_scatter_csr(const long long* rowptr, const int* col, const flo
                               unsigned* err);
 
 __global__ void k_selftest_wait(unsigned long long limit_ns, unsigned* err);
-__global__ void k_symmetrize(const double* R, int ldr, int sb, double* G);
 
 // tcgen05 Gram (ca_gram_tc.cu): host-side launcher.  Returns a cudaError_t.
 // Computes FP32 partials part[c][j][i] (c < P, stride sbp; stored transposed) of

@@ -34,8 +34,7 @@ constexpr size_t kErrOff = 0;                                              // er
 constexpr size_t kV2Off = 256;                                             // kMaxK float2
 constexpr size_t kPartOff = kV2Off + (size_t)kMaxK * 8;                    // kSplits x 128 x 128 doubles
 constexpr size_t kPPartOff = kPartOff + (size_t)kSplits * 128 * 128 * 8;   // kSplits x 128 doubles
-constexpr size_t kROff = kPPartOff + (size_t)kSplits * 128 * 8;            // 128 x 128 doubles
-constexpr size_t kTotal = kROff + (size_t)128 * 128 * 8;
+constexpr size_t kTotal = kPPartOff + (size_t)kSplits * 128 * 8;
 
 }  // namespace
 
@@ -101,7 +100,6 @@ extern "C" int ca_gram_project_noalloc(void* cuda_stream, int xfmt, int prec, co
   float2* v2 = reinterpret_cast<float2*>(base + kV2Off);
   void* part = base + kPartOff;
   double* ppart = reinterpret_cast<double*>(base + kPPartOff);
-  double* R = reinterpret_cast<double*>(base + kROff);
 
   // only the error word must start at zero; every other region read below is
   // first written by this call
@@ -131,8 +129,7 @@ extern "C" int ca_gram_project_noalloc(void* cuda_stream, int xfmt, int prec, co
   SolveArgs sa{idx, N, 1, 0, sb, sbp, 0.0, 0.0, 0.0, 0.0, nullptr, nullptr, nullptr};
   const long long entries = (long long)sb * (sb + 1) / 2 + sb;
   launch_reduce(tc, (int)std::min<long long>((entries + 31) / 32, 256), 0, stream, part, ppart, P,
-                sbp, R, nullptr, p, nullptr, 0, sa, err);
-  k_symmetrize<<<(unsigned)(((long long)sb * sb + 255) / 256), 256, 0, stream>>>(R, sbp, sb, G);
+                sbp, nullptr, nullptr, p, nullptr, 0, sa, err, G);
   if (cudaGetLastError() != cudaSuccess) return CA_ERR_CUDA;
   unsigned host_err = 0;
   if (cudaMemcpyAsync(&host_err, err, sizeof(unsigned), cudaMemcpyDeviceToHost, stream) !=

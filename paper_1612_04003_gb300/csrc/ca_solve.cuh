@@ -29,7 +29,7 @@ template <int EPT, int NT = 256, int BAR = 1>
 __device__ void cta_sweep_inverse(float2 (&a)[EPT], int b, float2* __restrict__ colbuf,
                                   float2* __restrict__ out, unsigned* __restrict__ err,
                                   int tix = -1) {
-  static_assert(NT == 256 || NT == 64, "a CTA of 256 threads or two of its warps");
+  static_assert(NT == 1024 || NT == 256 || NT == 64, "a whole CTA or two of its warps");
   const int t = tix >= 0 ? tix : (int)(threadIdx.x % NT);  // index among the NT threads
   int ri[EPT], ci[EPT];
 #pragma unroll
@@ -48,7 +48,7 @@ __device__ void cta_sweep_inverse(float2 (&a)[EPT], int b, float2* __restrict__ 
         if (ri[q] == k && !(a[q].x > 0.f)) ca_flag(err, CA_DEV_ERR_NOT_SPD);
       }
     }
-    if constexpr (NT < 256 || BAR != 1) asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
+    if constexpr (NT == 64 || BAR != 1) asm volatile("bar.sync %0, %1;" ::"n"(BAR), "n"(NT) : "memory");
     else __syncthreads();
     if (active) {
       // every thread forms 1 / a_kk itself (shorter than a broadcast)
