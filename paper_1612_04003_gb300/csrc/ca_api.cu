@@ -176,6 +176,21 @@ bool check_says_stop(const ca_opts* o, const ca_info& in) {
   return check_stops(o->stop == CA_STOP_OBJECTIVE, o->tol, in.res0, in.res, in.gap, in.fval);
 }
 
+// The sparse dual's side streams and their events, made on first use.
+int make_side(ca_ctx* ctx) {
+  auto event = [](cudaEvent_t* e) {
+    return *e ? cudaSuccess : cudaEventCreateWithFlags(e, cudaEventDisableTiming);
+  };
+  CA_TRY_CUDA(event(&ctx->evs));
+  for (int q = 0; q < 3; ++q) {
+    CA_TRY_CUDA(event(&ctx->ev_ready[q]));
+    CA_TRY_CUDA(event(&ctx->ev_read[q]));
+  }
+  for (cudaStream_t& sd : ctx->side)
+    if (!sd) CA_TRY_CUDA(cudaStreamCreateWithFlags(&sd, cudaStreamNonBlocking));
+  return CA_OK;
+}
+
 int launch_recompute(ca_ctx* ctx, const DenseProblem& pb, double* vout, const double* y0,
                      double c0, double c1) {
   prof_mark(ctx, PC_OTHER);
@@ -736,12 +751,16 @@ void ca_bcd_destroy(ca_ctx* ctx) {
   if (!ctx) return;
   cudaSetDevice(ctx->device);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  if (ctx->side) {
-    cudaStreamSynchronize(ctx->side);
-    cudaStreamDestroy(ctx->side);
+  for (cudaStream_t sd : ctx->side) {
+    if (!sd) continue;
+    cudaStreamSynchronize(sd);
+    cudaStreamDestroy(sd);
   }
-  for (cudaEvent_t e : ctx->ev)
-    if (e) cudaEventDestroy(e);
+  if (ctx->evs) cudaEventDestroy(ctx->evs);
+  for (int q = 0; q < 3; ++q) {
+    if (ctx->ev_ready[q]) cudaEventDestroy(ctx->ev_ready[q]);
+    if (ctx->ev_read[q]) cudaEventDestroy(ctx->ev_read[q]);
+  }
   for (cudaEvent_t e : ctx->prof.pool) cudaEventDestroy(e);
   if (ctx->arena) cudaFree(ctx->arena);
   if (ctx->d_err) cudaFree(ctx->d_err);
@@ -919,6 +938,9 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
     const size_t sbp = (size_t)(sbm + 31) / 32 * 32;
     need += 5 * align256(sbp * sbp * 8) + 3 * align256(sbp * 8) + 2 * align256(sbp * CA_FAST_B * 8) +
             4096;
+    // a third set of buffers lets the Grams of two later steps be formed at
+    // once; a tight scratch bound does without
+    const size_t third = 2 * align256(sbp * sbp * 8) + align256(sbp * CA_FAST_B * 8);
     if (o->check_every > 0) need += align256((size_t)check_rows(o, n, d) * 8) + 512;
     // the dense-sparse split of the Gram (s*b >= 32): column counts, the
     // dense map, and Xd (nrows x fd FP32, 64 MB at most)
@@ -933,6 +955,8 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
     const size_t roff_bytes = csr_rangeoff_bytes(n, d);
     const bool use_roff = split && roff_bytes <= ((size_t)256 << 20);
     if (use_roff) need += align256(roff_bytes);
+    const int nbuf = ctx->scratch_max && need + third > ctx->scratch_max ? 2 : 3;
+    if (nbuf == 3) need += third;
     CA_TRY(ensure_arena(ctx, need));
     Carve cv{static_cast<char*>(ctx->arena)};
     bool st;
@@ -949,11 +973,16 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
     float2* Ginv = cv.take<float2>(sbp * CA_FAST_B);
     float2* Rs = cv.take<float2>(sbp * sbp);
     // the Gram (transposed lower triangle), Rs and the diagonal-block
-    // inverses, two buffers each: what step k+1 needs of them is formed on
-    // the side stream while step k's solves read the other
-    double* Gbuf[2] = {cv.take<double>(sbp * sbp), cv.take<double>(sbp * sbp)};
-    float2* RsB[2] = {Rs, cv.take<float2>(sbp * sbp)};
-    float2* GinvB[2] = {Ginv, cv.take<float2>(sbp * CA_FAST_B)};
+    // inverses, nbuf buffers each: what steps k+1 (and k+2) need of them is
+    // formed on side streams while step k's solves read another
+    double* Gbuf[3] = {cv.take<double>(sbp * sbp), cv.take<double>(sbp * sbp), nullptr};
+    float2* RsB[3] = {Rs, cv.take<float2>(sbp * sbp), nullptr};
+    float2* GinvB[3] = {Ginv, cv.take<float2>(sbp * CA_FAST_B), nullptr};
+    if (nbuf == 3) {
+      Gbuf[2] = cv.take<double>(sbp * sbp);
+      RsB[2] = cv.take<float2>(sbp * sbp);
+      GinvB[2] = cv.take<float2>(sbp * CA_FAST_B);
+    }
     double* rn = cv.take<double>((size_t)n);  // row norms (the Grams' diagonals)
     double* pp1 = cv.take<double>(sbp);       // its projections
     CA_TRY(clear_err(ctx));
@@ -1028,132 +1057,100 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
       CA_TRY(residual(&ctx->info.res0, 0));
       ctx->info.res = ctx->info.res0;
     }
-    // s*b <= 4096: the strict lower triangle of each step's Gram (the split,
-    // or one warp per pair) has no input that the solves change, so it runs
-    // on the side stream one step ahead; events: ev[0] the start and the
-    // join, ev[1 + k%2] buffer k%2 formed, ev[3 + k%2] buffer k%2 read
-    const bool two = sbm <= 4096;
-    if (two && !ctx->side) {
-      for (cudaEvent_t& e : ctx->ev)
-        if (!e) CA_TRY_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-      CA_TRY_CUDA(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
-    }
-    struct SideJoin {  // every exit: the main stream waits for the side stream's work
+    // The strict lower triangle of each step's Gram (the split, or one warp per
+    // pair) has no input that the solves change: it is formed on side streams,
+    // nbuf - 1 steps ahead, each step on the stream of its turn.  Events: evs the
+    // start and the join, ev_ready[k % nbuf] buffer formed, ev_read[k % nbuf]
+    // buffer read.
+    const int ahead = nbuf - 1;
+    CA_TRY(make_side(ctx));
+    struct SideJoin {  // every exit: the main stream waits for the side streams' work
       ca_ctx* c;
       bool on;
       void operator()() {
         if (!on) return;
         on = false;
-        cudaEventRecord(c->ev[0], c->side);
-        cudaStreamWaitEvent(c->stream, c->ev[0], 0);
+        for (cudaStream_t sd : c->side) {
+          cudaEventRecord(c->evs, sd);
+          cudaStreamWaitEvent(c->stream, c->evs, 0);
+        }
       }
       ~SideJoin() { (*this)(); }
     } join{ctx, false};
-    // the fast a4 (b <= 16) with s*b >= 128: the diagonal blocks' inverses
-    // and Rs come from the side stream too, and the library stream runs the
-    // projections, the chain and the scatter (below 128 rows the extra
-    // launch on the side stream costs more than the reduction it moves)
-    constexpr int kPrepMinSB = 128;
+    // the fast a4 (b <= 16): the diagonal blocks' inverses and Rs come from the
+    // side streams too, and the library stream runs the projections, the chain
+    // and the scatter
     const bool f64solve = o->solve == CA_SOLVE_F64;
-    auto fast_step = [&](int sbk) {
-      return two && fast_solve(b, sbk, f64solve) && b <= 16 && sbk >= kPrepMinSB;
-    };
+    auto fast_step = [&](int sbk) { return fast_solve(b, sbk, f64solve) && b <= 16; };
     auto step_args = [&](long long kk) {
       const int skk = (int)std::min<long long>(s, o->H - (long long)s * kk);
       return SolveArgs{idx + (size_t)s * kk * b, n, b, skk, skk * b, (int)sbp, 1.0 / ln, 1.0, 1.0,
                        1.0, ad, yd, delta};
     };
-    auto offdiag = [&](long long kk) {
+    auto form_gram = [&](long long kk) -> int {  // step kk's, on its side stream
       const SolveArgs sk_args = step_args(kk);
-      const int sbk = sk_args.sb;
+      const int sbk = sk_args.sb, q = (int)(kk % nbuf);
       const bool sp = split && sbk >= kSplitMinSB;
-      launch_csr_offdiag(ctx->side, cdev, sk_args.idx, n, d, sbk, (int)sbp, Gbuf[kk & 1], dmap, Xd,
-                         fd, sp, roff);
+      cudaStream_t sd = ctx->side[kk % ahead];
+      // buffer q was last read by the solves of step kk - nbuf
+      if (kk >= nbuf) CA_TRY_CUDA(cudaStreamWaitEvent(sd, ctx->ev_read[q], 0));
+      launch_csr_offdiag(sd, cdev, sk_args.idx, n, d, sbk, (int)sbp, Gbuf[q], dmap, Xd, fd, sp, roff);
       ctx->prof.kernel_launches += sbk <= 1 ? 0 : (sp ? 2 : 1);
       if (fast_step(sbk)) {
-        launch_csr_prep(ctx->side, ctx->num_sms, rn, n, Gbuf[kk & 1], sk_args, RsB[kk & 1],
-                        GinvB[kk & 1], ctx->d_err);
+        launch_csr_prep(sd, ctx->num_sms, rn, n, Gbuf[q], sk_args, RsB[q], GinvB[q], ctx->d_err);
         ctx->prof.kernel_launches += 1;
       }
+      CA_TRY_CUDA(cudaEventRecord(ctx->ev_ready[q], sd));
+      return CA_OK;
     };
-    if (fast_step(sbm)) {  // before the side stream starts
+    if (fast_step(b)) {  // before the side streams start
       launch_csr_rownorm(ctx->stream, cdev, n, rn);
       ctx->prof.kernel_launches += 1;
     }
-    if (two && n_outer > 0) {
-      CA_TRY_CUDA(cudaEventRecord(ctx->ev[0], ctx->stream));
-      CA_TRY_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev[0], 0));
-      join.on = true;
-      offdiag(0);
-      CA_TRY_CUDA(cudaEventRecord(ctx->ev[1], ctx->side));
-    }
+    CA_TRY_CUDA(cudaEventRecord(ctx->evs, ctx->stream));
+    for (cudaStream_t sd : ctx->side) CA_TRY_CUDA(cudaStreamWaitEvent(sd, ctx->evs, 0));
+    join.on = true;
+    for (long long kk = 0; kk < std::min<long long>(ahead, n_outer); ++kk) CA_TRY(form_gram(kk));
     for (long long k = 0; k < n_outer; ++k) {
       const int sk = (int)std::min<long long>(s, o->H - (long long)s * k);
-      const int sb = sk * b;
+      const int sb = sk * b, q = (int)(k % nbuf);
       const int* ik = idx + (size_t)s * k * b;
-      double* Gt = Gbuf[k & 1];
-      // a2+a3: the projections here (with the diagonal when s*b < 128); the
-      // rest of the Gram comes from the side stream (all of it, by the row
-      // hash tables, when s*b > 4096)
+      double* Gt = Gbuf[q];
+      if (k + ahead < n_outer) CA_TRY(form_gram(k + ahead));
+      CA_TRY_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev_ready[q], 0));
+      // a2+a3: the projections here (with the diagonal on the general path);
+      // the rest of the Gram comes from the side streams
       const bool fk = fast_step(sb);
       prof_mark(ctx, PC_GRAM);
-      if (fk) {
-        launch_csr_proj(ctx->stream, cdev, ik, n, d, sb, wd, pp1, ctx->d_err);
-        ctx->prof.kernel_launches += 1;
-      } else if (two) {
-        launch_csr_rows(ctx->stream, cdev, ik, n, d, sb, (int)sbp, wd, Gt, pp1, ctx->d_err);
-        ctx->prof.kernel_launches += 1;
-      } else {
-        launch_csr_gram(ctx->stream, ctx->num_sms, cdev, ik, n, d, sb, (int)sbp, wd, Gt, pp1,
-                        ctx->d_err);
-        ctx->prof.kernel_launches += sb > 1 ? 2 : 1;
-      }
+      if (fk) launch_csr_proj(ctx->stream, cdev, ik, n, d, sb, wd, pp1, ctx->d_err);
+      else launch_csr_rows(ctx->stream, cdev, ik, n, d, sb, (int)sbp, wd, Gt, pp1, ctx->d_err);
+      ctx->prof.kernel_launches += 1;
       prof_mark(ctx, PC_GRAM);
-      if (two) {
-        if (k + 1 < n_outer) {  // buffer (k+1)%2 was last read by the solves of step k-1
-          if (k >= 1) CA_TRY_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev[3 + ((k + 1) & 1)], 0));
-          offdiag(k + 1);
-          CA_TRY_CUDA(cudaEventRecord(ctx->ev[1 + ((k + 1) & 1)], ctx->side));
-        }
-        CA_TRY_CUDA(cudaStreamWaitEvent(ctx->stream, ctx->ev[1 + (k & 1)], 0));
-      }
-      // a4: with b <= 16 the chain alone (its other inputs are ready), or
-      // the Gram through the dense path's reduction as its one FP64
-      // partial: reduce + diagonal inverses + chain in one launch, else the
-      // general form
+      // a4: with b <= 16 the chain alone (its other inputs are ready), else the
+      // general form on the Gram as one FP64 partial
       const SolveArgs sa = step_args(k);
       if (fk) {
         prof_mark(ctx, PC_SOLVE);
-        launch_chain(b, chain_smem(b, sb), ctx->stream, RsB[k & 1], pp1, GinvB[k & 1], sa,
-                     ctx->d_err);
+        // (shared memory enough that no CTA of the side streams' Gram kernels
+        // shares the chain's SM: they would take its issue slots)
+        launch_chain(b, std::max<size_t>(chain_smem(b, sb), 200 * 1024), ctx->stream, RsB[q], pp1,
+                     GinvB[q], sa, ctx->d_err);
         prof_mark(ctx, PC_SOLVE);
         ctx->prof.kernel_launches += 1;
-      } else if (fast_solve(b, sb, f64solve) && b <= 16) {
-        const long long entries = (long long)sb * (sb + 1) / 2 + sb;
-        const int grid = (int)std::max<long long>(
-                             1, std::min<long long>((entries + 63) / 64 + sk, ctx->num_sms - 1)) + 1;
-        prof_mark(ctx, PC_SOLVE);
-        const int e = launch_reduce_chain_f64(grid, chain_smem(b, sb), ctx->stream, Gt, pp1,
-                                              (int)sbp, R, RsB[k & 1], pvec, GinvB[k & 1], sk, sa,
-                                              ctx->d_err, ctx->d_ticket);
-        prof_mark(ctx, PC_SOLVE);
-        ctx->prof.kernel_launches += 1;
-        if (e != 0) return cuda_fail((cudaError_t)e, __LINE__);
       } else {
         GramPlan g{};
         g.tc = false;
         g.sbp = (int)sbp;
         g.P = 1;
-        // (Rs and Ginv of this step's parity: the side stream may be
-        // writing the other pair for the next step)
-        CA_TRY(launch_reduce_solve(ctx, g, Gt, pp1, R, RsB[k & 1], pvec, GinvB[k & 1], sa,
-                                   f64solve));
+        CA_TRY(launch_reduce_solve(ctx, g, Gt, pp1, R, RsB[q], pvec, GinvB[q], sa, f64solve));
       }
-      if (two) CA_TRY_CUDA(cudaEventRecord(ctx->ev[3 + (k & 1)], ctx->stream));
       // a5: w -= Y Delta/(lambda n)
       launch_scatter_csr(ctx->stream, cdev, ik, n, d, sb, delta, -1.0 / ln, wd, ctx->d_err);
       ctx->prof.kernel_launches += 1;
       CA_TRY_CUDA(cudaGetLastError());
+      // (after the scatter: a stream operation between two kernels would keep
+      // the second from starting early)
+      CA_TRY_CUDA(cudaEventRecord(ctx->ev_read[q], ctx->stream));
       if (o->recompute_every > 0 && (k + 1) % o->recompute_every == 0) recompute();
       if (o->check_every > 0 && ((k + 1) % o->check_every == 0 || k + 1 == n_outer)) {
         CA_TRY(residual(&ctx->info.res, std::min<long long>((k + 1) * (long long)s, o->H)));

@@ -34,11 +34,13 @@ struct Profile {
 struct ca_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
-  // the sparse dual's second stream (the next step's off-diagonal Gram, and
-  // for s*b >= 128 its diagonal-block inverses and Rs, run on it while the
-  // current step's solves run) and its events; made on first use
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+  // the sparse dual's side streams (later steps' off-diagonal Grams, diagonal-
+  // block inverses and Rs run on them while the current step's solves run) and
+  // their events; made on first use
+  cudaStream_t side[2] = {nullptr, nullptr};
+  cudaEvent_t evs = nullptr;
+  cudaEvent_t ev_ready[3] = {nullptr, nullptr, nullptr};
+  cudaEvent_t ev_read[3] = {nullptr, nullptr, nullptr};
   size_t scratch_max = 0;
   int num_sms = 0;
   void* arena = nullptr;

@@ -536,9 +536,13 @@ __global__ void __launch_bounds__(256, 1)
 k_chain(const float2* __restrict__ Rs, const double* __restrict__ pvec,
         const float2* __restrict__ Ginv, SolveArgs a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
-  pdl_wait();  // (as a programmatic dependent: p from the launch before it)
+  pdl_trigger();  // (the scatter's CTAs load their rows while the chain runs)
+  if constexpr (BMAX > 16) pdl_wait();  // p from the launch before it
   if constexpr (BMAX <= 16)
-    chain_la_body<BMAX, DEPTH>(Rs, pvec, Ginv, a, err, smem_d, [] { return true; });
+    chain_la_body<BMAX, DEPTH>(Rs, pvec, Ginv, a, err, smem_d, [] {
+      pdl_wait();  // p (and what precedes it) from the launches before
+      return true;
+    });
   else
     chain_body<BMAX, DEPTH>(Rs, pvec, Ginv, a, err, smem_d);
 }
@@ -584,13 +588,6 @@ template __global__ void k_reduce_chain<float, 8, 4>(const float*, const double*
 template __global__ void k_reduce_chain<float, 16, 3>(const float*, const double*, int, int,
                                                       double*, float2*, double*, float2*, int,
                                                       SolveArgs, unsigned*, unsigned*);
-template __global__ void k_reduce_chain<double, 8, 4>(const double*, const double*, int, int,
-                                                      double*, float2*, double*, float2*, int,
-                                                      SolveArgs, unsigned*, unsigned*);
-template __global__ void k_reduce_chain<double, 16, 3>(const double*, const double*, int, int,
-                                                       double*, float2*, double*, float2*, int,
-                                                       SolveArgs, unsigned*, unsigned*);
-
 // Shared launches over several problems (the batched solves): one grid
 // reduces every problem's split-K partials (role table: problem and CTA index
 // within it), one grid runs one chain CTA per problem.  No CTA waits on
@@ -904,34 +901,40 @@ k_csr_proj(const long long* __restrict__ rowptr, const int* __restrict__ col,
            long long ncols, const double* __restrict__ w, double* __restrict__ pvec,
            unsigned* __restrict__ err) {
   __shared__ double red[8];
-  pdl_wait();  // w (the previous step's update)
-  pdl_trigger();
   const int r = blockIdx.x, tid = threadIdx.x;
   const int ir = idx[r];
   double sp = 0.0;
-  if (ir >= 0 && ir < nrows) {
-    const long long e1 = rowptr[ir + 1];
-    for (long long eb = rowptr[ir] + tid; eb < e1; eb += 4 * 256) {
-      int fs[4];
-      float vs[4];
+  const bool ok = ir >= 0 && ir < nrows;
+  const long long e0 = ok ? rowptr[ir] : 0, e1 = ok ? rowptr[ir + 1] : 0;
+  int fs[4];
+  float vs[4];
+  auto load = [&](long long eb) {  // (entries past the row: the last one again)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const long long e = eb + 256 * u;
-        fs[u] = e < e1 ? col[e] : -1;
-        vs[u] = e < e1 ? val[e] : 0.f;
-      }
-      double ws[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const bool in = fs[u] >= 0 && fs[u] < ncols;
-        if (!in && eb + 256 * u < e1) ca_flag(err, CA_DEV_ERR_ARG);
-        ws[u] = in ? w[fs[u]] : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) sp = fma((double)vs[u], ws[u], sp);
+    for (int u = 0; u < 4; ++u) {
+      const long long e = min(eb + 256 * u, e1 - 1);
+      fs[u] = __ldg(col + e);
+      vs[u] = __ldg(val + e);
     }
-  } else if (tid == 0) {
-    ca_flag(err, CA_DEV_ERR_ARG);
+  };
+  // the row's first entries load before the wait for w (the previous step's update)
+  if (e0 < e1) load(e0 + tid);
+  pdl_wait();
+  pdl_trigger();
+  if (!ok && tid == 0) ca_flag(err, CA_DEV_ERR_ARG);
+  for (long long eb = e0 + tid; eb < e1; eb += 4 * 256) {
+    double ws[4];
+    float vc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const bool in = fs[u] >= 0 && fs[u] < ncols;
+      if (!in) ca_flag(err, CA_DEV_ERR_ARG);
+      ws[u] = __ldcg(w + (in ? fs[u] : 0));
+      vc[u] = in && eb + 256 * u < e1 ? vs[u] : 0.f;
+      if (!(in && eb + 256 * u < e1)) ws[u] = 0.0;
+    }
+    if (eb + 4 * 256 < e1) load(eb + 4 * 256);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) sp = fma((double)vc[u], ws[u], sp);
   }
   for (int o = 16; o > 0; o >>= 1) sp += __shfl_xor_sync(0xffffffffu, sp, o);
   if ((tid & 31) == 0) red[tid >> 5] = sp;
@@ -993,7 +996,7 @@ k_csr_prep(const double* __restrict__ rn, const int* __restrict__ idx, long long
     if (tid < b * b) {
       const int i = tid / b, c = tid - (tid / b) * b;
       const double v = i == c ? dsum[i]
-                              : G[(long long)(jb + (i < c ? i : c)) * ldr + jb + (i < c ? c : i)];
+                              : __ldcg(G + (long long)(jb + (i < c ? i : c)) * ldr + jb + (i < c ? c : i));
       float2 m = df_mul(cG2, split_f64(v));
       if (i == c) m = df_add(m, cI2);
       Mb[tid] = m;
@@ -1015,7 +1018,7 @@ k_csr_prep(const double* __restrict__ rn, const int* __restrict__ idx, long long
   const long long stride = (long long)(gridDim.x - sa.s_cur) * 256;
   for (long long e = (long long)(blockIdx.x - sa.s_cur) * 256 + tid; e < ne; e += stride) {
     const int c = (int)(e / sb), i = (int)(e - (long long)c * sb);
-    if (i > c) Rs[(long long)c * ldr + i] = df_mul(cG2, split_f64(G[(long long)c * ldr + i]));
+    if (i > c) Rs[(long long)c * ldr + i] = df_mul(cG2, split_f64(__ldcg(G + (long long)c * ldr + i)));
   }
 }
 
@@ -1060,154 +1063,6 @@ k_csr_gram_pairs(const long long* __restrict__ rowptr, const int* __restrict__ c
   }
 }
 
-// The sparse Gram of one outer step (steps a2+a3, Alg. 4 "compute the Gram
-// matrix" on the CSR of X^T): G[p][q] = x_{I_p}^T x_{I_q} for q < p.  The
-// lower triangle is cut into tiles of kCsrPB
-// rows p by kCsrQC rows q, one CTA each: the CTA puts its rows p into
-// shared-memory hash tables (feature -> value), then its warps stream the
-// rows q of the tile once, four entries per lane in flight, each entry
-// probing every table.  The work is the streamed row lengths times the
-// tables, with no atomics and each Gram entry written by one warp.  Products
-// of two FP32 values are exact as (p, e) by a fused multiply-add and are
-// summed in double-float (~2^-44 of sum |terms|); a row p longer than its
-// table is searched in its sorted global columns instead.  The diagonal and
-// the projections come from k_csr_rows.  The Gram goes out as the one split-K
-// "partial" of the dense path's reduction (transposed: entry (i, j), i >= j,
-// at G[j * ldr + i]).
-constexpr int kCsrPB = 4;                      // rows p of a tile (rows q: qc, a launch argument)
-constexpr int kCsrHashBits = 11;               // a table of 2048 entries per row p
-constexpr int kCsrHash = 1 << kCsrHashBits;
-constexpr int kCsrHashMaxRow = kCsrHash / 2;   // load factor <= 1/2
-constexpr int kCsrSmem = kCsrPB * kCsrHash * 8;  // dynamic shared memory of k_csr_gram
-
-__device__ __forceinline__ unsigned csr_hash(int f) {
-  return ((unsigned)f * 2654435761u) >> (32 - kCsrHashBits);
-}
-
-// tiles of the lower triangle: row block pb has ceil(min(sb, (pb+1) PB) / qc)
-__host__ __device__ __forceinline__ int csr_tiles_of(int pb, int sb, int qc) {
-  const int pmax = min(sb, (pb + 1) * kCsrPB);
-  return (pmax + qc - 1) / qc;
-}
-
-__global__ void __launch_bounds__(256)
-k_csr_gram(const long long* __restrict__ rowptr, const int* __restrict__ col,
-           const float* __restrict__ val, const int* __restrict__ idx, long long nrows,
-           long long ncols, int sb, int ldr, int qcs, const double* __restrict__ w,
-           double* __restrict__ G, double* __restrict__ pvec, unsigned* __restrict__ err) {
-  // dynamic shared memory: kCsrPB tables of kCsrHash keys and values
-  extern __shared__ int csr_smem[];
-  int (*hkey)[kCsrHash] = reinterpret_cast<int (*)[kCsrHash]>(csr_smem);
-  float (*hval)[kCsrHash] = reinterpret_cast<float (*)[kCsrHash]>(csr_smem + kCsrPB * kCsrHash);
-  pdl_wait();  // w (the previous step's update) and the previous use of G
-  pdl_trigger();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // this CTA's tile: row block pb, q chunk qc
-  int pb = 0, rem = blockIdx.x;
-  while (rem >= csr_tiles_of(pb, sb, qcs)) rem -= csr_tiles_of(pb, sb, qcs), ++pb;
-  const int qc = rem;
-  const int pl = pb * kCsrPB, ph = min(sb, pl + kCsrPB);  // rows p: [pl, ph)
-  const int ql = qc * qcs, qh = min(ph, ql + qcs);         // rows q: [ql, qh), q <= p
-  long long p0[kCsrPB], p1[kCsrPB];
-  bool hashed[kCsrPB];
-#pragma unroll
-  for (int j = 0; j < kCsrPB; ++j) {
-    const int p = pl + j;
-    const int ip = p < ph ? idx[p] : -1;
-    const bool okp = ip >= 0 && ip < nrows;
-    if (p < ph && !okp && tid == 0) ca_flag(err, CA_DEV_ERR_ARG);
-    p0[j] = okp ? rowptr[ip] : 0;
-    p1[j] = okp ? rowptr[ip + 1] : 0;
-    hashed[j] = p1[j] - p0[j] <= kCsrHashMaxRow;
-  }
-  for (int k = tid; k < kCsrPB * kCsrHash; k += 256) (&hkey[0][0])[k] = -1;
-  __syncthreads();
-  // the tables: every row p's entries, four loads in flight per thread
-#pragma unroll
-  for (int j = 0; j < kCsrPB; ++j) {
-    if (!hashed[j]) continue;
-    for (long long eb = p0[j] + tid; eb < p1[j]; eb += 1024) {
-      int fs[4];
-      float vs[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const long long e = eb + 256 * u;
-        fs[u] = e < p1[j] ? col[e] : -1;
-        vs[u] = e < p1[j] ? val[e] : 0.f;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (fs[u] < 0) continue;
-        unsigned h = csr_hash(fs[u]);
-        while (atomicCAS(&hkey[j][h], -1, fs[u]) != -1) h = (h + 1) & (kCsrHash - 1);
-        hval[j][h] = vs[u];
-      }
-    }
-  }
-  __syncthreads();
-  // value of feature f in row p = pl + j (0 when absent)
-  auto lookup = [&](int j, int f) -> float {
-    if (hashed[j]) {
-      unsigned h = csr_hash(f);
-      for (;;) {
-        const int k = hkey[j][h];
-        if (k == f) return hval[j][h];
-        if (k == -1) return 0.f;
-        h = (h + 1) & (kCsrHash - 1);
-      }
-    }
-    long long lo = p0[j], hi = p1[j];  // a long row: its sorted global columns
-    while (lo < hi) {
-      const long long mid = (lo + hi) >> 1;
-      if (col[mid] < f) lo = mid + 1; else hi = mid;
-    }
-    return (lo < p1[j] && col[lo] == f) ? val[lo] : 0.f;
-  };
-  for (int q = ql + warp; q < qh; q += 8) {
-    const int iq = idx[q];
-    float hi[kCsrPB], lo[kCsrPB];
-#pragma unroll
-    for (int j = 0; j < kCsrPB; ++j) hi[j] = lo[j] = 0.f;
-    if (iq >= 0 && iq < nrows) {
-      const long long e0 = rowptr[iq], e1 = rowptr[iq + 1];
-      for (long long eb = e0 + lane; eb < e1; eb += 128) {
-        int fs[4];
-        float vs[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {  // four entries in flight per lane
-          const long long e = eb + 32 * u;
-          fs[u] = e < e1 ? col[e] : -1;
-          vs[u] = e < e1 ? val[e] : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (fs[u] < 0) continue;
-#pragma unroll
-          for (int j = 0; j < kCsrPB; ++j) {
-            if (pl + j <= q || pl + j >= ph) continue;  // pairs q < p (k_csr_rows: q = p)
-            const float vp = lookup(j, fs[u]);
-            if (vp != 0.f) {
-              const float pr = vp * vs[u];
-              const float pe = fmaf(vp, vs[u], -pr);  // vp vq = pr + pe exactly
-              float s2, t2;
-              two_sum(hi[j], pr, s2, t2);
-              hi[j] = s2;
-              lo[j] += t2 + pe;
-            }
-          }
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < kCsrPB; ++j) {
-      if (pl + j <= q || pl + j >= ph) continue;
-      float2 acc = df_norm(hi[j], lo[j]);
-      for (int o = 16; o > 0; o >>= 1) acc = df_add(acc, df_shfl_xor(acc, o));
-      if (lane == 0) G[(long long)q * ldr + pl + j] = (double)acc.x + (double)acc.y;
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // Sparse Gram by a dense-sparse split of the features (steps a2+a3 of Alg. 4
 // on the CSR of X^T).  A feature present in a large share of the samples
@@ -1222,7 +1077,7 @@ k_csr_gram(const long long* __restrict__ rowptr, const int* __restrict__ col,
 // in its sorted columns), buckets them by feature in shared memory and adds
 // the exact product of every pair of entries of a feature to G with FP64
 // atomics.  Together with k_csr_rows (diagonal, projections) this is the
-// same G as the pair kernels form, up to the order of FP64 additions.
+// same G as the pair kernel forms, up to the order of FP64 additions.
 // ---------------------------------------------------------------------------
 // cnt[f] += 1 for every stored entry of column f (cnt zero on entry)
 __global__ void __launch_bounds__(256)
@@ -1507,30 +1362,38 @@ k_scatter_csr_rows(const long long* __restrict__ rowptr, const int* __restrict__
                    const float* __restrict__ val, const int* __restrict__ idx,
                    long long nrows_total, long long ncols, const double* __restrict__ coef,
                    double c, double* __restrict__ v, unsigned* __restrict__ err) {
-  pdl_wait();  // coef (the solve's Delta)
-  pdl_trigger();
   const int r = blockIdx.x, tid = threadIdx.x;
   const long long row = idx[r];
-  if (row < 0 || row >= nrows_total) {
+  const bool ok = row >= 0 && row < nrows_total;
+  const long long e0 = ok ? rowptr[row] : 0, e1 = ok ? rowptr[row + 1] : 0;
+  int fs[4];
+  float vs[4];
+  auto load = [&](long long eb) {  // (entries past the row: the last one again)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const long long e = min(eb + 256 * u, e1 - 1);
+      fs[u] = __ldg(col + e);
+      vs[u] = __ldg(val + e);
+    }
+  };
+  // the row's first entries load before the wait for coef (the solve's Delta)
+  if (e0 < e1) load(e0 + tid);
+  pdl_wait();
+  pdl_trigger();
+  if (!ok) {
     if (tid == 0) ca_flag(err, CA_DEV_ERR_ARG);
     return;
   }
-  const double cr = c * coef[r];
-  const long long e1 = rowptr[row + 1];
-  for (long long eb = rowptr[row] + tid; eb < e1; eb += 4 * 256) {
-    int fs[4];
-    float vs[4];
+  const double cr = c * __ldcg(coef + r);
+  for (long long eb = e0 + tid; eb < e1; eb += 4 * 256) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const long long e = eb + 256 * u;
-      fs[u] = e < e1 ? col[e] : -1;
-      vs[u] = e < e1 ? val[e] : 0.f;
+      if (eb + 256 * u < e1) {
+        if (fs[u] >= 0 && fs[u] < ncols) atomicAdd(v + fs[u], (double)vs[u] * cr);
+        else ca_flag(err, CA_DEV_ERR_ARG);
+      }
     }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (fs[u] >= 0 && fs[u] < ncols) atomicAdd(v + fs[u], (double)vs[u] * cr);
-      else if (eb + 256 * u < e1) ca_flag(err, CA_DEV_ERR_ARG);
-    }
+    if (eb + 4 * 256 < e1) load(eb + 4 * 256);
   }
 }
 
@@ -2005,30 +1868,6 @@ void launch_csr_prep(cudaStream_t st, int num_sms, const double* rn, long long n
                       Rs, Ginv, err);
 }
 
-void launch_csr_gram(cudaStream_t st, int num_sms, const ca_csr_dev& csr, const int* idx,
-                     long long nrows, long long ncols, int sb, int ldr, const double* w, double* G,
-                     double* pvec, unsigned* err) {
-  // q rows per tile: 32, halved while the tiles are fewer than two per SM
-  auto count = [&](int qc) {
-    int t = 0;
-    for (int pb = 0; pb * kCsrPB < sb; ++pb) t += csr_tiles_of(pb, sb, qc);
-    return t;
-  };
-  int qc = 32;
-  while (qc > 1 && count(qc) < 2 * num_sms) qc >>= 1;
-  launch_programmatic(k_csr_rows, (unsigned)((sb + 7) / 8), 0, st, csr.rowptr, csr.col, csr.val,
-                      idx, nrows, ncols, sb, ldr, w, G, pvec, err);
-  if (sb <= 1) return;
-  if (sb <= 128) {  // few pairs: one warp per pair
-    const long long npairs = (long long)sb * (sb - 1) / 2;
-    launch_programmatic(k_csr_gram_pairs, (unsigned)std::max(1LL, (npairs + 7) / 8), 0, st,
-                        csr.rowptr, csr.col, csr.val, idx, nrows, sb, ldr, G);
-    return;
-  }
-  launch_programmatic(k_csr_gram, (unsigned)count(qc), kCsrSmem, st, csr.rowptr, csr.col,
-                      csr.val, idx, nrows, ncols, sb, ldr, qc, w, G, pvec, err);
-}
-
 void launch_csr_prepare(cudaStream_t st, int num_sms, const ca_csr_dev& csr, long long nrows,
                         long long ncols, long long nnz, int* cnt, const int* dmap, int fd,
                         float* Xd, bool fill) {
@@ -2078,24 +1917,8 @@ void launch_csr_offdiag(cudaStream_t st, const ca_csr_dev& csr, const int* idx, 
                       idx, nrows, ncols, sb, dmap, ldr, G, roff, nr);
 }
 
-int launch_reduce_chain_f64(int grid, size_t smem, cudaStream_t st, const double* part,
-                            const double* ppart, int sbp, double* R, float2* Rs, double* pvec,
-                            float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err,
-                            unsigned* ticket) {
-  cudaError_t e;
-  if (sa.b <= 8)
-    e = launch_programmatic(k_reduce_chain<double, 8, 4>, (unsigned)grid, smem, st, part, ppart, 1,
-                            sbp, R, Rs, pvec, Ginv, ndiag, sa, err, ticket);
-  else if (sa.b <= 16)
-    e = launch_programmatic(k_reduce_chain<double, 16, 3>, (unsigned)grid, smem, st, part, ppart, 1,
-                            sbp, R, Rs, pvec, Ginv, ndiag, sa, err, ticket);
-  else
-    e = cudaErrorInvalidValue;
-  return (int)e;
-}
-
 int set_solve_smem_limit(int bytes) {
-  cudaError_t e[15] = {set_dyn_smem(k_solve, bytes), set_dyn_smem(k_csr_gram, kCsrSmem),
+  cudaError_t e[12] = {set_dyn_smem(k_solve, bytes),
                       set_dyn_smem(k_sgram, kSgSmem),
                       set_dyn_smem(k_dgram, 2 * kDgT * (kCsrDenseMax + 4) * 4),
                       set_dyn_smem(k_chain<8, 4>, bytes),
@@ -2106,9 +1929,7 @@ int set_solve_smem_limit(int bytes) {
                       set_dyn_smem(k_reduce_chain<float, 16, 3>, bytes),
                       set_dyn_smem(k_reduce<double>, bytes),
                       set_dyn_smem(k_chain_batch<8, 4>, bytes),
-                      set_dyn_smem(k_chain_batch<16, 3>, bytes),
-                      set_dyn_smem(k_reduce_chain<double, 8, 4>, bytes),
-                      set_dyn_smem(k_reduce_chain<double, 16, 3>, bytes)};
+                      set_dyn_smem(k_chain_batch<16, 3>, bytes)};
   for (cudaError_t x : e)
     if (x != cudaSuccess) return (int)x;
   return 0;

@@ -248,13 +248,6 @@ void launch_csr_prep(cudaStream_t st, int num_sms, const double* rn, long long n
                      unsigned* err);
 void launch_csr_proj(cudaStream_t st, const ca_csr_dev& csr, const int* idx, long long nrows,
                      long long ncols, int sb, const double* w, double* pvec, unsigned* err);
-void launch_csr_gram(cudaStream_t st, int num_sms, const ca_csr_dev& csr, const int* idx,
-                     long long nrows, long long ncols, int sb, int ldr, const double* w, double* G,
-                     double* pvec, unsigned* err);
-int launch_reduce_chain_f64(int grid, size_t smem, cudaStream_t st, const double* part,
-                            const double* ppart, int sbp, double* R, float2* Rs, double* pvec,
-                            float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err,
-                            unsigned* ticket);
 void launch_scatter_csr(cudaStream_t st, const ca_csr_dev& csr, const int* idx, long long nrows,
                         long long ncols, long long nlist, const double* coef, double c, double* v,
                         unsigned* err);
