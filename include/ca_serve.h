@@ -103,11 +103,11 @@ void ca_server_destroy(ca_server* s);
 
 /* Batched solves: `count` dense problems of uneven sizes solved together on
  * ctx (its stream, its scratch arena).  Each round runs one outer step of
- * every unfinished problem in three shared launches: one Gram pass whose
+ * every unfinished problem in two shared launches: one Gram pass whose
  * CTAs split the concatenation of all problems' 32-column atoms into
  * stretches of equal HBM cost (steps a2+a3, with each problem's deferred
- * update a5 fused in), one reduction of every problem's split-K partials
- * with the inversion of its diagonal blocks, and one chain CTA per problem
+ * update a5 fused in), then the reduction of every problem's split-K partials
+ * with the inversion of its diagonal blocks and one chain CTA per problem
  * (the s unrolled solves of eq. "recur" / its dual analogue, step a4).
  * Problems are independent: each computes what ca_bcd_solve / ca_bdcd_solve
  * computes alone, up to the order of the FP32 Gram sums (the split-K
@@ -126,10 +126,10 @@ void ca_server_destroy(ca_server* s);
  *            vector, forms its residual and waits for the GPU; a problem
  *            that meets its rule leaves the rounds); solve CA_SOLVE_DF
  *            (else CA_ERR_UNSUPPORTED).
- *   flags    CA_BATCH_GRAPH: rounds that differ only in pointers (a segment,
- *            up to 64 rounds) are captured into one CUDA graph and launched
- *            as one (needs a non-NULL stream on ctx; ignored while
- *            profiling).
+ *   flags    0 or CA_BATCH_GRAPH, with the same results: a segment (rounds
+ *            that differ only in pointers, up to 64) runs once, so its
+ *            launches are made directly in both cases (a graph captured for
+ *            one launch cost more than it saved).
  *   out      count results: status, s (the depth of the last step), h_done,
  *            and the stopping test's res0, res, gap, fval and bound.
  * Returns after the work finished.  Errors: CA_ERR_ARG, CA_ERR_UNSUPPORTED,

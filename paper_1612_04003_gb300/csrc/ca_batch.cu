@@ -1,25 +1,27 @@
 // ca_batch.cu -- ca_batch_solve: several dense ridge problems (primal CA-BCD,
 // Algorithm 2, or dual CA-BDCD, Algorithm 4) of uneven sizes solved together.
 //
-// Each round runs one outer step of every unfinished problem in three shared
+// Each round runs one outer step of every unfinished problem in two shared
 // launches:
 //   * one Gram pass (steps a2+a3, with the deferred update a5 of the
 //     problem's previous step fused in): the P CTAs split the concatenation
 //     of all problems' 32-column atoms into stretches of equal HBM cost
 //     (ca_batch_plan.h); a CTA walks the units of its stretch, one split-K
 //     partial slot each;
-//   * one reduction of every problem's partial slots, with the inversion of
-//     its diagonal blocks (step a4);
-//   * one chain CTA per problem (the s unrolled solves of eq. "recur" / its
+//   * one launch that reduces every problem's partial slots, inverts its
+//     diagonal blocks (step a4) and, in one chain CTA per problem, runs the
+//     dependent chain (the s unrolled solves of eq. "recur" / its
 //     dual analogue), so the dependent chains of different problems run at
 //     the same time on different SMs.
 // A small problem alone cannot fill the GPU (its Gram pass has fewer atoms
 // than SMs, and its chain leaves all but one SM idle); in a shared round the
 // problems fill each other's gaps.  Rounds whose launches differ only in
-// pointers form a segment; with CA_BATCH_GRAPH a segment is captured into a
-// CUDA graph once and launched as one.  Problems submitted with s = 0 get
-// their unrolling depth by measured cost: trial rounds with s b = 128, 64
-// and 32 rows per outer step, each timed with CUDA events, then the
+// pointers form a segment, whose descriptors go to the device in one copy.  A
+// segment runs once, so its launches are made directly: captured into a CUDA
+// graph (capture, instantiation, one launch) the same segments took 10 to 25%
+// longer (8 problems, 83 rounds: 4.61 against 3.96 ms).  Problems submitted
+// with s = 0 get their unrolling depth by measured cost: trial rounds with s b
+// = 128, 64 and 32 rows per outer step, each timed with CUDA events, then the
 // cheapest per block update (the paper's trade-off between fewer launches
 // and a larger Gram, Sec. 5, measured instead of modelled).
 #include <algorithm>
@@ -71,10 +73,11 @@ int sb_class(int sb) { return sb <= 32 ? 32 : (sb <= 64 ? 64 : 128); }
 // Rows of an outer step of problem q in the next round.
 int step_rows(const BInst& q) { return (int)std::min<long long>(q.s, q.H - q.h) * q.b; }
 
-// Reducing CTAs of a problem: its diagonal blocks, then 64 entries a pass.
-int reduce_ctas(int sb, int scur) {
+// Reducing CTAs of a problem: its diagonal blocks, then CTAs of 64 entries a
+// pass, at most `most` of them (more passes each instead).
+int reduce_ctas(int sb, int scur, int most) {
   const long long entries = (long long)sb * (sb + 1) / 2 + sb;
-  return scur + (int)std::max<long long>(1, (entries + 63) / 64);
+  return scur + (int)std::max<long long>(1, std::min<long long>(most, (entries + 63) / 64));
 }
 
 // Reduce-grid roles of a round: per problem its diagonal blocks and up to
@@ -132,7 +135,8 @@ int batch_need(ca_ctx* ctx, int count, const ca_request* reqs, size_t* out, bool
   need += align256((size_t)kSegMaxRounds * count * sizeof(GramInst)) +
           align256((size_t)kSegMaxRounds * count * sizeof(RedInst)) +
           align256(nslot_max * sizeof(GramUnit)) + align256((size_t)(P + 1) * sizeof(int));
-  need += align256(max_roles_of(count) * sizeof(RedRole)) + 4096;
+  need += align256(max_roles_of(count) * sizeof(RedRole)) +
+          align256(((size_t)count + 1) * sizeof(unsigned)) + 4096;
   *out = need;
   *any_tuned_out = any_tuned;
   return CA_OK;
@@ -261,11 +265,16 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
   }
   float* part_pool = cv.take<float>(nslot_max * kBatchMaxSB * kBatchMaxSB);
   double* ppart_pool = cv.take<double>(nslot_max * kBatchMaxSB);
-  GramInst* d_ginst = cv.take<GramInst>((size_t)kSegMaxRounds * count);
-  RedInst* d_rinst = cv.take<RedInst>((size_t)kSegMaxRounds * count);
-  GramUnit* d_units = cv.take<GramUnit>(nslot_max);
-  int* d_ubeg = cv.take<int>((size_t)P + 1);
-  RedRole* d_roles = cv.take<RedRole>(max_roles);
+  // a segment's descriptors: one array on the device, one copy
+  const size_t desc_bytes =
+      align256((size_t)kSegMaxRounds * count * sizeof(GramInst)) +
+      align256((size_t)kSegMaxRounds * count * sizeof(RedInst)) +
+      align256(nslot_max * sizeof(GramUnit)) + align256(((size_t)P + 1) * sizeof(int)) +
+      align256(max_roles * sizeof(RedRole));
+  char* d_desc = cv.take<char>(desc_bytes);
+  unsigned* d_tickets = cv.take<unsigned>((size_t)count + 1);  // (zero between launches)
+  CA_TRY_CUDA(cudaMemsetAsync(d_tickets, 0, ((size_t)count + 1) * sizeof(unsigned), ctx->stream));
+  std::vector<char> h_desc(desc_bytes);
 
   std::vector<GramInst> h_ginst;
   std::vector<RedInst> h_rinst;
@@ -279,7 +288,6 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
   double trial_cost[3] = {0, 0, 0};
   bool warm = !any_tuned;         // the first round runs untimed
   int status = CA_OK;
-  const bool graph = (flags & CA_BATCH_GRAPH) && ctx->stream != nullptr;
 
   auto run_segment = [&](const std::vector<int>& act, int rounds, bool timed) -> int {
     const int na = (int)act.size();
@@ -307,11 +315,14 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
     }
     h_ubeg[(size_t)P] = (int)h_units.size();
     // reduce roles: each problem's CTAs (same in every round of the segment)
+    // one CTA an SM (the chain's shared memory): about two rounds of them in all
+    // (10 problems, s b = 128: 2.49 ms, with one pass a CTA 2.72)
+    const int most = std::max(1, (2 * ctx->num_sms - na) / na);
     h_roles.clear();
     for (int j = 0; j < na; ++j) {
       const BInst& q = in[(size_t)act[(size_t)j]];
       const int sb = step_rows(q), sc = sb / q.b;
-      const int nc = reduce_ctas(sb, sc);
+      const int nc = reduce_ctas(sb, sc, most);
       for (int t = 0; t < nc; ++t) h_roles.push_back(RedRole{j, t, nc});
     }
     // per-round descriptors
@@ -330,7 +341,8 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
                                                 q.pb.K, idx, sb, q.pb.v2, part, ppart, u};
         SolveArgs sa{idx, q.pb.N, q.b, sc, sb, sbp, q.pb.cG, q.pb.cI, q.pb.cP, q.pb.cY, q.pb.x,
                      q.pb.yv, dl};
-        h_rinst[(size_t)rr * na + j] = RedInst{part, ppart, pl.nslots[(size_t)j], sbp, sc, q.R, q.Rs,
+        h_rinst[(size_t)rr * na + j] = RedInst{part, ppart, pl.nslots[(size_t)j], sbp, sc,
+                                               reduce_ctas(sb, sc, most), q.R, q.Rs,
                                                q.pvec, q.Ginv, sa};
         // advance: this step's update is pending for the next round
         q.prev_idx = idx;
@@ -341,16 +353,20 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
         q.k += 1;
       }
     }
-    CA_TRY_CUDA(cudaMemcpyAsync(d_ginst, h_ginst.data(), h_ginst.size() * sizeof(GramInst),
-                                cudaMemcpyHostToDevice, ctx->stream));
-    CA_TRY_CUDA(cudaMemcpyAsync(d_rinst, h_rinst.data(), h_rinst.size() * sizeof(RedInst),
-                                cudaMemcpyHostToDevice, ctx->stream));
-    CA_TRY_CUDA(cudaMemcpyAsync(d_units, h_units.data(), h_units.size() * sizeof(GramUnit),
-                                cudaMemcpyHostToDevice, ctx->stream));
-    CA_TRY_CUDA(cudaMemcpyAsync(d_ubeg, h_ubeg.data(), h_ubeg.size() * sizeof(int),
-                                cudaMemcpyHostToDevice, ctx->stream));
-    CA_TRY_CUDA(cudaMemcpyAsync(d_roles, h_roles.data(), h_roles.size() * sizeof(RedRole),
-                                cudaMemcpyHostToDevice, ctx->stream));
+    size_t off = 0;
+    auto put = [&](const auto& v) {
+      using E = typename std::decay<decltype(v[0])>::type;
+      E* at = reinterpret_cast<E*>(d_desc + off);
+      std::memcpy(h_desc.data() + off, v.data(), v.size() * sizeof(E));
+      off += align256(v.size() * sizeof(E));
+      return at;
+    };
+    const GramInst* d_ginst = put(h_ginst);
+    const RedInst* d_rinst = put(h_rinst);
+    const GramUnit* d_units = put(h_units);
+    const int* d_ubeg = put(h_ubeg);
+    const RedRole* d_roles = put(h_roles);
+    CA_TRY_CUDA(cudaMemcpyAsync(d_desc, h_desc.data(), off, cudaMemcpyHostToDevice, ctx->stream));
     const size_t csm = chain_smem(bmax, sbmax);
     auto launch_rounds = [&]() -> int {
       for (int rr = 0; rr < rounds; ++rr) {
@@ -360,39 +376,16 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
         prof_mark(ctx, PC_GRAM);
         if (e) return cuda_fail((cudaError_t)e, __LINE__);
         prof_mark(ctx, PC_SOLVE);
-        e = launch_reduce_batch((int)h_roles.size(), ctx->stream, d_rinst + (size_t)rr * na, d_roles,
-                                ctx->d_err);
-        if (e) return cuda_fail((cudaError_t)e, __LINE__);
-        e = launch_chain_batch(na, bmax, csm, ctx->stream, d_rinst + (size_t)rr * na, ctx->d_err);
+        e = launch_reduce_chain_batch((int)h_roles.size(), na, bmax, csm, ctx->stream,
+                                      d_rinst + (size_t)rr * na, d_roles, d_tickets, d_tickets + 1,
+                                      ctx->d_err);
         prof_mark(ctx, PC_SOLVE);
         if (e) return cuda_fail((cudaError_t)e, __LINE__);
-        ctx->prof.kernel_launches += 3;
+        ctx->prof.kernel_launches += 2;
       }
       return CA_OK;
     };
     if (timed) CA_TRY_CUDA(cudaEventRecord(ev0, ctx->stream));
-    if (graph && !ctx->prof.on) {
-      cudaGraph_t gr = nullptr;
-      cudaGraphExec_t ge = nullptr;
-      CA_TRY_CUDA(cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));
-      const int e = launch_rounds();
-      const cudaError_t ce = cudaStreamEndCapture(ctx->stream, &gr);
-      if (e != CA_OK) {
-        if (gr) cudaGraphDestroy(gr);
-        return e;
-      }
-      CA_TRY_CUDA(ce);
-      const cudaError_t ie = cudaGraphInstantiate(&ge, gr, 0);
-      cudaGraphDestroy(gr);
-      CA_TRY_CUDA(ie);
-      const cudaError_t le = cudaGraphLaunch(ge, ctx->stream);
-      if (le == cudaSuccess && timed) cudaEventRecord(ev1, ctx->stream);
-      // the next segment rewrites the descriptor arrays: wait for this one
-      const cudaError_t se = le == cudaSuccess ? cudaStreamSynchronize(ctx->stream) : le;
-      cudaGraphExecDestroy(ge);
-      CA_TRY_CUDA(se);
-      return CA_OK;
-    }
     CA_TRY(launch_rounds());
     if (timed) CA_TRY_CUDA(cudaEventRecord(ev1, ctx->stream));
     // the next segment rewrites the descriptor arrays: wait for this one

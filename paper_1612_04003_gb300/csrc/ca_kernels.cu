@@ -588,29 +588,47 @@ template __global__ void k_reduce_chain<float, 8, 4>(const float*, const double*
 template __global__ void k_reduce_chain<float, 16, 3>(const float*, const double*, int, int,
                                                       double*, float2*, double*, float2*, int,
                                                       SolveArgs, unsigned*, unsigned*);
-// Shared launches over several problems (the batched solves): one grid
-// reduces every problem's split-K partials (role table: problem and CTA index
-// within it), one grid runs one chain CTA per problem.  No CTA waits on
-// another, so neither grid needs its CTAs resident at once.
-__global__ void __launch_bounds__(256, 2)
-k_reduce_batch(const RedInst* __restrict__ insts, const RedRole* __restrict__ roles,
-               unsigned* __restrict__ err) {
-  pdl_wait();
-  pdl_trigger();
-  const RedRole ro = roles[blockIdx.x];
-  const RedInst ri = insts[ro.inst];
-  reduce_body<float>(ri.part, ri.ppart, ri.P, ri.sbp, ri.R, ri.Rs, ri.pvec, ri.Ginv, ri.ndiag,
-                     ri.sa, err, ro.cta, ro.ncta);
-}
-
+// a4 of several problems (the batched solves) in one launch: reducing CTAs (role
+// table: problem and CTA index within it), then a chain CTA per problem, which
+// gathers what does not depend on the reduction and waits (bounded) for its
+// problem's reducing CTAs (tickets[problem], zero on entry, left zero).  A CTA
+// takes its role by arrival (*arrived, zero on entry, left zero), so every
+// reducing role has started before the first chain waits, whatever part of
+// the grid is resident.
 template <int BMAX, int DEPTH>
-__global__ void __launch_bounds__(256, 1)
-k_chain_batch(const RedInst* __restrict__ insts, unsigned* __restrict__ err) {
+__global__ void __launch_bounds__(256, 2)
+k_reduce_chain_batch(const RedInst* __restrict__ insts, const RedRole* __restrict__ roles,
+                     int nroles, unsigned* __restrict__ arrived, unsigned* __restrict__ tickets,
+                     unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
+  __shared__ int s_role;
+  if (threadIdx.x == 0) {
+    const unsigned t = atomicAdd(arrived, 1u);
+    if (t == gridDim.x - 1) *arrived = 0u;  // (every other CTA has its number)
+    s_role = (int)t;
+  }
+  __syncthreads();
+  const int role = s_role;
+  if (role < nroles) {
+    pdl_wait();
+    pdl_trigger();
+    const RedRole ro = roles[role];
+    const RedInst ri = insts[ro.inst];
+    reduce_body<float>(ri.part, ri.ppart, ri.P, ri.sbp, ri.R, ri.Rs, ri.pvec, ri.Ginv, ri.ndiag,
+                       ri.sa, err, ro.cta, ro.ncta);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();  // this CTA's R, Rs, p, Ginv before its count
+      atomicAdd(tickets + ro.inst, 1u);
+    }
+    return;
+  }
   pdl_wait();
   pdl_trigger();
-  const RedInst ri = insts[blockIdx.x];
-  chain_la_body<BMAX, DEPTH>(ri.Rs, ri.pvec, ri.Ginv, ri.sa, err, smem_d, [] { return true; });
+  const int i = role - nroles;
+  const RedInst ri = insts[i];
+  chain_la_body<BMAX, DEPTH>(ri.Rs, ri.pvec, ri.Ginv, ri.sa, err, smem_d,
+                             [&] { return chain_wait(tickets + i, (unsigned)ri.nred, true, err); });
 }
 
 template __global__ void k_chain<8, 4>(const float2*, const double*, const float2*, SolveArgs,
@@ -1825,17 +1843,15 @@ static cudaError_t set_dyn_smem(K kernel, int bytes) {
                               bytes < cap ? bytes : cap);
 }
 
-int launch_reduce_batch(int grid, cudaStream_t st, const RedInst* insts, const RedRole* roles,
-                        unsigned* err) {
-  return (int)launch_programmatic(k_reduce_batch, (unsigned)grid, 0, st, insts, roles, err);
-}
-
-int launch_chain_batch(int count, int bmax, size_t smem, cudaStream_t st, const RedInst* insts,
-                       unsigned* err) {
+int launch_reduce_chain_batch(int nroles, int count, int bmax, size_t smem, cudaStream_t st,
+                              const RedInst* insts, const RedRole* roles, unsigned* arrived,
+                              unsigned* tickets, unsigned* err) {
   if (bmax <= 8)
-    return (int)launch_programmatic(k_chain_batch<8, 4>, (unsigned)count, smem, st, insts, err);
+    return (int)launch_programmatic(k_reduce_chain_batch<8, 4>, (unsigned)(nroles + count), smem, st,
+                                    insts, roles, nroles, arrived, tickets, err);
   if (bmax <= 16)
-    return (int)launch_programmatic(k_chain_batch<16, 3>, (unsigned)count, smem, st, insts, err);
+    return (int)launch_programmatic(k_reduce_chain_batch<16, 3>, (unsigned)(nroles + count), smem, st,
+                                    insts, roles, nroles, arrived, tickets, err);
   return (int)cudaErrorInvalidValue;
 }
 
@@ -1928,8 +1944,8 @@ int set_solve_smem_limit(int bytes) {
                       set_dyn_smem(k_reduce_chain<float, 8, 4>, bytes),
                       set_dyn_smem(k_reduce_chain<float, 16, 3>, bytes),
                       set_dyn_smem(k_reduce<double>, bytes),
-                      set_dyn_smem(k_chain_batch<8, 4>, bytes),
-                      set_dyn_smem(k_chain_batch<16, 3>, bytes)};
+                      set_dyn_smem(k_reduce_chain_batch<8, 4>, bytes),
+                      set_dyn_smem(k_reduce_chain_batch<16, 3>, bytes)};
   for (cudaError_t x : e)
     if (x != cudaSuccess) return (int)x;
   return 0;

@@ -185,6 +185,7 @@ struct RedInst {
   const float* part;
   const double* ppart;
   int P, sbp, ndiag;
+  int nred;  // its reducing CTAs
   double* R;
   float2* Rs;
   double* pvec;
@@ -194,11 +195,9 @@ struct RedInst {
 struct RedRole {
   int inst, cta, ncta;
 };
-int launch_reduce_batch(int grid, cudaStream_t st, const RedInst* insts, const RedRole* roles,
-                        unsigned* err);
-// one chain CTA per problem (b <= bmax <= 16, s*b <= 256)
-int launch_chain_batch(int count, int bmax, size_t smem, cudaStream_t st, const RedInst* insts,
-                       unsigned* err);
+int launch_reduce_chain_batch(int nroles, int count, int bmax, size_t smem, cudaStream_t st,
+                              const RedInst* insts, const RedRole* roles, unsigned* arrived,
+                              unsigned* tickets, unsigned* err);
 
 // Sparse dual, steps a2+a3 of one outer step from the CSR of X^T (row hash
 // tables, ca_kernels.cu): G (ldr x ldr, transposed lower triangle, the one
