@@ -5,6 +5,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <utility>
 #include <vector>
 
 #include "ca_bcd.h"
@@ -949,7 +950,8 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
     // (a multiple of 8: Xd's rows are zero-padded to 16-byte multiples)
     const int fdmax = (int)std::min<long long>(
         CA_CSR_DENSE_MAX, ((64LL << 20) / (4 * std::max(1LL, n))) & ~7LL);
-    if (split) need += 2 * align256((size_t)d * 4) + align256((size_t)n * std::max(fdmax, 8) * 4) + 512;
+    if (split)
+      need += 2 * align256((size_t)d * 4) + align256((size_t)n * std::max(fdmax, 8) * 4) + 512;
     need += align256((size_t)n * 8);  // row norms
     // where each feature range starts in every row (256 MB at most, else searched)
     const size_t roff_bytes = csr_rangeoff_bytes(n, d);
@@ -1007,62 +1009,15 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
                                                                        ctx->d_err);
       ctx->prof.kernel_launches += 2;
     };
-    recompute();
-    k_sample<<<(unsigned)((o->H + 7) / 8), 256, 0, ctx->stream>>>(o->seed, o->h0, o->H, o->b, n, idx);
-    CA_TRY_CUDA(cudaGetLastError());
-    // heavy features (in at least a quarter of the rows; the heaviest fdmax
-    // at most) become the columns of Xd, chosen on the host from the counts
-    int fd = 0;
-    int* dmap = nullptr;
-    float* Xd = nullptr;
-    if (split) {
-      int* cnt = cv.take<int>((size_t)d);
-      dmap = cv.take<int>((size_t)d);
-      CA_TRY_CUDA(cudaMemsetAsync(cnt, 0, (size_t)d * 4, ctx->stream));
-      launch_csr_prepare(ctx->stream, ctx->num_sms, cdev, n, d, nnz, cnt, nullptr, 0, nullptr, false);
-      std::vector<int> hc((size_t)d);
-      CA_TRY_CUDA(cudaMemcpyAsync(hc.data(), cnt, (size_t)d * 4, cudaMemcpyDeviceToHost, ctx->stream));
-      CA_TRY_CUDA(cudaStreamSynchronize(ctx->stream));
-      const long long heavy = (n + 3) / 4;
-      std::vector<int> cand;
-      for (long long f = 0; f < d; ++f)
-        if (hc[(size_t)f] >= heavy) cand.push_back((int)f);
-      if ((int)cand.size() > fdmax) {
-        std::stable_sort(cand.begin(), cand.end(), [&](int x, int y2) { return hc[x] > hc[y2]; });
-        cand.resize((size_t)fdmax);
-        std::sort(cand.begin(), cand.end());
-      }
-      std::vector<int> hm((size_t)d, -1);
-      for (size_t j = 0; j < cand.size(); ++j) hm[(size_t)cand[j]] = (int)j;
-      fd = ((int)cand.size() + 7) & ~7;  // row length of Xd; the padding stays zero
-      CA_TRY_CUDA(cudaMemcpy(dmap, hm.data(), (size_t)d * 4, cudaMemcpyHostToDevice));
-      Xd = cv.take<float>((size_t)n * std::max(fd, 8));
-      if (fd > 0) {
-        CA_TRY_CUDA(cudaMemsetAsync(Xd, 0, (size_t)n * fd * 4, ctx->stream));
-        launch_csr_prepare(ctx->stream, ctx->num_sms, cdev, n, d, nnz, nullptr, dmap, fd, Xd, true);
-      }
-      ctx->prof.kernel_launches += fd > 0 ? 2 : 1;
-    }
-    int* roff = nullptr;
-    if (use_roff) {
-      roff = cv.take<int>(roff_bytes / sizeof(int));
-      launch_csr_rangeoff(ctx->stream, cdev, n, d, roff);
-      ctx->prof.kernel_launches += 1;
-    }
     const int b = o->b, s = o->s;
-    const long long n_outer = (o->H + s - 1) / s;
-    ctx->info = ca_info{o->H, 0, 0.0, 0.0, 0.0, 0.0, -1.0};
-    ctx->trace.clear();
-    if (o->check_every > 0) {
-      CA_TRY(residual(&ctx->info.res0, 0));
-      ctx->info.res = ctx->info.res0;
-    }
-    // The strict lower triangle of each step's Gram (the split, or one warp per
-    // pair) has no input that the solves change: it is formed on side streams,
-    // nbuf - 1 steps ahead, each step on the stream of its turn.  Events: evs the
-    // start and the join, ev_ready[k % nbuf] buffer formed, ev_read[k % nbuf]
-    // buffer read.
-    const int ahead = nbuf - 1;
+    // the fast a4 (b <= 16): the diagonal blocks' inverses and Rs come from the
+    // side streams too, and the library stream runs the projections, the chain
+    // and the scatter
+    const bool f64solve = o->solve == CA_SOLVE_F64;
+    auto fast_step = [&](int sbk) { return fast_solve(b, sbk, f64solve) && b <= 16; };
+    // What a solve forms once, on three streams at a time: the start w_0 and the
+    // sample here, the column counts on one side stream, row norms and range
+    // offsets on the other.
     CA_TRY(make_side(ctx));
     struct SideJoin {  // every exit: the main stream waits for the side streams' work
       ca_ctx* c;
@@ -1077,11 +1032,93 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
       }
       ~SideJoin() { (*this)(); }
     } join{ctx, false};
-    // the fast a4 (b <= 16): the diagonal blocks' inverses and Rs come from the
-    // side streams too, and the library stream runs the projections, the chain
-    // and the scatter
-    const bool f64solve = o->solve == CA_SOLVE_F64;
-    auto fast_step = [&](int sbk) { return fast_solve(b, sbk, f64solve) && b <= 16; };
+    CA_TRY_CUDA(cudaEventRecord(ctx->evs, ctx->stream));
+    for (cudaStream_t sd : ctx->side) CA_TRY_CUDA(cudaStreamWaitEvent(sd, ctx->evs, 0));
+    join.on = true;
+    int* cnt = nullptr;
+    int* dmap = nullptr;
+    float* Xd = nullptr;
+    int ncand = 0;  // candidates dmap's memory holds ([0] their number, then from [2] on pairs)
+    if (split) {
+      cnt = cv.take<int>((size_t)d);
+      dmap = cv.take<int>((size_t)d);
+      Xd = cv.take<float>((size_t)n * std::max(fdmax, 8));
+      ncand = (int)std::max(0LL, std::min<long long>(kCsrCand, (d - 2) / 2));
+      // (Xd, filled later, holds the copies of the counters)
+      const int copies = (size_t)n * std::max(fdmax, 8) >= (size_t)8 * d ? 8 : 1;
+      CA_TRY_CUDA(cudaMemsetAsync(copies > 1 ? (void*)Xd : (void*)cnt, 0, (size_t)copies * d * 4,
+                                  ctx->side[0]));
+      CA_TRY_CUDA(cudaMemsetAsync(dmap, 0, sizeof(int), ctx->side[0]));
+      launch_csr_count(ctx->side[0], ctx->num_sms, cdev, d, nnz,
+                       copies > 1 ? reinterpret_cast<int*>(Xd) : cnt, copies, cnt,
+                       (int)std::min<long long>((n + 3) / 4, 2147483647LL), dmap, ncand);
+      ctx->prof.kernel_launches += 2;
+    }
+    if (fast_step(b)) {
+      launch_csr_rownorm(ctx->side[1], cdev, n, rn);
+      ctx->prof.kernel_launches += 1;
+    }
+    int* roff = nullptr;
+    if (use_roff) {
+      roff = cv.take<int>(roff_bytes / sizeof(int));
+      launch_csr_rangeoff(ctx->side[1], cdev, n, d, roff);
+      ctx->prof.kernel_launches += 1;
+    }
+    recompute();
+    k_sample<<<(unsigned)((o->H + 7) / 8), 256, 0, ctx->stream>>>(o->seed, o->h0, o->H, o->b, n, idx);
+    CA_TRY_CUDA(cudaGetLastError());
+    // heavy features (in at least a quarter of the rows; the heaviest fdmax
+    // at most) become the columns of Xd, chosen on the host from the candidates
+    int fd = 0;
+    if (split) {
+      // (a first part of the list that holds the usual number, the rest if need be)
+      std::vector<int> hc((size_t)std::min<long long>(d, 2 + 2 * ncand));
+      const size_t first = std::min<size_t>(hc.size(), 2 + 2 * CA_CSR_DENSE_MAX);
+      CA_TRY_CUDA(cudaMemcpyAsync(hc.data(), dmap, first * 4, cudaMemcpyDeviceToHost, ctx->side[0]));
+      CA_TRY_CUDA(cudaStreamSynchronize(ctx->side[0]));
+      if (hc[0] > CA_CSR_DENSE_MAX && hc[0] <= ncand)
+        CA_TRY_CUDA(cudaMemcpy(hc.data(), dmap, hc.size() * 4, cudaMemcpyDeviceToHost));
+      std::vector<std::pair<int, int>> cand;  // (feature, count), by feature
+      if (hc[0] <= ncand) {
+        for (int j = 0; j < hc[0]; ++j) cand.emplace_back(hc[2 + 2 * j], hc[3 + 2 * j]);
+        std::sort(cand.begin(), cand.end());
+      } else {  // more than the list holds: from all counts
+        hc.resize((size_t)d);
+        CA_TRY_CUDA(cudaMemcpy(hc.data(), cnt, (size_t)d * 4, cudaMemcpyDeviceToHost));
+        for (long long f = 0; f < d; ++f)
+          if (hc[(size_t)f] >= (n + 3) / 4) cand.emplace_back((int)f, hc[(size_t)f]);
+      }
+      if ((int)cand.size() > fdmax) {
+        std::stable_sort(cand.begin(), cand.end(),
+                         [](const auto& x, const auto& y2) { return x.second > y2.second; });
+        cand.resize((size_t)fdmax);
+        std::sort(cand.begin(), cand.end());
+      }
+      fd = ((int)cand.size() + 7) & ~7;  // row length of Xd; the padding stays zero
+      CA_TRY_CUDA(cudaMemsetAsync(dmap, 0xff, (size_t)d * 4, ctx->stream));
+      if (fd > 0) {
+        std::vector<int> feats;
+        for (const auto& c : cand) feats.push_back(c.first);
+        CA_TRY_CUDA(cudaMemcpyAsync(cnt, feats.data(), feats.size() * 4, cudaMemcpyHostToDevice,
+                                    ctx->stream));
+        CA_TRY_CUDA(cudaMemsetAsync(Xd, 0, (size_t)n * fd * 4, ctx->stream));
+        launch_csr_dense(ctx->stream, cdev, n, d, cnt, (int)feats.size(), dmap, fd, Xd);
+        ctx->prof.kernel_launches += 2;
+      }
+    }
+    const long long n_outer = (o->H + s - 1) / s;
+    ctx->info = ca_info{o->H, 0, 0.0, 0.0, 0.0, 0.0, -1.0};
+    ctx->trace.clear();
+    if (o->check_every > 0) {
+      CA_TRY(residual(&ctx->info.res0, 0));
+      ctx->info.res = ctx->info.res0;
+    }
+    // The strict lower triangle of each step's Gram (the split, or one warp per
+    // pair) has no input that the solves change: it is formed on side streams,
+    // nbuf - 1 steps ahead, each step on the stream of its turn.  Events: evs the
+    // start and the join, ev_ready[k % nbuf] buffer formed, ev_read[k % nbuf]
+    // buffer read.
+    const int ahead = nbuf - 1;
     auto step_args = [&](long long kk) {
       const int skk = (int)std::min<long long>(s, o->H - (long long)s * kk);
       return SolveArgs{idx + (size_t)s * kk * b, n, b, skk, skk * b, (int)sbp, 1.0 / ln, 1.0, 1.0,
@@ -1103,13 +1140,12 @@ int ca_bdcd_solve(ca_ctx* ctx, int xfmt, const void* XT, long long d, long long 
       CA_TRY_CUDA(cudaEventRecord(ctx->ev_ready[q], sd));
       return CA_OK;
     };
-    if (fast_step(b)) {  // before the side streams start
-      launch_csr_rownorm(ctx->stream, cdev, n, rn);
-      ctx->prof.kernel_launches += 1;
+    // each side stream: what the other streams formed
+    for (cudaStream_t from : {ctx->stream, ctx->side[1]}) {
+      CA_TRY_CUDA(cudaEventRecord(ctx->evs, from));
+      for (cudaStream_t to : ctx->side)
+        if (to != from) CA_TRY_CUDA(cudaStreamWaitEvent(to, ctx->evs, 0));
     }
-    CA_TRY_CUDA(cudaEventRecord(ctx->evs, ctx->stream));
-    for (cudaStream_t sd : ctx->side) CA_TRY_CUDA(cudaStreamWaitEvent(sd, ctx->evs, 0));
-    join.on = true;
     for (long long kk = 0; kk < std::min<long long>(ahead, n_outer); ++kk) CA_TRY(form_gram(kk));
     for (long long k = 0; k < n_outer; ++k) {
       const int sk = (int)std::min<long long>(s, o->H - (long long)s * k);

@@ -1097,14 +1097,43 @@ k_csr_gram_pairs(const long long* __restrict__ rowptr, const int* __restrict__ c
 // atomics.  Together with k_csr_rows (diagonal, projections) this is the
 // same G as the pair kernel forms, up to the order of FP64 additions.
 // ---------------------------------------------------------------------------
-// cnt[f] += 1 for every stored entry of column f (cnt zero on entry)
+// cnt[c d + f] += 1 for every stored entry of column f (zero on entry), c = the
+// CTA's copy of the counters: with one copy the additions to the features that
+// most rows hold wait for one another.
 __global__ void __launch_bounds__(256)
-k_colcount(const int* __restrict__ col, long long nnz, long long ncols, int* __restrict__ cnt) {
+k_colcount(const int* __restrict__ col, long long nnz, long long ncols, int* __restrict__ cnt,
+           int copies) {
+  int* mine = cnt + (long long)(blockIdx.x % copies) * ncols;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nnz;
        e += (long long)gridDim.x * blockDim.x) {
     const int f = col[e];
-    if (f >= 0 && f < ncols) atomicAdd(cnt + f, 1);
+    if (f >= 0 && f < ncols) atomicAdd(mine + f, 1);
   }
+}
+
+// out[f] = the sum of the copies; the features with at least `heavy` entries go
+// to cand: cand[0] their number, then (feature, count) pairs (ncand at most).
+__global__ void __launch_bounds__(256)
+k_colcand(const int* cnt, int copies, long long ncols, int heavy,
+          int* out, int* __restrict__ cand, int ncand) {
+  const long long f = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (f >= ncols) return;
+  int t = 0;
+  for (int c = 0; c < copies; ++c) t += cnt[(long long)c * ncols + f];
+  out[f] = t;
+  if (t >= heavy) {
+    const int j = atomicAdd(cand, 1);
+    if (j < ncand) {
+      cand[2 + 2 * j] = (int)f;
+      cand[3 + 2 * j] = t;
+    }
+  }
+}
+
+// dmap[feats[j]] = j
+__global__ void k_dense_map(const int* __restrict__ feats, int n, int* __restrict__ dmap) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < n) dmap[feats[j]] = j;
 }
 
 // Xd[r][dmap[f]] = X^T[r][f] for the mapped (heavy) features (Xd zero on entry)
@@ -1884,17 +1913,20 @@ void launch_csr_prep(cudaStream_t st, int num_sms, const double* rn, long long n
                       Rs, Ginv, err);
 }
 
-void launch_csr_prepare(cudaStream_t st, int num_sms, const ca_csr_dev& csr, long long nrows,
-                        long long ncols, long long nnz, int* cnt, const int* dmap, int fd,
-                        float* Xd, bool fill) {
-  if (!fill) {
-    const long long blocks = std::max(1LL, std::min<long long>((nnz + 255) / 256, 8LL * num_sms));
-    k_colcount<<<(unsigned)blocks, 256, 0, st>>>(csr.col, nnz, ncols, cnt);
-    return;
-  }
-  if (fd > 0)
-    k_dense_fill<<<(unsigned)((nrows + 7) / 8), 256, 0, st>>>(csr.rowptr, csr.col, csr.val, nrows,
-                                                                ncols, dmap, fd, Xd);
+void launch_csr_count(cudaStream_t st, int num_sms, const ca_csr_dev& csr, long long ncols,
+                      long long nnz, int* copies_cnt, int copies, int* cnt, int heavy, int* cand,
+                      int ncand) {
+  const long long blocks = std::max(1LL, std::min<long long>((nnz + 255) / 256, 8LL * num_sms));
+  k_colcount<<<(unsigned)blocks, 256, 0, st>>>(csr.col, nnz, ncols, copies_cnt, copies);
+  k_colcand<<<(unsigned)((ncols + 255) / 256), 256, 0, st>>>(copies_cnt, copies, ncols, heavy, cnt,
+                                                             cand, ncand);
+}
+
+void launch_csr_dense(cudaStream_t st, const ca_csr_dev& csr, long long nrows, long long ncols,
+                      const int* feats, int nf, int* dmap, int fd, float* Xd) {
+  k_dense_map<<<(unsigned)((nf + 255) / 256), 256, 0, st>>>(feats, nf, dmap);
+  k_dense_fill<<<(unsigned)((nrows + 7) / 8), 256, 0, st>>>(csr.rowptr, csr.col, csr.val, nrows,
+                                                            ncols, dmap, fd, Xd);
 }
 
 void launch_csr_rows(cudaStream_t st, const ca_csr_dev& csr, const int* idx, long long nrows,

@@ -208,18 +208,26 @@ int launch_reduce_chain_batch(int nroles, int count, int bmax, size_t smem, cuda
 struct ca_csr_dev;
 // Dense-sparse split of the sparse Gram: heavy features (columns of X^T in
 // at least a quarter of the rows, CA_CSR_DENSE_MAX at most) get a column of
-// the dense nrows x fd matrix Xd.  launch_csr_prepare: fill = false counts
-// each column's entries into cnt (zero on entry); fill = true scatters the
-// mapped entries into Xd (zero on entry; fd, the row length of Xd, a
-// multiple of 8 with the columns past the mapped ones left zero).  The split
+// the dense nrows x fd matrix Xd (launch_csr_count, then launch_csr_dense;
+// fd, the row length of Xd, is a multiple of 8 with the columns past the
+// mapped ones left zero).  The split
 // Gram of a step: the
 // Gram of the sampled rows of Xd (k_dgram, writes the strict lower
 // triangle), then the remaining features' pair products (k_sgram, FP64
 // atomics); sb <= 4096.
 #define CA_CSR_DENSE_MAX 512
-void launch_csr_prepare(cudaStream_t st, int num_sms, const ca_csr_dev& csr, long long nrows,
-                        long long ncols, long long nnz, int* cnt, const int* dmap, int fd,
-                        float* Xd, bool fill);
+constexpr int kCsrCand = 4096;  // heavy features a candidate list holds at most
+// cnt[f] = entries of column f (summed over copies_cnt, `copies` x ncols, zero on
+// entry; may be cnt itself with one copy); the features with at least `heavy`
+// entries in cand ([0], zero on entry: their number; from [2] on (feature,
+// count) pairs, the first ncand).
+void launch_csr_count(cudaStream_t st, int num_sms, const ca_csr_dev& csr, long long ncols,
+                      long long nnz, int* copies_cnt, int copies, int* cnt, int heavy, int* cand,
+                      int ncand);
+// dmap[feats[j]] = j (the rest -1 on entry), and the columns feats of Xd (zero on
+// entry).
+void launch_csr_dense(cudaStream_t st, const ca_csr_dev& csr, long long nrows, long long ncols,
+                      const int* feats, int nf, int* dmap, int fd, float* Xd);
 // The diagonal and projections of the sampled rows (k_csr_rows), and the
 // strict lower triangle of their Gram: the split (k_dgram + k_sgram) or,
 // split = false, one warp per pair (k_csr_gram_pairs, sb <= 128).
