@@ -329,15 +329,15 @@ int launch_reduce_solve(ca_ctx* ctx, const GramPlan& g, const void* part, const 
                                                         ctx->num_sms - 1)) + 1;
     prof_mark(ctx, PC_SOLVE);
     const int e = launch_reduce_chain(grid, chain_smem(sa.b, sa.sb), ctx->stream,
-                                      static_cast<const float*>(part), ppart, g.P, g.sbp, R, Rs,
+                                      static_cast<const float*>(part), ppart, g.P, g.sbp, Rs,
                                       pvec, Ginv, ndiag, sa, ctx->d_err, ctx->d_ticket);
     prof_mark(ctx, PC_SOLVE);
     ctx->prof.kernel_launches += 1;
     return e != 0 ? cuda_fail((cudaError_t)e, __LINE__) : CA_OK;
   }
   prof_mark(ctx, PC_SOLVE);
-  launch_reduce(g.tc, G + ndiag, 0, ctx->stream, part, ppart, g.P, g.sbp, R, fast ? Rs : nullptr,
-                pvec, ndiag ? Ginv : nullptr, ndiag, sa, ctx->d_err);
+  launch_reduce(g.tc, G + ndiag, 0, ctx->stream, part, ppart, g.P, g.sbp,
+                ndiag ? nullptr : R, fast ? Rs : nullptr, pvec, ndiag ? Ginv : nullptr, ndiag, sa, ctx->d_err);
   ctx->prof.kernel_launches += 1;
   if (fast && !ndiag) {
     launch_factor(ctx->stream, R, sa, Ginv, ctx->d_err);
@@ -524,7 +524,6 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
       pa.rscale = pb.rscale;
       pa.part = static_cast<float*>(part);
       pa.ppart = ppart;
-      pa.R = R;
       pa.Rs = Rs;
       pa.pvec = pvec;
       pa.Ginv = Ginv;

@@ -52,7 +52,6 @@ struct BInst {
   long long k = 0;         // outer steps done
   int recompute_every = 0;
   int* idx_all = nullptr;  // H x b sampled indices (from opts.h0)
-  double* R = nullptr;
   float2* Rs = nullptr;
   double* pvec = nullptr;
   float2* Ginv = nullptr;
@@ -124,7 +123,7 @@ int batch_need(ca_ctx* ctx, int count, const ca_request* reqs, size_t* out, bool
     if (!pre) need += align256(panel_bytes(N, K)) + 256;
     need += align256((size_t)Kp * 8) + align256((size_t)N * 8) + align256((size_t)o.H * o.b * 4);
     if (r.method == 0) need += align256((size_t)K * 8);  // rho
-    need += 2 * align256((size_t)kBatchMaxSB * kBatchMaxSB * 8) + 3 * align256((size_t)kBatchMaxSB * 8) +
+    need += align256((size_t)kBatchMaxSB * kBatchMaxSB * 8) + 3 * align256((size_t)kBatchMaxSB * 8) +
             align256((size_t)kBatchMaxSB * kBatchMaxB * 8);
     if (prec == CA_GRAM_FP16_SCALED) need += align256((size_t)N * 4);
     if (o.check_every > 0) need += align256((size_t)check_rows(&o, N, K) * 8) + 512;
@@ -235,7 +234,6 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
       pb.c0 = 0.0;
       pb.c1 = -1.0 / ln;
     }
-    q.R = cv.take<double>((size_t)kBatchMaxSB * kBatchMaxSB);
     q.Rs = cv.take<float2>((size_t)kBatchMaxSB * kBatchMaxSB);
     q.pvec = cv.take<double>(kBatchMaxSB);
     q.delta[0] = cv.take<double>(kBatchMaxSB);
@@ -342,7 +340,7 @@ extern "C" int ca_batch_solve(ca_ctx* ctx, int count, const ca_request* reqs, in
         SolveArgs sa{idx, q.pb.N, q.b, sc, sb, sbp, q.pb.cG, q.pb.cI, q.pb.cP, q.pb.cY, q.pb.x,
                      q.pb.yv, dl};
         h_rinst[(size_t)rr * na + j] = RedInst{part, ppart, pl.nslots[(size_t)j], sbp, sc,
-                                               reduce_ctas(sb, sc, most), q.R, q.Rs,
+                                               reduce_ctas(sb, sc, most), q.Rs,
                                                q.pvec, q.Ginv, sa};
         // advance: this step's update is pending for the next round
         q.prev_idx = idx;

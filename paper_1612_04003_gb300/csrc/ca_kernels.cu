@@ -235,7 +235,7 @@ __device__ void block_solve(const double* __restrict__ R, const double* __restri
 // ---------------------------------------------------------------------------
 
 // Reduce the split-K partials (entry (i, j), i >= j, of partial c at
-// part[c][j][i]) into R (lower triangle) and p.  Rs (when not
+// part[c][j][i]) into R (lower triangle; null: not wanted) and p.  Rs (when not
 // null) receives the cG-scaled FP32 pairs of the lower-triangle entries,
 // stored transposed (entry (i, j), i >= j, at Rs[j * ldr + i]) so that the
 // chain reads a column block with coalesced loads.  CTAs 0 .. ndiag-1 each
@@ -362,12 +362,12 @@ __device__ void reduce_body(const PT* __restrict__ part, const double* __restric
         Gout[(long long)i * sb + j] = g;
         Gout[(long long)j * sb + i] = g;
       } else if constexpr (sizeof(PT) == 8) {
-        R[(long long)i * ldr + j] = t64;
+        if (R) R[(long long)i * ldr + j] = t64;
         if (Rs) Rs[(long long)j * ldr + i] = df_mul(cG2, split_f64(t64));
       } else {
         const float2 t = df_add(df_add(red[w][lane], red[w + 1][lane]),
                                 df_add(red[w + 2][lane], red[w + 3][lane]));
-        R[(long long)i * ldr + j] = (double)t.x + (double)t.y;
+        if (R) R[(long long)i * ldr + j] = (double)t.x + (double)t.y;
         if (Rs) Rs[(long long)j * ldr + i] = df_mul(cG2, t);
       }
     }
@@ -562,7 +562,7 @@ k_chain(const float2* __restrict__ Rs, const double* __restrict__ pvec,
 template <typename PT, int BMAX, int DEPTH>
 __global__ void __launch_bounds__(256, 1)
 k_reduce_chain(const PT* __restrict__ part, const double* __restrict__ ppart, int P, int sbp,
-               double* __restrict__ R, float2* __restrict__ Rs, double* __restrict__ pvec,
+               float2* __restrict__ Rs, double* __restrict__ pvec,
                float2* __restrict__ Ginv, int ndiag, SolveArgs sa, unsigned* __restrict__ err,
                unsigned* __restrict__ ticket) {
   extern __shared__ double smem_d[];
@@ -570,7 +570,8 @@ k_reduce_chain(const PT* __restrict__ part, const double* __restrict__ ppart, in
   pdl_trigger();
   const int nred = (int)gridDim.x - 1;
   if ((int)blockIdx.x < nred) {
-    reduce_body<PT>(part, ppart, P, sbp, R, Rs, pvec, Ginv, ndiag, sa, err, (int)blockIdx.x, nred);
+    reduce_body<PT>(part, ppart, P, sbp, nullptr, Rs, pvec, Ginv, ndiag, sa, err, (int)blockIdx.x,
+                    nred);
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();  // this CTA's R, Rs, p, Ginv before its count
@@ -582,12 +583,12 @@ k_reduce_chain(const PT* __restrict__ part, const double* __restrict__ ppart, in
                              [&] { return chain_wait(ticket, (unsigned)nred, true, err); });
 }
 
-template __global__ void k_reduce_chain<float, 8, 4>(const float*, const double*, int, int, double*,
-                                                     float2*, double*, float2*, int, SolveArgs,
-                                                     unsigned*, unsigned*);
+template __global__ void k_reduce_chain<float, 8, 4>(const float*, const double*, int, int, float2*,
+                                                     double*, float2*, int, SolveArgs, unsigned*,
+                                                     unsigned*);
 template __global__ void k_reduce_chain<float, 16, 3>(const float*, const double*, int, int,
-                                                      double*, float2*, double*, float2*, int,
-                                                      SolveArgs, unsigned*, unsigned*);
+                                                      float2*, double*, float2*, int, SolveArgs,
+                                                      unsigned*, unsigned*);
 // a4 of several problems (the batched solves) in one launch: reducing CTAs (role
 // table: problem and CTA index within it), then a chain CTA per problem, which
 // gathers what does not depend on the reduction and waits (bounded) for its
@@ -614,7 +615,7 @@ k_reduce_chain_batch(const RedInst* __restrict__ insts, const RedRole* __restric
     pdl_trigger();
     const RedRole ro = roles[role];
     const RedInst ri = insts[ro.inst];
-    reduce_body<float>(ri.part, ri.ppart, ri.P, ri.sbp, ri.R, ri.Rs, ri.pvec, ri.Ginv, ri.ndiag,
+    reduce_body<float>(ri.part, ri.ppart, ri.P, ri.sbp, nullptr, ri.Rs, ri.pvec, ri.Ginv, ri.ndiag,
                        ri.sa, err, ro.cta, ro.ncta);
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1522,16 +1523,15 @@ cudaError_t launch_programmatic_t(K kernel, unsigned grid, unsigned threads, siz
 }
 
 int launch_reduce_chain(int grid, size_t smem, cudaStream_t st, const float* part,
-                        const double* ppart, int P, int sbp, double* R, float2* Rs, double* pvec,
-                        float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err,
-                        unsigned* ticket) {
+                        const double* ppart, int P, int sbp, float2* Rs, double* pvec, float2* Ginv,
+                        int ndiag, const SolveArgs& sa, unsigned* err, unsigned* ticket) {
   cudaError_t e;
   if (sa.b <= 8)
     e = launch_programmatic(k_reduce_chain<float, 8, 4>, (unsigned)grid, smem, st, part, ppart, P,
-                            sbp, R, Rs, pvec, Ginv, ndiag, sa, err, ticket);
+                            sbp, Rs, pvec, Ginv, ndiag, sa, err, ticket);
   else if (sa.b <= 16)
     e = launch_programmatic(k_reduce_chain<float, 16, 3>, (unsigned)grid, smem, st, part, ppart, P,
-                            sbp, R, Rs, pvec, Ginv, ndiag, sa, err, ticket);
+                            sbp, Rs, pvec, Ginv, ndiag, sa, err, ticket);
   else
     e = cudaErrorInvalidValue;
   return (int)e;

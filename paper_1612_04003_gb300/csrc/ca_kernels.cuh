@@ -26,9 +26,8 @@ void launch_factor(cudaStream_t st, const double* R, const SolveArgs& sa, float2
 // with the diagonal-block inverses (ndiag = s_cur CTAs), then the chain on the
 // CTA that finishes last.  Returns a cudaError_t.
 int launch_reduce_chain(int grid, size_t smem, cudaStream_t st, const float* part,
-                        const double* ppart, int P, int sbp, double* R, float2* Rs, double* pvec,
-                        float2* Ginv, int ndiag, const SolveArgs& sa, unsigned* err,
-                        unsigned* ticket);
+                        const double* ppart, int P, int sbp, float2* Rs, double* pvec, float2* Ginv,
+                        int ndiag, const SolveArgs& sa, unsigned* err, unsigned* ticket);
 #define CA_FAST_B 32
 #define CA_FAST_SB 256
 // panel: FP32 A stored as 32-column panels [K/32][N][32] (k_pack_panels).
@@ -125,7 +124,6 @@ struct PersistArgs {
   const float* rscale;   // scaled FP16: power-of-two multiplier of each row of A
   float* part;           // Pg x sbp x sbp FP32 Gram partials (transposed)
   double* ppart;         // Pg x sbp projection partials
-  double* R;
   float2* Rs;
   double* pvec;
   float2* Ginv;
@@ -186,7 +184,6 @@ struct RedInst {
   const double* ppart;
   int P, sbp, ndiag;
   int nred;  // its reducing CTAs
-  double* R;
   float2* Rs;
   double* pvec;
   float2* Ginv;

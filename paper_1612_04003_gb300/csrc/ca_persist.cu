@@ -672,7 +672,6 @@ __global__ void __launch_bounds__(kThreadsP, 1) k_persist(PersistArgs a, unsigne
           asm volatile("bar.sync %0, %1;" ::"n"(kBarSide), "n"(kSideT) : "memory");
           if (half == 0 && kind == 1) {
             const float2 tt = kHalves > 1 ? df_add(red2[ent], red2[ent + 64]) : red2[ent];
-            a.R[(long long)i * ldr + j] = (double)tt.x + (double)tt.y;
             a.Rs[(long long)j * ldr + i] = df_mul(cG2, tt);
           } else if (half == 0 && kind == 2) {
             a.pvec[i] = kHalves > 1 ? redp[ent] + redp[ent + 64] : redp[ent];
