@@ -299,8 +299,8 @@ def secondary_workloads(ctx, stream):
                                 "nnz per feature), lambda 1e-5, b=8, H=2048, CUDA-core FP64 Gram "
                                 "(s*b < 32: one warp per row pair; s*b >= 32: dense part of the "
                                 "features in at least a quarter of the samples + bucketed pair "
-                                "products of the rest), next step's w-independent part on a "
-                                "second stream",
+                                "products of the rest), the w-independent part of the next two "
+                                "steps on two side streams",
                     "nnz": int(sp.rowptr[-1]), "s": s_, "ms_per_solve": t,
                     "block_updates_per_s": h_sp / (t * 1e-3),
                     "us_per_outer_step": t * 1e3 / -(-h_sp // s_)})
@@ -359,7 +359,7 @@ def batch_study(ctx, stream, count=24):
     """The batched solves (ca_batch_solve) on uneven problems shaped like the
     served-batch workload, scaled to a short run (d 256-2048, n 4096-32768):
     the same problems one after another (each its own solve), in shared
-    launches (plain and CUDA-graph-captured), and with the depth chosen by
+    launches (with and without CA_BATCH_GRAPH), and with the depth chosen by
     measured cost.  Block updates per second of the whole set."""
     import torch
     probs = _uneven_problems(count, 5, (256, 2048), (4096, 32768))

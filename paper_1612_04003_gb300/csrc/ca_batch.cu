@@ -42,7 +42,7 @@ using namespace caint;
 
 constexpr int kBatchMaxSB = 128;     // s*b of a problem in a shared round
 constexpr int kBatchMaxB = 16;       // b of a problem (chain with lookahead)
-constexpr int kSegMaxRounds = 64;    // rounds per segment (graph size)
+constexpr int kSegMaxRounds = 64;    // rounds per segment (descriptors copied at once)
 constexpr int kTrialSB[3] = {128, 64, 32};
 
 struct BInst {

@@ -6,7 +6,7 @@
 // A segment of at most kSeg columns: every row gets one power of two above its
 // largest magnitude there, each element becomes a 55-bit fixed-point integer
 // (to nearest) and the integer seven signed base-256 digits.  A digit is exact
-// in BF16; so is every product, and the sums of the products of digits i and
+// in FP16; so is every product (in FP32), and the sums of the products of digits i and
 // j with one i + j = l stay below 2^24 (l - 1 pairs of at most 2^14 over kSeg
 // columns, l <= 6), so the FP32 accumulators of the levels l = 2 .. 6 are
 // exact integers.  Levels 7 .. 9 share one accumulator (their FP32 rounding is

@@ -45,7 +45,11 @@ __global__ void k_sample(unsigned long long seed, long long h0, long long H, int
 // projection on v, split over K.  Grid (P, tile pairs): CTA (c, t) computes
 // the 64x64 tile (I, J), I >= J, of sum_{k in split c} Y[i][k] Y[j][k],
 // stored transposed (entry (i, j) at [j][i], like the tensor-core partials);
-// diagonal-tile CTAs also form sum_k Y[i][k] v[k].
+// diagonal-tile CTAs also form sum_k Y[i][k] v[k].  Bound by the FP64 pipe (two
+// FMAs a clock and SM: 557 us at 128 rows x 24001 columns), so only what
+// k_gram64 and k_persist64 (ca_persist64.cu) do not take comes here: FP32 X with
+// the exact Gram, FP64 X with more than 128 rows a step, and the form that
+// allocates nothing.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256)
@@ -762,7 +766,8 @@ template __global__ void k_update_dense<float, true>(const float*, long long, lo
 // before one FP64 atomic addition a column.  FP32 A: x split in two FP32
 // halves, exact products summed in double-float over the split's rows, then
 // FP64.  PANEL (FP32 only): A stored as 32-column panels [K/32][N][32]
-// (zero-padded).  Bound by HBM (FP32) or the FP64 pipe.
+// (zero-padded).  Bound by HBM (FP32) or the FP64 pipe.  FP32 panels 8192 x
+// 131072: 0.66 ms, 6.5 TB/s (1.10 ms with a thread walking four columns).
 // ---------------------------------------------------------------------------
 template <typename T, bool PANEL>
 __global__ void __launch_bounds__(256)
@@ -913,7 +918,9 @@ k_csr_rows(const long long* __restrict__ rowptr, const int* __restrict__ col,
 
 // Projections x_{I_p}^T w of the sampled rows alone (the part of a2+a3 that
 // needs the current w), one CTA per row: thread t takes entries t, t + 256,
-// ... of the row, four in flight, then a CTA sum (FP64 products and sums).
+// ... of the row, four in flight, then a CTA sum (FP64 products and sums).  The
+// first entries load before the wait for w: it is latency that bounds it (6.3 us
+// alone in a cold launch of 256 rows).
 __global__ void __launch_bounds__(256)
 k_csr_proj(const long long* __restrict__ rowptr, const int* __restrict__ col,
            const float* __restrict__ val, const int* __restrict__ idx, long long nrows,
@@ -1041,7 +1048,7 @@ k_csr_prep(const double* __restrict__ rn, const int* __restrict__ idx, long long
   }
 }
 
-// The off-diagonal Gram entries of few sampled rows (s*b <= 64) by sorted-list
+// The off-diagonal Gram entries of few sampled rows (s*b < 32) by sorted-list
 // intersection, one warp per pair q < p: lanes walk the shorter row and
 // binary-search the longer, products exact in FP64.
 __global__ void __launch_bounds__(256)
@@ -1088,19 +1095,23 @@ k_csr_gram_pairs(const long long* __restrict__ rowptr, const int* __restrict__ c
 // makes almost every sampled pair nonzero: its contribution to G = Y Y^T is
 // a dense rank-one term, cheaper to form as part of a small dense Gram than
 // pair by pair.  Once per solve the heavy features get a column of the dense
-// n x fd matrix Xd (k_colcount, host choice, k_dense_fill); every outer step
+// n x fd matrix Xd (k_colcount, k_colcand, host choice, k_dense_map,
+// k_dense_fill); every outer step
 // k_dgram forms the Gram of the sampled rows of Xd (exact products summed
 // in double-float) and writes the strict lower triangle of G, then k_sgram
 // adds the products of the remaining features: each CTA takes a range of
-// features, gathers the sampled rows' entries in it (a binary search per row
-// in its sorted columns), buckets them by feature in shared memory and adds
-// the exact product of every pair of entries of a feature to G with FP64
-// atomics.  Together with k_csr_rows (diagonal, projections) this is the
-// same G as the pair kernel forms, up to the order of FP64 additions.
+// features, gathers the sampled rows' entries in it (from the offset table, or
+// a binary search per row in its sorted columns), buckets them by feature in
+// shared memory and adds the exact product of every pair of entries of a
+// feature to G with FP64 atomics.  Together with the row norms (or k_csr_rows)
+// for the diagonal this is the same G as the pair kernel forms, up to the
+// order of FP64 additions.
 // ---------------------------------------------------------------------------
 // cnt[c d + f] += 1 for every stored entry of column f (zero on entry), c = the
 // CTA's copy of the counters: with one copy the additions to the features that
-// most rows hold wait for one another.
+// most rows hold wait for one another.  Eight copies, the list below in place
+// of all counts read by the host, and the set-up's other passes on streams of
+// their own: 590 -> 370 us a solve (16384 rows, 10.6 M entries).
 __global__ void __launch_bounds__(256)
 k_colcount(const int* __restrict__ col, long long nnz, long long ncols, int* __restrict__ cnt,
            int copies) {
@@ -1404,7 +1415,7 @@ k_scatter_csr(const long long* __restrict__ rowptr, const int* __restrict__ col,
 
 // a5 for the sampled rows of the sparse dual: v[col] += c * val * coef[r],
 // one CTA per listed row (entries t, t + 256, ... of the row, four in
-// flight; FP64 atomics).
+// flight; FP64 atomics).  The first entries load before the wait for Delta.
 __global__ void __launch_bounds__(256)
 k_scatter_csr_rows(const long long* __restrict__ rowptr, const int* __restrict__ col,
                    const float* __restrict__ val, const int* __restrict__ idx,
@@ -1553,7 +1564,9 @@ int launch_reduce_chain(int grid, size_t smem, cudaStream_t st, const float* par
 // in double-float (v2 zero-padded to a multiple of 32); FP64 A: FP64.
 // v and v2 change between calls (the solves update them): read through L2
 // (ld.global.cg), never the non-coherent read-only path; A is constant.
-// q starts at zero (k_residual_norm clears it after use).
+// q starts at zero (k_residual_norm clears it after use).  Bound by HBM at many
+// columns, else by the latency of its loads: the next rows' loads are in flight
+// while a set is summed (X^T 20003 x 1000: 41 us before).
 template <typename T, bool PANEL>
 __global__ void __launch_bounds__(256)
 k_rowdot_dense(const T* __restrict__ A, long long lda, long long N, long long K,
@@ -1802,7 +1815,9 @@ void launch_split(cudaStream_t st, const double* v, long long K, float2* v2) {
 // rows) into 32-column panels: P[(a N + r) 32 + c] = A[r][32 a + c], zero past
 // K.  A CTA takes 8 rows x 64 panels: a warp reads 512 contiguous bytes of its
 // row (four panels), the eight warps write 1 KB of each panel.  rmax (when not
-// null, zero on entry): the bits of each row's largest magnitude, NaN left out.
+// null, zero on entry): the bits of each row's largest magnitude, NaN left out
+// (a pass of its own over the panels took 0.71 ms at 8192 x 131072, this pass
+// 1.49 ms before and after).  Bound by HBM, a read and a write of X.
 __global__ void __launch_bounds__(256)
 k_pack_panels(const float* __restrict__ A, long long N, long long K, long long lda,
               float* __restrict__ Pn, unsigned* __restrict__ rmax) {

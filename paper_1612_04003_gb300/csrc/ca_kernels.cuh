@@ -196,12 +196,12 @@ int launch_reduce_chain_batch(int nroles, int count, int bmax, size_t smem, cuda
                               const RedInst* insts, const RedRole* roles, unsigned* arrived,
                               unsigned* tickets, unsigned* err);
 
-// Sparse dual, steps a2+a3 of one outer step from the CSR of X^T (row hash
-// tables, ca_kernels.cu): G (ldr x ldr, transposed lower triangle, the one
-// "partial" of the reduction) and the projections pvec[r] = x_{I_r}^T w, in
-// one programmatic-dependent launch.  Then a4 by the reduction of that
-// single FP64 partial, the diagonal inverses and the chain in one launch
-// (b <= 16), and a5 by the scatter (programmatic dependent).
+// Sparse dual, one outer step from the CSR of X^T.  The strict lower triangle of
+// G (ldr x ldr, transposed) by the pair kernel or the split below; b <= 16: the
+// diagonal from the row norms, the inverses and Rs (launch_csr_prep) follow it on
+// its side stream, and the library stream runs the projections pvec[r] =
+// x_{I_r}^T w, the chain and the scatter.  b > 16 or FP64 solves: diagonal and
+// projections by launch_csr_rows, then the general reduce, factor and solve.
 struct ca_csr_dev;
 // Dense-sparse split of the sparse Gram: heavy features (columns of X^T in
 // at least a quarter of the rows, CA_CSR_DENSE_MAX at most) get a column of
