@@ -1361,13 +1361,19 @@ int ca_gram_project(ca_ctx* ctx, int xfmt, int prec, const void* A, long long N,
                         (const void*)p})
     if (!is_device_ptr(q)) return CA_ERR_ARG;
   CA_TRY_CUDA(cudaSetDevice(ctx->device));
-  const GramPlan g = gram_plan(ctx, xfmt, prec, sb, K);
+  GramPlan g = gram_plan(ctx, xfmt, prec, sb, K);
   const size_t el = g.tc ? 4 : 8;
   const long long Kp = (K + 31) / 32 * 32;
-  const size_t need = align256((size_t)g.P * g.sbp * g.sbp * el) + align256((size_t)g.P * g.sbp * 8) +
-                      align256((size_t)g.sbp * g.sbp * 8) + align256((size_t)g.sbp * 8) +
-                      align256((size_t)Kp * 8) + align256((size_t)N * 4) + 1024;
-  CA_TRY(ensure_arena(ctx, need));
+  auto need = [&] {
+    return align256((size_t)g.P * g.sbp * g.sbp * el) + align256((size_t)g.P * g.sbp * 8) +
+           align256((size_t)g.sbp * g.sbp * 8) + align256((size_t)g.sbp * 8) +
+           align256((size_t)Kp * 8) + align256((size_t)N * 4) + 1024;
+  };
+  // a tight scratch bound: a partial for two CTAs per SM and 64 x 64 tile
+  // (k_gram_simt's number) instead of one per SM, if that is fewer
+  if (xfmt == CA_DENSE_F64 && ctx->scratch_max && need() > ctx->scratch_max)
+    g.P = std::min(g.P, std::max(1, 2 * ctx->num_sms / g.ntiles));
+  CA_TRY(ensure_arena(ctx, need()));
   Carve cv{static_cast<char*>(ctx->arena)};
   const bool f16 = g.tc && prec == CA_GRAM_FP16_SCALED;
   float* rsc = f16 ? cv.take<float>((size_t)N) : nullptr;  // per-row FP16 multipliers

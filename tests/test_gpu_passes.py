@@ -193,3 +193,26 @@ def test_sparse_at_a_scratch_bound(ctx):
         pytest.fail("no bound accepted")
     assert bound > 1 << 20
     assert _rel(a, a_ref.cpu().numpy()) < TOL64 and _rel(w, w_ref.cpu().numpy()) < TOL64
+
+
+def test_fp64_gram_at_a_scratch_bound(ctx):
+    """128 rows: 16 MB hold two partials per SM and three 64 x 64 tiles, not one per SM (2^-52 K
+    m_i m_j as without a bound); 8 MB hold neither."""
+    import paper_1612_04003_gb300 as ca
+    rng = np.random.default_rng(2)
+    A, v = rng.standard_normal((128, 9001)), rng.standard_normal(9001)
+    idx = torch.arange(128, dtype=torch.int32, device="cuda")
+    G = torch.empty(128, 128, dtype=torch.float64, device="cuda")
+    p = torch.empty(128, dtype=torch.float64, device="cuda")
+    c = ca.Context(0, scratch_bytes_max=16 << 20)
+    c.ca_gram_project(_dev(A), idx, _dev(v), G, p, prec="f64")
+    c.close()
+    m = np.abs(A).max(1)
+    Y = A.astype(np.longdouble)
+    assert (np.abs(G.cpu().numpy() - Y @ Y.T) <= 2.0 ** -52 * 9001 * np.outer(m, m)).all()
+    assert (np.abs(p.cpu().numpy() - Y @ v) <= 2.0 ** -52 * 9001 * m * np.abs(v).max()).all()
+    c = ca.Context(0, scratch_bytes_max=8 << 20)
+    with pytest.raises(ca.CaError) as e:
+        c.ca_gram_project(_dev(A), idx, _dev(v), G, p, prec="f64")
+    c.close()
+    assert e.value.status == ca.CA_ERR_OOM
