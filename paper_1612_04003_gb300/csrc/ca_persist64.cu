@@ -10,7 +10,7 @@
 //   column CTA, step k, main warps: wait Delta_{k-1} -> v -= cU Y_{k-1}^T
 //     Delta_{k-1} on its columns, p partial -> count P -> Gram partial of step
 //     k+1 -> count G; side warps: all G -> its share of the entries summed (Rs,
-//     the diagonal blocks) -> count E (s b >= 64: then all P -> its rows of p
+//     the diagonal blocks) -> count E (s b >= 32: then all P -> its rows of p
 //     -> count Q)
 //   inverse CTA, step k:  all E -> its diagonal blocks inverted -> count R
 //   chain CTA, step k:    all R and P (or Q) -> p -> the s dependent solves ->
@@ -42,7 +42,10 @@ constexpr int kSide = 96;    // side threads of a column CTA (reduction); twelve
 constexpr int kMma = 32;     // and the warp that issues the MMAs of the digit Gram
 constexpr int kBarSide = 7;  // named barrier of the side warps
 constexpr int kSmemMax = 200 * 1024;  // dynamic shared memory a launch may ask for
-constexpr int kSmallSB = 16;  // rows of a step the CUDA-core Gram takes
+// Rows of a step up to which the Gram is formed on CUDA cores, digits above (ms a
+// solve, CUDA cores against digits: 16 rows x 1024 columns 0.627 / 0.692, 32
+// rows x 8190 columns 1.63 / 1.15).
+constexpr int kSmallSB = 16;
 
 // Counts in cnt[].  A fast CTA may form the Gram partial of step p + 1 (and its
 // side warps reduce it) before a slow one has done step p, but not that of
@@ -52,7 +55,10 @@ struct Cnt {
   enum { G = 0, E = 2, R = 4, P = 6, Q = 7, D = 8 };
 };
 constexpr int kMaxInv = 16;  // inverse CTAs
-constexpr int kRowsSB = 64;  // s b from which the column CTAs sum p
+// s b from which the column CTAs' side warps sum p, a row a warp, and not the
+// chain CTA (ms a solve, chain CTA against side warps: 4 rows 1.72 / 1.96, 16
+// rows 0.643 / 0.647, 32 rows 1.157 / 1.096)
+constexpr int kRowsSB = 32;
 
 // thread 0 waits, the main warps follow; false once a wait of the grid gave up
 __device__ __forceinline__ bool main_wait(const unsigned* p, unsigned target, unsigned* err, bool ok) {
@@ -305,10 +311,10 @@ k_gram64(Persist64Args a, unsigned* __restrict__ err) {
   }
 }
 
-// p[r] = the sum of the P partials, all threads.  An FP64 addition holds a
-// scheduler for 64 cycles whatever the lanes in use: for few rows a warp sums
-// a row (lanes over the partials), for more the lanes take 32 rows and the
-// warps share the partials (sm: 256 sums).
+// p[r] = the sum of the P partials of sb < kRowsSB rows, all threads.  An FP64
+// addition holds a scheduler for 64 cycles whatever the lanes in use: for few
+// rows a warp sums a row (lanes over the partials), for more the lanes take the
+// rows and the warps share the partials (sm: 256 sums).
 __device__ __forceinline__ void sum_rows(const Persist64Args& a, int P, int sbp, int sb, double* sm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (sb <= 8) {
@@ -320,18 +326,16 @@ __device__ __forceinline__ void sum_rows(const Persist64Args& a, int P, int sbp,
       if (lane == 0) a.pvec[warp] = t;
     }
   } else {
-    const int gw = sb <= 32 ? 8 : 4;  // warps a group of 32 rows
-    const int grp = warp / gw, sub = warp % gw, r = 32 * grp + lane;
     double t = 0.0;
-    if (r < sb) {
+    if (lane < sb) {
 #pragma unroll 16
-      for (int q = sub; q < P; q += gw) t += __ldcg(a.ppart + (long long)q * sbp + r);
+      for (int q = warp; q < P; q += 8) t += __ldcg(a.ppart + (long long)q * sbp + lane);
     }
     sm[threadIdx.x] = t;
     main_sync();
-    if (sub == 0 && r < sb) {
-      for (int w = 1; w < gw; ++w) t += sm[threadIdx.x + 32 * w];
-      a.pvec[r] = t;
+    if (warp == 0 && lane < sb) {
+      for (int w = 1; w < 8; ++w) t += sm[lane + 32 * w];
+      a.pvec[lane] = t;
     }
   }
   main_sync();
