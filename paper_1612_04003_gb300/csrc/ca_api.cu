@@ -239,8 +239,8 @@ GramPlan gram_plan(ca_ctx* ctx, int xfmt, int prec, int sbm, long long K) {
     const int t = g.sbp / 64;
     g.ntiles = t * (t + 1) / 2;
     const long long nchunks = (K + 31) / 32;
-    if (xfmt == CA_DENSE_F64 && sbm <= gram64_max_sb()) {  // k_gram64: a CTA per SM
-      g.P = (int)std::min<long long>(ctx->num_sms, nchunks);
+    if (xfmt == CA_DENSE_F64) {  // k_gram64
+      g.P = gram64_splits(sbm, K, ctx->num_sms);
       return g;
     }
     long long Pm = std::max(1LL, (long long)(2 * ctx->num_sms) / g.ntiles);

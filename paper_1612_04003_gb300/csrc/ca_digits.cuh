@@ -83,6 +83,13 @@ struct DigitGram {
   int64_t* diag;        // [SBP] (SBP = 128)
   uint32_t gt = 0;      // stages so far (buffers and phases run on)
   uint32_t ph = 0;      // passes so far
+  // gram<true>: two groups of 64 rows of a larger Gram, at rows and columns lo
+  // and hi + 64 of the partial; the diagonal block of a group only if owned
+  int lo = 0, hi = 0;
+  bool own_lo = true, own_hi = true;
+  __device__ __forceinline__ bool owned(int i, int j) const {  // i >= j
+    return i >= 64 ? (j < 64 || own_hi) : own_lo;
+  }
 
   // This thread's rows 2 (warp + 8 i) + lane / 16, columns 2 (lane % 16) and
   // the next of a stage.
@@ -234,10 +241,12 @@ struct DigitGram {
 
   // Gram of rows off[0 .. sb) over columns [k0, k1), added to (add) or stored
   // in part[j * sbp + i], i >= j.  All 256 threads; false once a wait gave up.
+  template <bool PAIR = false>
   __device__ bool gram(const double* __restrict__ A, const long long* off, int sb, long long k0,
                        long long k1, double* __restrict__ part, int sbp, bool add, unsigned* err,
                        bool ok) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    auto at_ = [&](int r) { return PAIR ? r + (r < 64 ? lo : hi) : r; };  // a row's place in part
     // largest exponent of each row in the segment
     bool plain = false;
     constexpr int RB = 4;  // rows in flight a warp
@@ -270,9 +279,11 @@ struct DigitGram {
       for (int e = tid; e < sb * (sb + 1) / 2; e += 256) {
         int i, j;
         tri_decode(e, i, j);
-        double s = add ? part[(long long)j * sbp + i] : 0.0;
+        if (PAIR && !owned(i, j)) continue;
+        double* at = part + (long long)at_(j) * sbp + at_(i);
+        double s = add ? *at : 0.0;
         for (long long k = k0; k < k1; ++k) s = fma(__ldg(A + off[i] + k), __ldg(A + off[j] + k), s);
-        part[(long long)j * sbp + i] = s;
+        *at = s;
       }
       main_sync();
       return ok;
@@ -312,7 +323,7 @@ struct DigitGram {
         if (j > row) break;
         // units of level 7 (2^-40 of level 2), then 2^(er + ej - 2098)
         const double g = fixed_to_double(v[q] * 256 + __float2int_rn(low[q]), er + emax[j]);
-        double* at = part + (long long)j * sbp + row;
+        double* at = part + (long long)at_(j) * sbp + at_(row);
         *at = add ? *at + g : g;
       }
     };
@@ -325,7 +336,8 @@ struct DigitGram {
     const int ccn = (warp & 3) * 32 + 31;  // last column of the quadrant's triangle
     auto chunks = [&](auto&& f) {
       if (act)
-        for (int cc = 16 * (warp >> 2); cc < sb && cc <= ccn; cc += 32) f(cc);
+        for (int cc = 16 * (warp >> 2); cc < sb && cc <= ccn; cc += 32)
+          if (!PAIR || owned(ccn, cc)) f(cc);
     };
     if constexpr (SBP <= 64) {
       ok = pass<2, 9>(A, rw, sb, k0, k1, err, ok);
@@ -345,7 +357,7 @@ struct DigitGram {
     } else {
       // the integers of levels 2 .. 5 wait in the half of the partial that holds
       // no entry: (row, j) at [row * sbp + j], j < row, and the diagonal in diag
-      int64_t* hold = reinterpret_cast<int64_t*>(part) + (long long)min(row, sb - 1) * sbp;
+      int64_t* hold = reinterpret_cast<int64_t*>(part) + (long long)at_(min(row, sb - 1)) * sbp;
       ok = pass<2, 5>(A, rw, sb, k0, k1, err, ok);
       chunks([&](int cc) {
         int64_t v[16];
@@ -358,7 +370,7 @@ struct DigitGram {
         if (row < sb) {
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
-            if (cc + q < row) hold[cc + q] = v[q];
+            if (cc + q < row) hold[at_(cc + q)] = v[q];
             if (cc + q == row) diag[row] = v[q];
           }
         }
@@ -369,7 +381,7 @@ struct DigitGram {
       chunks([&](int cc) {
         int64_t v[16];
 #pragma unroll
-        for (int q = 0; q < 16; ++q) v[q] = hold[min(cc + q, SBP - 1)];
+        for (int q = 0; q < 16; ++q) v[q] = hold[at_(min(cc + q, SBP - 1))];
 #pragma unroll
         for (int q = 0; q < 16; ++q)
           if (cc + q == row) v[q] = diag[row];

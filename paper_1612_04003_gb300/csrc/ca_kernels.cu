@@ -48,8 +48,7 @@ __global__ void k_sample(unsigned long long seed, long long h0, long long H, int
 // diagonal-tile CTAs also form sum_k Y[i][k] v[k].  Bound by the FP64 pipe (two
 // FMAs a clock and SM: 557 us at 128 rows x 24001 columns), so only what
 // k_gram64 and k_persist64 (ca_persist64.cu) do not take comes here: FP32 X with
-// the exact Gram, FP64 X with more than 128 rows a step, and the form that
-// allocates nothing.
+// the exact Gram, and the form that allocates nothing.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256)
@@ -1816,8 +1815,9 @@ void launch_split(cudaStream_t st, const double* v, long long K, float2* v2) {
 // K.  A CTA takes 8 rows x 64 panels: a warp reads 512 contiguous bytes of its
 // row (four panels), the eight warps write 1 KB of each panel.  rmax (when not
 // null, zero on entry): the bits of each row's largest magnitude, NaN left out
-// (a pass of its own over the panels took 0.71 ms at 8192 x 131072, this pass
-// 1.49 ms before and after).  Bound by HBM, a read and a write of X.
+// (a pass of its own over the panels took 0.71 ms).  Bound by HBM, a read and a
+// write of X: 8192 x 131072 1.25 ms, 6.9 TB/s (1.49 ms with a warp writing one
+// row of four panels at a time).
 __global__ void __launch_bounds__(256)
 k_pack_panels(const float* __restrict__ A, long long N, long long K, long long lda,
               float* __restrict__ Pn, unsigned* __restrict__ rmax) {

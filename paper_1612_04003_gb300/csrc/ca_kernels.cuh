@@ -160,9 +160,9 @@ struct Persist64Args {
   SolveArgs sa;          // solve constants (idx and delta are set per step); ldr = sbp
   unsigned* cnt;         // 9 counts, zero on entry
 };
-// The Gram pass of dense FP64 X alone, sb <= gram64_max_sb(): P <= ceil(K / 32)
-// split-K partials (P x sbp^2, transposed) and projections (P x sbp).
-int gram64_max_sb();
+// The Gram pass of dense FP64 X alone: P <= gram64_splits() split-K partials (P x
+// sbp^2, transposed, sbp a multiple of 64) and projections (P x sbp).
+int gram64_splits(int sb, long long K, int num_sms);
 int launch_gram64(const double* A, long long lda, long long N, long long K, const int* idx, int sb,
                   const double* v, int P, int sbp, double* part, double* ppart, unsigned* err,
                   cudaStream_t st);

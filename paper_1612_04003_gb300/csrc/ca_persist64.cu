@@ -262,7 +262,7 @@ __device__ __forceinline__ void digits_end(const DigitGram<8 * RQ>& dg) {
 }
 
 // Gram partial of the CTA's columns [c0, c1).
-template <int RQ>
+template <int RQ, bool PAIR = false>
 __device__ __forceinline__ bool gram_columns(DigitGram<8 * RQ>& dg, const double* __restrict__ A,
                                              const long long* off, int sb, long long c0,
                                              long long c1, double* smem_d, double* __restrict__ part,
@@ -274,24 +274,41 @@ __device__ __forceinline__ bool gram_columns(DigitGram<8 * RQ>& dg, const double
   // segments of equal length, whole 32-column stages
   const long long nst = (c1 - c0 + 31) / 32, nseg = (nst + kSeg / 32 - 1) / (kSeg / 32);
   for (long long g = 0; g < nseg && ok; ++g)
-    ok = dg.gram(A, off, sb, c0 + nst * g / nseg * 32, min(c1, c0 + nst * (g + 1) / nseg * 32), part,
+    ok = dg.template gram<PAIR>(A, off, sb, c0 + nst * g / nseg * 32, min(c1, c0 + nst * (g + 1) / nseg * 32), part,
                  sbp, g > 0, err, ok);
   return ok;
 }
 
 // The Gram pass alone (steps a2+a3): split-K partials over gridDim.x CTAs and
-// the projection partials on v.
-template <int RQ>
+// the projection partials on v.  PAIR (more than 128 rows): blockIdx.y is a pair
+// of groups of 64 rows, whose 128-row Gram the CTA forms and of which it stores
+// the off-diagonal block, the diagonal block of a group being stored with the
+// next group (the last one's with the one before).  (ng - 1) ng / 2
+// tiles, of which a group pair is one; 256 x 24001 0.36 ms, 512 x 24001 1.55 ms
+// (1.80 and 6.42 ms as FP64 FMAs in 64 x 64 tiles), error 2.1e-16 K against
+// 4.9e-15 K at 1000 columns.
+template <int RQ, bool PAIR>
 __global__ void __launch_bounds__(kT + kMma, 1)
 k_gram64(Persist64Args a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
   __shared__ long long soff[8 * RQ];
   __shared__ double ured[64 * RQ];
   __shared__ DigitShared<RQ> sh;
-  const int P = (int)gridDim.x, c = blockIdx.x, sb = a.sb, sbp = a.sa.ldr;
+  const int P = (int)gridDim.x, c = blockIdx.x, sbp = a.sa.ldr;
   const long long nch = (a.K + 15) / 16;
   const long long c0 = nch * c / P * 16, c1 = min(a.K, nch * (c + 1) / P * 16);
   DigitGram<8 * RQ> dg;
+  int sb = a.sb, ga = 0, gb = 1;  // rows, and the groups of a pair
+  if constexpr (PAIR) {
+    const int ng = (a.sb + 63) / 64;
+    tri_decode((int)blockIdx.y, gb, ga);
+    ++gb;
+    sb = 64 + min(64, a.sb - 64 * gb);
+    dg.lo = 64 * ga;
+    dg.hi = 64 * (gb - 1);
+    dg.own_lo = gb == ga + 1;
+    dg.own_hi = dg.own_lo && gb == ng - 1;
+  }
   const bool digits = sb > kSmallSB;
   if (digits) digits_begin<RQ>(dg, sh, smem_d);
   if (threadIdx.x >= kT) {
@@ -301,10 +318,18 @@ k_gram64(Persist64Args a, unsigned* __restrict__ err) {
     }
     return;
   }
-  row_offsets(a.idx_all, sb, a.N, a.lda, soff, err);
+  if constexpr (PAIR) {
+    row_offsets(a.idx_all + 64 * ga, 64, a.N, a.lda, soff, err);
+    row_offsets(a.idx_all + 64 * gb, sb - 64, a.N, a.lda, soff + 64, err);
+  } else {
+    row_offsets(a.idx_all, sb, a.N, a.lda, soff, err);
+  }
   main_sync();
-  gram_columns<RQ>(dg, a.A, soff, sb, c0, c1, smem_d, a.part + (long long)c * sbp * sbp, sbp, err, true);
-  update_project<RQ>(a, soff, soff, nullptr, sb, 0, c0, c1, ured, a.ppart + (long long)c * sbp);
+  gram_columns<RQ, PAIR>(dg, a.A, soff, sb, c0, c1, smem_d, a.part + (long long)c * sbp * sbp, sbp,
+                         err, true);
+  if (!PAIR || dg.own_lo)  // (the last pair's groups follow each other)
+    update_project<RQ>(a, soff, soff, nullptr, !PAIR || dg.own_hi ? sb : 64, 0, c0, c1, ured,
+                       a.ppart + (long long)c * sbp + 64 * ga);
   if (digits) {
     dg.stop();
     digits_end<RQ>(dg);
@@ -530,7 +555,7 @@ size_t column_smem(int sb) {
 
 template <typename Kern>
 int launch64(Kern kern, std::atomic<unsigned long long>& configured, const Persist64Args& a,
-             int grid, size_t smem, bool coop, unsigned* err, cudaStream_t st) {
+             dim3 grid, size_t smem, bool coop, unsigned* err, cudaStream_t st) {
   if (smem > (size_t)kSmemMax) return (int)cudaErrorInvalidConfiguration;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -542,7 +567,7 @@ int launch64(Kern kern, std::atomic<unsigned long long>& configured, const Persi
     configured.fetch_or(bit, std::memory_order_release);
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(coop ? kT + kMma + kSide : kT + kMma);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
@@ -562,15 +587,24 @@ int launch_steps(const Persist64Args& a, int P, size_t chain_smem, unsigned* err
                   std::max(chain_smem, column_smem<RQ>(a.sb)), true, err, st);
 }
 
-template <int RQ>
-int launch_gram(const Persist64Args& a, int P, unsigned* err, cudaStream_t st) {
+template <int RQ, bool PAIR = false>
+int launch_gram(const Persist64Args& a, dim3 grid, unsigned* err, cudaStream_t st) {
   static std::atomic<unsigned long long> configured{0ull};
-  return launch64(k_gram64<RQ>, configured, a, P, column_smem<RQ>(a.sb), false, err, st);
+  return launch64(k_gram64<RQ, PAIR>, configured, a, grid, column_smem<RQ>(a.sb), false, err, st);
+}
+
+// pairs of groups of 64 rows (one: all rows in one CTA)
+int gram64_pairs(int sb) {
+  const int ng = (sb + 63) / 64;
+  return sb <= 128 ? 1 : ng * (ng - 1) / 2;
 }
 
 }  // namespace
 
-int gram64_max_sb() { return 128; }
+// One CTA per SM over the column splits and row pairs.
+int gram64_splits(int sb, long long K, int num_sms) {
+  return (int)std::min<long long>(std::max(1, num_sms / gram64_pairs(sb)), (K + 31) / 32);
+}
 
 int launch_gram64(const double* A, long long lda, long long N, long long K, const int* idx, int sb,
                   const double* v, int P, int sbp, double* part, double* ppart, unsigned* err,
@@ -586,10 +620,10 @@ int launch_gram64(const double* A, long long lda, long long N, long long K, cons
   a.part = part;
   a.ppart = ppart;
   a.sa.ldr = sbp;
-  if (sb <= 32) return launch_gram<4>(a, P, err, st);
-  if (sb <= 64) return launch_gram<8>(a, P, err, st);
-  if (sb <= 128) return launch_gram<16>(a, P, err, st);
-  return (int)cudaErrorInvalidValue;
+  if (sb <= 32) return launch_gram<4>(a, dim3(P), err, st);
+  if (sb <= 64) return launch_gram<8>(a, dim3(P), err, st);
+  if (sb <= 128) return launch_gram<16>(a, dim3(P), err, st);
+  return launch_gram<16, true>(a, dim3(P, gram64_pairs(sb)), err, st);
 }
 
 // Column CTAs of the persistent launch (0: not for this block size, rows of a

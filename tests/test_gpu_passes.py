@@ -216,3 +216,40 @@ def test_fp64_gram_at_a_scratch_bound(ctx):
         c.ca_gram_project(_dev(A), idx, _dev(v), G, p, prec="f64")
     c.close()
     assert e.value.status == ca.CA_ERR_OOM
+
+
+@pytest.mark.parametrize("rows,K", [(129, 1), (191, 3000), (192, 40), (193, 999), (256, 2401),
+                                    (300, 33), (700, 200)])
+def test_fp64_gram_of_row_pairs(ctx, rows, K):
+    """More than 128 rows: pairs of groups of 64, the last one ragged; rows of magnitudes 1e-6 ..
+    1e6, one group with a row outside the digits' exponent range (plain FP64 sums), one with an
+    infinity.  2^-52 K m_i m_j, as for up to 128 rows, and K 2^-1074 where the square of the
+    small row is a subnormal number."""
+    rng = np.random.default_rng(rows)
+    A = rng.standard_normal((rows, K)) * 10.0 ** rng.uniform(-6, 6, (rows, 1))
+    A[70] *= 1e-160
+    A[rows - 1, K // 2] = np.inf
+    v = rng.standard_normal(K)
+    idx = rng.permutation(rows).astype(np.int32)
+    G = torch.full((rows, rows), 7.0, dtype=torch.float64, device="cuda")
+    p = torch.empty(rows, dtype=torch.float64, device="cuda")
+    ctx.ca_gram_project(_dev(A), _dev(idx), _dev(v), G, p, prec="f64")
+    g, h, keep = G.cpu().numpy(), p.cpu().numpy(), np.isfinite(A[idx]).all(1)
+    Y = A[idx][keep].astype(np.longdouble)
+    m = np.abs(A[idx][keep]).max(1)
+    assert (g == g.T)[np.ix_(keep, keep)].all() and not np.isfinite(g[~keep]).any()
+    tol = 2.0 ** -52 * K * np.outer(m, m) + K * 2.0 ** -1074
+    assert (np.abs(g[np.ix_(keep, keep)] - Y @ Y.T) <= tol).all()
+    assert (np.abs(h[keep] - Y @ v) <= 2.0 ** -52 * K * m * np.abs(v).max()).all()
+    assert not np.isfinite(h[~keep]).any()
+
+
+@pytest.mark.parametrize("b,s", [(16, 16), (16, 9), (32, 5), (8, 40)])
+def test_fp64_solve_of_row_pairs(ctx, b, s):
+    """The same in a solve whose last step is short (fewer groups, or one CTA's rows)."""
+    p = synth.tiny_primal(d=300, n=2001, seed=s)
+    w, z = _zeros(300), _zeros(2001)
+    H = 3 * s + s // 2 + 1
+    ctx.ca_bcd_solve(_dev(p.X), _dev(p.y), w, z, b=b, s=s, H=H, lam=1e-1, seed=4, prec="f64")
+    w_ref, z_ref = oracle.ca_bcd(p.X, p.y, 1e-1, b=b, s=s, H=H, seed=4)
+    assert _rel(w, w_ref) < TOL64 and _rel(z, z_ref) < TOL64
