@@ -413,11 +413,12 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
     __shared__ float2 colbuf[66];
     for (int p = 0; p < npass && ok; ++p) {
       ok = main_wait(a.cnt + Cnt::E + (p & 1), (unsigned)(nred * (p / 2 + 1)), err, ok);
-      for (int j = c - P; j < s; j += ninv) {  // (each block replaced by its inverse)
+      int done = 0;  // pivots: the blocks of this CTA share colbuf without a barrier between them
+      for (int j = c - P; j < s; j += ninv, done += b) {  // (each block replaced by its inverse)
         float2* out = a.Ginv[(a.k0 + p) & 1] + (long long)j * b * b;
         float2 m[1] = {tid < b * b ? __ldcg(out + tid) : make_float2(0.f, 0.f)};
-        if (BMAX > 8) cta_sweep_inverse<1, kT, 8>(m, b, colbuf, out, err, tid);
-        else if (tid < 64) cta_sweep_inverse<1, 64, 8>(m, b, colbuf, out, err, tid);
+        if (BMAX > 8) cta_sweep_inverse<1, kT, 8>(m, b, colbuf, out, err, tid, done);
+        else if (tid < 64) cta_sweep_inverse<1, 64, 8>(m, b, colbuf, out, err, tid, done);
       }
       main_count(a.cnt + Cnt::R + (p & 1));
     }

@@ -24,11 +24,14 @@
 // barrier BAR over their 64 threads (NT = 256 with BAR other than 1: named
 // barrier BAR over 256 threads of a larger CTA).
 // Writes Gamma^{-1} (FP32 pairs, row-major) to out; a non-positive pivot
-// raises CA_DEV_ERR_NOT_SPD.
+// raises CA_DEV_ERR_NOT_SPD.  Threads that invert several blocks one after another
+// with no barrier of their own in between pass the pivots they have done so far
+// as `done`: the buffers then alternate from block to block too (after an odd b
+// pivot 0 would write the buffer that the last pivot still reads).
 template <int EPT, int NT = 256, int BAR = 1>
 __device__ void cta_sweep_inverse(float2 (&a)[EPT], int b, float2* __restrict__ colbuf,
                                   float2* __restrict__ out, unsigned* __restrict__ err,
-                                  int tix = -1) {
+                                  int tix = -1, int done = 0) {
   static_assert(NT == 1024 || NT == 256 || NT == 64, "a whole CTA or two of its warps");
   const int t = tix >= 0 ? tix : (int)(threadIdx.x % NT);  // index among the NT threads
   int ri[EPT], ci[EPT];
@@ -40,7 +43,7 @@ __device__ void cta_sweep_inverse(float2 (&a)[EPT], int b, float2* __restrict__ 
   }
   const bool active = t < b * b;
   for (int k = 0; k < b; ++k) {
-    float2* ck = colbuf + (k & 1) * 33;  // [0, b): column k
+    float2* ck = colbuf + ((done + k) & 1) * 33;  // [0, b): column k
 #pragma unroll
     for (int q = 0; q < EPT; ++q) {
       if (ci[q] == k) {

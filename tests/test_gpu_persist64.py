@@ -123,3 +123,24 @@ def test_gram_fp64_non_finite(ctx):
     assert (np.isnan(g) == np.isnan(ref)).all() and (np.isinf(g) == np.isinf(ref)).all()
     fin = np.isfinite(ref)
     assert np.abs(g[fin] - ref[fin]).max() <= 2.0 ** -52 * 500 * 25
+
+
+@pytest.mark.parametrize("method,d,n,b,s", [("primal", 150, 2003, 7, 17), ("dual", 2003, 150, 7, 18),
+                                            ("primal", 140, 999, 5, 25), ("dual", 700, 140, 3, 42)])
+def test_odd_blocks_in_turn(ctx, method, d, n, b, s):
+    """Odd b with more than 16 blocks a step: an inverse CTA takes several blocks one after another,
+    and the last pivot of one and the first of the next are both even.  Seven steps, the last one
+    short; 1e-10, as for every FP64 solve."""
+    p = synth.tiny_primal(d=d, n=n, seed=b + s)
+    lam, H = 1e-1, 6 * s + 5
+    x = torch.zeros(d if method == "primal" else n, dtype=torch.float64, device="cuda")
+    aux = torch.zeros(n if method == "primal" else d, dtype=torch.float64, device="cuda")
+    kw = dict(b=b, s=s, H=H, seed=9)
+    if method == "primal":
+        ctx.ca_bcd_solve(_dev(p.X), _dev(p.y), x, aux, lam=lam, prec="f64", **kw)
+        ref = oracle.ca_bcd(p.X, p.y, lam, **kw)
+    else:
+        ctx.ca_bdcd_solve(_dev(p.X.T), _dev(p.y), x, aux, lam=lam, prec="f64", **kw)
+        ref = oracle.ca_bdcd(p.X, p.y, lam, **kw)
+    assert _rel(x.cpu().numpy(), np.asarray(ref[0])) < 1e-10
+    assert _rel(aux.cpu().numpy(), np.asarray(ref[1])) < 1e-10
