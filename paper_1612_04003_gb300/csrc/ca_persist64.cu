@@ -214,6 +214,9 @@ __device__ void update_project(const Persist64Args& a, const long long* off, con
 template <int RQ>
 struct DigitShared {
   int emax[8 * RQ];
+  float wt[8 * RQ];
+  int nlist;
+  uint32_t tmin[16];
   int64_t diag[RQ == 16 ? 128 : 1];
   uint64_t bars[5];
   uint32_t cmd[2];
@@ -230,6 +233,9 @@ __device__ __forceinline__ void digits_begin(DigitGram<8 * RQ>& dg, DigitShared<
                                             ~uintptr_t(1023));
   dg.bars = sh.bars;
   dg.emax = sh.emax;
+  dg.wt = sh.wt;
+  dg.nlist = &sh.nlist;
+  dg.tmin = sh.tmin;
   dg.diag = sh.diag;
   dg.cmd = sh.cmd;
   if (threadIdx.x == 0) {

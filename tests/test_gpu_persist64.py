@@ -144,3 +144,67 @@ def test_odd_blocks_in_turn(ctx, method, d, n, b, s):
         ref = oracle.ca_bdcd(p.X, p.y, lam, **kw)
     assert _rel(x.cpu().numpy(), np.asarray(ref[0])) < 1e-10
     assert _rel(aux.cpu().numpy(), np.asarray(ref[1])) < 1e-10
+
+
+def _uneven(rng, rows, K, kind):
+    """Rows whose entries of G are far below the product of the two rows' largest magnitudes."""
+    A = rng.standard_normal((rows, K))
+    if kind == "spikes":  # one large element a row, in different columns
+        A[np.arange(rows), rng.permutation(max(rows, K))[:rows] % K] *= 1e9
+    elif kind == "one":  # one such row
+        A[rows // 2, K // 2] *= 1e9
+    elif kind == "spread":  # elements of any magnitude
+        A *= 10.0 ** rng.uniform(-12, 12, (rows, K))
+    elif kind == "supports":  # a few nonzero columns a row, and a tiny one that all rows share
+        A *= rng.random((rows, K)) < 0.1
+        A[:, K // 3] = 1e-9 * (1.0 + rng.random(rows))
+    elif kind == "groups":  # groups of columns in units of their own, each row at home in one
+        unit = 10.0 ** rng.uniform(-8, 8, 4)
+        home = rng.integers(0, 4, rows)
+        A *= np.where(np.arange(K)[None] % 4 == home[:, None], unit[home][:, None], 1e-10)
+    return A
+
+
+@pytest.mark.parametrize("kind", ["even", "spikes", "one", "spread", "supports", "groups"])
+@pytest.mark.parametrize("rows,K", [(16, 180), (17, 31), (32, 4000), (33, 180), (64, 5003),
+                                    (100, 16), (128, 180), (20, 30011),
+                                    (40, 30011), (128, 30011), (200, 700), (300, 5003)])
+def test_fp64_gram_entry_by_entry(ctx, rows, K, kind):
+    """G = Y Y^T of FP64 rows, every entry against its own terms: S_ij = sum |y_ik y_jk|.  A segment
+    of n <= 192 columns is within 1.2 x 128 or (n > 128) n 2^-53 S; the sums of a CTA's
+    segments, of the at most 152 partials and the last rounding add one 2^-53 S each; K <= 30011
+    gives a CTA two segments, or (row pairs, K <= 5003) nine on at least four CTAs."""
+    rng = np.random.default_rng(rows * 7 + K)
+    A = _uneven(rng, rows, K, kind)
+    v = rng.standard_normal(K)
+    G = torch.empty(rows, rows, dtype=torch.float64, device="cuda")
+    p = torch.empty(rows, dtype=torch.float64, device="cuda")
+    idx = rng.permutation(rows).astype(np.int32)
+    ctx.ca_gram_project(_dev(A), _dev(idx), _dev(v), G, p, prec="f64")
+    cols = np.sort(rng.permutation(rows)[:24])  # (extended precision is slow: 24 columns of G)
+    Y = A[idx].astype(np.longdouble)
+    S = np.abs(Y) @ np.abs(Y[cols]).T
+    g = G.cpu().numpy()
+    assert (g == g.T).all()
+    assert (np.abs(g[:, cols] - Y @ Y[cols].T) <= 2.0 ** -53 * (198 + 9 + 152 + 1) * S).all()
+
+
+@pytest.mark.parametrize("rows", [20, 70])
+def test_fp64_gram_zero_rows_and_infinities(ctx, rows):
+    """A row of zeros loses nothing to digits, but times an infinity or a NaN it is a NaN."""
+    rng = np.random.default_rng(4)
+    A = rng.standard_normal((rows, 700))
+    A[2], A[3, 100:400] = 0.0, 0.0
+    A[5, 120], A[7, 20], A[9] = -np.inf, np.nan, 1e-310
+    G = torch.empty(rows, rows, dtype=torch.float64, device="cuda")
+    p = torch.empty(rows, dtype=torch.float64, device="cuda")
+    ctx.ca_gram_project(_dev(A), torch.arange(rows, dtype=torch.int32, device="cuda"),
+                        _dev(rng.standard_normal(700)), G, p, prec="f64")
+    g = G.cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        ref = (A[:, None] * A[None]).sum(-1)
+        S = (np.abs(A[:, None]) * np.abs(A[None])).sum(-1)
+    assert (np.isnan(g) == np.isnan(ref)).all() and (np.isinf(g) == np.isinf(ref)).all()
+    fin = np.isfinite(ref)
+    # (numpy's pairwise sum and ours; products with the small row round to 2^-1075 each)
+    assert (np.abs(g[fin] - ref[fin]) <= 2.0 ** -53 * 700 * S[fin] + 700 * 2.0 ** -1074).all()
