@@ -289,10 +289,11 @@ __device__ __forceinline__ bool gram_columns(DigitGram<8 * RQ>& dg, const double
 // the projection partials on v.  PAIR (more than 128 rows): blockIdx.y is a pair
 // of groups of 64 rows, whose 128-row Gram the CTA forms and of which it stores
 // the off-diagonal block, the diagonal block of a group being stored with the
-// next group (the last one's with the one before).  (ng - 1) ng / 2
-// tiles, of which a group pair is one; 256 x 24001 0.36 ms, 512 x 24001 1.55 ms
-// (1.80 and 6.42 ms as FP64 FMAs in 64 x 64 tiles), error 2.1e-16 K against
-// 4.9e-15 K at 1000 columns.
+// next group (the last one's with the first: both with the last pair made that
+// one the last to end).  (ng - 1) ng / 2 tiles, of which a group pair is one;
+// normal numbers 256 x 24001 0.33 ms, 512 x 24001 1.47 ms (1.80 and 6.42 ms as
+// FP64 FMAs in 64 x 64 tiles); four fifths zeros 1.80 and 8.7 ms; elements of 24
+// decades, every entry off the diagonal by FP64, 2.31 and 11.1 ms.
 template <int RQ, bool PAIR>
 __global__ void __launch_bounds__(kT + kMma, 1)
 k_gram64(Persist64Args a, unsigned* __restrict__ err) {
@@ -313,7 +314,7 @@ k_gram64(Persist64Args a, unsigned* __restrict__ err) {
     dg.lo = 64 * ga;
     dg.hi = 64 * (gb - 1);
     dg.own_lo = gb == ga + 1;
-    dg.own_hi = dg.own_lo && gb == ng - 1;
+    dg.own_hi = ga == 0 && gb == ng - 1;
   }
   const bool digits = sb > kSmallSB;
   if (digits) digits_begin<RQ>(dg, sh, smem_d);
@@ -333,9 +334,18 @@ k_gram64(Persist64Args a, unsigned* __restrict__ err) {
   main_sync();
   gram_columns<RQ, PAIR>(dg, a.A, soff, sb, c0, c1, smem_d, a.part + (long long)c * sbp * sbp, sbp,
                          err, true);
-  if (!PAIR || dg.own_lo)  // (the last pair's groups follow each other)
-    update_project<RQ>(a, soff, soff, nullptr, !PAIR || dg.own_hi ? sb : 64, 0, c0, c1, ured,
-                       a.ppart + (long long)c * sbp + 64 * ga);
+  double* pp = a.ppart + (long long)c * sbp;
+  if constexpr (PAIR) {
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      if (!(h == 0 ? dg.own_lo : dg.own_hi)) continue;
+      update_project<RQ>(a, soff + 64 * h, soff, nullptr, h == 0 ? 64 : sb - 64, 0, c0, c1, ured,
+                         pp + 64 * (h == 0 ? ga : gb));
+      main_sync();  // (ured is free again)
+    }
+  } else {
+    update_project<RQ>(a, soff, soff, nullptr, sb, 0, c0, c1, ured, pp);
+  }
   if (digits) {
     dg.stop();
     digits_end<RQ>(dg);
