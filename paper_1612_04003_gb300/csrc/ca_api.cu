@@ -449,10 +449,7 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
     const int sb = sk * b;
     const int* idx = idx_all + (size_t)s * k * b;
     double* delta = delta2[k & 1];
-    // (a persistent FP64 launch applies a pending update itself)
-    const bool fuse_k = fuse || (persist64 && sk == s && k + 1 < n_outer &&
-                                 (long long)s * (k + 2) <= H && !boundary_after(k));
-    if (pending && (!fuse_k || due(k - 1))) {
+    if (pending && (!fuse || due(k - 1))) {
       CA_TRY(update_alone());                                   // a5 of step k-1 (clears after_rc)
       if (due(k - 1)) CA_TRY(launch_recompute(ctx, pb, pb.v, pb.y0, pb.c0, pb.c1));  // a6
     }
@@ -470,8 +467,6 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
       pa.sb = sb;
       pa.k0 = k;
       pa.npass = (int)(k1 - k);
-      pa.prev_idx = pending ? prev_idx : nullptr;
-      pa.prev_sb = pending ? prev_sb : 0;
       pa.delta2[0] = delta2[0];
       pa.delta2[1] = delta2[1];
       pa.v = pb.v;
@@ -492,7 +487,6 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
       if (e == (int)cudaErrorCooperativeLaunchTooLarge || e == (int)cudaErrorInvalidConfiguration) {
         (void)cudaGetLastError();  // not resident at once here: the launches per step instead
         persist64 = false;
-        if (pending) CA_TRY(update_alone());
       } else if (e != 0) {
         return cuda_fail((cudaError_t)e, __LINE__);
       } else {

@@ -147,10 +147,8 @@ struct Persist64Args {
   int sb;                // s * b of every step of the launch
   long long k0;
   int npass;
-  const int* prev_idx;   // rows of step k0 - 1, update pending (prev_sb = 0: none)
-  int prev_sb;
   double* delta2[2];     // Delta of step k in delta2[k & 1]
-  double* v;             // K, updated in place
+  double* v;             // K, updated in place (the last step's update is left to the caller)
   double cU;
   double* part;          // 2 x P x sbp^2 Gram partials (transposed), by step parity
   double* ppart;         // P x sbp projection partials

@@ -533,12 +533,11 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   };
 
   row_offsets(a.idx_all + a.k0 * sb, sb, a.N, a.lda, soff[0], err);
-  if (a.prev_sb > 0) row_offsets(a.prev_idx, a.prev_sb, a.N, a.lda, soff[1], err);
   main_sync();
   gram(0, soff[0]);
   for (int p = 0; p < npass && ok; ++p) {
     const long long k = a.k0 + p;
-    const int psb = p == 0 ? a.prev_sb : sb;
+    const int psb = p == 0 ? 0 : sb;  // (no update is pending where a run starts)
     if (p > 0) ok = main_wait(a.cnt + Cnt::D, (unsigned)p, err, ok);
     if (!ok) break;
     if (psb > 0) {
