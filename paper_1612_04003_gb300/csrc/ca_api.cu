@@ -307,16 +307,15 @@ void launch_solve(ca_ctx* ctx, const double* R, const float2* Rs, const double* 
 
 // Whether launch_reduce_solve runs a4 as the single reduce + chain launch.
 bool uses_reduce_chain(const GramPlan& g, const SolveArgs& sa, bool f64solve) {
-  return g.tc && sa.s_cur > 0 && fast_solve(sa.b, sa.sb, f64solve) && sa.b <= 16;
+  return g.tc && fast_solve(sa.b, sa.sb, f64solve) && sa.b <= 16;
 }
 
 // a4 entry: reduce the partials to R, p and invert the diagonal blocks (in
-// the reduce launch for b <= 16, by k_factor otherwise), then (s_cur > 0) the
-// inner solves.
+// the reduce launch for b <= 16, by k_factor otherwise), then the inner solves.
 int launch_reduce_solve(ca_ctx* ctx, const GramPlan& g, const void* part, const double* ppart,
                         double* R, float2* Rs, double* pvec, float2* Ginv, const SolveArgs& sa,
                         bool f64solve = false) {
-  const bool fast = sa.s_cur > 0 && fast_solve(sa.b, sa.sb, f64solve);
+  const bool fast = fast_solve(sa.b, sa.sb, f64solve);
   const long long entries = (long long)sa.sb * (sa.sb + 1) / 2 + sa.sb;
   const long long passes = (entries + 31) / 32;
   const int G = (int)std::max(1LL, std::min<long long>(passes, 8LL * ctx->num_sms));
@@ -344,12 +343,10 @@ int launch_reduce_solve(ca_ctx* ctx, const GramPlan& g, const void* part, const 
     ctx->prof.kernel_launches += 1;
   }
   prof_mark(ctx, PC_SOLVE);
-  if (sa.s_cur > 0) {
-    prof_mark(ctx, PC_CHAIN);
-    launch_solve(ctx, R, Rs, pvec, Ginv, sa, f64solve);
-    prof_mark(ctx, PC_CHAIN);
-    ctx->prof.kernel_launches += 1;
-  }
+  prof_mark(ctx, PC_CHAIN);
+  launch_solve(ctx, R, Rs, pvec, Ginv, sa, f64solve);
+  prof_mark(ctx, PC_CHAIN);
+  ctx->prof.kernel_launches += 1;
   return cuda_status(cudaGetLastError());
 }
 
