@@ -152,10 +152,9 @@ k_gram_tc(const float* __restrict__ A, long long lda, long long N, long long K,
     }
   };
 
-  // Shared memory is not cleared: rows >= sb of a tile (never loaded) only
-  // reach accumulator rows / columns >= sb and projection entries >= sb,
-  // which are never stored or never read; the K tail past the last column is
-  // zero-filled by the copies (row-major) or zero in the panels.
+  // Shared memory is not cleared: rows >= sb of a tile are zero-filled by the
+  // copies, and so is the K tail past the last column (row-major; zero in the
+  // panels).
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {  // (3xTF32 uses the first MS pairs)
       mbar_init(&full[s], kLoaderWarps);  // one arrival per loader warp

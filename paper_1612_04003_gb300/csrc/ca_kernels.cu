@@ -577,7 +577,7 @@ k_reduce_chain(const PT* __restrict__ part, const double* __restrict__ ppart, in
                     nred);
     __syncthreads();
     if (threadIdx.x == 0) {
-      __threadfence();  // this CTA's R, Rs, p, Ginv before its count
+      __threadfence();  // this CTA's Rs, p, Ginv before its count
       atomicAdd(ticket, 1u);
     }
     return;
@@ -622,7 +622,7 @@ k_reduce_chain_batch(const RedInst* __restrict__ insts, const RedRole* __restric
                        ri.sa, err, ro.cta, ro.ncta);
     __syncthreads();
     if (threadIdx.x == 0) {
-      __threadfence();  // this CTA's R, Rs, p, Ginv before its count
+      __threadfence();  // this CTA's Rs, p, Ginv before its count
       atomicAdd(tickets + ro.inst, 1u);
     }
     return;
@@ -1749,9 +1749,6 @@ void launch_factor(cudaStream_t st, const double* R, const SolveArgs& sa, float2
                    unsigned* err) {
   launch_programmatic_t(k_factor, (unsigned)sa.s_cur, 1024u, 0, st, R, sa, Ginv, err);
 }
-
-// Rs[j][i] = FP32 split of cG R[i][j] (transposed, as k_reduce writes it) for
-// the lower-triangle entries outside the diagonal blocks (the sparse path
 
 int launch_update_dense(bool f64, cudaStream_t st, const void* A, long long lda, long long N,
                         long long K, const int* idx, int sb, const double* delta, double cU,

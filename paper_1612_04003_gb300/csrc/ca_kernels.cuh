@@ -225,7 +225,7 @@ void launch_csr_dense(cudaStream_t st, const ca_csr_dev& csr, long long nrows, l
                       const int* feats, int nf, int* dmap, int fd, float* Xd);
 // The diagonal and projections of the sampled rows (k_csr_rows), and the
 // strict lower triangle of their Gram: the split (k_dgram + k_sgram) or,
-// split = false, one warp per pair (k_csr_gram_pairs, sb <= 128).
+// split = false, one warp per pair (k_csr_gram_pairs, sb < 32).
 void launch_csr_rows(cudaStream_t st, const ca_csr_dev& csr, const int* idx, long long nrows,
                      long long ncols, int sb, int ldr, const double* w, double* G, double* pvec,
                      unsigned* err);
