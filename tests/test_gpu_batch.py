@@ -217,3 +217,18 @@ def test_batch_certified_stop_matches_solo(ca_ctx):
     assert _rel(wb, w) < TOL32
     for p, q in zip(others, res[1:]):
         assert q["h_done"] == p["H"] and q["bound"] is None
+
+
+def test_more_rounds_than_a_segment(ca_ctx):
+    """More than 64 rounds of the same problems: a segment's descriptors and counters are used again
+    by the next one (a change of the set of problems starts a segment too)."""
+    ca, ctx, _ = ca_ctx
+    probs = _problems([("primal", 96, 1000, 4, 2, 301, 1e-2), ("dual", 640, 200, 8, 2, 282, 1e-1),
+                       ("primal", 256, 4096, 8, 2, 150, 1e-3)])
+    res = ctx.ca_batch_solve(probs)
+    for p, r in zip(probs, res):
+        assert r["status"] == ca.CA_OK and r["h_done"] == p["H"]
+        x_ref, aux_ref = _oracle(p)
+        assert _rel(p["x"], x_ref) < TOL32 and _rel(p["aux"], aux_ref) < TOL32
+        xs, auxs = _solo(ctx, p)
+        assert _rel(p["x"], xs) < TOL32 and _rel(p["aux"], auxs) < TOL32
