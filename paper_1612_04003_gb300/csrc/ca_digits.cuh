@@ -13,25 +13,27 @@
 // rounded in FP32 past 2^24; higher levels are left out.  The levels are put
 // together in 64-bit integers and converted once.
 //
-// What that loses is relative to M_i M_j, not to the entry: at most (1.27 n + 1)
-// 2^-55 M_i M_j, of which n 2^-55 is the elements' rounding.  FP64 FMAs lose at most
-// n 2^-53 S with S = sum |y_ik y_jk|, which for uneven rows is far less.  So
-// an entry is formed by digits only where S >= 0.0026 min(n, 128) M_i M_j; it is
-// then within 1.2 max(n, 128) 2^-53 S.  The other entries are summed in FP64.
-//  - With t the mean of min(|y| / M, 1/8) over a row, in eighths, S >= n M_i M_j (t_i +
-//    t_j - 1) / 64, as a b >= (a + b - 1/8) / 8 for a, b <= 1/8, and S >= n M^2 t^2 /
-//    64 on the diagonal: the two smallest t of a segment, summed with the first
-//    conversion, say whether all its entries have that.  A row of normal numbers
-//    has t = 0.8 (largest magnitude 2 to 4 times the deviation) or 0.63 (4 to 8
-//    times), and 2 x 0.583 suffices: 4 of 9408 segments of 32 x 8190 in 64 steps
-//    were not cleared (128 x 24001 of normal numbers 82 us, as without the test).  A
-//    row of zeros loses nothing.
+// What that loses is relative to M_i M_j, not to the entry: the elements' rounding
+// at most n 2^-56 (l_i + l_j) M_i M_j, l <= 1 the mean of |y| / M over a row, and the
+// rest (0.27 n + 1) 2^-55 M_i M_j (0.02 n up to 160 columns).  FP64 FMAs lose at most n
+// 2^-53 S with S = sum |y_ik y_jk|, which for uneven rows is far less.  So an
+// entry is formed by digits only where S is known to be large enough for it to
+// be within 1.2 max(n, 128) 2^-53 S; the other entries are summed in FP64.
+//  - With t the mean of min(|y| / M, 1/8) over a row, in eighths: l <= t, S >= n M_i M_j
+//    (t_i + t_j - 1) / 64, as a b >= (a + b - 1/8) / 8 for a, b <= 1/8, and S >= n M^2
+//    t^2 / 64 on the diagonal.  So the two smallest t of a segment, summed with the
+//    first conversion, clear all its entries if they add up to 1.07 + 0.1 / n, the
+//    smaller at least 0.3.  A row of normal numbers has t = 0.8 (largest magnitude 2
+//    to 4 times the deviation) or 0.63 (4 to 8 times): with a line at 1.17 four of
+//    the 9408 segments of 32 x 8190 in 64 steps were not cleared, 40 us of 1.13 ms;
+//    with this one next to none.  A row of zeros loses nothing.
 //  - Any other segment starts again with one more product of the same form, of the
 //    elements' leading seven bits rounded down (exact integers: S' 2^-14 M_i M_j <=
-//    S), and an entry goes by its S' (128 x 24001: exponentially distributed 108
-//    us; four fifths zeros 413; elements of 24 decades, every entry by FP64, 498,
-//    where FP64 tiles of 64 x 64 took 557).  Rows with an infinity, a NaN or a magnitude
-//    outside 2^-480 .. 2^490 fail with every other row.
+//    S), and an entry goes by S' >= 42 min(n, 128), that is S >= 0.0026 min(n, 128) M_i M_j
+//    (128 x 24001: exponentially distributed 108 us; four fifths zeros 413;
+//    elements of 24 decades, every entry by FP64, 498, where FP64 tiles of 64 x 64
+//    took 557; normal numbers, all cleared, 82).  Rows with an infinity, a NaN or a
+//    magnitude outside 2^-480 .. 2^490 fail with every other row.
 //
 // Why: the FP64 pipe does two FMAs a clock and SM (1.25 TFLOP/s).  The 34
 // digit products of a 128-row tile and 32 columns take ~4,400 cycles of the
@@ -44,6 +46,15 @@ namespace {
 
 constexpr int kSeg = 192;  // columns whose level sums stay exact in FP32
 constexpr int kDigits = 7;
+
+// threadIdx.x as a value of its own: what is derived from it is formed anew and
+// not kept over the steps of a solve in registers that then spill (2003 x 24001,
+// s b = 128: 1.90 ms a solve, so 1.87).
+__device__ __forceinline__ int fresh_tid() {
+  int t = (int)threadIdx.x;
+  asm volatile("" : "+r"(t));
+  return t;
+}
 
 // Named barrier 1 over the eight warps that form a Gram partial (a CTA may have
 // others), and the same with a vote.
@@ -172,6 +183,7 @@ struct DigitGram {
   int* nlist;           // entries to sum in FP64
   uint32_t* tmin;       // [16] each warp's two smallest t n
   int64_t* diag;        // [SBP] (SBP = 128)
+  int tid0 = 0;         // fresh_tid() of the segment
   uint32_t gt = 0;      // stages so far (buffers and phases run on)
   uint32_t ph = 0;      // passes so far
   // gram<true>: two groups of 64 rows of a larger Gram, at rows and columns lo
@@ -198,7 +210,7 @@ struct DigitGram {
   // each load makes branches that wait for one load after another)
   __device__ __forceinline__ void load(const double* __restrict__ A, const Rows& rw, long long k,
                                        long long k1, double (&x)[kRows][2]) const {
-    const long long kk = k + 2 * (threadIdx.x & 15);
+    const long long kk = k + 2 * (tid0 & 15);
     const long long ka = min(kk, k1 - 1), kb = min(kk + 1, k1 - 1);
 #pragma unroll
     for (int i = 0; i < kRows; ++i) {
@@ -219,7 +231,7 @@ struct DigitGram {
   template <int ND, bool SUM>
   __device__ __forceinline__ void convert(const Rows& rw, const double (&x)[kRows][2],
                                           unsigned char* buf, uint32_t (&ts)[kRows]) const {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane & 15;
+    const int warp = tid0 >> 5, lane = tid0 & 31, l = lane & 15;
 #pragma unroll
     for (int i = 0; i < kRows; ++i) {
       const int r = 2 * (warp + 8 * i) + (lane >> 4);
@@ -331,13 +343,13 @@ struct DigitGram {
       if (gt >= 2 && ok) ok = mbar_wait_grid(&bars[bi], ((gt >> 1) - 1) & 1, err);
       convert<(L1 - 1 < kDigits ? L1 - 1 : kDigits), SUM>(rw, x, buf, ts);
       load(A, rw, k + 32, k1, x);  // (lands while the MMAs of this stage run)
-      if (threadIdx.x == 0)
+      if (tid0 == 0)
         cmd[bi] = (uint32_t)(L1 == 1 ? 3 : L0 == 6 ? 2 : L1 == 5 ? 1 : 0) | (k == k0 ? kFirst : 0u) |
                   (k + 32 >= k1 ? kLast : 0u) | (k + 16 >= k1 ? kHalf : 0u) | (uint32_t)nb << 8;
       fence_proxy_async_smem();
       tc_fence_before();
       __syncwarp();
-      if ((threadIdx.x & 31) == 0) mbar_arrive(&bars[3 + bi]);
+      if ((tid0 & 31) == 0) mbar_arrive(&bars[3 + bi]);
     }
     return ok;
   }
@@ -351,7 +363,7 @@ struct DigitGram {
   // Whether the two smallest t of the segment's sb rows let every entry be formed
   // by digits (all main warps; ts from the conversion).
   __device__ __forceinline__ bool even(const uint32_t (&ts)[kRows], int sb, uint32_t n) const {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = tid0 >> 5, lane = tid0 & 31;
     constexpr uint32_t kNone = 0x3fffffffu;
     uint32_t t1 = kNone, t2 = kNone;
 #pragma unroll
@@ -376,9 +388,8 @@ struct DigitGram {
     t1 = __reduce_min_sync(0xffffffffu, t2);
     if (__popc(__ballot_sync(0xffffffffu, t2 == t1)) > 1) t2 = t1;
     else t2 = __reduce_min_sync(0xffffffffu, t2 == t1 ? kNone : t2);
-    // t n in units of 2^-20: t1 + t2 >= n + 0.166 min(n, 128) (0.0026 64 = 0.164), t1 >=
-    // 0.41 n (0.41^2 > 0.164)
-    return t1 + t2 >= (n << 20) + 174064u * min(n, 128u) && t1 >= 429917u * n;
+    // t n in units of 2^-20: t1 + t2 >= 1.07 + 0.1 / n, t1 >= 0.3
+    return t1 + t2 >= 1121977u * n + 104858u && t1 >= 314573u * n;
   }
 
   // The passes of a segment whose emax and wt stand, and its entries into part; false,
@@ -388,7 +399,7 @@ struct DigitGram {
   __device__ __forceinline__ bool passes(const double* __restrict__ A, const long long* off, int sb,
                                          long long k0, long long k1, double* __restrict__ part,
                                          int sbp, bool add, unsigned* err, bool& ok) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = tid0, warp = tid >> 5, lane = tid & 31;
     auto at_ = [&](int r) { return PAIR ? r + (r < 64 ? lo : hi) : r; };  // a row's place in part
     Rows rw;
 #pragma unroll
@@ -558,7 +569,8 @@ struct DigitGram {
   __device__ bool gram(const double* __restrict__ A, const long long* off, int sb, long long k0,
                        long long k1, double* __restrict__ part, int sbp, bool add, unsigned* err,
                        bool ok) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    tid0 = fresh_tid();
+    const int warp = tid0 >> 5, lane = tid0 & 31;
     // largest exponent of each row in the segment
     bool plain = false;
     constexpr int RB = 4;  // rows in flight a warp

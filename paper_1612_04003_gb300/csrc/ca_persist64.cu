@@ -152,7 +152,7 @@ template <int RQ>
 __device__ void update_project(const Persist64Args& a, const long long* off, const long long* poff,
                                const double* sdl, int sb, int psb, long long k0, long long k1,
                                double* red, double* __restrict__ pp) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2;
+  const int tid = fresh_tid(), warp = tid >> 5, lane = tid & 31, g = lane >> 2;
   double pacc[RQ], y[RQ], x[RQ], vk;
 #pragma unroll
   for (int q = 0; q < RQ; ++q) pacc[q] = 0.0;
