@@ -83,7 +83,15 @@ typedef enum {
  * the stopping test first rebuilds the maintained vector that way.  The
  * b x b solves (a4) run in double-float by default or in FP64 (ca_solve). */
 typedef enum {
-  CA_GRAM_F64 = 0,        /* FP64 on CUDA cores (any dense X)                   */
+  CA_GRAM_F64 = 0,        /* FP64 (any dense X).  FP32 X, and FP64 X with up to 16
+                           * rows a step: FMAs on CUDA cores.  FP64 X with
+                           * more rows: products of base-256 digits on the
+                           * tensor cores, each element rounded to 2^-55 of
+                           * its row's largest magnitude among up to 192
+                           * columns, wherever that is as accurate as FP64
+                           * sums (else those): the n = up to 192 products of
+                           * an entry are summed to within 1.2 max(n, 128)
+                           * 2^-53 of the sum of their magnitudes             */
   CA_GRAM_FP32_EXACT = 1, /* FP32 X: 3xTF32 split products on tcgen05, FP32 acc. */
   CA_GRAM_TF32 = 2,       /* FP32 X: TF32 tcgen05 products, FP32 accumulate     */
   CA_GRAM_BF16X3 = 3,     /* FP32 X: x = b0 + b1 in BF16, b0 b0^T + b0 b1^T +
@@ -282,14 +290,17 @@ int ca_bcd_release_scratch(ca_ctx* ctx);
 int ca_gram_project(ca_ctx* ctx, int xfmt, int prec, const void* A, long long N, long long K,
                     long long ld, const int* idx, int sb, const double* v, double* G, double* p);
 
-/* Steps a2+a3 as ca_gram_project computes them (the same kernels; the split-K
- * partials are summed in a different order, so the results agree to
- * rounding: within 1e-12 relative on FP64 A, and within the Gram mode's
- * product bound on FP32 A), for callers that must not allocate device memory
- * (the paper has no counterpart: this is an interface convenience).  Such callers include code running while a host
- * framework owns every device allocation through its own pool, code on a
- * latency-critical path where an allocation's implicit synchronisation is not
- * acceptable, and code that may only enqueue work on a stream it was given.
+/* Steps a2+a3 as ca_gram_project computes them, for callers that must not
+ * allocate device memory (the paper has no counterpart: this is an interface
+ * convenience).  FP32 A: the same kernels, the split-K partials summed in a
+ * different order, so the results agree within the Gram mode's product bound
+ * (CA_GRAM_F64: to FP64 rounding).  FP64 A: FP64 FMAs on CUDA cores whatever sb,
+ * where ca_gram_project takes digit products from 17 rows on; an entry of the
+ * two differs by at most (K + 400) 2^-53 sum_k |y_ik y_jk|.  Such callers
+ * include code running while a host framework owns every device allocation
+ * through its own pool, code on a latency-critical path where an allocation's
+ * implicit synchronisation is not acceptable, and code that may only enqueue
+ * work on a stream it was given.
  * No context is needed and nothing is allocated: the scratch is one fixed
  * device array inside the library (6.5 MiB, held on every GPU that loads the
  * library until the process exits).
@@ -327,19 +338,22 @@ const char* ca_last_error(ca_ctx* ctx);
 /* Name of a status code (static string). */
 const char* ca_status_str(int status);
 
-/* Tuning of the dense tensor-core solves on ctx (kept until changed).
+/* Tuning of the dense solves on ctx (kept until changed).
  *   CA_TUNE_PERSISTENT  1 (default): a run of full outer steps between two
  *       host decisions (a check of the stopping test, a due recomputation,
  *       the short last step) runs as one persistent cooperative launch when
- *       the solve fits it (FP32 X in 32-column panels, BF16x3 or scaled-FP16
- *       Gram, s*b <= 128, b <= 8, CA_SOLVE_DF, at least s + 1 Gram CTAs):
+ *       the solve fits it.  FP32 X in 32-column panels, BF16x3 or scaled-FP16
+ *       Gram, s*b <= 128, b <= 8, CA_SOLVE_DF, at least s + 1 Gram CTAs:
  *       the s unrolled solves of step k (eq. "recur", Algorithms 2 and 4)
  *       then run while the Gram pass of step k+1 streams its rows, and that
  *       pass corrects its projection by the cross Gram of the two steps'
- *       rows (the same sums in exact arithmetic).  0: one Gram launch and
- *       one solve launch per outer step.
- *   CA_TUNE_OVERLAP  share in [0, 1] of each Gram CTA's columns streamed
- *       before the previous step's solve is known (default 0.4; 0: none).
+ *       rows (the same sums in exact arithmetic).  FP64 X, s*b <= 128, b <=
+ *       16, CA_SOLVE_DF: the Gram of step k+1 is formed while the solves of
+ *       step k run, the projection after them.  0: a few launches per outer
+ *       step (FP32 X: one Gram launch and one solve launch).
+ *   CA_TUNE_OVERLAP  FP32 X: share in [0, 1] of each Gram CTA's columns
+ *       streamed before the previous step's solve is known (default 0.4; 0:
+ *       none).
  * Errors: CA_ERR_ARG (NULL context, unknown key, value out of range). */
 #define CA_TUNE_PERSISTENT 1
 #define CA_TUNE_OVERLAP 2

@@ -69,3 +69,26 @@ def test_noalloc_rejects_sizes_beyond_its_scratch(setup):
     with pytest.raises(ca.CaError) as e:
         ca.gram_project_noalloc(A, idx, v, G, p, prec="tf32")
     assert e.value.status == ca.CA_ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("rows", [16, 40, 128])
+def test_noalloc_matches_on_uneven_fp64_rows(setup, rows):
+    """FP64 A whose rows have one element far above the rest, each in a column of its own: the two
+    entries sum the same products, each to FP64 rounding (at most K additions here, 198 + 9 + 152 + 1
+    of 2^-53 sum |y_ik y_jk| there), so an entry differs by at most (K + 400) 2^-53 of that sum."""
+    ca, ctx = setup
+    rng = np.random.default_rng(rows)
+    K = 5003
+    A = rng.standard_normal((rows, K))
+    A[np.arange(rows), rng.permutation(K)[:rows]] *= 1e9
+    Ad, v = torch.as_tensor(A).cuda(), torch.as_tensor(rng.standard_normal(K)).cuda()
+    idx = torch.arange(rows, dtype=torch.int32, device="cuda")
+    G = [torch.empty((rows, rows), dtype=torch.float64, device="cuda") for _ in range(2)]
+    p = [torch.empty(rows, dtype=torch.float64, device="cuda") for _ in range(2)]
+    ctx.ca_gram_project(Ad, idx, v, G[0], p[0], prec="f64")
+    ca.gram_project_noalloc(Ad, idx, v, G[1], p[1], prec="f64")
+    torch.cuda.synchronize()
+    S = np.abs(A) @ np.abs(A).T
+    assert (np.abs((G[0] - G[1]).cpu().numpy()) <= (K + 400) * 2.0 ** -53 * S).all()
+    Sp = np.abs(A) @ np.abs(v.cpu().numpy())
+    assert (np.abs((p[0] - p[1]).cpu().numpy()) <= (2 * K + 400) * 2.0 ** -53 * Sp).all()
