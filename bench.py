@@ -359,8 +359,7 @@ def batch_study(ctx, stream, count=24):
     """The batched solves (ca_batch_solve) on uneven problems shaped like the
     served-batch workload, scaled to a short run (d 256-2048, n 4096-32768):
     the same problems one after another (each its own solve), in shared
-    launches (with and without CA_BATCH_GRAPH), and with the depth chosen by
-    measured cost.  Block updates per second of the whole set."""
+    launches, and with the depth chosen by measured cost.  Block updates per second of the whole set."""
     import torch
     probs = _uneven_problems(count, 5, (256, 2048), (4096, 32768))
     total_h = sum(p["kw"]["H"] for p in probs)
@@ -392,14 +391,13 @@ def batch_study(ctx, stream, count=24):
                        "s b = 64, H = min(2048, 4 N / b), BF16x3 Gram"}
     t = timed(seq)
     out["one_after_another"] = {"seconds": t, "block_updates_per_s": total_h / t}
-    for name, graph in (("shared_launches", False), ("shared_launches_graph", True)):
-        t = timed(lambda: ctx.ca_batch_solve([fresh(p) for p in probs], graph=graph))
-        out[name] = {"seconds": t, "block_updates_per_s": total_h / t}
+    t = timed(lambda: ctx.ca_batch_solve([fresh(p) for p in probs]))
+    out["shared_launches"] = {"seconds": t, "block_updates_per_s": total_h / t}
     tuned = [dict(fresh(p), s=0) for p in probs]
     t = timed(lambda: ctx.ca_batch_solve([dict(q, x=torch.zeros_like(q["x"]),
                                                aux=torch.zeros_like(q["aux"])) for q in tuned]))
     res = ctx.ca_batch_solve(tuned)
-    out["shared_launches_graph_depth_by_cost"] = {
+    out["shared_launches_depth_by_cost"] = {
         "seconds": t, "block_updates_per_s": total_h / t,
         "rows_per_step_chosen": sorted({r["s"] * p["kw"]["b"] for r, p in zip(res, probs)})}
     del probs

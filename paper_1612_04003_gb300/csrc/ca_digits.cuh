@@ -30,8 +30,8 @@
 //  - Any other segment starts again with one more product of the same form, of the
 //    elements' leading seven bits rounded down (exact integers: S' 2^-14 M_i M_j <=
 //    S), and an entry goes by S' >= 42 min(n, 128), that is S >= 0.0026 min(n, 128) M_i M_j
-//    (128 x 24001: exponentially distributed 108 us; four fifths zeros 413;
-//    elements of 24 decades, every entry by FP64, 498, where FP64 tiles of 64 x 64
+//    (128 x 24001: exponentially distributed 107 us; four fifths zeros 416;
+//    elements of 24 decades, next to every entry by FP64, 500, where FP64 tiles of 64 x 64
 //    took 557; normal numbers, all cleared, 82).  Rows with an infinity, a NaN or a
 //    magnitude outside 2^-480 .. 2^490 fail with every other row.
 //
@@ -548,8 +548,8 @@ struct DigitGram {
     }
     return true;
   }
-  // (a function of its own, on a copy: inlined, with its test in the other
-  // segments' loops, X^T 1500 x 8190, s b = 32, took 1.15 ms, so 1.13)
+  // (a function of its own, on a copy: inlined, its registers cost the loops of
+  // the other segments 20 us of 1.1 ms, X^T 1500 x 8190, s b = 32)
   struct After {
     uint32_t gt, ph;
     bool ok;

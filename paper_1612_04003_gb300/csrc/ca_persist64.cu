@@ -24,8 +24,8 @@
 // Bound by latency at few columns a CTA, by the FP64 conversions of the digits
 // and FP64 projections at many.  Against four launches a step and a Gram tile
 // of 64 x 64 FP64 products whatever s b (ms a solve): X 64 x 1024, b = 4, 200
-// solves: s = 1 1.80 against 11.7 (9 us a step), s = 4 0.64 against 3.13 (13
-// us); X^T 1500 x 8190, b = 8, s = 4: 1.14 against 6.84 (18 us); 2003 x 24001,
+// solves: s = 1 1.75 against 11.7 (9 us a step), s = 4 0.64 against 3.13 (13
+// us); X^T 1500 x 8190, b = 8, s = 4: 1.10 against 6.84 (17 us); 2003 x 24001,
 // b = 16, s = 8: 1.89 against 10.2 (70 us a step between recomputations).
 #include <algorithm>
 #include <atomic>
