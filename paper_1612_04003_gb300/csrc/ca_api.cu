@@ -12,6 +12,7 @@
 #include "ca_check.h"
 #include "ca_internal.h"
 #include "ca_kernels.cuh"
+#include "ca_steps_plan.h"
 
 namespace caint {
 
@@ -451,8 +452,7 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
       if (due(k - 1)) CA_TRY(launch_recompute(ctx, pb, pb.v, pb.y0, pb.c0, pb.c1));  // a6
     }
     long long k1 = k + 1;  // end of the run that starts at k
-    if ((persist_ok || persist64) && sk == s)
-      while (k1 < n_outer && (long long)s * (k1 + 1) <= H && !boundary_after(k1 - 1)) ++k1;
+    if ((persist_ok || persist64) && sk == s) k1 = casteps::run_end(k, s, H, boundary_after);
     bool persisted = false;
     if (persist64 && sk == s && k1 - k >= 2) {
       Persist64Args pa{};
@@ -496,6 +496,7 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
         prev_delta = delta2[k & 1];
       }
     } else if (persist_ok && sk == s && k1 - k >= 2) {
+      if (pending) CA_TRY(update_alone());  // (a run that ended at kMaxRun steps)
       PersistArgs pa{};
       pa.A = static_cast<const float*>(pb.A);
       pa.N = pb.N;

@@ -147,3 +147,17 @@ def test_tuning_refuses_bad_values(ctx):
         with pytest.raises(ca.CaError) as e:
             ctx.ca_set_tuning(**kw)
         assert e.value.status == ca.CA_ERR_ARG
+
+
+def test_persistent_more_steps_than_a_launch(ctx, dual):
+    """65536 outer steps go to one launch; the next one starts after the update of its last step."""
+    X32, y = dual
+    kw = dict(b=1, s=1, H=65536 + 6, seed=3)
+    ctx.ca_set_tuning(persistent=True, overlap=0.4)
+    a = torch.zeros(512, dtype=torch.float64, device="cuda")
+    w = torch.zeros(65536, dtype=torch.float64, device="cuda")
+    XT, yd = _dev(X32.T), _dev(y)
+    n = _launches(ctx, lambda: ctx.ca_bdcd_solve(XT, yd, a, w, lam=1e-2, prec="bf16x3", **kw))
+    assert n < 20
+    a_ref, w_ref = oracle.ca_bdcd(X32.astype(np.float64), y, 1e-2, **kw)
+    assert _rel(a, a_ref) < TOL32 and _rel(w, w_ref) < TOL32

@@ -208,3 +208,21 @@ def test_fp64_gram_zero_rows_and_infinities(ctx, rows):
     fin = np.isfinite(ref)
     # (numpy's pairwise sum and ours; products with the small row round to 2^-1075 each)
     assert (np.abs(g[fin] - ref[fin]) <= 2.0 ** -53 * 700 * S[fin] + 700 * 2.0 ** -1074).all()
+
+
+@pytest.mark.parametrize("method,d,n,b,s", [("primal", 6, 70, 1, 1), ("dual", 40, 9, 2, 1)])
+def test_more_steps_than_a_launch(ctx, method, d, n, b, s):
+    """65536 steps go to one launch; the update of its last one is applied before the next launch."""
+    p = synth.tiny_primal(d=d, n=n, seed=2)
+    lam, H = 1e-1, 65536 * s + 5
+    x = torch.zeros(d if method == "primal" else n, dtype=torch.float64, device="cuda")
+    aux = torch.zeros(n if method == "primal" else d, dtype=torch.float64, device="cuda")
+    kw = dict(b=b, s=s, H=H, seed=3)
+    if method == "primal":
+        ctx.ca_bcd_solve(_dev(p.X), _dev(p.y), x, aux, lam=lam, prec="f64", **kw)
+        ref = oracle.ca_bcd(p.X, p.y, lam, **kw)
+    else:
+        ctx.ca_bdcd_solve(_dev(p.X.T), _dev(p.y), x, aux, lam=lam, prec="f64", **kw)
+        ref = oracle.ca_bdcd(p.X, p.y, lam, **kw)
+    assert _rel(x.cpu().numpy(), np.asarray(ref[0])) < 1e-10
+    assert _rel(aux.cpu().numpy(), np.asarray(ref[1])) < 1e-10
