@@ -372,7 +372,7 @@ int run_dense(ca_ctx* ctx, const DenseProblem& pb, const ca_opts* o, int* idx_al
   // FP64 X: runs of full steps go to one persistent launch (ca_persist64.cu)
   // of P64 column CTAs, with two sets of partials
   const int P64 = pb.xfmt == CA_DENSE_F64 && !f64solve
-                      ? persist64_columns(b, sbm / b, K, ctx->num_sms) : 0;
+                      ? casteps::persist64_columns(b, sbm / b, K, ctx->num_sms) : 0;
   bool persist64 = ctx->persist && P64 > 0;
   const int Pmax = persist64 ? std::max(P, 2 * P64) : P;
   void* part = g.tc ? (void*)cv.take<float>((size_t)P * sbp * sbp)

@@ -164,9 +164,7 @@ int gram64_splits(int sb, long long K, int num_sms);
 int launch_gram64(const double* A, long long lda, long long N, long long K, const int* idx, int sb,
                   const double* v, int P, int sbp, double* part, double* ppart, unsigned* err,
                   cudaStream_t st);
-// Column CTAs of the persistent launch: 0 where it does not cover the call.
-int persist64_columns(int b, int s, long long K, int num_sms);
-// P = persist64_columns().  Returns a cudaError_t.
+// P = casteps::persist64_columns().  Returns a cudaError_t.
 int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,
                      cudaStream_t st);
 

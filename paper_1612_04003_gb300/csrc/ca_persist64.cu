@@ -33,8 +33,11 @@
 #include "ca_digits.cuh"
 #include "ca_kernels.cuh"
 #include "ca_solve.cuh"
+#include "ca_steps_plan.h"
 
 namespace {
+
+using casteps::kMaxInv;
 
 constexpr int kT = 256;      // main threads of a CTA (the Gram pass, the chain)
 constexpr int kSide = 96;    // side threads of a column CTA (reduction); twelve warps in all
@@ -54,7 +57,6 @@ constexpr int kSmallSB = 16;
 struct Cnt {
   enum { G = 0, E = 2, R = 4, P = 6, Q = 7, D = 8 };
 };
-constexpr int kMaxInv = 16;  // inverse CTAs
 // s b from which the column CTAs' side warps sum p, a row a warp, and not the
 // chain CTA (ms a solve, chain CTA against side warps: 4 rows 1.72 / 1.96, 16
 // rows 0.643 / 0.647, 32 rows 1.157 / 1.096)
@@ -640,13 +642,6 @@ int launch_gram64(const double* A, long long lda, long long N, long long K, cons
   if (sb <= 64) return launch_gram<8>(a, dim3(P), err, st);
   if (sb <= 128) return launch_gram<16>(a, dim3(P), err, st);
   return launch_gram<16, true>(a, dim3(P, gram64_pairs(sb)), err, st);
-}
-
-// Column CTAs of the persistent launch (0: not for this block size, rows of a
-// step or GPU).
-int persist64_columns(int b, int s, long long K, int num_sms) {
-  if (b > 16 || s * b > 128) return 0;
-  return (int)std::max(0LL, std::min<long long>(num_sms - 1 - std::min(s, kMaxInv), (K + 31) / 32));
 }
 
 int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,
