@@ -538,13 +538,14 @@ struct DigitGram {
       });
     }
     tc_fence_before();
-    main_sync();  // the accumulators are read, the list is complete
-    if constexpr (UNEVEN) {
-      if (*nlist > 0) {
-        sum_listed<SBP>(A, off, sb, k0, k1, *nlist, add, dig, part, sbp, PAIR ? lo : 0,
-                        PAIR ? hi : 0);
-        main_sync();  // (the digits' memory, the list and its length are free again)
-      }
+    if constexpr (!UNEVEN) {
+      main_sync();  // the accumulators are read
+    } else if (!main_any(!ok) && *nlist > 0) {
+      // (the list is complete; with a wait given up, digits written late might
+      // have taken its place, and nothing is summed)
+      sum_listed<SBP>(A, off, sb, k0, k1, *nlist, add, dig, part, sbp, PAIR ? lo : 0,
+                      PAIR ? hi : 0);
+      main_sync();  // (the digits' memory, the list and its length are free again)
     }
     return true;
   }
