@@ -24,8 +24,8 @@
 // Bound by latency at few columns a CTA, by the FP64 conversions of the digits
 // and FP64 projections at many.  Against four launches a step and a Gram tile
 // of 64 x 64 FP64 products whatever s b (ms a solve): X 64 x 1024, b = 4, 200
-// solves: s = 1 1.75 against 11.7 (9 us a step), s = 4 0.64 against 3.13 (13
-// us); X^T 1500 x 8190, b = 8, s = 4: 1.10 against 6.84 (17 us); 2003 x 24001,
+// solves: s = 1 1.69 against 11.7 (8 us a step), s = 4 0.62 against 3.13 (12
+// us); X^T 1500 x 8190, b = 8, s = 4: 1.11 against 6.84 (17 us); 2003 x 24001,
 // b = 16, s = 8: 1.89 against 10.2 (70 us a step between recomputations).
 #include <algorithm>
 #include <atomic>
@@ -269,21 +269,21 @@ __device__ __forceinline__ void digits_end(const DigitGram<8 * RQ>& dg) {
   }
 }
 
-// Gram partial of the CTA's columns [c0, c1).
-template <int RQ, bool PAIR = false>
+// Gram partial of the CTA's columns [c0, c1).  DIG: more than kSmallSB rows.
+template <int RQ, bool DIG, bool PAIR = false>
 __device__ __forceinline__ bool gram_columns(DigitGram<8 * RQ>& dg, const double* __restrict__ A,
                                              const long long* off, int sb, long long c0,
                                              long long c1, double* smem_d, double* __restrict__ part,
                                              int sbp, unsigned* err, bool ok) {
-  if (sb <= kSmallSB) {
+  if constexpr (!DIG) {
     gram_small(A, off, sb, c0, c1, smem_d, part, sbp);
-    return ok;
+  } else {
+    // segments of equal length, whole 32-column stages
+    const long long nst = (c1 - c0 + 31) / 32, nseg = (nst + kSeg / 32 - 1) / (kSeg / 32);
+    for (long long g = 0; g < nseg && ok; ++g)
+      ok = dg.template gram<PAIR>(A, off, sb, c0 + nst * g / nseg * 32,
+                                  min(c1, c0 + nst * (g + 1) / nseg * 32), part, sbp, g > 0, err, ok);
   }
-  // segments of equal length, whole 32-column stages
-  const long long nst = (c1 - c0 + 31) / 32, nseg = (nst + kSeg / 32 - 1) / (kSeg / 32);
-  for (long long g = 0; g < nseg && ok; ++g)
-    ok = dg.template gram<PAIR>(A, off, sb, c0 + nst * g / nseg * 32, min(c1, c0 + nst * (g + 1) / nseg * 32), part,
-                 sbp, g > 0, err, ok);
   return ok;
 }
 
@@ -296,7 +296,7 @@ __device__ __forceinline__ bool gram_columns(DigitGram<8 * RQ>& dg, const double
 // normal numbers 256 x 24001 0.33 ms, 512 x 24001 1.47 ms (1.80 and 6.42 ms as
 // FP64 FMAs in 64 x 64 tiles); four fifths zeros 1.80 and 8.7 ms; elements of 24
 // decades, every entry off the diagonal by FP64, 2.31 and 11.1 ms.
-template <int RQ, bool PAIR>
+template <int RQ, bool DIG, bool PAIR>
 __global__ void __launch_bounds__(kT + kMma, 1)
 k_gram64(Persist64Args a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
@@ -318,10 +318,9 @@ k_gram64(Persist64Args a, unsigned* __restrict__ err) {
     dg.own_lo = gb == ga + 1;
     dg.own_hi = ga == 0 && gb == ng - 1;
   }
-  const bool digits = sb > kSmallSB;
-  if (digits) digits_begin<RQ>(dg, sh, smem_d);
+  if constexpr (DIG) digits_begin<RQ>(dg, sh, smem_d);
   if (threadIdx.x >= kT) {
-    if (digits) {
+    if constexpr (DIG) {
       dg.mma_loop(err);
       digits_end<RQ>(dg);
     }
@@ -334,7 +333,7 @@ k_gram64(Persist64Args a, unsigned* __restrict__ err) {
     row_offsets(a.idx_all, sb, a.N, a.lda, soff, err);
   }
   main_sync();
-  gram_columns<RQ, PAIR>(dg, a.A, soff, sb, c0, c1, smem_d, a.part + (long long)c * sbp * sbp, sbp,
+  gram_columns<RQ, DIG, PAIR>(dg, a.A, soff, sb, c0, c1, smem_d, a.part + (long long)c * sbp * sbp, sbp,
                          err, true);
   double* pp = a.ppart + (long long)c * sbp;
   if constexpr (PAIR) {
@@ -348,7 +347,7 @@ k_gram64(Persist64Args a, unsigned* __restrict__ err) {
   } else {
     update_project<RQ>(a, soff, soff, nullptr, sb, 0, c0, c1, ured, pp);
   }
-  if (digits) {
+  if constexpr (DIG) {
     dg.stop();
     digits_end<RQ>(dg);
   }
@@ -392,7 +391,10 @@ __device__ __forceinline__ int entries_a_role(int E, int P) {
   return epr;
 }
 
-template <int BMAX, int DEPTH, int RQ>
+// (DIG false, up to kSmallSB rows: a kernel of its own, whose registers the
+// digits' loops have no part in: X 64 x 1024, s = 1 1.75 -> 1.69 ms, s = 4 0.64 ->
+// 0.62 a solve)
+template <int BMAX, int DEPTH, int RQ, bool DIG>
 __global__ void __launch_bounds__(kT + kMma + kSide, 1)
 k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   extern __shared__ double smem_d[];
@@ -517,10 +519,9 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   }
   __shared__ DigitShared<RQ> sh;
   DigitGram<8 * RQ> dg;
-  const bool digits = sb > kSmallSB;
-  if (digits) digits_begin<RQ>(dg, sh, smem_d);
+  if constexpr (DIG) digits_begin<RQ>(dg, sh, smem_d);
   if (tid >= kT) {
-    if (digits) {
+    if constexpr (DIG) {
       dg.mma_loop(err);
       digits_end<RQ>(dg);
     }
@@ -530,7 +531,7 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
   const long long c0 = nch * c / P * 16, c1 = min(a.K, nch * (c + 1) / P * 16);
   auto gram = [&](int p, const long long* off) {  // the partial of step k0 + p
     double* part = a.part + ((a.k0 + p) & 1) * (long long)P * sq;
-    ok = gram_columns<RQ>(dg, a.A, off, sb, c0, c1, smem_d, part + c * sq, sbp, err, ok);
+    ok = gram_columns<RQ, DIG>(dg, a.A, off, sb, c0, c1, smem_d, part + c * sq, sbp, err, ok);
     main_count(a.cnt + Cnt::G + (p & 1));
   };
 
@@ -556,7 +557,7 @@ k_persist64(Persist64Args a, unsigned* __restrict__ err) {
       gram(p + 1, soff[(p + 1) & 1]);
     }
   }
-  if (digits) {
+  if constexpr (DIG) {
     dg.stop();
     digits_end<RQ>(dg);
   }
@@ -598,17 +599,17 @@ int launch64(Kern kern, std::atomic<unsigned long long>& configured, const Persi
   return (int)(e != cudaSuccess ? e : cudaGetLastError());
 }
 
-template <int BMAX, int DEPTH, int RQ>
+template <int BMAX, int DEPTH, int RQ, bool DIG>
 int launch_steps(const Persist64Args& a, int P, size_t chain_smem, unsigned* err, cudaStream_t st) {
   static std::atomic<unsigned long long> configured{0ull};
-  return launch64(k_persist64<BMAX, DEPTH, RQ>, configured, a, P + 1 + std::min(a.sa.s_cur, kMaxInv),
+  return launch64(k_persist64<BMAX, DEPTH, RQ, DIG>, configured, a, P + 1 + std::min(a.sa.s_cur, kMaxInv),
                   std::max(chain_smem, column_smem<RQ>(a.sb)), true, err, st);
 }
 
-template <int RQ, bool PAIR = false>
+template <int RQ, bool DIG = true, bool PAIR = false>
 int launch_gram(const Persist64Args& a, dim3 grid, unsigned* err, cudaStream_t st) {
   static std::atomic<unsigned long long> configured{0ull};
-  return launch64(k_gram64<RQ, PAIR>, configured, a, grid, column_smem<RQ>(a.sb), false, err, st);
+  return launch64(k_gram64<RQ, DIG, PAIR>, configured, a, grid, column_smem<RQ>(a.sb), false, err, st);
 }
 
 // pairs of groups of 64 rows (one: all rows in one CTA)
@@ -638,20 +639,22 @@ int launch_gram64(const double* A, long long lda, long long N, long long K, cons
   a.part = part;
   a.ppart = ppart;
   a.sa.ldr = sbp;
+  if (sb <= kSmallSB) return launch_gram<4, false>(a, dim3(P), err, st);
   if (sb <= 32) return launch_gram<4>(a, dim3(P), err, st);
   if (sb <= 64) return launch_gram<8>(a, dim3(P), err, st);
   if (sb <= 128) return launch_gram<16>(a, dim3(P), err, st);
-  return launch_gram<16, true>(a, dim3(P, gram64_pairs(sb)), err, st);
+  return launch_gram<16, true, true>(a, dim3(P, gram64_pairs(sb)), err, st);
 }
 
 int launch_persist64(const Persist64Args& a, int P, size_t chain_smem, unsigned* err,
                      cudaStream_t st) {
-#define CA_P64(RQ)                                                       \
-  return a.sa.b <= 8 ? launch_steps<8, 4, RQ>(a, P, chain_smem, err, st) \
-                     : launch_steps<16, 3, RQ>(a, P, chain_smem, err, st);
-  if (a.sb <= 32) CA_P64(4)
-  if (a.sb <= 64) CA_P64(8)
-  if (a.sb <= 128) CA_P64(16)
+#define CA_P64(RQ, DIG)                                                       \
+  return a.sa.b <= 8 ? launch_steps<8, 4, RQ, DIG>(a, P, chain_smem, err, st) \
+                     : launch_steps<16, 3, RQ, DIG>(a, P, chain_smem, err, st);
+  if (a.sb <= kSmallSB) CA_P64(4, false)
+  if (a.sb <= 32) CA_P64(4, true)
+  if (a.sb <= 64) CA_P64(8, true)
+  if (a.sb <= 128) CA_P64(16, true)
 #undef CA_P64
   return (int)cudaErrorInvalidValue;
 }
