@@ -25,7 +25,7 @@
 // and FP64 projections at many.  Against four launches a step and a Gram tile
 // of 64 x 64 FP64 products whatever s b (ms a solve): X 64 x 1024, b = 4, 200
 // solves: s = 1 1.69 against 11.7 (8 us a step), s = 4 0.62 against 3.13 (12
-// us); X^T 1500 x 8190, b = 8, s = 4: 1.11 against 6.84 (17 us); 2003 x 24001,
+// us); X^T 1500 x 8190, b = 8, s = 4: 1.12 against 6.84 (17 us); 2003 x 24001,
 // b = 16, s = 8: 1.89 against 10.2 (70 us a step between recomputations).
 #include <algorithm>
 #include <atomic>
